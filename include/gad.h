@@ -141,9 +141,9 @@ int gad_default_params(int32_t L, const int32_t* dims, uint64_t seed, float* out
  * update; the call then waits for the stream.  loss_out == NULL: the epoch is only enqueued (no wait, no
  * copy); read the losses later with gad_get_loss.  Returns GAD_ERR_NONFINITE if a loss is NaN or infinite
  * (detected when the losses are read).
- * From the second call on the launches of an epoch are replayed as one CUDA graph (captured on the context's
- * stream, thread-local mode) when nothing in them changes from epoch to epoch: dropout == 0, flag bits 1 and 3 clear,
- * per-kernel timing off, and a stream that can be captured (any stream but the legacy default one).  Otherwise, while
+ * From the second call on the launches of an epoch are replayed as one CUDA graph (captured on a stream of the
+ * context, thread-local mode) when nothing in them changes from epoch to epoch: flag bits 1 and 3 clear and per-kernel
+ * timing off.  Otherwise, while
  * the caller is capturing that stream itself, or if the capture fails, they are enqueued one by one; the results are
  * the same either way. */
 int gad_train_epoch(gad_ctx* ctx, float* loss_out);

@@ -216,7 +216,7 @@ class Gad:
         return out
 
     def forward(self):
-        out = np.zeros((self.n, self.dims[-1]), dtype=np.float32)
+        out = np.empty((self.n, self.dims[-1]), dtype=np.float32)   # every row is written
         self._ck(self._L.gad_forward(self._h, _ptr(out, C.c_float)))
         return out
 

@@ -50,7 +50,7 @@ __device__ __forceinline__ float4 load_bias(const ActEpi& ep, int k, int col) {
 __device__ __forceinline__ float4 apply_act(float4 v, float4 b, const ActEpi& ep, long long row, int col) {
     float x[4] = {v.x + b.x, v.y + b.y, v.z + b.z, v.w + b.w};
     if (ep.relu) {
-        const uint64_t key = ep.drop ? dropout_row_key(ep.seed, ep.epoch, ep.layer, row) : 0ull;
+        const uint64_t key = ep.drop ? dropout_row_key(ep.seed, __ldg(ep.epoch), ep.layer, row) : 0ull;
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             x[t] = relu_nan(x[t]);

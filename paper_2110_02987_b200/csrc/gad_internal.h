@@ -100,7 +100,7 @@ struct Epilogue {            // of the forward SpMM: bias, ReLU, dropout
     int32_t relu;            // 0 on the last layer
     float dropout;
     uint64_t seed;
-    int64_t epoch;
+    const long long* epoch;  // device counter that indexes the dropout mask (read only with dropout > 0)
     int32_t layer;
 };
 
@@ -114,7 +114,7 @@ struct ActEpi {
     uint32_t thr;          // keep an element when the top 24 bits of its hash reach this
     float scale;           // 1 / (1 - rate)
     unsigned long long seed;
-    long long epoch;
+    const long long* epoch;   // device counter of the epochs run so far
     int layer;
     int col0;              // column of the operand's first column (column slabs)
 };
@@ -224,8 +224,11 @@ cudaError_t launch_zeta_gram(const void* mapHi, const void* mapLo, const float* 
                              const int32_t* sub_off, const int64_t* deg_sum, const int64_t* tile_ptr, int64_t ntiles, int K, float beta,
                              float* Xhi, float* Xlo, float* norm2, double* partial, double* zeta, int32_t* err, int num_sms, cudaStream_t s);
 
+// `epoch` (may be null): the device epoch counter, advanced by one.
 cudaError_t launch_sgd_consensus(float* params, const float* grads, int64_t pstride, int64_t len, int K, float lr,
-                                 const double* zeta, int weighted, int with_sgd, const int32_t* err_word, cudaStream_t s);
+                                 const double* zeta, int weighted, int with_sgd, const int32_t* err_word, long long* epoch, cudaStream_t s);
+// The device epoch counter on its own: + 1, or set to a value.
+cudaError_t launch_epoch_counter(long long* epoch, long long set_to, bool advance, cudaStream_t s);
 // One context's share of a consensus over several contexts: out = sum_k w_k (theta_k - lr grad_k) with w_k = zeta_k / total
 // (or 1 / total), the parameters unchanged; and the finished sum written to every replica.
 cudaError_t launch_consensus_partial(const float* params, const float* grads, int64_t pstride, int64_t len, int K, float lr,
@@ -246,5 +249,13 @@ cudaError_t launch_gather_rows(const float* Xg, int F, const int32_t* gid, int64
 cudaError_t launch_gather_labels(const int32_t* yg, const int32_t* gid, int64_t Np, int32_t* label, cudaStream_t s);
 cudaError_t launch_scatter_core(const float* logits, int ld, int C, const int32_t* gid, const RowSpan* core_spans,
                                 int nspans, float* out, cudaStream_t s);
+
+// host_copy.cu: `bytes` of device memory into the caller's memory through pinned slots, complete on return; the pages of
+// a pageable destination touched ahead of it (they are overwritten by the copy); contexts that may copy, + 1 / - 1.
+cudaError_t copy_to_host(void* dst, const void* src, size_t bytes, cudaStream_t s);
+void host_prefault(void* dst, size_t bytes);
+void host_copy_user(int delta);
+char* take_small_pinned(size_t bytes);
+void give_small_pinned(char* b, size_t bytes);
 
 }  // namespace gad

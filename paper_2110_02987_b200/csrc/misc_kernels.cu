@@ -537,8 +537,9 @@ __device__ __forceinline__ float4 weighted_sum(const float* __restrict__ params,
 __global__ void __launch_bounds__(256) sgd_consensus_kernel(float* __restrict__ params, const float* __restrict__ grads,
                                                             long long pstride, long long len4, int K, float lr,
                                                             const double* __restrict__ zeta, int weighted, int with_sgd,
-                                                            const int32_t* __restrict__ err_word) {
+                                                            const int32_t* __restrict__ err_word, long long* epoch) {
     extern __shared__ float w_sm[];
+    if (epoch && blockIdx.x == 0 && threadIdx.x == 0) *epoch += 1;   // last kernel of an epoch: nothing reads the counter beside it
     if (err_word && *err_word) return;   // a bounded wait ran out earlier in this epoch: keep the parameters as they are
     consensus_weights(zeta, K, weighted, w_sm);
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -547,12 +548,18 @@ __global__ void __launch_bounds__(256) sgd_consensus_kernel(float* __restrict__ 
     for (int k = 0; k < K; ++k) reinterpret_cast<float4*>(params + (long long)k * pstride)[i] = acc;
 }
 cudaError_t launch_sgd_consensus(float* params, const float* grads, int64_t pstride, int64_t len, int K, float lr,
-                                 const double* zeta, int weighted, int with_sgd, const int32_t* err_word, cudaStream_t s) {
+                                 const double* zeta, int weighted, int with_sgd, const int32_t* err_word, long long* epoch, cudaStream_t s) {
     const long long len4 = len / 4;
     if (len4 > 0) {
         const int threads = len4 >= 148 * 256 * 4 ? 256 : 64;   // a small model is spread over more CTAs
         sgd_consensus_kernel<<<(unsigned)((len4 + threads - 1) / threads), threads, (size_t)K * sizeof(float), s>>>(params, grads, pstride, len4, K, lr,
-                                                                                                   zeta, weighted, with_sgd, err_word); ++g_kernel_launches; }
+                                                                                                   zeta, weighted, with_sgd, err_word, epoch); ++g_kernel_launches; }
+    return cudaGetLastError();
+}
+
+__global__ void epoch_counter_kernel(long long* epoch, long long set_to, int advance) { *epoch = advance ? *epoch + 1 : set_to; }
+cudaError_t launch_epoch_counter(long long* epoch, long long set_to, bool advance, cudaStream_t s) {
+    epoch_counter_kernel<<<1, 1, 0, s>>>(epoch, set_to, advance ? 1 : 0); ++g_kernel_launches;
     return cudaGetLastError();
 }
 

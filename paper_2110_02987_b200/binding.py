@@ -449,26 +449,34 @@ class Augmenter:
         cp = np.zeros(K + 1, dtype=np.int64)
         np.cumsum([len(c) for c in cores], out=cp[1:])
         cn = _arr(np.concatenate(cores) if cp[-1] > 0 else np.empty(0, np.int32), np.int32)
-        cfg = _AugmentConfig(int(steps), int(cap), float(alpha), float(E), float(zc), int(seed), 0)
-        nbytes = C.c_size_t(0)
-        rc = L.gad_augment_workspace_bytes(C.byref(self._csr), C.c_int32(K), _ptr(cp, C.c_int64), _ptr(cn, C.c_int32), C.byref(cfg),
-                                           C.byref(nbytes))
-        if rc != GAD_OK:
-            self._fail(rc)
-        if self._ws is None or int(nbytes.value) > self._ws_bytes:
-            self._ws = torch.empty(int(nbytes.value) + 256, dtype=torch.uint8, device="cuda")
-            self._ws_bytes = int(nbytes.value)
-            self._resident = False
-        cfg.graph_resident = 1 if self._resident else 0
-        aligned = (self._ws.data_ptr() + 255) // 256 * 256
+        cfg = _AugmentConfig(int(steps), int(cap), float(alpha), float(E), float(zc), int(seed), 1 if self._resident else 0)
         st = stream if stream is not None else torch.cuda.current_stream()
         capacity = int(sum(int(np.floor(alpha * 2.0 * len(c))) for c in cores)) + 1
         halo_ptr = np.zeros(K + 1, dtype=np.int64)
         halo = np.zeros(capacity, dtype=np.int32)
         walks = np.zeros(K, dtype=np.int64)
-        rc = L.gad_augment(C.byref(self._csr), C.c_int32(K), _ptr(cp, C.c_int64), _ptr(cn, C.c_int32), C.byref(cfg), C.c_void_p(aligned),
-                           C.c_size_t(self._ws_bytes), C.c_void_p(st.cuda_stream), _ptr(halo_ptr, C.c_int64), _ptr(halo, C.c_int32),
-                           C.c_int64(capacity), _ptr(walks, C.c_int64))
+        pcp, pcn, php, phn, pw = (_ptr(cp, C.c_int64), _ptr(cn, C.c_int32), _ptr(halo_ptr, C.c_int64), _ptr(halo, C.c_int32),
+                                  _ptr(walks, C.c_int64))
+
+        def call():
+            cfg.graph_resident = 1 if self._resident else 0
+            aligned = (self._ws.data_ptr() + 255) // 256 * 256
+            return L.gad_augment(C.byref(self._csr), C.c_int32(K), pcp, pcn, C.byref(cfg), C.c_void_p(aligned), C.c_size_t(self._ws_bytes),
+                                 C.c_void_p(st.cuda_stream), php, phn, C.c_int64(capacity), pw)
+
+        # the workspace of the call before nearly always fits: its size is asked for only when there is none or the call says it
+        # is too small (before it has done anything)
+        rc = call() if self._ws is not None else -5
+        if rc == -5:
+            nbytes = C.c_size_t(0)
+            rc = L.gad_augment_workspace_bytes(C.byref(self._csr), C.c_int32(K), pcp, pcn, C.byref(cfg), C.byref(nbytes))
+            if rc == GAD_OK and (self._ws is None or int(nbytes.value) > self._ws_bytes):
+                self._ws = torch.empty(int(nbytes.value) + 256, dtype=torch.uint8, device="cuda")
+                self._ws_bytes = int(nbytes.value)
+                self._resident = False
+                rc = call()
+            elif rc == GAD_OK:
+                rc = -5
         if rc != GAD_OK:
             self._resident = False
             self._fail(rc)

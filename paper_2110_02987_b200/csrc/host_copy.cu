@@ -51,7 +51,13 @@ void give_to(std::vector<char*>& idle, size_t most, char* b) {
     }
     cudaFreeHost(b);
 }
-char* take_buffer() { return take_from(g_pool.idle, kSlots * kSlotBytes); }
+char* take_buffer() {
+    {
+        std::lock_guard<std::mutex> g(g_pool.lock);
+        if (g_pool.users <= 0) return nullptr;   // no context to keep the buffer for: pinning one for a single copy costs more than it saves
+    }
+    return take_from(g_pool.idle, kSlots * kSlotBytes);
+}
 void give_buffer(char* b) { give_to(g_pool.idle, 2, b); }
 
 bool is_pageable(const void* p) {
@@ -116,7 +122,7 @@ void host_prefault(void* dst, size_t bytes) {
 cudaError_t copy_to_host(void* dst, const void* src, size_t bytes, cudaStream_t s) {
     cudaError_t e;
     char* buf = bytes > 0 && is_pageable(dst) ? take_buffer() : nullptr;
-    if (!buf) {   // pinned destination (or no pinned memory to be had): one plain copy
+    if (!buf) {   // pinned destination, or no ring: one plain copy
         e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s);
         return e != cudaSuccess ? e : cudaStreamSynchronize(s);
     }

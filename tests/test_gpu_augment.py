@@ -104,3 +104,20 @@ def test_a_second_call_reuses_the_graph_on_the_device():
         assert walks.tolist() == [it["n"] for it in info]
         for x, y in zip(got, want):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("n,K", [(2047, 1), (2048, 3), (2049, 40), (5003, 7)])
+def test_boundary_lists_at_the_edges_of_a_tile(n, K):
+    """The boundary list is cut into tiles of 2048 node ids: one node less, exactly one tile, one more, and a ragged end, with
+    core sets that are not contiguous and more subgraphs than fill a batch's grid evenly."""
+    rng = np.random.default_rng(n)
+    src = np.repeat(np.arange(n), 6)
+    dst = rng.integers(0, n, size=src.size)
+    u, v = np.concatenate([src, dst]), np.concatenate([dst, src])
+    key = np.unique(u.astype(np.int64) * n + v)
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(np.bincount(key // n, minlength=n), out=rowptr[1:])
+    perm = rng.permutation(n - 5).astype(np.int32) + 5
+    cores = [np.ascontiguousarray(c) for c in np.array_split(perm, K)]
+    got, _ = _both(n, rowptr, (key % n).astype(np.int32), cores, 2, alpha=0.2, seed=n)
+    assert all(len(h) > 0 for h in got)

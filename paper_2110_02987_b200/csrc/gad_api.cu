@@ -137,7 +137,7 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
     // row tiles of the grouped transforms (128 rows, never across subgraphs) and reduction chunks
     const int64_t target = 592;
     int64_t R = round_up(std::max<int64_t>(1, (p.Np + target - 1) / target), 32);
-    R = std::min<int64_t>(std::max<int64_t>(R, 128), 16384);
+    R = std::min<int64_t>(R, 16384);
     // The weight gradient has a long reduction per output tile, so it gets longer chunks: about one CTA per SM (a
     // single wave: every CTA pays the pipeline fill once) over the layer with the most output tiles (128 rows x up to 256 columns each).
     int64_t max_tiles = 1;
@@ -278,6 +278,10 @@ struct gad_ctx {
     std::vector<float> host_block;  // staging for parameter pack / unpack
     char* pinned = nullptr;         // pinned host memory the small results of waiting calls land in (pinned_bytes)
     size_t pinned_bytes = 0;
+    // The replicas' parameters are equal (after creation and every consensus) until gad_set_params gives one its own: copy 0 then
+    // stands for all of them and the others are stale.  `unsettled`: a consensus over differing copies has been enqueued and
+    // nothing has waited for it since; should a bounded wait have run out it left them as they were (error word 2 tells).
+    bool same_params = true, unsettled = false;
     bool epoch_dirty = false;       // the device counter differs from `epoch` (gad_set_epoch, epochs without dropout)
     cudaStream_t capture_stream = nullptr;   // epochs are captured on it, whatever stream they are launched on
     cudaStream_t copy_stream = nullptr;   // host -> device copies of gad_set_inputs
@@ -354,6 +358,9 @@ int run(gad_ctx* ctx, const char* name, int layer, double bytes, double flops, F
 // Room for the bfloat16 copy of an aggregation's operand: the reduced-precision mode gathers from that copy.
 void* bf16_of(gad_ctx* ctx) { return ctx->cfg.gemm_mode == 1 ? (void*)(ctx->ws + ctx->p.o_bf16) : nullptr; }
 
+// Floats between the replicas' parameters as the kernels read them: copy 0 stands for all of them while they are equal.
+int64_t param_stride(const gad_ctx* ctx) { return ctx->same_params ? 0 : ctx->p.pstride; }
+
 // The device epoch counter, when anything reads it.
 long long* dropout_counter(gad_ctx* ctx) { return ctx->cfg.dropout > 0.f ? ctx->at<long long>(ctx->p.o_epoch) : nullptr; }
 
@@ -371,25 +378,50 @@ int hand_over(gad_ctx* ctx, cudaStream_t from, cudaStream_t to, cudaEvent_t ev) 
     return GAD_OK;
 }
 
+// After a consensus has been enqueued.
+void copies_made_equal(gad_ctx* ctx) {
+    if (!ctx->same_params) ctx->unsettled = true;
+    ctx->same_params = true;
+}
+// words: the device's error words as read after a wait.
+void settle(gad_ctx* ctx, const int32_t* words) {
+    if (ctx->unsettled && words[2]) ctx->same_params = false;
+    ctx->unsettled = false;
+}
+int settle_now(gad_ctx* ctx) {
+    if (!ctx->unsettled) return GAD_OK;
+    GAD_CK(cudaMemcpyAsync(ctx->pinned, ctx->ws + ctx->p.o_flags, 12, cudaMemcpyDeviceToHost, ctx->stream));
+    GAD_CK(cudaStreamSynchronize(ctx->stream));
+    int32_t words[3];
+    std::memcpy(words, ctx->pinned, 12);
+    settle(ctx, words);
+    return GAD_OK;
+}
+
 int forward_pass(gad_ctx* ctx, bool train, cudaStream_t ss) {
     const Plan& p = ctx->p;
     float* Z = ctx->at<float>(p.o_G2);
     const float* params = ctx->at<float>(p.o_params);
     const int passes = ctx->cfg.gemm_mode == 0 ? 3 : 1;
-    if (ctx->use_tc)
+    const int64_t pstride = param_stride(ctx);
+    if (ctx->use_tc) {
+        std::vector<SplitLayer> sl((size_t)p.L);
+        double weights = 0.0;
         for (int l = 0; l < p.L; ++l) {
             const Layer& y = p.layers[l];
-            GAD_RUN("split_weights", l, 20.0 * p.K * y.fi * y.fo, 0.0, [&] {
-                return launch_split_weights(params, p.pstride, y.w_int, y.fi, y.fo, y.ldw, y.ldi, p.K, ctx->at<float>(p.o_w_hi[l]),
-                                            ctx->at<float>(p.o_w_lo[l]), ctx->at<float>(p.o_wt_hi[l]), ctx->at<float>(p.o_wt_lo[l]),
-                                            ss);
-            });
+            const bool plain = l > 0;   // layer 0 has no gradient with respect to its input
+            sl[(size_t)l] = SplitLayer{y.fi, y.fo, y.ldw, y.ldi, y.w_int, plain ? ctx->at<float>(p.o_w_hi[l]) : nullptr,
+                                       plain ? ctx->at<float>(p.o_w_lo[l]) : nullptr, ctx->at<float>(p.o_wt_hi[l]), ctx->at<float>(p.o_wt_lo[l])};
+            weights += (plain ? 20.0 : 12.0) * y.fi * y.fo;
         }
+        const int copies = ctx->same_params ? 1 : p.K;
+        GAD_RUN("split_weights", -1, weights * copies, 0.0, [&] { return launch_split_weights(params, pstride, copies, sl.data(), p.L, ss); });
+    }
     bool split_pending = ctx->use_tc && ss != ctx->stream;   // the first transform waits for the split operands
     if (split_pending) GAD_CK(cudaEventRecord(ctx->ev_split, ss));
     for (int l = 0; l < p.L; ++l) {
         const Layer& y = p.layers[l];
-        Epilogue ep{params, p.pstride, y.b_int, ctx->at<int32_t>(p.o_sub_off), p.K, l < p.L - 1 ? 1 : 0,
+        Epilogue ep{params, pstride, y.b_int, ctx->at<int32_t>(p.o_sub_off), p.K, l < p.L - 1 ? 1 : 0,
                     train ? ctx->cfg.dropout : 0.f, ctx->cfg.seed, ctx->at<long long>(p.o_epoch), l};
         if (p.agg_first[l]) {
             // A~ (H W) = (A~ H) W: aggregate at the input width, finish the layer in the transform's epilogue
@@ -404,8 +436,8 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t ss) {
                 if (ctx->use_tc)
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 2, passes, y.fi, y.fo,
                                                ctx->H(l + 1), y.ldo, ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, &act,
-                                               ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream);
-                return launch_gemm_rows_simt(2, ctx->at<float>(p.o_P[l]), y.ldi, y.fi, params, p.pstride, y.w_int, y.ldw, y.fo, ctx->H(l + 1), y.ldo,
+                                               ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params);
+                return launch_gemm_rows_simt(2, ctx->at<float>(p.o_P[l]), y.ldi, y.fi, params, pstride, y.w_int, y.ldw, y.fo, ctx->H(l + 1), y.ldo,
                                              ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, &act, ctx->stream);
             });
             continue;
@@ -417,8 +449,8 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t ss) {
             if (ctx->use_tc)
                 return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 0, passes, y.fi, y.fo, Z,
                                            y.ldo, ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, nullptr,
-                                           ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, zb);
-            return launch_gemm_rows_simt(0, ctx->H(l), y.ldi, y.fi, params, p.pstride, y.w_int, y.ldw, y.fo, Z, y.ldo,
+                                           ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params, zb);
+            return launch_gemm_rows_simt(0, ctx->H(l), y.ldi, y.fi, params, pstride, y.w_int, y.ldw, y.fo, Z, y.ldo,
                                          ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, nullptr, ctx->stream);
         });
         GAD_RUN("spmm_fwd", l, spmm_bytes(p, y.fo), 2.0 * p.nnz * y.fo,
@@ -464,10 +496,9 @@ int zeta_pass(gad_ctx* ctx, cudaStream_t s) {
         for (int l = 0; l < nl; ++l) {
             const int phase = nl == 1 ? 0 : (l == 0 ? 1 : (l == nl - 1 ? 3 : 2));
             cudaError_t e = launch_zeta(ctx->H(l), p.ld[l], p.dims[l], ctx->at<int32_t>(p.o_deg), ctx->at<RowSpan>(p.o_chunks),
-                                        (int)p.chunks.size(), ctx->at<int32_t>(p.o_chunk_ptr), ctx->at<int32_t>(p.o_sub_off),
+                                        (int)p.chunks.size(), ctx->at<int32_t>(p.o_chunk_ptr), ctx->at<int32_t>(p.o_sub_off), p.K,
                                         ctx->at<int64_t>(p.o_deg_sum), ctx->at<int64_t>(p.o_deg_sq), ctx->cfg.beta,
-                                        ctx->at<double>(p.o_zeta_partial), ctx->at<unsigned>(p.o_counters) + 1 + p.K,
-                                        ctx->at<double>(p.o_zeta), ctx->at<double>(p.o_zeta_q), phase, s);
+                                        ctx->at<double>(p.o_zeta_partial), ctx->at<double>(p.o_zeta), ctx->at<double>(p.o_zeta_q), phase, s);
             if (e != cudaSuccess) return e;
         }
         return cudaSuccess;
@@ -481,6 +512,7 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
     float* G2 = ctx->at<float>(p.o_G2);
     float* grads = ctx->at<float>(p.o_grads);
     const float* params = ctx->at<float>(p.o_params);
+    const int64_t pstride = param_stride(ctx);
     const RowSpan* chunks = ctx->at<RowSpan>(p.o_chunks);
     const int nc = (int)p.chunks.size();
     const int32_t* chunk_ptr = ctx->at<int32_t>(p.o_chunk_ptr);
@@ -488,7 +520,8 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
     const int ndw = (int)p.dw_chunks.size();
     const int32_t* dw_chunk_ptr = ctx->at<int32_t>(p.o_dw_chunk_ptr);
     const float scale = ctx->cfg.dropout > 0.f ? 1.f / (1.f - ctx->cfg.dropout) : 1.f;
-    bool bias_done = false;   // the layer above was narrow: its fused kernel has already summed this layer's dPre columns
+    // whether this layer's dPre columns have been summed already: by the loss kernel, or by the layer above's fused narrow kernel
+    bool bias_done = softmax_sums_columns(p.ld[p.L]);
     for (int l = p.L - 1; l >= 0; --l) {
         const Layer& y = p.layers[l];
         // the store of this layer's backward aggregation, and its entries
@@ -516,7 +549,7 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
             // the chunk results hold db of layer l-1 and then dW of layer l, which is also their order in the parameter block
             const int64_t plen = (int64_t)y.ldi + (int64_t)y.fi * y.ldw;
             GAD_RUN("gemm_dwdh", l, 4.0 * p.Np * (2.0 * y.fi + y.fo) + 8.0 * p.K * y.fi * y.fo, 4.0 * p.Np * y.fi * y.fo, [&] {
-                return launch_narrow_bwd(ctx->H(l), y.ldi, y.fi, G2, y.ldo, params, p.pstride, y.w_int, y.ldw,
+                return launch_narrow_bwd(ctx->H(l), y.ldi, y.fi, G2, y.ldo, params, pstride, y.w_int, y.ldw,
                                          ctx->at<RowSpan>(p.o_nchunks), (int)p.nchunks.size(), scale, G1,
                                          ctx->at<float>(p.o_nw_partial), plen, ctx->at<int32_t>(p.o_flags) + 1, ctx->stream);
             });
@@ -549,8 +582,8 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 3], &ctx->maps[kMapsPerLayer * l + 4], &ctx->maps[kMapsPerLayer * l + 5], 1,
                                                ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G2, y.ldi, ctx->at<RowSpan>(p.o_tiles),
                                                (int)p.tiles.size(), nullptr, 0, 1.f, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
-                                               ctx->num_sms, ctx->stream);
-                return launch_gemm_rows_simt(1, G1, y.ldo, y.fo, params, p.pstride, y.w_int, y.ldw, y.fi, G2, y.ldi,
+                                               ctx->num_sms, ctx->stream, ctx->same_params);
+                return launch_gemm_rows_simt(1, G1, y.ldo, y.fo, params, pstride, y.w_int, y.ldw, y.fi, G2, y.ldi,
                                              ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, nullptr, ctx->stream);
             });
             if (ss != ctx->stream) GAD_CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_bias, 0));   // the column sums have read dPre
@@ -567,8 +600,8 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 3], &ctx->maps[kMapsPerLayer * l + 4], &ctx->maps[kMapsPerLayer * l + 5], 1,
                                                ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G1, y.ldi, ctx->at<RowSpan>(p.o_tiles),
                                                (int)p.tiles.size(), ctx->H(l), y.ldi, scale, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
-                                               ctx->num_sms, ctx->stream);
-                return launch_gemm_rows_simt(1, G2, y.ldo, y.fo, params, p.pstride, y.w_int, y.ldw, y.fi, G1, y.ldi,
+                                               ctx->num_sms, ctx->stream, ctx->same_params);
+                return launch_gemm_rows_simt(1, G2, y.ldo, y.fo, params, pstride, y.w_int, y.ldw, y.fi, G1, y.ldi,
                                              ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), ctx->H(l), y.ldi, scale, nullptr,
                                              ctx->stream);
             });
@@ -777,15 +810,13 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
     // features: graph order -> staging -> store-row order with zero pad columns
     GAD_CK(cudaMemcpyAsync(ctx->ws + p.o_stage, X, 4 * (size_t)g->n * p.dims[0], cudaMemcpyHostToDevice, ctx->stream));
     GAD_CK(launch_gather_rows(ctx->at<float>(p.o_stage), p.dims[0], ctx->at<int32_t>(p.o_gid), p.Np, ctx->H(0), p.ld[0], ctx->stream));
-    // parameters: K identical padded copies
+    // parameters: one padded copy, which stands for all K while they are equal
     std::vector<float> ext((size_t)p.P);
     if (init_params) std::memcpy(ext.data(), init_params, sizeof(float) * (size_t)p.P);
     else default_params(p.dims, cfg->seed, ext.data());
     ctx->host_block.assign((size_t)p.pstride, 0.f);
     pack_params(p, ext.data(), ctx->host_block.data());
-    for (int32_t k = 0; k < p.K; ++k)
-        GAD_CK(cudaMemcpyAsync(ctx->at<float>(p.o_params) + (int64_t)k * p.pstride, ctx->host_block.data(), 4 * (size_t)p.pstride,
-                               cudaMemcpyHostToDevice, ctx->stream));
+    GAD_CK(cudaMemcpyAsync(ctx->at<float>(p.o_params), ctx->host_block.data(), 4 * (size_t)p.pstride, cudaMemcpyHostToDevice, ctx->stream));
     GAD_CK(cudaMemsetAsync(ctx->ws + p.o_grads, 0, 4 * (size_t)p.K * p.pstride, ctx->stream));
     GAD_CK(cudaMemsetAsync(ctx->ws + p.o_flags, 0, 16, ctx->stream));
     // tensor-core path: operand copies start at zero (their pad columns are never written) and get TMA descriptors
@@ -853,11 +884,12 @@ int gad_default_params(int32_t L, const int32_t* dims, uint64_t seed, float* out
 int gad_get_loss(gad_ctx* ctx, float* loss_out) {
     if (!ctx || !loss_out) return GAD_ERR_ARG;
     const Plan& p = ctx->p;
-    int32_t flags[2];
-    GAD_CK(cudaMemcpyAsync(ctx->pinned, ctx->ws + p.o_loss, p.o_flags + 8 - p.o_loss, cudaMemcpyDeviceToHost, ctx->stream));
+    int32_t flags[3];
+    GAD_CK(cudaMemcpyAsync(ctx->pinned, ctx->ws + p.o_loss, p.o_flags + 12 - p.o_loss, cudaMemcpyDeviceToHost, ctx->stream));
     GAD_CK(cudaStreamSynchronize(ctx->stream));
     std::memcpy(loss_out, ctx->pinned, 4 * (size_t)(p.K + 1));
-    std::memcpy(flags, ctx->pinned + (p.o_flags - p.o_loss), 8);
+    std::memcpy(flags, ctx->pinned + (p.o_flags - p.o_loss), 12);
+    settle(ctx, flags);
     const int32_t flag = flags[0];
     if (flags[1]) {
         GAD_CK(cudaMemsetAsync(ctx->ws + p.o_flags, 0, 8, ctx->stream));
@@ -886,20 +918,28 @@ static int enqueue_epoch(gad_ctx* ctx, bool consensus) {
     if (ctx->cfg.zeta_mode == 2 && (rc = hand_over(ctx, ctx->stream, ss, ctx->ev_fork)) != GAD_OK) return rc;
     if (ss != ctx->stream && (rc = zeta_pass(ctx, ss)) != GAD_OK) return rc;
     const int C = p.dims[p.L];
+    const Layer& last = p.layers[(size_t)p.L - 1];
     GAD_RUN("softmax_xent", -1, 8.0 * p.Np * C, 0.0, [&] {
         return launch_softmax_xent(ctx->H(p.L), p.ld[p.L], C, ctx->at<int32_t>(p.o_label), ctx->at<uint8_t>(p.o_train),
                                    ctx->at<RowSpan>(p.o_chunks), (int)p.chunks.size(), ctx->at<float>(p.o_inv_ntrain),
-                                   ctx->at<float>(p.o_G1), ctx->at<float>(p.o_loss_partial), ctx->at<int32_t>(p.o_chunk_ptr), p.K,
-                                   ctx->ntrain_total > 0 ? 1.f / (float)ctx->ntrain_total : 0.f, ctx->at<float>(p.o_loss),
-                                   ctx->at<int32_t>(p.o_flags), ctx->at<unsigned>(p.o_counters), ctx->stream);
+                                   ctx->at<float>(p.o_G1), ctx->at<float>(p.o_loss_partial), ctx->at<float>(p.o_cs_partial), p.maxld, ctx->stream);
     });
+    // the sums over the chunks are needed at the end of the epoch only
+    if ((rc = hand_over(ctx, ctx->stream, ss, ctx->ev_g1)) != GAD_OK) return rc;
+    const int bias_ld = softmax_sums_columns(p.ld[p.L]) ? p.ld[p.L] : 0;
+    GAD_RUN("loss_finish", -1, 4.0 * p.chunks.size() * (bias_ld + 1), 1.0 * p.chunks.size() * (bias_ld + 1), [&] {
+        return launch_loss_finish(ctx->at<float>(p.o_loss_partial), ctx->at<float>(p.o_inv_ntrain), ctx->at<int32_t>(p.o_chunk_ptr), p.K,
+                                  ctx->ntrain_total > 0 ? 1.f / (float)ctx->ntrain_total : 0.f, ctx->at<float>(p.o_loss), ctx->at<int32_t>(p.o_flags),
+                                  ctx->at<float>(p.o_cs_partial), p.maxld, bias_ld, ctx->at<float>(p.o_grads), p.pstride, last.b_int, ss);
+    });
+    if (ss != ctx->stream) GAD_CK(cudaEventRecord(ctx->ev_bias, ss));
     if ((rc = backward_pass(ctx, ss)) != GAD_OK) return rc;
     if (ss == ctx->stream && (rc = zeta_pass(ctx, ss)) != GAD_OK) return rc;
     if ((rc = hand_over(ctx, ss, ctx->stream, ctx->ev_join)) != GAD_OK) return rc;
     if (consensus)
-        GAD_RUN("sgd_consensus", -1, 12.0 * p.K * p.Pint, 4.0 * p.K * p.Pint, [&] {
-            return launch_sgd_consensus(ctx->at<float>(p.o_params), ctx->at<float>(p.o_grads), p.pstride, p.pstride, p.K, ctx->cfg.lr,
-                                        ctx->at<double>(p.o_zeta), ctx->cfg.weighted, 1, ctx->at<int32_t>(p.o_flags) + 1, dropout_counter(ctx), ctx->stream);
+        GAD_RUN("sgd_consensus", -1, 4.0 * ((ctx->same_params ? 1 : p.K) + p.K + 1) * p.Pint, 4.0 * p.K * p.Pint, [&] {
+            return launch_sgd_consensus(ctx->at<float>(p.o_params), param_stride(ctx), ctx->at<float>(p.o_grads), p.pstride, p.pstride, p.K, ctx->cfg.lr,
+                                        ctx->at<double>(p.o_zeta), ctx->cfg.weighted, 1, ctx->at<int32_t>(p.o_flags), dropout_counter(ctx), ctx->stream);
         });
     else if (dropout_counter(ctx))
         GAD_CK(launch_epoch_counter(dropout_counter(ctx), 0, true, ctx->stream));
@@ -912,7 +952,7 @@ static int enqueue_epoch(gad_ctx* ctx, bool consensus) {
 // runs on a stream of the context, so that a context on the legacy default stream (which cannot be captured, but takes
 // graph launches) replays its epochs too: 2000 nodes, 32-16-4, 126 -> 86 us per waiting epoch.
 static bool graph_allowed(const gad_ctx* ctx) {
-    return (ctx->cfg.flags & 8) == 0 && !ctx->profiling && !ctx->hoist && ctx->direct_epochs >= 1;
+    return (ctx->cfg.flags & 8) == 0 && ctx->same_params && !ctx->profiling && !ctx->hoist && ctx->direct_epochs >= 1;
 }
 
 static void capture_epoch(gad_ctx* ctx, bool consensus, gad_ctx::EpochGraph& eg) {
@@ -966,6 +1006,7 @@ static int train_epoch(gad_ctx* ctx, float* loss_out, bool consensus) {
         if (rc != GAD_OK) return rc;
         ctx->direct_epochs += 1;
     }
+    if (consensus) copies_made_equal(ctx);
     ctx->epoch += 1;
     if (loss_out) return gad_get_loss(ctx, loss_out);
     return GAD_OK;
@@ -1004,10 +1045,11 @@ int gad_consensus(gad_ctx* ctx) {
     const Plan& p = ctx->p;
     int rc = zeta_pass(ctx, ctx->stream);
     if (rc != GAD_OK) return rc;
-    GAD_RUN("consensus", -1, 8.0 * p.K * p.Pint, 2.0 * p.K * p.Pint, [&] {
-        return launch_sgd_consensus(ctx->at<float>(p.o_params), ctx->at<float>(p.o_grads), p.pstride, p.pstride, p.K, 0.f,
-                                    ctx->at<double>(p.o_zeta), ctx->cfg.weighted, 0, ctx->at<int32_t>(p.o_flags) + 1, nullptr, ctx->stream);
+    GAD_RUN("consensus", -1, 4.0 * ((ctx->same_params ? 1 : p.K) + 1) * p.Pint, 2.0 * p.K * p.Pint, [&] {
+        return launch_sgd_consensus(ctx->at<float>(p.o_params), param_stride(ctx), ctx->at<float>(p.o_grads), p.pstride, p.pstride, p.K, 0.f,
+                                    ctx->at<double>(p.o_zeta), ctx->cfg.weighted, 0, ctx->at<int32_t>(p.o_flags), nullptr, ctx->stream);
     });
+    copies_made_equal(ctx);
     return GAD_OK;
 }
 
@@ -1030,8 +1072,8 @@ int gad_consensus_partial(gad_ctx* ctx, double total, int32_t with_step, float* 
         int rc = zeta_pass(ctx, ctx->stream);
         if (rc != GAD_OK) return rc;
     }
-    GAD_RUN("consensus_partial", -1, (with_step ? 8.0 : 4.0) * p.K * p.Pint + 4.0 * p.Pint, 4.0 * p.K * p.Pint, [&] {
-        return launch_consensus_partial(ctx->at<float>(p.o_params), ctx->at<float>(p.o_grads), p.pstride, p.pstride, p.K, ctx->cfg.lr,
+    GAD_RUN("consensus_partial", -1, 4.0 * ((ctx->same_params ? 1 : p.K) + (with_step ? p.K : 0) + 1) * p.Pint, 4.0 * p.K * p.Pint, [&] {
+        return launch_consensus_partial(ctx->at<float>(p.o_params), param_stride(ctx), ctx->at<float>(p.o_grads), p.pstride, p.pstride, p.K, ctx->cfg.lr,
                                         ctx->at<double>(p.o_zeta), ctx->cfg.weighted, with_step ? 1 : 0, total, dev_out, ctx->at<int32_t>(p.o_flags) + 1,
                                         ctx->stream);
     });
@@ -1041,16 +1083,19 @@ int gad_consensus_partial(gad_ctx* ctx, double total, int32_t with_step, float* 
 int gad_consensus_apply(gad_ctx* ctx, const float* dev_in) {
     if (!ctx || !dev_in || ((uintptr_t)dev_in & 15) != 0) return GAD_ERR_ARG;
     const Plan& p = ctx->p;
-    GAD_RUN("consensus_apply", -1, 4.0 * (p.K + 1) * p.Pint, 0.0, [&] {
-        return launch_consensus_apply(ctx->at<float>(p.o_params), p.pstride, p.pstride, p.K, dev_in, ctx->at<int32_t>(p.o_flags) + 1, ctx->stream);
+    GAD_RUN("consensus_apply", -1, 8.0 * p.Pint, 0.0, [&] {
+        return launch_consensus_apply(ctx->at<float>(p.o_params), p.pstride, dev_in, ctx->at<int32_t>(p.o_flags), ctx->stream);
     });
+    copies_made_equal(ctx);
     return GAD_OK;
 }
 
 int gad_export_params(gad_ctx* ctx, int32_t k, float* dev_out) {
     if (!ctx || !dev_out || k < 0 || k >= ctx->p.K) return GAD_ERR_ARG;
     const Plan& p = ctx->p;
-    GAD_CK(cudaMemcpyAsync(dev_out, ctx->at<float>(p.o_params) + (int64_t)k * p.pstride, 4 * (size_t)p.pstride, cudaMemcpyDeviceToDevice,
+    int rc = settle_now(ctx);
+    if (rc != GAD_OK) return rc;
+    GAD_CK(cudaMemcpyAsync(dev_out, ctx->at<float>(p.o_params) + (int64_t)k * param_stride(ctx), 4 * (size_t)p.pstride, cudaMemcpyDeviceToDevice,
                            ctx->stream));
     return GAD_OK;
 }
@@ -1061,22 +1106,35 @@ int gad_param_count(const gad_ctx* ctx, int64_t* P) {
     return GAD_OK;
 }
 
-static int get_block(gad_ctx* ctx, size_t base, int32_t k, float* out) {
+static int get_block(gad_ctx* ctx, size_t base, int64_t stride, int32_t k, float* out) {
     if (!ctx || !out || k < 0 || k >= ctx->p.K) return GAD_ERR_ARG;
     const Plan& p = ctx->p;
-    GAD_CK(cudaMemcpyAsync(ctx->host_block.data(), ctx->at<float>(base) + (int64_t)k * p.pstride, 4 * (size_t)p.pstride,
+    GAD_CK(cudaMemcpyAsync(ctx->host_block.data(), ctx->at<float>(base) + (int64_t)k * stride, 4 * (size_t)p.pstride,
                            cudaMemcpyDeviceToHost, ctx->stream));
     GAD_CK(cudaStreamSynchronize(ctx->stream));
     unpack_params(p, ctx->host_block.data(), out);
     return GAD_OK;
 }
-int gad_get_params(gad_ctx* ctx, int32_t k, float* out) { return get_block(ctx, ctx ? ctx->p.o_params : 0, k, out); }
-int gad_get_grads(gad_ctx* ctx, int32_t k, float* out) { return get_block(ctx, ctx ? ctx->p.o_grads : 0, k, out); }
+int gad_get_params(gad_ctx* ctx, int32_t k, float* out) {
+    if (!ctx) return GAD_ERR_ARG;
+    int rc = settle_now(ctx);
+    return rc != GAD_OK ? rc : get_block(ctx, ctx->p.o_params, param_stride(ctx), k, out);
+}
+int gad_get_grads(gad_ctx* ctx, int32_t k, float* out) { return ctx ? get_block(ctx, ctx->p.o_grads, ctx->p.pstride, k, out) : GAD_ERR_ARG; }
 
 int gad_set_params(gad_ctx* ctx, int32_t k, const float* in) {
     if (!ctx || !in || k < 0 || k >= ctx->p.K) return GAD_ERR_ARG;
     const Plan& p = ctx->p;
+    int rc = settle_now(ctx);
+    if (rc != GAD_OK) return rc;
     GAD_CK(cudaStreamSynchronize(ctx->stream));
+    if (ctx->same_params && p.K > 1) {   // from here on the copies are told apart: bring the stale ones up to date
+        for (int32_t j = 1; j < p.K; ++j)
+            GAD_CK(cudaMemcpyAsync(ctx->at<float>(p.o_params) + (int64_t)j * p.pstride, ctx->at<float>(p.o_params), 4 * (size_t)p.pstride,
+                                   cudaMemcpyDeviceToDevice, ctx->stream));
+        GAD_CK(cudaMemsetAsync(ctx->ws + p.o_flags + 8, 1, 4, ctx->stream));
+        ctx->same_params = false;
+    }
     pack_params(p, in, ctx->host_block.data());
     GAD_CK(cudaMemcpyAsync(ctx->at<float>(p.o_params) + (int64_t)k * p.pstride, ctx->host_block.data(), 4 * (size_t)p.pstride,
                            cudaMemcpyHostToDevice, ctx->stream));
@@ -1167,10 +1225,12 @@ int gad_synchronize(gad_ctx* ctx) {
     if (!ctx) return GAD_ERR_ARG;
     GAD_CK(cudaStreamSynchronize(ctx->copy_stream));
     GAD_CK(cudaStreamSynchronize(ctx->side_stream));
-    int32_t timed_out = 0;
-    GAD_CK(cudaMemcpyAsync(ctx->pinned, ctx->ws + ctx->p.o_flags + 4, 4, cudaMemcpyDeviceToHost, ctx->stream));
+    int32_t words[3];
+    GAD_CK(cudaMemcpyAsync(ctx->pinned, ctx->ws + ctx->p.o_flags, 12, cudaMemcpyDeviceToHost, ctx->stream));
     GAD_CK(cudaStreamSynchronize(ctx->stream));
-    std::memcpy(&timed_out, ctx->pinned, 4);
+    std::memcpy(words, ctx->pinned, 12);
+    settle(ctx, words);
+    const int32_t timed_out = words[1];
     if (timed_out) {
         GAD_CK(cudaMemsetAsync(ctx->ws + ctx->p.o_flags + 4, 0, 4, ctx->stream));
         return fail(ctx, GAD_ERR_DEVICE_TIMEOUT, "a bounded device-side wait ran out (role " + std::to_string(timed_out) + ")");

@@ -155,13 +155,22 @@ int tc_bn_for(int n_cols);
 int tc_tn_rows();   // rows of the row-box descriptors the weight-gradient kernel reads (mapH / mapZ of launch_gemm_tn_tc)
 bool tc_make_map(void* out_map, const void* base, uint64_t inner, uint64_t rows, uint64_t outer, uint64_t row_stride_bytes,
                  uint64_t outer_stride_bytes, uint32_t box_rows, bool mn_major = false);
-cudaError_t launch_split_weights(const float* params, int64_t pstride, int64_t w_int, int fi, int fo, int ldw, int ldkt, int K,
-                                 float* w_hi, float* w_lo, float* wt_hi, float* wt_lo, cudaStream_t s);
+struct SplitLayer {
+    int fi, fo, ldw, ldkt;
+    long long w_int;
+    float *w_hi, *w_lo, *wt_hi, *wt_lo;   // w_hi, w_lo: null where no kernel reads the plain copies
+};
+struct SplitLayers {
+    static constexpr int MAX = 8;
+    SplitLayer y[MAX];
+};
+cudaError_t launch_split_weights(const float* params, int64_t pstride, int K, const SplitLayer* layers, int L, cudaStream_t s);
+// one_b: the operand copies of replica 0 serve every subgraph.
 // Cbf16 (mode 0 only, may be null): the result goes there as bfloat16 [rows x ldc] INSTEAD of to C - the operand copy the
 // reduced-precision aggregation gathers, written by its producer.
 cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols,
                                 float* C, int ldc, const RowSpan* tiles, int ntiles, const float* Hmask, int ldh, float scale,
-                                const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, void* Cbf16 = nullptr);
+                                const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16 = nullptr);
 
 // Tensor-core version of launch_gemm_tn_simt; mapH / mapZ are row-box descriptors (tc_tn_rows rows) of H^(l) and dZ.
 cudaError_t launch_gemm_tn_tc(const void* mapH, const void* mapZ, int passes, int M, int n_cols, int ldw, const RowSpan* chunks,
@@ -184,25 +193,28 @@ cudaError_t launch_gemm_tn_simt(const float* H, int ldh, int M, const float* dZ,
 cudaError_t launch_reduce_chunks(const float* partial, int64_t pstride_chunk, const int32_t* chunk_ptr, int K,
                                  float* out, int64_t ostride, int64_t off, int64_t len, cudaStream_t s);
 
-// The three launchers below are single kernels whose last-arriving CTA (per subgraph, or overall for the loss)
-// finishes the reduction over the chunks in chunk order; `counters` are monotonic arrival counters, zero at creation.
-
-// out[k][off + j] = sum over the rows of subgraph k of G[row][j], j < ld  (counters: one per subgraph).
+// out[k][off + j] = sum over the rows of subgraph k of G[row][j], j < ld.  A single kernel whose last-arriving CTA of a subgraph
+// adds the chunk sums in chunk order; counters: one per subgraph, monotonic, zero at creation.
 cudaError_t launch_colsum_chunks(const float* G, int ld, const RowSpan* chunks, int nchunks, float* partial,
                                  int64_t pstride_chunk, const int32_t* chunk_ptr, unsigned* counters, float* out,
                                  int64_t ostride, int64_t off, cudaStream_t s);
 
-// dlogits, and loss[0..K-1] = mean loss of each subgraph, loss[K] = mean over all training rows  (counter: one).
+// dlogits and per chunk the loss, and where softmax_sums_columns(ld) holds the column sums of dlogits (cs_partial).
+bool softmax_sums_columns(int ld);
 cudaError_t launch_softmax_xent(const float* logits, int ld, int C, const int32_t* label, const uint8_t* train,
                                 const RowSpan* chunks, int nchunks, const float* inv_ntrain, float* dlogits,
-                                float* loss_partial, const int32_t* chunk_ptr, int K, float inv_total, float* loss,
-                                int32_t* nonfinite, unsigned* counter, cudaStream_t s);
+                                float* loss_partial, float* cs_partial, int64_t pstride_chunk, cudaStream_t s);
+// loss[0..K-1] = mean loss of each subgraph, loss[K] = mean over all training rows, and with bias_ld > 0 out[k][off + j] = sum of
+// the column sums of subgraph k's chunks, j < bias_ld.
+cudaError_t launch_loss_finish(const float* loss_partial, const float* inv_ntrain, const int32_t* chunk_ptr, int K, float inv_total, float* loss,
+                               int32_t* nonfinite, const float* bias_partial, int64_t pstride_chunk, int bias_ld, float* out, int64_t ostride,
+                               int64_t off, cudaStream_t s);
 
-// zeta[k] of every subgraph that has rows  (counters: one per subgraph).  phase 0: from the matrix X alone; phases 1, 2, 3:
-// X is the first, a further, the last of several matrices whose squared distances add up (q_acc: one double per subgraph).
+// zeta[k] of every subgraph that has rows.  phase 0: from the matrix X alone; phases 1, 2, 3: X is the first, a further, the last
+// of several matrices whose squared distances add up (q_acc: one double per subgraph).
 cudaError_t launch_zeta(const float* X, int ld, int F, const int32_t* deg, const RowSpan* chunks, int nchunks,
-                        const int32_t* chunk_ptr, const int32_t* sub_off, const int64_t* deg_sum, const int64_t* deg_sq,
-                        float beta, double* partial, unsigned* counters, double* zeta, double* q_acc, int phase, cudaStream_t s);
+                        const int32_t* chunk_ptr, const int32_t* sub_off, int K, const int64_t* deg_sum, const int64_t* deg_sq,
+                        float beta, double* partial, double* zeta, double* q_acc, int phase, cudaStream_t s);
 
 // zeta_k in the literal pairwise form, sum_{i<j} p_i p_j / (|x_i - x_j| + beta), 64 x 64 tiles of pairs (one CTA each,
 // pair_ptr[k] = first tile of subgraph k); counters: one per subgraph; partial: one double per tile.
@@ -225,15 +237,17 @@ cudaError_t launch_zeta_gram(const void* mapHi, const void* mapLo, const float* 
                              float* Xhi, float* Xlo, float* norm2, double* partial, double* zeta, int32_t* err, int num_sms, cudaStream_t s);
 
 // `epoch` (may be null): the device epoch counter, advanced by one.
-cudaError_t launch_sgd_consensus(float* params, const float* grads, int64_t pstride, int64_t len, int K, float lr,
-                                 const double* zeta, int weighted, int with_sgd, const int32_t* err_word, long long* epoch, cudaStream_t s);
+// pstride_p: floats between the replicas' parameters, 0 while they are equal (copy 0 then stands for all of them; the result always
+// goes to copy 0).  words: the context's error words {non-finite loss, wait that ran out, copies differ}.
+cudaError_t launch_sgd_consensus(float* params, int64_t pstride_p, const float* grads, int64_t pstride, int64_t len, int K, float lr,
+                                 const double* zeta, int weighted, int with_sgd, int32_t* words, long long* epoch, cudaStream_t s);
 // The device epoch counter on its own: + 1, or set to a value.
 cudaError_t launch_epoch_counter(long long* epoch, long long set_to, bool advance, cudaStream_t s);
 // One context's share of a consensus over several contexts: out = sum_k w_k (theta_k - lr grad_k) with w_k = zeta_k / total
 // (or 1 / total), the parameters unchanged; and the finished sum written to every replica.
-cudaError_t launch_consensus_partial(const float* params, const float* grads, int64_t pstride, int64_t len, int K, float lr,
+cudaError_t launch_consensus_partial(const float* params, int64_t pstride_p, const float* grads, int64_t pstride, int64_t len, int K, float lr,
                                      const double* zeta, int weighted, int with_sgd, double total, float* out, const int32_t* err_word, cudaStream_t s);
-cudaError_t launch_consensus_apply(float* params, int64_t pstride, int64_t len, int K, const float* in, const int32_t* err_word, cudaStream_t s);
+cudaError_t launch_consensus_apply(float* params, int64_t len, const float* in, int32_t* words, cudaStream_t s);
 
 // One CTA waits, with the transforms' bounded wait and a limit of `polls` polls, on a barrier that nothing arrives at, and
 // reports it in `err` like a transform would (role 99).  For testing the time-out path; returns at once.

@@ -53,44 +53,66 @@ __device__ __forceinline__ int segments_for(int cols) {
     return 256 / p;
 }
 
-struct LossTail {
-    const int32_t* chunk_ptr;   // [K+1]
-    int K;
-    float inv_total;
-    float* loss;                // [K+1]
-    int32_t* nonfinite;
-    unsigned* counter;
-};
-
-// The chunk sums are first brought into shared memory by the whole CTA (4096 at a time); one thread per subgraph
-// then adds its subgraph's sums in chunk order, and thread 0 adds the K subgraph sums in ascending k for the global
-// loss sum_k |T_k| L_k / sum_k |T_k|.
-__device__ __forceinline__ void loss_finalize(const float* loss_partial, const float* __restrict__ inv_ntrain, const LossTail& t) {
+// What follows the loss kernel, beside the backward pass: the CTA of subgraph k adds up the column sums of its chunks' d logits
+// (the bias gradient of the last layer; bias_ld == 0: none were taken), the last CTA the losses.  The chunk losses are first
+// brought into shared memory by the whole CTA (4096 at a time); one thread per subgraph then adds its subgraph's sums in chunk order,
+// and thread 0 adds the K subgraph sums in ascending k for the global loss sum_k |T_k| L_k / sum_k |T_k|.
+__global__ void __launch_bounds__(256) loss_finish_kernel(const float* __restrict__ loss_partial, const float* __restrict__ inv_ntrain,
+                                                          const int32_t* __restrict__ chunk_ptr, int K, float inv_total, float* __restrict__ loss,
+                                                          int32_t* __restrict__ nonfinite, const float* __restrict__ bias_partial,
+                                                          long long pstride_chunk, int bias_ld, float* __restrict__ out, long long ostride,
+                                                          long long off) {
+    if ((int)blockIdx.x < K && bias_ld > 0) {
+        __shared__ float seg_sm[256];
+        const int k = blockIdx.x, c0 = chunk_ptr[k], c1 = chunk_ptr[k + 1];
+        const int nseg = segments_for(bias_ld), per = 256 / nseg;
+        const int jl = threadIdx.x % per, seg = threadIdx.x / per;
+        for (int j0 = 0; j0 < bias_ld; j0 += per) {
+            const int j = j0 + jl;
+            seg_sm[threadIdx.x] = j < bias_ld ? segment_sum(bias_partial, pstride_chunk, j, c0, c1, seg, nseg) : 0.f;
+            __syncthreads();
+            if (seg == 0 && j < bias_ld) {
+                float t = seg_sm[jl];
+                for (int q = 1; q < nseg; ++q) t += seg_sm[q * per + jl];
+                out[(long long)k * ostride + off + j] = t;
+            }
+            __syncthreads();
+        }
+        return;
+    }
     __shared__ float stage[4096];
     __shared__ float sums[1024];
-    const int nchunks = t.chunk_ptr[t.K];
+    const int nchunks = chunk_ptr[K];
     const bool staged = nchunks <= 4096;
     if (staged)
-        for (int c = threadIdx.x; c < nchunks; c += blockDim.x) stage[c] = __ldcg(loss_partial + c);
+        for (int c = threadIdx.x; c < nchunks; c += blockDim.x) stage[c] = loss_partial[c];
     __syncthreads();
-    for (int k = threadIdx.x; k < t.K; k += blockDim.x) {
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
         float s = 0.f;
-        for (int c = t.chunk_ptr[k]; c < t.chunk_ptr[k + 1]; ++c) s += staged ? stage[c] : __ldcg(loss_partial + c);
+        for (int c = chunk_ptr[k]; c < chunk_ptr[k + 1]; ++c) s += staged ? stage[c] : loss_partial[c];
         if (k < 1024) sums[k] = s;
-        t.loss[k] = s * inv_ntrain[k];
-        if (!isfinite(s)) atomicExch(t.nonfinite, 1);
+        loss[k] = s * inv_ntrain[k];
+        if (!isfinite(s)) atomicExch(nonfinite, 1);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         float s = 0.f;
-        for (int k = 0; k < t.K; ++k) {
+        for (int k = 0; k < K; ++k) {
             if (k < 1024) { s += sums[k]; continue; }
             float sk = 0.f;
-            for (int c = t.chunk_ptr[k]; c < t.chunk_ptr[k + 1]; ++c) sk += staged ? stage[c] : __ldcg(loss_partial + c);
+            for (int c = chunk_ptr[k]; c < chunk_ptr[k + 1]; ++c) sk += staged ? stage[c] : loss_partial[c];
             s += sk;
         }
-        t.loss[t.K] = s * t.inv_total;
+        loss[K] = s * inv_total;
     }
+}
+cudaError_t launch_loss_finish(const float* loss_partial, const float* inv_ntrain, const int32_t* chunk_ptr, int K, float inv_total, float* loss,
+                               int32_t* nonfinite, const float* bias_partial, int64_t pstride_chunk, int bias_ld, float* out, int64_t ostride,
+                               int64_t off, cudaStream_t s) {
+    loss_finish_kernel<<<(unsigned)(bias_ld > 0 ? K + 1 : 1), 256, 0, s>>>(loss_partial, inv_ntrain, chunk_ptr, K, inv_total, loss, nonfinite, bias_partial,
+                                                                          pstride_chunk, bias_ld, out, ostride, off);
+    ++g_kernel_launches;
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -103,7 +125,7 @@ __global__ void __launch_bounds__(256) softmax_xent_kernel(const float* __restri
                                                            const uint8_t* __restrict__ train,
                                                            const RowSpan* __restrict__ chunks,
                                                            const float* __restrict__ inv_ntrain,
-                                                           float* __restrict__ dlogits, float* loss_partial, LossTail fin) {
+                                                           float* __restrict__ dlogits, float* __restrict__ loss_partial) {
     __shared__ float wsum[8];
     const RowSpan c = chunks[blockIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -141,19 +163,22 @@ __global__ void __launch_bounds__(256) softmax_xent_kernel(const float* __restri
         for (int w = 0; w < 8; ++w) s += wsum[w];
         loss_partial[blockIdx.x] = s;
     }
-    if (cta_arrive_last(fin.counter, gridDim.x)) loss_finalize(loss_partial, inv_ntrain, fin);
 }
 
-// Up to 128 classes: L lanes hold one row (a float4 each), 32/L rows per warp step, the row stays in registers.
+// Up to 128 classes: L lanes hold one row (a float4 each), 32/L rows per warp step, the row stays in registers.  The column sums of
+// d logits (the bias gradient of the last layer) come out of the same pass: per chunk into cs_partial.
 template <int L>
 __global__ void __launch_bounds__(256) softmax_xent_small_kernel(const float* __restrict__ logits, int ld, int C,
                                                                  const int32_t* __restrict__ label,
                                                                  const uint8_t* __restrict__ train,
                                                                  const RowSpan* __restrict__ chunks,
                                                                  const float* __restrict__ inv_ntrain,
-                                                                 float* __restrict__ dlogits, float* loss_partial, LossTail fin) {
+                                                                 float* __restrict__ dlogits, float* __restrict__ loss_partial,
+                                                                 float* __restrict__ cs_partial, long long pstride_chunk) {
     constexpr int RPW = 32 / L;
     __shared__ float wsum[8];
+    __shared__ float4 csum[8][L];
+    float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
     const RowSpan c = chunks[blockIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane / L, gl = lane & (L - 1);
@@ -215,36 +240,46 @@ __global__ void __launch_bounds__(256) softmax_xent_small_kernel(const float* __
                 o4[t] = j < C ? (expf(z[t] - lse) - (j == y ? 1.f : 0.f)) * inv : 0.f;
             }
             gout[gl] = make_float4(o4[0], o4[1], o4[2], o4[3]);
+            cs.x += o4[0]; cs.y += o4[1]; cs.z += o4[2]; cs.w += o4[3];
         }
         cur = nxt;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+#pragma unroll
+    for (int o = 16; o >= L; o >>= 1) {   // the row groups of the warp
+        cs.x += __shfl_xor_sync(0xffffffffu, cs.x, o); cs.y += __shfl_xor_sync(0xffffffffu, cs.y, o);
+        cs.z += __shfl_xor_sync(0xffffffffu, cs.z, o); cs.w += __shfl_xor_sync(0xffffffffu, cs.w, o);
+    }
     if (lane == 0) wsum[warp] = acc;
+    if (lane < L) csum[warp][lane] = cs;
     __syncthreads();
     if (threadIdx.x == 0) {
         float s = 0.f;
         for (int w = 0; w < 8; ++w) s += wsum[w];
         loss_partial[blockIdx.x] = s;
     }
-    if (cta_arrive_last(fin.counter, gridDim.x)) loss_finalize(loss_partial, inv_ntrain, fin);
+    if ((int)threadIdx.x < ld4) {
+        float4 t = csum[0][threadIdx.x];
+        for (int w = 1; w < 8; ++w) { const float4 u = csum[w][threadIdx.x]; t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w; }
+        reinterpret_cast<float4*>(cs_partial + (long long)blockIdx.x * pstride_chunk)[threadIdx.x] = t;
+    }
 }
 
+bool softmax_sums_columns(int ld) { return ld <= 128; }
 cudaError_t launch_softmax_xent(const float* logits, int ld, int C, const int32_t* label, const uint8_t* train,
                                 const RowSpan* chunks, int nchunks, const float* inv_ntrain, float* dlogits,
-                                float* loss_partial, const int32_t* chunk_ptr, int K, float inv_total, float* loss,
-                                int32_t* nonfinite, unsigned* counter, cudaStream_t s) {
+                                float* loss_partial, float* cs_partial, int64_t pstride_chunk, cudaStream_t s) {
     if (nchunks > 0) {
         const int ld4 = ld >> 2;
-        const LossTail fin{chunk_ptr, K, inv_total, loss, nonfinite, counter};
-#define GAD_SMALL(L) softmax_xent_small_kernel<L><<<(unsigned)nchunks, 256, 0, s>>>(logits, ld, C, label, train, chunks, inv_ntrain, dlogits, loss_partial, fin)
+#define GAD_SMALL(L) softmax_xent_small_kernel<L><<<(unsigned)nchunks, 256, 0, s>>>(logits, ld, C, label, train, chunks, inv_ntrain, dlogits, loss_partial, cs_partial, pstride_chunk)
         if (ld4 <= 1) GAD_SMALL(1);
         else if (ld4 <= 2) GAD_SMALL(2);
         else if (ld4 <= 4) GAD_SMALL(4);
         else if (ld4 <= 8) GAD_SMALL(8);
         else if (ld4 <= 16) GAD_SMALL(16);
         else if (ld4 <= 32) GAD_SMALL(32);
-        else softmax_xent_kernel<<<(unsigned)nchunks, 256, 0, s>>>(logits, ld, C, label, train, chunks, inv_ntrain, dlogits, loss_partial, fin);
+        else softmax_xent_kernel<<<(unsigned)nchunks, 256, 0, s>>>(logits, ld, C, label, train, chunks, inv_ntrain, dlogits, loss_partial);
 #undef GAD_SMALL
         ++g_kernel_launches;
     }
@@ -357,16 +392,18 @@ cudaError_t launch_reduce_chunks(const float* partial, int64_t pstride_chunk, co
 // for any shift c_f; c_f = the subgraph's first row keeps the two sums small.  This kernel accumulates the
 // two weighted sums per chunk and per feature in double precision.
 // ---------------------------------------------------------------------------------------------
-// zeta_k = S_k / (D_k + beta) from the chunk sums of subgraph k, chunks added in order; run by one whole CTA.
+// zeta_k = S_k / (D_k + beta) from the chunk sums of subgraph k, chunks added in order; one CTA per subgraph.
 // `phase` spreads one zeta over several matrices (the layers' inputs, zeta_mode 2): 0 = this matrix alone; 1 = the first
 // of several (its distance sum goes to q_acc[k]); 2 = a further one (added to q_acc[k]); 3 = the last one (added, then zeta).
-__device__ __forceinline__ void zeta_finalize(int k, const double* partial, int F, int ld, const int32_t* __restrict__ chunk_ptr,
+__global__ void __launch_bounds__(256) zeta_finish_kernel(const double* __restrict__ partial, int F, int ld, const int32_t* __restrict__ chunk_ptr,
                                               const int32_t* __restrict__ sub_off, const int64_t* __restrict__ deg_sum,
                                               const int64_t* __restrict__ deg_sq, float beta, double* __restrict__ zeta,
                                               double* __restrict__ q_acc, int phase) {
     __shared__ double red[256];
     __shared__ double seg_a[256], seg_b[256];
+    const int k = blockIdx.x;
     const long long n = sub_off[k + 1] - sub_off[k];
+    if (n == 0) return;   // zero since creation
     const bool uniform = deg_sum[k] == 0;
     const double D = uniform ? (double)n : (double)deg_sum[k];
     double q = 0.0;
@@ -412,77 +449,62 @@ __device__ __forceinline__ void zeta_finalize(int k, const double* partial, int 
     }
 }
 
-__global__ void __launch_bounds__(256) zeta_partial_kernel(const float* __restrict__ X, int ld, int F,
-                                                           const int32_t* __restrict__ deg,
-                                                           const RowSpan* __restrict__ chunks,
-                                                           const int32_t* __restrict__ sub_off,
-                                                           const int64_t* __restrict__ deg_sum, double* partial,
-                                                           const int32_t* __restrict__ chunk_ptr,
-                                                           const int64_t* __restrict__ deg_sq, float beta,
-                                                           unsigned* counters, double* __restrict__ zeta,
-                                                           double* __restrict__ q_acc, int phase) {
-    // threads = 8 row lanes x 32 column lanes of one float4 each (as in the column sums above)
+// Grid: (row chunks, blocks of 128 columns); threads = 8 row lanes x 32 column lanes of one float4 each (as in the column sums above).
+// The columns are spread over CTAs because the chunks of a small graph are few: with one CTA per chunk 2843 rows of 1433 features
+// took 58 us on 24 CTAs.
+__global__ void __launch_bounds__(256) zeta_partial_kernel(const float* __restrict__ X, int ld, const int32_t* __restrict__ deg,
+                                                           const RowSpan* __restrict__ chunks, const int32_t* __restrict__ sub_off,
+                                                           const int64_t* __restrict__ deg_sum, double* __restrict__ partial) {
     __shared__ double sm[8][32][8];
     const RowSpan c = chunks[blockIdx.x];
     const bool uniform = deg_sum[c.k] == 0;
     const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
-    const int ld4 = ld >> 2;
-    const float4* x0 = reinterpret_cast<const float4*>(X + (long long)sub_off[c.k] * ld);
+    const int ld4 = ld >> 2, v = (int)blockIdx.y * 32 + cx;
     double* P = partial + (long long)blockIdx.x * 2 * ld;
-    for (int v0 = 0; v0 < ld4; v0 += 32) {
-        const int v = v0 + cx;
-        double a[4] = {0.0, 0.0, 0.0, 0.0}, b[4] = {0.0, 0.0, 0.0, 0.0};
-        if (v < ld4) {
-            const float4 sh = x0[v];
-            const float4* g = reinterpret_cast<const float4*>(X + (long long)c.row0 * ld) + v;
-            const int32_t* dg = deg + c.row0;
-            int r = ry;
-            for (; r + 8 < c.nrows; r += 16) {
-                const float4 u0 = g[(long long)r * ld4], u1 = g[(long long)(r + 8) * ld4];
-                const double w0 = uniform ? 1.0 : (double)dg[r], w1 = uniform ? 1.0 : (double)dg[r + 8];
-                const double d0[4] = {(double)(u0.x - sh.x), (double)(u0.y - sh.y), (double)(u0.z - sh.z), (double)(u0.w - sh.w)};
-                const double d1[4] = {(double)(u1.x - sh.x), (double)(u1.y - sh.y), (double)(u1.z - sh.z), (double)(u1.w - sh.w)};
+    double a[4] = {0.0, 0.0, 0.0, 0.0}, b[4] = {0.0, 0.0, 0.0, 0.0};
+    if (v < ld4) {
+        const float4 sh = reinterpret_cast<const float4*>(X + (long long)sub_off[c.k] * ld)[v];
+        const float4* g = reinterpret_cast<const float4*>(X + (long long)c.row0 * ld) + v;
+        const int32_t* dg = deg + c.row0;
+        auto add = [&](const float4& u, int d) {
+            const double w = uniform ? 1.0 : (double)d;
+            const double x[4] = {(double)(u.x - sh.x), (double)(u.y - sh.y), (double)(u.z - sh.z), (double)(u.w - sh.w)};
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    a[t] = fma(w0, d0[t], a[t]); b[t] = fma(w0 * d0[t], d0[t], b[t]);
-                    a[t] = fma(w1, d1[t], a[t]); b[t] = fma(w1 * d1[t], d1[t], b[t]);
-                }
-            }
-            for (; r < c.nrows; r += 8) {
-                const float4 u0 = g[(long long)r * ld4];
-                const double w0 = uniform ? 1.0 : (double)dg[r];
-                const double d0[4] = {(double)(u0.x - sh.x), (double)(u0.y - sh.y), (double)(u0.z - sh.z), (double)(u0.w - sh.w)};
+            for (int t = 0; t < 4; ++t) { a[t] = fma(w, x[t], a[t]); b[t] = fma(w * x[t], x[t], b[t]); }
+        };
+        int r = ry;
+        for (; r + 24 < c.nrows; r += 32) {   // four rows in flight
+            float4 u[4];
+            int d[4];
 #pragma unroll
-                for (int t = 0; t < 4; ++t) { a[t] = fma(w0, d0[t], a[t]); b[t] = fma(w0 * d0[t], d0[t], b[t]); }
-            }
+            for (int q = 0; q < 4; ++q) { u[q] = g[(long long)(r + 8 * q) * ld4]; d[q] = dg[r + 8 * q]; }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) add(u[q], d[q]);
         }
-#pragma unroll
-        for (int t = 0; t < 4; ++t) { sm[ry][cx][t] = a[t]; sm[ry][cx][4 + t] = b[t]; }
-        __syncthreads();
-        if (ry == 0 && v < ld4) {
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                double sa = 0.0, sb = 0.0;
-                for (int w = 0; w < 8; ++w) { sa += sm[w][cx][t]; sb += sm[w][cx][4 + t]; }
-                P[4 * v + t] = sa;
-                P[ld + 4 * v + t] = sb;
-            }
-        }
-        __syncthreads();
+        for (; r < c.nrows; r += 8) add(g[(long long)r * ld4], dg[r]);
     }
-    // the last CTA of this subgraph turns the chunk sums into zeta_k
-    if (cta_arrive_last(counters + c.k, (unsigned)(chunk_ptr[c.k + 1] - chunk_ptr[c.k])))
-        zeta_finalize(c.k, partial, F, ld, chunk_ptr, sub_off, deg_sum, deg_sq, beta, zeta, q_acc, phase);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) { sm[ry][cx][t] = a[t]; sm[ry][cx][4 + t] = b[t]; }
+    __syncthreads();
+    if (ry == 0 && v < ld4) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            double sa = 0.0, sb = 0.0;
+            for (int w = 0; w < 8; ++w) { sa += sm[w][cx][t]; sb += sm[w][cx][4 + t]; }
+            P[4 * v + t] = sa;
+            P[ld + 4 * v + t] = sb;
+        }
+    }
 }
 
 // zeta[k] for every subgraph that has rows (the entry of an empty subgraph is left as it is: zero since creation).
 cudaError_t launch_zeta(const float* X, int ld, int F, const int32_t* deg, const RowSpan* chunks, int nchunks,
-                        const int32_t* chunk_ptr, const int32_t* sub_off, const int64_t* deg_sum, const int64_t* deg_sq,
-                        float beta, double* partial, unsigned* counters, double* zeta, double* q_acc, int phase, cudaStream_t s) {
+                        const int32_t* chunk_ptr, const int32_t* sub_off, int K, const int64_t* deg_sum, const int64_t* deg_sq,
+                        float beta, double* partial, double* zeta, double* q_acc, int phase, cudaStream_t s) {
     if (nchunks > 0) {
-        zeta_partial_kernel<<<(unsigned)nchunks, 256, 0, s>>>(X, ld, F, deg, chunks, sub_off, deg_sum, partial, chunk_ptr, deg_sq, beta,
-                                                              counters, zeta, q_acc, phase);
-        ++g_kernel_launches;
+        zeta_partial_kernel<<<dim3((unsigned)nchunks, (unsigned)((ld / 4 + 31) / 32)), 256, 0, s>>>(X, ld, deg, chunks, sub_off, deg_sum, partial);
+        zeta_finish_kernel<<<(unsigned)K, 256, 0, s>>>(partial, F, ld, chunk_ptr, sub_off, deg_sum, deg_sq, beta, zeta, q_acc, phase);
+        g_kernel_launches += 2;
     }
     return cudaGetLastError();
 }
@@ -507,7 +529,7 @@ __device__ __forceinline__ void consensus_weights(const double* __restrict__ zet
 // sum_k w_k (theta_k - lr grad_k) for the four parameters at float4 index i, k ascending.  The copies are read eight at a time,
 // all sixteen loads of a batch issued before the first is used: with many copies of a small model (K = 64 copies of a
 // 256-256 layer are 50 MB spread over 65 CTAs) the kernel is a chain of dependent loads otherwise.
-__device__ __forceinline__ float4 weighted_sum(const float* __restrict__ params, const float* __restrict__ grads, long long pstride,
+__device__ __forceinline__ float4 weighted_sum(const float* params, long long pstride_p, const float* __restrict__ grads, long long pstride,
                                                long long i, int K, float lr, int with_sgd, const float* w_sm) {
     constexpr int B = 8;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -516,7 +538,7 @@ __device__ __forceinline__ float4 weighted_sum(const float* __restrict__ params,
 #pragma unroll
         for (int t = 0; t < B; ++t) {
             const int k = min(k0 + t, K - 1);   // past the end: the last copy again, with weight 0 below
-            p[t] = reinterpret_cast<const float4*>(params + (long long)k * pstride)[i];
+            p[t] = reinterpret_cast<const float4*>(params + (long long)k * pstride_p)[i];
             g[t] = with_sgd ? reinterpret_cast<const float4*>(grads + (long long)k * pstride)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
@@ -533,27 +555,32 @@ __device__ __forceinline__ float4 weighted_sum(const float* __restrict__ params,
 }
 
 // theta_k <- theta_k - lr * grad_k (each replica's own step, update equation of Section 3.3), then
-// theta_k <- sum_j w_j theta_j for every k (weighted global consensus, Section 3.4.2).  One float4 per thread.
-__global__ void __launch_bounds__(256) sgd_consensus_kernel(float* __restrict__ params, const float* __restrict__ grads,
+// theta_k <- sum_j w_j theta_j for every k (weighted global consensus, Section 3.4.2).  One float4 per thread.  All copies come out
+// equal, so only copy 0 is written, and while they are equal it is the only one read (pstride_p == 0): K gradient sets and one
+// parameter set in, one out, where K of each went both ways (50 copies of a 500-128-128-128-7 net: 13.5 -> XX us).  words[2] says on
+// the device whether the copies differ.
+__global__ void __launch_bounds__(256) sgd_consensus_kernel(float* params, long long pstride_p, const float* __restrict__ grads,
                                                             long long pstride, long long len4, int K, float lr,
                                                             const double* __restrict__ zeta, int weighted, int with_sgd,
-                                                            const int32_t* __restrict__ err_word, long long* epoch) {
+                                                            int32_t* words, long long* epoch) {
     extern __shared__ float w_sm[];
     if (epoch && blockIdx.x == 0 && threadIdx.x == 0) *epoch += 1;   // last kernel of an epoch: nothing reads the counter beside it
-    if (err_word && *err_word) return;   // a bounded wait ran out earlier in this epoch: keep the parameters as they are
+    if (words[1]) return;   // a bounded wait ran out earlier in this epoch: keep the parameters as they are
     consensus_weights(zeta, K, weighted, w_sm);
+    if (blockIdx.x == 0 && threadIdx.x == 0 && pstride_p != 0) words[2] = 0;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= len4) return;
-    const float4 acc = weighted_sum(params, grads, pstride, i, K, lr, with_sgd, w_sm);
-    for (int k = 0; k < K; ++k) reinterpret_cast<float4*>(params + (long long)k * pstride)[i] = acc;
+    reinterpret_cast<float4*>(params)[i] = weighted_sum(params, pstride_p, grads, pstride, i, K, lr, with_sgd, w_sm);
 }
-cudaError_t launch_sgd_consensus(float* params, const float* grads, int64_t pstride, int64_t len, int K, float lr,
-                                 const double* zeta, int weighted, int with_sgd, const int32_t* err_word, long long* epoch, cudaStream_t s) {
+cudaError_t launch_sgd_consensus(float* params, int64_t pstride_p, const float* grads, int64_t pstride, int64_t len, int K, float lr,
+                                 const double* zeta, int weighted, int with_sgd, int32_t* words, long long* epoch, cudaStream_t s) {
     const long long len4 = len / 4;
     if (len4 > 0) {
         const int threads = len4 >= 148 * 256 * 4 ? 256 : 64;   // a small model is spread over more CTAs
-        sgd_consensus_kernel<<<(unsigned)((len4 + threads - 1) / threads), threads, (size_t)K * sizeof(float), s>>>(params, grads, pstride, len4, K, lr,
-                                                                                                   zeta, weighted, with_sgd, err_word, epoch); ++g_kernel_launches; }
+        sgd_consensus_kernel<<<(unsigned)((len4 + threads - 1) / threads), threads, (size_t)K * sizeof(float), s>>>(
+            params, pstride_p, grads, pstride, len4, K, lr, zeta, weighted, with_sgd, words, epoch);
+        ++g_kernel_launches;
+    }
     return cudaGetLastError();
 }
 
@@ -566,8 +593,8 @@ cudaError_t launch_epoch_counter(long long* epoch, long long set_to, bool advanc
 // The same sum over the replicas of one context when the subgraphs are spread over several contexts:
 //   out = sum_k w_k (theta_k - lr * grad_k),  w_k = zeta_k / total (weighted) or 1 / total,
 // with `total` the sum over ALL contexts, so that the contexts' results add up to the consensus.  The parameters
-// themselves are left alone; consensus_apply_kernel writes the finished sum to every replica.
-__global__ void __launch_bounds__(256) consensus_partial_kernel(const float* __restrict__ params, const float* __restrict__ grads,
+// themselves are left alone; consensus_apply_kernel writes the finished sum (to copy 0: the copies are equal from then on).
+__global__ void __launch_bounds__(256) consensus_partial_kernel(const float* __restrict__ params, long long pstride_p, const float* __restrict__ grads,
                                                                 long long pstride, long long len4, int K, float lr,
                                                                 const double* __restrict__ zeta, int weighted, int with_sgd,
                                                                 double total, float* __restrict__ out, const int32_t* __restrict__ err_word) {
@@ -577,30 +604,28 @@ __global__ void __launch_bounds__(256) consensus_partial_kernel(const float* __r
     __syncthreads();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= len4) return;
-    const float4 acc = weighted_sum(params, grads, pstride, i, K, lr, with_sgd, w_sm);
-    reinterpret_cast<float4*>(out)[i] = acc;
+    reinterpret_cast<float4*>(out)[i] = weighted_sum(params, pstride_p, grads, pstride, i, K, lr, with_sgd, w_sm);
 }
-__global__ void __launch_bounds__(256) consensus_apply_kernel(float* __restrict__ params, long long pstride, long long len4, int K,
-                                                              const float* __restrict__ in, const int32_t* __restrict__ err_word) {
+__global__ void __launch_bounds__(256) consensus_apply_kernel(float* __restrict__ params, long long len4, const float* __restrict__ in, int32_t* words) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= len4 || (err_word && *err_word)) return;
-    const float4 v = reinterpret_cast<const float4*>(in)[i];
-    for (int k = 0; k < K; ++k) reinterpret_cast<float4*>(params + (long long)k * pstride)[i] = v;
+    if (i >= len4 || words[1]) return;
+    reinterpret_cast<float4*>(params)[i] = reinterpret_cast<const float4*>(in)[i];
+    if (i == 0) words[2] = 0;
 }
-cudaError_t launch_consensus_partial(const float* params, const float* grads, int64_t pstride, int64_t len, int K, float lr,
+cudaError_t launch_consensus_partial(const float* params, int64_t pstride_p, const float* grads, int64_t pstride, int64_t len, int K, float lr,
                                      const double* zeta, int weighted, int with_sgd, double total, float* out, const int32_t* err_word, cudaStream_t s) {
     const long long len4 = len / 4;
     if (len4 > 0) {
         const int threads = len4 >= 148 * 256 * 4 ? 256 : 64;
-        consensus_partial_kernel<<<(unsigned)((len4 + threads - 1) / threads), threads, (size_t)K * sizeof(float), s>>>(params, grads, pstride, len4, K, lr,
+        consensus_partial_kernel<<<(unsigned)((len4 + threads - 1) / threads), threads, (size_t)K * sizeof(float), s>>>(params, pstride_p, grads, pstride, len4, K, lr,
                                                                                                        zeta, weighted, with_sgd, total, out, err_word);
         ++g_kernel_launches;
     }
     return cudaGetLastError();
 }
-cudaError_t launch_consensus_apply(float* params, int64_t pstride, int64_t len, int K, const float* in, const int32_t* err_word, cudaStream_t s) {
+cudaError_t launch_consensus_apply(float* params, int64_t len, const float* in, int32_t* words, cudaStream_t s) {
     const long long len4 = len / 4;
-    if (len4 > 0) { consensus_apply_kernel<<<(unsigned)((len4 + 255) / 256), 256, 0, s>>>(params, pstride, len4, K, in, err_word); ++g_kernel_launches; }
+    if (len4 > 0) { consensus_apply_kernel<<<(unsigned)((len4 + 255) / 256), 256, 0, s>>>(params, len4, in, words); ++g_kernel_launches; }
     return cudaGetLastError();
 }
 

@@ -68,12 +68,21 @@ def load():
         L.gad_last_error.argtypes = [C.c_void_p]
         L.gad_destroy.restype = None
         L.gad_destroy.argtypes = [C.c_void_p]
+        # the calls of a training loop: addresses go in as plain integers
+        L.gad_train_epoch.argtypes = L.gad_train_epoch_local.argtypes = L.gad_read_loss_async.argtypes = [C.c_void_p, C.c_void_p]
+        L.gad_export_params.argtypes = [C.c_void_p, C.c_int32, C.c_void_p]
+        L.gad_consensus_apply.argtypes = [C.c_void_p, C.c_void_p]
         _lib = L
     return _lib
 
 
 def _ptr(a, t):
     return a.ctypes.data_as(C.POINTER(t)) if a is not None else None
+
+
+def _address(a):
+    """Address of a float32 array that the library reads or writes in place."""
+    return a.ctypes.data
 
 
 def _arr(a, dtype):
@@ -130,6 +139,7 @@ class Gad:
         L = load()
         self._L = L
         self._h = None
+        self._consensus_floats = None
         self.n = int(n)
         self.dims = tuple(int(d) for d in dims)
         inp = _Inputs(n, rowptr, col, weights, core_ptr, core_nodes, halo_ptr, halo_nodes, dims, lr, dropout, seed,
@@ -200,10 +210,10 @@ class Gad:
         if not wait:
             self._ck(self._L.gad_train_epoch(self._h, None))
             if loss_out is not None:
-                self._ck(self._L.gad_read_loss_async(self._h, _ptr(loss_out, C.c_float)))
+                self._ck(self._L.gad_read_loss_async(self._h, _address(loss_out)))
             return None
         out = loss_out if loss_out is not None else np.zeros(self.K + 1, dtype=np.float32)
-        self._ck(self._L.gad_train_epoch(self._h, _ptr(out, C.c_float)))
+        self._ck(self._L.gad_train_epoch(self._h, _address(out)))
         return out
 
     def synchronize(self):
@@ -237,7 +247,7 @@ class Gad:
             self._ck(self._L.gad_train_epoch_local(self._h, None))
             return None
         out = np.zeros(self.K + 1, dtype=np.float32)
-        self._ck(self._L.gad_train_epoch_local(self._h, _ptr(out, C.c_float)))
+        self._ck(self._L.gad_train_epoch_local(self._h, _address(out)))
         return out
 
     def ntrain(self):
@@ -247,9 +257,11 @@ class Gad:
         return out
 
     def consensus_floats(self) -> int:
-        n = C.c_int64(0)
-        self._ck(self._L.gad_consensus_floats(self._h, C.byref(n)))
-        return int(n.value)
+        if self._consensus_floats is None:
+            n = C.c_int64(0)
+            self._ck(self._L.gad_consensus_floats(self._h, C.byref(n)))
+            self._consensus_floats = int(n.value)
+        return self._consensus_floats
 
     def new_consensus_buffer(self):
         """A float32 CUDA tensor of gad_consensus_floats elements on this context's device."""
@@ -265,11 +277,11 @@ class Gad:
 
     def consensus_apply(self, buf):
         self._check_buffer(buf)
-        self._ck(self._L.gad_consensus_apply(self._h, C.c_void_p(buf.data_ptr())))
+        self._ck(self._L.gad_consensus_apply(self._h, buf.data_ptr()))
 
     def export_params(self, k, out):
         self._check_buffer(out)
-        self._ck(self._L.gad_export_params(self._h, C.c_int32(k), C.c_void_p(out.data_ptr())))
+        self._ck(self._L.gad_export_params(self._h, k, out.data_ptr()))
         return out
 
     def _check_buffer(self, t):

@@ -46,6 +46,15 @@ __device__ __forceinline__ float4 load_bias(const ActEpi& ep, int k, int col) {
     return __ldg(reinterpret_cast<const float4*>(ep.params + (long long)k * ep.pstride + ep.b_int + col));
 }
 
+__device__ __forceinline__ float2 load_bias2(const ActEpi& ep, int k, int col) {
+    return __ldg(reinterpret_cast<const float2*>(ep.params + (long long)k * ep.pstride + ep.b_int + col));
+}
+
+__device__ __forceinline__ uint64_t dropout_row_key(const ActEpi& ep, long long row) {
+    return dropout_row_key(ep.seed, __ldg(ep.epoch), ep.layer, row);
+}
+__device__ __forceinline__ float relu_unless(float x, int relu) { return relu ? relu_nan(x) : x; }
+
 // v = four consecutive pre-activation sums of `row`, columns col .. col+3 (before the bias b).
 __device__ __forceinline__ float4 apply_act(float4 v, float4 b, const ActEpi& ep, long long row, int col) {
     float x[4] = {v.x + b.x, v.y + b.y, v.z + b.z, v.w + b.w};

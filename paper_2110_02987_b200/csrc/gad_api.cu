@@ -57,14 +57,17 @@ struct Plan {
     std::vector<Layer> layers;
     std::vector<int32_t> ld;          // [L+1]
     int32_t maxld = 0;
-    std::vector<RowSpan> tiles, chunks, dw_chunks, core_spans;
-    std::vector<int32_t> chunk_ptr, dw_chunk_ptr;   // [K+1]
+    std::vector<RowSpan> pair_tiles;  // 128-row tiles, an even number per subgraph (the last may be empty)
+    size_t o_pair_tiles = 0;
+    std::vector<RowSpan> tiles, chunks, core_spans;
+    std::vector<int32_t> chunk_ptr;   // [K+1]
+    struct DwChunks { std::vector<RowSpan> spans; std::vector<int32_t> ptr; size_t o_spans = 0, o_ptr = 0; };
+    std::vector<DwChunks> dw;         // [L] row chunks of each layer's weight gradient, their first chunk per subgraph [K+1]
     std::vector<int64_t> pair_ptr;    // [K+1] tiles of pairs per subgraph (zeta_mode 1 on the FP32 ALUs), else empty
     size_t o_pair_ptr = 0, o_pair_partial = 0;
     std::vector<int64_t> gram_ptr;    // [K+1] 128 x 128 tiles of pairs per subgraph (zeta_mode 1 on the tensor cores)
     size_t o_gram_ptr = 0, o_gram_partial = 0, o_norm2 = 0, o_xhi = 0, o_xlo = 0;
     bool pair_alu_ok = false;         // every subgraph is small enough for the FP32-ALU pairwise kernel
-    int64_t dw_partial = 0;           // floats per chunk
     std::vector<uint8_t> agg_first;   // [L] the layer aggregates before it transforms: sigma((A~ H^(l)) W + b)
     std::vector<size_t> o_P;          // [L] A~ H^(l)  [Np x ld_l] of those layers
     size_t o_epoch = 0;               // device epoch counter (indexes the dropout mask)
@@ -80,7 +83,7 @@ struct Plan {
     // offsets into the workspace
     size_t o_growptr = 0, o_gecv = 0, o_gfin = 0, o_gitems = 0;   // the loss rows' store (see gad_ctx::Ag)
     size_t o_rowptr, o_ecv, o_fin, o_items, o_trowptr, o_tecv, o_tfin, o_titems, o_spmm_scratch, o_sub_off, o_gid, o_deg, o_label, o_train,
-        o_deg_sum, o_deg_sq, o_inv_ntrain, o_tiles, o_chunks, o_chunk_ptr, o_dw_chunks, o_dw_chunk_ptr, o_core_spans, o_G1, o_G2, o_params, o_grads,
+        o_deg_sum, o_deg_sq, o_inv_ntrain, o_tiles, o_chunks, o_chunk_ptr, o_core_spans, o_G1, o_G2, o_params, o_grads,
         o_dw_partial, o_cs_partial, o_loss_partial, o_zeta_partial, o_zeta, o_loss, o_flags, o_zeta_f, o_w_f, o_stage,
         o_stage_lab, o_stage2, o_stage_lab2;
     std::vector<size_t> o_H, o_w_hi, o_w_lo, o_wt_hi, o_wt_lo;   // per layer
@@ -123,7 +126,6 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
     for (int l = 1; l < p.L; ++l) p.agg_first[l] = (cfg->flags & 32) == 0 && p.dims[l] < p.dims[l + 1];
     p.layers.resize(p.L);
     int64_t oi = 0, oe = 0;
-    p.dw_partial = 0;
     for (int l = 0; l < p.L; ++l) {
         Layer& y = p.layers[l];
         y.fi = p.dims[l]; y.fo = p.dims[l + 1]; y.ldi = p.ld[l]; y.ldo = p.ld[l + 1]; y.ldw = p.ld[l + 1];
@@ -131,31 +133,35 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
         y.b_int = oi; oi += y.ldo;
         y.w_ext = oe; oe += (int64_t)y.fi * y.fo;
         y.b_ext = oe; oe += y.fo;
-        p.dw_partial = std::max(p.dw_partial, (int64_t)y.fi * y.ldw);
     }
     p.P = oe; p.Pint = oi; p.pstride = round_up(oi, 64);
     // row tiles of the grouped transforms (128 rows, never across subgraphs) and reduction chunks
     const int64_t target = 592;
     int64_t R = round_up(std::max<int64_t>(1, (p.Np + target - 1) / target), 32);
     R = std::min<int64_t>(R, 16384);
-    // The weight gradient has a long reduction per output tile, so it gets longer chunks: about one CTA per SM (a
-    // single wave: every CTA pays the pipeline fill once) over the layer with the most output tiles (128 rows x up to 256 columns each).
-    int64_t max_tiles = 1;
-    for (const Layer& y : p.layers) {
-        const int bn = tc_bn_for(y.fo);
-        max_tiles = std::max<int64_t>(max_tiles, ((y.fi + 127) / 128) * (int64_t)((y.ldw + bn - 1) / bn));
+    p.dw.resize(p.L);
+    size_t dw_floats = 0;
+    for (int l = 0; l < p.L; ++l) {
+        const Layer& y = p.layers[l];
+        const int64_t Rdw = tn_chunk_rows(sub_off, tn_shape(y.fi, y.ldw), y.fi, y.ldw, 148);
+        Plan::DwChunks& d = p.dw[l];
+        d.ptr.assign(K + 1, 0);
+        for (int32_t k = 0; k < K; ++k) {
+            for (int64_t r = sub_off[k]; r < sub_off[k + 1]; r += Rdw)
+                d.spans.push_back(RowSpan{(int32_t)r, (int32_t)std::min<int64_t>(Rdw, sub_off[k + 1] - r), k, 0});
+            d.ptr[k + 1] = (int32_t)d.spans.size();
+        }
+        dw_floats = std::max(dw_floats, d.spans.size() * (size_t)y.fi * y.ldw);
     }
-    int64_t Rdw = round_up(std::max<int64_t>(1, p.Np * max_tiles / std::max<int64_t>(74, 148 - K)), 32);
-    // (not longer than 4096 rows: the CTAs that share a chunk then stay close enough to share it in L2)
-    Rdw = std::min<int64_t>(std::max<int64_t>(Rdw, 256), 4096);
     p.chunk_ptr.assign(K + 1, 0);
-    p.dw_chunk_ptr.assign(K + 1, 0);
     for (int32_t k = 0; k < K; ++k) {
-        for (int64_t r = sub_off[k]; r < sub_off[k + 1]; r += Rdw)
-            p.dw_chunks.push_back(RowSpan{(int32_t)r, (int32_t)std::min<int64_t>(Rdw, sub_off[k + 1] - r), k, 0});
-        p.dw_chunk_ptr[k + 1] = (int32_t)p.dw_chunks.size();
         for (int32_t r = sub_off[k]; r < sub_off[k + 1]; r += 128)
             p.tiles.push_back(RowSpan{r, std::min<int32_t>(128, sub_off[k + 1] - r), k, 0});
+        for (int32_t r = sub_off[k]; r < sub_off[k + 1]; r += 256) {
+            p.pair_tiles.push_back(RowSpan{r, std::min<int32_t>(128, sub_off[k + 1] - r), k, 0});
+            const int32_t r2 = std::min(r + 128, sub_off[k + 1] - 1);   // (a row that exists, also when none is left)
+            p.pair_tiles.push_back(RowSpan{r2, std::max(0, std::min<int32_t>(128, sub_off[k + 1] - r - 128)), k, 0});
+        }
         for (int64_t r = sub_off[k]; r < sub_off[k + 1]; r += R)
             p.chunks.push_back(RowSpan{(int32_t)r, (int32_t)std::min<int64_t>(R, sub_off[k + 1] - r), k, 0});
         p.chunk_ptr[k + 1] = (int32_t)p.chunks.size();
@@ -180,9 +186,10 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
     p.o_sub_off = take(cur, 4 * (size_t)(K + 1)); p.o_gid = take(cur, 4 * Np); p.o_deg = take(cur, 4 * Np);
     p.o_label = take(cur, 4 * Np); p.o_train = take(cur, Np);
     p.o_deg_sum = take(cur, 8 * (size_t)K); p.o_deg_sq = take(cur, 8 * (size_t)K); p.o_inv_ntrain = take(cur, 4 * (size_t)K);
+    p.o_pair_tiles = take(cur, sizeof(RowSpan) * p.pair_tiles.size());
     p.o_tiles = take(cur, sizeof(RowSpan) * p.tiles.size()); p.o_chunks = take(cur, sizeof(RowSpan) * nc);
     p.o_chunk_ptr = take(cur, 4 * (size_t)(K + 1));
-    p.o_dw_chunks = take(cur, sizeof(RowSpan) * p.dw_chunks.size()); p.o_dw_chunk_ptr = take(cur, 4 * (size_t)(K + 1));
+    for (Plan::DwChunks& d : p.dw) { d.o_spans = take(cur, sizeof(RowSpan) * d.spans.size()); d.o_ptr = take(cur, 4 * (size_t)(K + 1)); }
     p.o_core_spans = take(cur, sizeof(RowSpan) * p.core_spans.size());
     p.o_H.resize(p.L + 1);
     for (int l = 0; l <= p.L; ++l) p.o_H[l] = take(cur, 4 * Np * (size_t)p.ld[l]);
@@ -192,7 +199,7 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
     if (cfg->gemm_mode == 1) p.o_bf16 = take(cur, 2 * Np * (size_t)max_spmm_ld);
     p.o_G1 = take(cur, 4 * Np * (size_t)p.maxld); p.o_G2 = take(cur, 4 * Np * (size_t)p.maxld);
     p.o_params = take(cur, 4 * (size_t)K * (size_t)p.pstride); p.o_grads = take(cur, 4 * (size_t)K * (size_t)p.pstride);
-    p.o_dw_partial = take(cur, 4 * p.dw_chunks.size() * (size_t)p.dw_partial); p.o_cs_partial = take(cur, 4 * nc * (size_t)p.maxld);
+    p.o_dw_partial = take(cur, 4 * dw_floats); p.o_cs_partial = take(cur, 4 * nc * (size_t)p.maxld);
     int32_t zeta_ld = p.ld[0];   // widest matrix the importance statistics run over: H^(0), or every layer's input (zeta_mode 2)
     if (cfg->zeta_mode == 2)
         for (int l = 0; l < p.L; ++l) zeta_ld = std::max(zeta_ld, p.ld[l]);
@@ -278,6 +285,7 @@ struct gad_ctx {
     std::vector<float> host_block;  // staging for parameter pack / unpack
     char* pinned = nullptr;         // pinned host memory the small results of waiting calls land in (pinned_bytes)
     size_t pinned_bytes = 0;
+    float* published = nullptr;     // second half of it: losses and error words as the last kernel of an epoch leaves them
     // The replicas' parameters are equal (after creation and every consensus) until gad_set_params gives one its own: copy 0 then
     // stands for all of them and the others are stale.  `unsettled`: a consensus over differing copies has been enqueued and
     // nothing has waited for it since; should a bounded wait have run out it left them as they were (error word 2 tells).
@@ -435,7 +443,7 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t ss) {
             GAD_RUN("gemm_fwd", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
                 if (ctx->use_tc)
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 2, passes, y.fi, y.fo,
-                                               ctx->H(l + 1), y.ldo, ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, &act,
+                                               ctx->H(l + 1), y.ldo, ctx->at<RowSpan>(p.o_pair_tiles), (int)(p.pair_tiles.size() / 2), nullptr, 0, 1.f, &act,
                                                ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params);
                 return launch_gemm_rows_simt(2, ctx->at<float>(p.o_P[l]), y.ldi, y.fi, params, pstride, y.w_int, y.ldw, y.fo, ctx->H(l + 1), y.ldo,
                                              ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, &act, ctx->stream);
@@ -448,7 +456,7 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t ss) {
         GAD_RUN("gemm_fwd", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
             if (ctx->use_tc)
                 return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 0, passes, y.fi, y.fo, Z,
-                                           y.ldo, ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, nullptr,
+                                           y.ldo, ctx->at<RowSpan>(p.o_pair_tiles), (int)(p.pair_tiles.size() / 2), nullptr, 0, 1.f, nullptr,
                                            ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params, zb);
             return launch_gemm_rows_simt(0, ctx->H(l), y.ldi, y.fi, params, pstride, y.w_int, y.ldw, y.fo, Z, y.ldo,
                                          ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, nullptr, ctx->stream);
@@ -516,9 +524,6 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
     const RowSpan* chunks = ctx->at<RowSpan>(p.o_chunks);
     const int nc = (int)p.chunks.size();
     const int32_t* chunk_ptr = ctx->at<int32_t>(p.o_chunk_ptr);
-    const RowSpan* dw_chunks = ctx->at<RowSpan>(p.o_dw_chunks);
-    const int ndw = (int)p.dw_chunks.size();
-    const int32_t* dw_chunk_ptr = ctx->at<int32_t>(p.o_dw_chunk_ptr);
     const float scale = ctx->cfg.dropout > 0.f ? 1.f / (1.f - ctx->cfg.dropout) : 1.f;
     // whether this layer's dPre columns have been summed already: by the loss kernel, or by the layer above's fused narrow kernel
     bool bias_done = softmax_sums_columns(p.ld[p.L]);
@@ -564,15 +569,17 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
             bias_done = true;
             continue;
         }
+        const RowSpan* dw_chunks = ctx->at<RowSpan>(p.dw[l].o_spans);
+        const int ndw = (int)p.dw[l].spans.size();
         GAD_RUN("gemm_dw", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
             cudaError_t e =
                 ctx->use_tc ? launch_gemm_tn_tc(&ctx->maps[kMapsPerLayer * l + 6], &ctx->maps[kMapsPerLayer * l + 7],
-                                                ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fi, y.fo, y.ldw, dw_chunks, ndw,
-                                                ctx->at<float>(p.o_dw_partial), ctx->at<int32_t>(p.o_flags) + 1, ctx->stream)
+                                                ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fi, y.ldw, dw_chunks, ndw,
+                                                ctx->at<float>(p.o_dw_partial), ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream)
                             : launch_gemm_tn_simt(agg_first ? ctx->at<float>(p.o_P[l]) : ctx->H(l), y.ldi, y.fi, agg_first ? G1 : G2, y.ldo,
                                                   y.fo, dw_chunks, ndw, ctx->at<float>(p.o_dw_partial), y.ldw, ctx->stream);
             if (e != cudaSuccess) return e;
-            return launch_reduce_chunks(ctx->at<float>(p.o_dw_partial), (int64_t)y.fi * y.ldw, dw_chunk_ptr, p.K, grads, p.pstride,
+            return launch_reduce_chunks(ctx->at<float>(p.o_dw_partial), (int64_t)y.fi * y.ldw, ctx->at<int32_t>(p.dw[l].o_ptr), p.K, grads, p.pstride,
                                         y.w_int, (int64_t)y.fi * y.ldw, ctx->stream);
         });
         if (l > 0 && agg_first) {
@@ -580,8 +587,8 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
             GAD_RUN("gemm_dh", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
                 if (ctx->use_tc)
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 3], &ctx->maps[kMapsPerLayer * l + 4], &ctx->maps[kMapsPerLayer * l + 5], 1,
-                                               ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G2, y.ldi, ctx->at<RowSpan>(p.o_tiles),
-                                               (int)p.tiles.size(), nullptr, 0, 1.f, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
+                                               ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G2, y.ldi, ctx->at<RowSpan>(p.o_pair_tiles),
+                                               (int)(p.pair_tiles.size() / 2), nullptr, 0, 1.f, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
                                                ctx->num_sms, ctx->stream, ctx->same_params);
                 return launch_gemm_rows_simt(1, G1, y.ldo, y.fo, params, pstride, y.w_int, y.ldw, y.fi, G2, y.ldi,
                                              ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, nullptr, ctx->stream);
@@ -598,8 +605,8 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
             GAD_RUN("gemm_dh", l, 4.0 * p.Np * (2.0 * y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
                 if (ctx->use_tc)
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 3], &ctx->maps[kMapsPerLayer * l + 4], &ctx->maps[kMapsPerLayer * l + 5], 1,
-                                               ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G1, y.ldi, ctx->at<RowSpan>(p.o_tiles),
-                                               (int)p.tiles.size(), ctx->H(l), y.ldi, scale, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
+                                               ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G1, y.ldi, ctx->at<RowSpan>(p.o_pair_tiles),
+                                               (int)(p.pair_tiles.size() / 2), ctx->H(l), y.ldi, scale, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
                                                ctx->num_sms, ctx->stream, ctx->same_params);
                 return launch_gemm_rows_simt(1, G2, y.ldo, y.fo, params, pstride, y.w_int, y.ldw, y.fi, G1, y.ldi,
                                              ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), ctx->H(l), y.ldi, scale, nullptr,
@@ -740,8 +747,10 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
     if (rc != GAD_OK) return fail(ctx, rc, ctx->err);
     ctx->cfg.dims = ctx->p.dims.data();
     const Plan& p = ctx->p;
-    ctx->pinned_bytes = std::max(p.o_flags + 16 - p.o_loss, 8 * (size_t)p.K);
+    const size_t report_bytes = (size_t)round_up((int64_t)std::max(p.o_flags + 16 - p.o_loss, 8 * (size_t)p.K), 128);
+    ctx->pinned_bytes = 2 * report_bytes;
     if (!(ctx->pinned = take_small_pinned(ctx->pinned_bytes))) return fail(ctx, GAD_ERR_OOM, "no pinned host memory");
+    ctx->published = reinterpret_cast<float*>(ctx->pinned + report_bytes);
     if (workspace_bytes < p.bytes) return fail(ctx, GAD_ERR_OOM, "workspace smaller than gad_workspace_bytes");
     const int C = p.dims[p.L];
     for (int32_t u = 0; u < g->n; ++u) {
@@ -801,12 +810,13 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
     if ((rc = upload(ctx, p.o_sub_off, st.sub_off)) || (rc = upload(ctx, p.o_gid, st.gid)) || (rc = upload(ctx, p.o_deg, st.deg)) ||
         (rc = upload(ctx, p.o_label, label)) || (rc = upload(ctx, p.o_train, train)) || (rc = upload(ctx, p.o_deg_sum, deg_sum)) ||
         (rc = upload(ctx, p.o_deg_sq, deg_sq)) || (rc = upload(ctx, p.o_inv_ntrain, inv_ntrain)) ||
-        (rc = upload(ctx, p.o_tiles, p.tiles)) || (rc = upload(ctx, p.o_chunks, p.chunks)) ||
-        (rc = upload(ctx, p.o_chunk_ptr, p.chunk_ptr)) || (rc = upload(ctx, p.o_dw_chunks, p.dw_chunks)) ||
-        (rc = upload(ctx, p.o_dw_chunk_ptr, p.dw_chunk_ptr)) || (rc = upload(ctx, p.o_core_spans, p.core_spans)) ||
+        (rc = upload(ctx, p.o_pair_tiles, p.pair_tiles)) || (rc = upload(ctx, p.o_tiles, p.tiles)) || (rc = upload(ctx, p.o_chunks, p.chunks)) ||
+        (rc = upload(ctx, p.o_chunk_ptr, p.chunk_ptr)) || (rc = upload(ctx, p.o_core_spans, p.core_spans)) ||
         (rc = upload(ctx, p.o_pair_ptr, p.pair_ptr)) || (rc = upload(ctx, p.o_gram_ptr, p.gram_ptr)) || (rc = upload(ctx, p.o_nchunks, p.nchunks)) ||
         (rc = upload(ctx, p.o_nchunk_ptr, p.nchunk_ptr)))
         return rc;
+    for (const Plan::DwChunks& d : p.dw)
+        if ((rc = upload(ctx, d.o_spans, d.spans)) || (rc = upload(ctx, d.o_ptr, d.ptr))) return rc;
     // features: graph order -> staging -> store-row order with zero pad columns
     GAD_CK(cudaMemcpyAsync(ctx->ws + p.o_stage, X, 4 * (size_t)g->n * p.dims[0], cudaMemcpyHostToDevice, ctx->stream));
     GAD_CK(launch_gather_rows(ctx->at<float>(p.o_stage), p.dims[0], ctx->at<int32_t>(p.o_gid), p.Np, ctx->H(0), p.ld[0], ctx->stream));
@@ -838,6 +848,7 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
                                                       std::to_string(kZetaPairMaxRows) + " rows");
     }
     if (ctx->use_tc) {
+        const int npairs = (int)(p.pair_tiles.size() / 2);
         ctx->maps.resize((size_t)kMapsPerLayer * p.L);
         bool ok = true;
         for (int l = 0; l < p.L && ok; ++l) {
@@ -851,12 +862,12 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
             const bool agg_first = p.agg_first[l] != 0;   // then the transform and the weight gradient read A~ H^(l), dW and dH read dPre (G1)
             float* Hin = agg_first ? ctx->at<float>(p.o_P[l]) : ctx->H(l);
             ok = ok && tc_make_map(&m[0], Hin, y.fi, p.Np, 0, 4ull * y.ldi, 0, 128);
-            ok = ok && tc_make_map(&m[1], ctx->at<float>(p.o_wt_hi[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, tc_bn_for(y.fo));
-            ok = ok && tc_make_map(&m[2], ctx->at<float>(p.o_wt_lo[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, tc_bn_for(y.fo));
+            ok = ok && tc_make_map(&m[1], ctx->at<float>(p.o_wt_hi[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, tc_rows_bn(y.fo, npairs) / 2);
+            ok = ok && tc_make_map(&m[2], ctx->at<float>(p.o_wt_lo[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, tc_rows_bn(y.fo, npairs) / 2);
             // input gradient: A = dZ [Np x fo] (in G2), B = W copies [K][fi][fo]
             ok = ok && tc_make_map(&m[3], ctx->at<float>(agg_first ? p.o_G1 : p.o_G2), y.fo, p.Np, 0, 4ull * y.ldo, 0, 128);
-            ok = ok && tc_make_map(&m[4], ctx->at<float>(p.o_w_hi[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, tc_bn_for(y.fi));
-            ok = ok && tc_make_map(&m[5], ctx->at<float>(p.o_w_lo[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, tc_bn_for(y.fi));
+            ok = ok && tc_make_map(&m[4], ctx->at<float>(p.o_w_hi[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, tc_rows_bn(y.fi, npairs) / 2);
+            ok = ok && tc_make_map(&m[5], ctx->at<float>(p.o_w_lo[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, tc_rows_bn(y.fi, npairs) / 2);
             // weight gradient: 32-row tiles of H^(l) and of dZ (in G2)
             ok = ok && tc_make_map(&m[6], Hin, y.fi, p.Np, 0, 4ull * y.ldi, 0, tc_tn_rows(), true);
             ok = ok && tc_make_map(&m[7], ctx->at<float>(agg_first ? p.o_G1 : p.o_G2), y.fo, p.Np, 0, 4ull * y.ldo, 0, tc_tn_rows(), true);
@@ -881,14 +892,22 @@ int gad_default_params(int32_t L, const int32_t* dims, uint64_t seed, float* out
     return GAD_OK;
 }
 
+static int take_report(gad_ctx* ctx, const char* report, float* loss_out);
+
 int gad_get_loss(gad_ctx* ctx, float* loss_out) {
     if (!ctx || !loss_out) return GAD_ERR_ARG;
     const Plan& p = ctx->p;
-    int32_t flags[3];
     GAD_CK(cudaMemcpyAsync(ctx->pinned, ctx->ws + p.o_loss, p.o_flags + 12 - p.o_loss, cudaMemcpyDeviceToHost, ctx->stream));
     GAD_CK(cudaStreamSynchronize(ctx->stream));
-    std::memcpy(loss_out, ctx->pinned, 4 * (size_t)(p.K + 1));
-    std::memcpy(flags, ctx->pinned + (p.o_flags - p.o_loss), 12);
+    return take_report(ctx, ctx->pinned, loss_out);
+}
+
+// The losses and error words in `report`, host memory laid out as in the workspace.
+static int take_report(gad_ctx* ctx, const char* report, float* loss_out) {
+    const Plan& p = ctx->p;
+    int32_t flags[3];
+    std::memcpy(loss_out, report, 4 * (size_t)(p.K + 1));
+    std::memcpy(flags, report + (p.o_flags - p.o_loss), 12);
     settle(ctx, flags);
     const int32_t flag = flags[0];
     if (flags[1]) {
@@ -939,7 +958,8 @@ static int enqueue_epoch(gad_ctx* ctx, bool consensus) {
     if (consensus)
         GAD_RUN("sgd_consensus", -1, 4.0 * ((ctx->same_params ? 1 : p.K) + p.K + 1) * p.Pint, 4.0 * p.K * p.Pint, [&] {
             return launch_sgd_consensus(ctx->at<float>(p.o_params), param_stride(ctx), ctx->at<float>(p.o_grads), p.pstride, p.pstride, p.K, ctx->cfg.lr,
-                                        ctx->at<double>(p.o_zeta), ctx->cfg.weighted, 1, ctx->at<int32_t>(p.o_flags), dropout_counter(ctx), ctx->stream);
+                                        ctx->at<double>(p.o_zeta), ctx->cfg.weighted, 1, ctx->at<int32_t>(p.o_flags), dropout_counter(ctx), ctx->at<float>(p.o_loss), ctx->published,
+                                        (int)((p.o_flags + 12 - p.o_loss) / 4), ctx->stream);
         });
     else if (dropout_counter(ctx))
         GAD_CK(launch_epoch_counter(dropout_counter(ctx), 0, true, ctx->stream));
@@ -985,6 +1005,7 @@ static void capture_epoch(gad_ctx* ctx, bool consensus, gad_ctx::EpochGraph& eg)
 
 static int train_epoch(gad_ctx* ctx, float* loss_out, bool consensus) {
     if (!ctx) return GAD_ERR_ARG;
+    const Plan& p = ctx->p;
     gad_ctx::EpochGraph& eg = ctx->graphs[consensus ? 1 : 0];
     bool done = false;
     if (dropout_counter(ctx) && ctx->epoch_dirty) {
@@ -1008,8 +1029,11 @@ static int train_epoch(gad_ctx* ctx, float* loss_out, bool consensus) {
     }
     if (consensus) copies_made_equal(ctx);
     ctx->epoch += 1;
-    if (loss_out) return gad_get_loss(ctx, loss_out);
-    return GAD_OK;
+    if (!loss_out) return GAD_OK;
+    if (!consensus || p.pstride == 0) return gad_get_loss(ctx, loss_out);
+    // the update kernel has left them in host memory: no copy to wait for behind it (8 us of a 2000-node epoch)
+    GAD_CK(cudaStreamSynchronize(ctx->stream));
+    return take_report(ctx, reinterpret_cast<const char*>(ctx->published), loss_out);
 }
 
 int gad_forward(gad_ctx* ctx, float* logits_out) {
@@ -1047,7 +1071,7 @@ int gad_consensus(gad_ctx* ctx) {
     if (rc != GAD_OK) return rc;
     GAD_RUN("consensus", -1, 4.0 * ((ctx->same_params ? 1 : p.K) + 1) * p.Pint, 2.0 * p.K * p.Pint, [&] {
         return launch_sgd_consensus(ctx->at<float>(p.o_params), param_stride(ctx), ctx->at<float>(p.o_grads), p.pstride, p.pstride, p.K, 0.f,
-                                    ctx->at<double>(p.o_zeta), ctx->cfg.weighted, 0, ctx->at<int32_t>(p.o_flags), nullptr, ctx->stream);
+                                    ctx->at<double>(p.o_zeta), ctx->cfg.weighted, 0, ctx->at<int32_t>(p.o_flags), nullptr, nullptr, nullptr, 0, ctx->stream);
     });
     copies_made_equal(ctx);
     return GAD_OK;

@@ -151,7 +151,7 @@ cudaError_t launch_gemm_rows_simt(int mode, const float* A, int lda, int Kd, con
 // Tensor-core (tcgen05) version of launch_gemm_rows_simt.  The operands come through TMA descriptors made by
 // tc_make_map (A: [rows x Kd]; B, B_lo: [K][N][Kd] copies written by launch_split_weights); passes = 3 gives fp32
 // accuracy by operand splitting, passes = 1 plain TF32 operands.  err receives a role code if a bounded wait runs out.
-int tc_bn_for(int n_cols);
+int tc_rows_bn(int n_cols, int npairs);
 int tc_tn_rows();   // rows of the row-box descriptors the weight-gradient kernel reads (mapH / mapZ of launch_gemm_tn_tc)
 bool tc_make_map(void* out_map, const void* base, uint64_t inner, uint64_t rows, uint64_t outer, uint64_t row_stride_bytes,
                  uint64_t outer_stride_bytes, uint32_t box_rows, bool mn_major = false);
@@ -165,16 +165,20 @@ struct SplitLayers {
     SplitLayer y[MAX];
 };
 cudaError_t launch_split_weights(const float* params, int64_t pstride, int K, const SplitLayer* layers, int L, cudaStream_t s);
-// one_b: the operand copies of replica 0 serve every subgraph.
+// pair_tiles: 2 npairs row tiles (at most 128 rows, or none), the two of a pair in the same subgraph; tc_rows_bn(n_cols, npairs) columns
+// per tile, half of them the rows of B's descriptor box.  one_b: the operand copies of replica 0 serve every subgraph.
 // Cbf16 (mode 0 only, may be null): the result goes there as bfloat16 [rows x ldc] INSTEAD of to C - the operand copy the
 // reduced-precision aggregation gathers, written by its producer.
 cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols,
-                                float* C, int ldc, const RowSpan* tiles, int ntiles, const float* Hmask, int ldh, float scale,
+                                float* C, int ldc, const RowSpan* pair_tiles, int npairs, const float* Hmask, int ldh, float scale,
                                 const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16 = nullptr);
 
 // Tensor-core version of launch_gemm_tn_simt; mapH / mapZ are row-box descriptors (tc_tn_rows rows) of H^(l) and dZ.
-cudaError_t launch_gemm_tn_tc(const void* mapH, const void* mapZ, int passes, int M, int n_cols, int ldw, const RowSpan* chunks,
-                              int nchunks, float* partial, int32_t* err, cudaStream_t s);
+struct TnShape { int cg, ntm, ntn, bn; };   // CTAs per work unit, output tiles (of 128 cg rows and bn columns)
+TnShape tn_shape(int fi, int ldw);
+int64_t tn_chunk_rows(const std::vector<int32_t>& sub_off, const TnShape& t, int fi, int ldw, int num_sms);
+cudaError_t launch_gemm_tn_tc(const void* mapH, const void* mapZ, int passes, int M, int ldw, const RowSpan* chunks, int nchunks, float* partial,
+                              int32_t* err, int num_sms, cudaStream_t s);
 
 // Backward transforms of a layer with at most 16 output columns as one stream on the FP32 ALUs (narrow.cu).  `chunks`
 // are runs of rows of one subgraph, one CTA each.  In one pass over H and dZ: dPre = (dZ W_k^T) masked by H > 0, times
@@ -238,9 +242,10 @@ cudaError_t launch_zeta_gram(const void* mapHi, const void* mapLo, const float* 
 
 // `epoch` (may be null): the device epoch counter, advanced by one.
 // pstride_p: floats between the replicas' parameters, 0 while they are equal (copy 0 then stands for all of them; the result always
-// goes to copy 0).  words: the context's error words {non-finite loss, wait that ran out, copies differ}.
+// goes to copy 0).  report_to (may be null): pinned host memory that receives the nreport words at `report`.  words: the context's error words {non-finite loss, wait that ran out, copies differ}.
 cudaError_t launch_sgd_consensus(float* params, int64_t pstride_p, const float* grads, int64_t pstride, int64_t len, int K, float lr,
-                                 const double* zeta, int weighted, int with_sgd, int32_t* words, long long* epoch, cudaStream_t s);
+                                 const double* zeta, int weighted, int with_sgd, int32_t* words, long long* epoch, const float* report, float* report_to,
+                                 int nreport, cudaStream_t s);
 // The device epoch counter on its own: + 1, or set to a value.
 cudaError_t launch_epoch_counter(long long* epoch, long long set_to, bool advance, cudaStream_t s);
 // One context's share of a consensus over several contexts: out = sum_k w_k (theta_k - lr grad_k) with w_k = zeta_k / total

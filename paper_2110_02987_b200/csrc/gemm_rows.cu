@@ -1,0 +1,424 @@
+// Grouped dense transforms on the 5th-generation tensor cores (tcgen05, accumulators in tensor memory):
+//   mode 0   Z_l  = H^(l) W_k^(l)                        (the H.W of the forward equation, Section 3.3)
+//   mode 1   dPre = (dZ_l W_k^(l)^T) masked by H^(l) > 0  (chain rule through the forward equation)
+//   mode 2   H^(l+1) = sigma((A~ H^(l)) W_k^(l) + b_k^(l)) with dropout: mode 0 finished in the epilogue, for a layer
+//            that aggregates before it transforms
+// All are C[rows x N] = A[rows x Kd] * B_k^T with A row-major (Kd contiguous) and B_k stored as N rows of Kd contiguous
+// values, i.e. both operands K-major.  Row tiles never cross a subgraph, so a tile uses one replica's B.
+//
+// fp32 accuracy from TF32 tensor cores: every operand value x is split into hi, a value with a 10-bit mantissa (exactly
+// representable in TF32), and lo = x - hi rounded to TF32, and the product is accumulated as A_hi B_hi + A_hi B_lo + A_lo B_hi
+// in fp32 (the dropped A_lo B_lo term and the rounding of lo are ~2^-20 relative).  B is split once per epoch by a small kernel
+// (hi = x rounded).  For A the tile as loaded is its own hi part, because the tensor core ignores the low 13 mantissa bits
+// of an fp32 operand (hi = x truncated); eight warps write only the lo tile beside it.  With passes = 1 only A B is issued
+// on the unsplit operands (TF32 operand precision).
+//
+// What bounds it is shared-memory bandwidth (128 B per clock and SM) under the tensor pipe, then HBM.  Per 32 values of the
+// reduction and 256 output columns the tensor pipe needs 1536 cycles.  One CTA alone moves 256 KB meanwhile (operand reads 144,
+// TMA 80, split 32) and another 32 for a drain that turns its tiles through shared memory: 2250 cycles.  Therefore
+//   - the CTAs of a cluster of two work as a pair (cta_group::2): each holds 128 rows of A and half of the B rows, and one
+//     MMA of M = 256 reads 4 KB of each from either CTA: 96 KB of operand reads and 48 of TMA instead of 144 and 80;
+//   - B stays in shared memory for all tiles of a CTA where it fits beside the ring (up to 256 columns x 128 values);
+//   - the drain reads tensor memory in the 16 x 256-bit shape, in which four lanes hold 32 consecutive bytes of a row: whole
+//     sectors go to global memory straight from the registers;
+//   - the ring of loaded tiles is separate from the two lo tiles, so that most of the space holds loads in flight (short
+//     reductions are a chain of TMA latency, split and MMA).
+// Before this kernel (one CTA per tile, B streamed, drain through shared memory) and with it, 525 000 rows: 100 -> 256 281 -> 165 us,
+// 256 -> 256 325 -> 282 us (the three passes alone: 252 us at the TF32 rate), 256 -> 47 167 -> 130 us; 110 000 rows, 128 -> 128:
+// 43 -> 29 us; 2843 rows, 1433 -> 128: 40 -> 27 us.
+// Roles of a CTA: warp 0 issues TMA loads, warps 2-9 split the A tile and tell the pair's leader, warp 1 of the leader
+// issues the MMAs, warps 10-17 drain.  Every mbarrier wait is bounded: on a time-out the CTA raises an error word, stops, meets its
+// peer at the cluster barrier, frees its tensor memory and returns.
+#include <cuda.h>
+
+#include "epilogue.cuh"
+#include "gad_internal.h"
+#include "tc_common.cuh"
+
+namespace gad {
+
+namespace {
+
+constexpr int BK = 32;                                    // values of the reduction per ring stage
+constexpr int A_BYTES = BM * BK * 4;                      // 16 KiB
+constexpr int MAX_STAGES = 8, MAX_LO = 4;
+constexpr int BAR_BYTES = 512;
+constexpr int DATA_BYTES = 232448 - 1024 - BAR_BYTES;     // 227 KiB less alignment and barriers
+constexpr int SMEM_BYTES = 232448;
+constexpr int SPLIT_WARPS = 8, EPI_WARPS = 8, EPI_WARP0 = 2 + SPLIT_WARPS;
+constexpr int THREADS = 32 * (EPI_WARP0 + EPI_WARPS);
+
+struct RowsArgs {
+    const RowSpan* tiles;     // an even number of them; tiles 2 p and 2 p + 1 belong to the same subgraph
+    int npairs, ntn, BN, Kd;
+    int nst, nlo;             // ring stages; lo tiles (2 or 4, at most nst: see the split)
+    int resident;             // B loaded once per (subgraph, column tile) instead of once per stage
+    float* C;
+    uint32_t* Cbf;            // mode 0: the result as bfloat16 (two values per word) instead of C, or null
+    int ldc;
+    const float* Hmask;
+    int ldh;
+    float scale;
+    int kmul;                 // 1: every subgraph has its own B; 0: one B for all (the replicas' parameters are equal)
+    int32_t* err;
+    ActEpi act;               // mode 2
+};
+
+// What the drain does with a value: nothing (mode 0, or 1 without a mask), bfloat16 (mode 0), the ReLU mask and dropout scale (mode
+// 1), bias and ReLU (mode 2), those with dropout.  A template parameter, like the number of passes: as branches inside the unrolled
+// drain they made the kernel wait for instructions, 10.7 us per 128 x 256 tile.
+enum Drain { kPlain, kBf16, kMask, kAct, kActDrop };
+
+// Tile t of the launch: resident, column tile by column tile (B changes rarely); otherwise the column tiles of a row tile
+// follow each other (A comes from L2 the second time).
+__device__ __forceinline__ void tile_of(const RowsArgs& a, int t, int& pair, int& n) {
+    if (a.resident) { n = t / a.npairs; pair = t % a.npairs; }
+    else { pair = t / a.ntn; n = t % a.ntn; }
+}
+
+template <int DRAIN, bool split>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
+gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBlo,
+                 const RowsArgs a) {
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw_addr = smem_u32(smem_raw);
+    const uint32_t pad = ((raw_addr + 1023u) & ~1023u) - raw_addr;   // the same in both CTAs (the 128B swizzle repeats every 1024 bytes)
+    uint8_t* sm = smem_raw + pad;
+    const uint32_t sm_addr = raw_addr + pad;
+    const uint32_t rank = cluster_rank();
+    const int nkb = (a.Kd + BK - 1) / BK;
+    const uint32_t b_bytes = (uint32_t)(a.BN / 2) * (BK * 4);              // this CTA's half of a B tile
+    constexpr uint32_t nb = split ? 2u : 1u;
+    const uint32_t off_lo = a.resident ? (uint32_t)nkb * b_bytes * nb : 0u;
+    const uint32_t off_ring = off_lo + (split ? (uint32_t)a.nlo * A_BYTES : 0u);
+    const uint32_t stage_bytes = (uint32_t)A_BYTES + (a.resident ? 0u : nb * b_bytes);
+    const int nst = a.nst;
+    const uint32_t bars = sm_addr + DATA_BYTES;
+    auto full = [&](int s) { return bars + 8u * s; };
+    auto empty = [&](int s) { return bars + 8u * (MAX_STAGES + s); };
+    auto xfull = [&](int q) { return bars + 8u * (2 * MAX_STAGES + q); };              // leader: both CTAs' operands of this step are ready
+    auto loempty = [&](int q) { return bars + 8u * (2 * MAX_STAGES + MAX_LO + q); };
+    auto tfull = [&](int i) { return bars + 8u * (2 * MAX_STAGES + 2 * MAX_LO + i); };
+    auto tempty = [&](int i) { return bars + 8u * (2 * MAX_STAGES + 2 * MAX_LO + 2 + i); };
+    const uint32_t bfull = bars + 8u * (2 * MAX_STAGES + 2 * MAX_LO + 4), bempty = bfull + 8u;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + DATA_BYTES + 8 * (2 * MAX_STAGES + 2 * MAX_LO + 6));
+    volatile uint32_t* abort_flag = tmem_slot + 1;
+    const uint32_t tmem_cols = a.BN < 16 ? 32u : 2u * (uint32_t)a.BN;
+
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (uniform, and known to be)
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
+        for (int q = 0; q < MAX_LO; ++q) { mbar_init(xfull(q), 2 * SPLIT_WARPS / (a.nlo == MAX_LO ? MAX_LO : 1)); mbar_init(loempty(q), 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(tfull(i), 1); mbar_init(tempty(i), 2 * EPI_WARPS); }
+        mbar_init(bfull, 1); mbar_init(bempty, 1);
+        *abort_flag = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) tmem_alloc2(smem_u32(tmem_slot), tmem_cols);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_sync();           // the peer's barriers exist before anything arrives at them
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = *tmem_slot;
+
+    // contiguous ranges of tiles: B changes as rarely as possible
+    const int ntiles = a.npairs * a.ntn, ncl = gridDim.x >> 1, cl = blockIdx.x >> 1;
+    const int t_begin = (int)((long long)ntiles * cl / ncl), t_end = (int)((long long)ntiles * (cl + 1) / ncl);
+    // calls f(tile, pair, n, B differs from the previous tile's) until it returns false
+    auto for_tiles = [&](auto&& f) {
+        int last_k = -1, last_n = -1;
+        for (int t = t_begin; t < t_end; ++t) {
+            int pair, n;
+            tile_of(a, t, pair, n);
+            const int k = a.kmul ? a.tiles[2 * pair].k : 0;
+            if (!f(pair, n, k, k != last_k || n != last_n)) return;
+            last_k = k; last_n = n;
+        }
+    };
+
+    if (warp == 0 && lane == 0) {
+        // ---------------- TMA producer ----------------
+        int stage = 0;
+        uint32_t phase = 0, bphase = 0;
+        for_tiles([&](int pair, int n, int k, bool new_b) {
+            const int row0 = a.tiles[2 * pair + (int)rank].row0, n0 = n * a.BN + (int)rank * (a.BN / 2);
+            if (a.resident && new_b) {
+                if (!mbar_wait(bempty, bphase ^ 1u, abort_flag, a.err, 1)) return false;
+                bphase ^= 1u;
+                mbar_expect_tx(bfull, (uint32_t)nkb * nb * b_bytes);
+                for (int kb = 0; kb < nkb; ++kb) {
+                    tma_load_3d(sm_addr + (uint32_t)kb * nb * b_bytes, &tmB, kb * BK, n0, k, bfull);
+                    if (split) tma_load_3d(sm_addr + ((uint32_t)kb * nb + 1u) * b_bytes, &tmBlo, kb * BK, n0, k, bfull);
+                }
+            }
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!mbar_wait(empty(stage), phase ^ 1u, abort_flag, a.err, 2)) return false;
+                mbar_expect_tx(full(stage), stage_bytes);
+                const uint32_t base = sm_addr + off_ring + (uint32_t)stage * stage_bytes;
+                tma_load_2d(base, &tmA, kb * BK, row0, full(stage));
+                if (!a.resident) {
+                    tma_load_3d(base + A_BYTES, &tmB, kb * BK, n0, k, full(stage));
+                    if (split) tma_load_3d(base + A_BYTES + b_bytes, &tmBlo, kb * BK, n0, k, full(stage));
+                }
+                if (++stage == nst) { stage = 0; phase ^= 1u; }
+            }
+            return true;
+        });
+    } else if (warp == 1 && rank == 0) {
+        // ---------------- MMA issuer (leader of the pair) ----------------
+        // The whole warp runs the loop and one elected lane issues: everything the MMAs take then stays in uniform registers, where
+        // the instruction wants it (with a loop of one lane alone an MMA took 75 cycles to issue).
+        int stage = 0, q = 0, acc = 0;
+        uint32_t qphase = 0, acc_phase = 0;
+        const uint32_t idesc = instr_desc(a.BN, 2 * BM);
+        bool first = true;
+        for_tiles([&](int, int, int, bool new_b) {
+            if (a.resident && new_b && !first && elect_one()) mma_commit2(bempty);   // every MMA on the previous B has been issued
+            first = false;
+            if (!__all_sync(0xffffffffu, mbar_wait(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 3))) return false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t d = tmem_base + (uint32_t)(acc * a.BN);
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!__all_sync(0xffffffffu, mbar_wait(xfull(q), qphase, abort_flag, a.err, 4))) return false;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t base = sm_addr + off_ring + (uint32_t)stage * stage_bytes;
+                const uint32_t bbase = a.resident ? sm_addr + (uint32_t)kb * nb * b_bytes : base + A_BYTES;
+                const uint64_t a_hi = smem_desc(base), a_lo = smem_desc(sm_addr + off_lo + (uint32_t)q * A_BYTES);
+                const uint64_t b_hi = smem_desc(bbase), b_lo = smem_desc(bbase + b_bytes);
+                const int nks = min(BK / 8, (a.Kd - kb * BK + 7) / 8);
+                if (elect_one()) {
+                    // 8 TF32 values = 32 bytes = 2 descriptor units along K
+#pragma unroll
+                    for (int ks = 0; ks < BK / 8; ++ks) {
+                        if (ks < nks) {
+                            mma_tf32_pair(d, a_hi + 2 * ks, b_hi + 2 * ks, idesc, (kb | ks) != 0 ? 1u : 0u);
+                            if (split) {
+                                mma_tf32_pair(d, a_hi + 2 * ks, b_lo + 2 * ks, idesc, 1u);
+                                mma_tf32_pair(d, a_lo + 2 * ks, b_hi + 2 * ks, idesc, 1u);
+                            }
+                        }
+                    }
+                    mma_commit2(empty(stage));     // the stage may be refilled, and the lo tile rewritten, in both CTAs once these MMAs
+                    mma_commit2(loempty(q));       // have read them
+                    if (kb == nkb - 1) mma_commit2(tfull(acc));   // accumulator complete, in both CTAs
+                }
+                __syncwarp();
+                if (++stage == nst) stage = 0;
+                if (++q == a.nlo) { q = 0; qphase ^= 1u; }
+            }
+            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            return true;
+        });
+    } else if (warp >= 2 && warp < EPI_WARP0) {
+        // ---------------- A split: lo = x - (x as the tensor core reads it); the pair's leader is told ----------------
+        // With two lo tiles (wide outputs: the tensor pipe sets the pace) all warps share a step.  With four they form four groups
+        // that take turns: what a step costs is then mostly waiting - for the barriers, the proxy fence and the arrival - so four
+        // steps are in hand at a time.  (A group's wait for a ring stage is unambiguous because nlo <= nst: once its own previous
+        // step has been multiplied, so has the step before in that stage.)
+        const int groups = a.nlo == MAX_LO ? MAX_LO : 1, gw = SPLIT_WARPS / groups, group = (warp - 2) / gw, tt = threadIdx.x - 64 - 32 * gw * group;
+        int stage = 0, q = 0;
+        uint32_t phase = 0, qphase = 0, bphase = 0;
+        for_tiles([&](int, int, int, bool new_b) {
+            // (the votes keep the warp together: lanes may see a time-out or an abort at different polls)
+            if (a.resident && new_b) {
+                if (!__all_sync(0xffffffffu, mbar_wait(bfull, bphase, abort_flag, a.err, 5))) return false;
+                bphase ^= 1u;
+            }
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (groups == 1 || q == group) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(loempty(q), qphase ^ 1u, abort_flag, a.err, 6))) return false;
+                    if (!__all_sync(0xffffffffu, mbar_wait(full(stage), phase, abort_flag, a.err, 7))) return false;
+                    if (split) {
+                        const float4* hi = reinterpret_cast<const float4*>(sm + off_ring + (uint32_t)stage * stage_bytes);
+                        float4* lo = reinterpret_cast<float4*>(sm + off_lo + (uint32_t)q * A_BYTES);
+#pragma unroll 4
+                        for (int i = tt; i < A_BYTES / 16; i += 32 * gw) {
+                            const float4 v = hi[i];   // stays where it is: the MMA reads it as the hi part
+                            lo[i] = make_float4(tf32_rest(v.x), tf32_rest(v.y), tf32_rest(v.z), tf32_rest(v.w));
+                        }
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tensor-core reads
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_leader(xfull(q));
+                }
+                if (++q == a.nlo) { q = 0; qphase ^= 1u; }
+                if (++stage == nst) { stage = 0; phase ^= 1u; }
+            }
+            return true;
+        });
+    } else if (warp >= EPI_WARP0) {
+        // ---------------- epilogue: tensor memory -> registers -> global ----------------
+        // This warp may read tensor-memory lanes 32 q .. 32 q + 31; the two warps of a quarter take alternate blocks of 32 columns.
+        // In a 16 x 256-bit read lane t gets, of every 8 columns, columns 2 (t % 4) and the next one of rows t / 4 and t / 4 + 8.
+        const int quarter = warp & 3, half = (warp - EPI_WARP0) >> 2;
+        const int sub_r = lane >> 2, sub_c = 2 * (lane & 3);
+        int acc = 0;
+        uint32_t acc_phase = 0;
+        for_tiles([&](int pair, int n, int, bool) {
+            const RowSpan sp = a.tiles[2 * pair + (int)rank];
+            const int n0 = n * a.BN;
+            const int r0 = quarter * 32 + sub_r;                 // this lane's rows: r0 + 8 i
+            float2 hm[4][4];
+            auto fetch_mask = [&](int c0) {
+                const int nc = n0 + c0 + sub_c, ng = min(4, (min(a.BN - c0, a.ldc - n0 - c0) - sub_c + 7) >> 3);
+                const float* h = a.Hmask + ((long long)sp.row0 + r0) * a.ldh + nc;
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+                        hm[i][g] = r0 + 8 * i < sp.nrows && g < ng ? __ldg(reinterpret_cast<const float2*>(h + 8 * i * a.ldh + 8 * g)) : make_float2(0.f, 0.f);
+            };
+            if (!__all_sync(0xffffffffu, mbar_wait(tfull(acc), acc_phase, abort_flag, a.err, 8))) return false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int c0 = 32 * half; c0 < a.BN && n0 + c0 < a.ldc; c0 += 64) {
+                const int nc = n0 + c0 + sub_c;                  // this lane's columns: nc + 8 g, nc + 8 g + 1
+                const int ng = min(4, (min(a.BN - c0, a.ldc - n0 - c0) - sub_c + 7) >> 3);   // groups it has columns in
+                const long long at0 = ((long long)sp.row0 + r0) * a.ldc + nc;
+                float2 bias[4];
+                if (DRAIN == kMask) fetch_mask(c0);
+                if (DRAIN == kAct || DRAIN == kActDrop)
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) bias[g] = g < ng ? load_bias2(a.act, sp.k, nc + 8 * g) : make_float2(0.f, 0.f);
+                float2 v[4][4];                                  // [row r0 + 8 i][columns nc + 8 g]
+                const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * a.BN + c0);
+                if (a.BN >= 32) tmem_ld_16x256b_x4(t0, v);
+                else tmem_ld_16x256b_x2(t0, v);
+                if (DRAIN == kMask) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            v[i][g].x = hm[i][g].x > 0.f ? v[i][g].x * a.scale : 0.f;
+                            v[i][g].y = hm[i][g].y > 0.f ? v[i][g].y * a.scale : 0.f;
+                        }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (r0 + 8 * i >= sp.nrows) break;
+                    uint64_t key = 0;
+                    if (DRAIN == kActDrop) key = dropout_row_key(a.act, (long long)sp.row0 + r0 + 8 * i);
+                    const long long at = at0 + 8 * i * a.ldc;
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        float2 o = v[i][g];
+                        if (DRAIN == kAct || DRAIN == kActDrop) {
+                            o.x = relu_unless(o.x + bias[g].x, a.act.relu);
+                            o.y = relu_unless(o.y + bias[g].y, a.act.relu);
+                        }
+                        if (DRAIN == kActDrop) {
+                            o.x = dropout_keep(key, nc + 8 * g, a.act.thr) ? o.x * a.act.scale : 0.f;
+                            o.y = dropout_keep(key, nc + 8 * g + 1, a.act.thr) ? o.y * a.act.scale : 0.f;
+                        }
+                        if (g < ng) {
+                            if (DRAIN == kBf16) a.Cbf[(at + 8 * g) >> 1] = bf16_bits(o.x) | (bf16_bits(o.y) << 16);
+                            else *reinterpret_cast<float2*>(a.C + at + 8 * g) = o;
+                        }
+                    }
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive_leader(tempty(acc));
+            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            return true;
+        });
+    }
+
+    // Tear-down.  After a time-out, give loads that may still be in flight a bounded chance to land before the shared memory is
+    // released.  Neither CTA leaves while the other may still read its operands or arrive at its barriers.
+    __syncthreads();
+    if (*abort_flag && threadIdx.x == 0)
+        for (int s = 0; s < nst; ++s)
+            for (uint32_t i = 0; i < 4096u; ++i)
+                if (mbar_try_wait(full(s), 0) || mbar_try_wait(full(s), 1)) break;
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_sync();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tmem_dealloc2(tmem_base, tmem_cols);
+    }
+}
+
+}  // namespace
+
+namespace {
+
+// Where the data of a CTA goes: four lo tiles if at least as many ring stages fit beside them, else two; B resident if at least
+// three ring stages fit beside it.
+void rows_layout(int BN, int Kd, int passes, RowsArgs& a) {
+    const int nkb = (Kd + BK - 1) / BK, nb = passes > 1 ? 2 : 1;
+    const int b_bytes = BN / 2 * (BK * 4);
+    for (a.nlo = 4;; a.nlo = 2) {
+        const long long room = (long long)DATA_BYTES - (passes > 1 ? a.nlo * A_BYTES : 0), room_a = room - (long long)nkb * nb * b_bytes;
+        a.resident = room_a >= (a.nlo > 3 ? a.nlo : 3) * A_BYTES ? 1 : 0;
+        const long long n = a.resident ? room_a / A_BYTES : room / (A_BYTES + nb * b_bytes);
+        a.nst = (int)(n < MAX_STAGES ? n : MAX_STAGES);
+        // (a resident B with two lo tiles is worth more than a streamed one with four)
+        if (a.nlo == 2 || (a.nst >= 4 && (a.resident || (long long)DATA_BYTES - 2 * A_BYTES - (long long)nkb * nb * b_bytes < 3 * A_BYTES))) return;
+    }
+}
+
+// Clusters of two CTAs that fit the GPU at once (a cluster stays inside a GPC).
+int max_clusters(int num_sms) {
+    static std::atomic<int> known{0};
+    int c = known.load();
+    if (c > 0) return c;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)num_sms); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = SMEM_BYTES; cfg.attrs = attr; cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&c, gemm_rows_kernel<kPlain, true>, &cfg) != cudaSuccess || c < 1) { cudaGetLastError(); c = num_sms / 2; }
+    known.store(c);
+    return c;
+}
+
+}  // namespace
+
+// Output columns per tile.  An MMA of M = 256, K = 8 costs about the same for any N up to 128 and twice that at 256, and every column
+// tile reads and splits A again, so the widest tile is the cheapest - unless the launch has so few row tiles that most SMs would
+// idle: then the columns are spread over more CTAs, down to 32 (2843 rows x 1433 -> 128: 24 row tiles, 40 us with 128 columns per
+// tile, 27 us with 32).
+int tc_rows_bn(int n_cols, int npairs) {
+    int bn = n_cols <= 16 ? 16 : n_cols <= 32 ? 32 : n_cols <= 64 ? 64 : n_cols <= 128 ? 128 : 256;
+    while (bn > 32 && (long long)npairs * ((n_cols + bn - 1) / bn) * 2 <= 74) bn /= 2;
+    return bn;
+}
+
+cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols,
+                                float* C, int ldc, const RowSpan* pair_tiles, int npairs, const float* Hmask, int ldh, float scale,
+                                const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16) {
+    if (npairs <= 0) return cudaSuccess;
+    if ((mode == 2 && !act) || (Cbf16 && mode != 0)) return cudaErrorInvalidValue;
+    RowsArgs a;
+    a.tiles = pair_tiles; a.npairs = npairs; a.BN = tc_rows_bn(n_cols, npairs); a.ntn = (ldc + a.BN - 1) / a.BN; a.Kd = Kd;
+    rows_layout(a.BN, Kd, passes, a);
+    a.C = C; a.Cbf = reinterpret_cast<uint32_t*>(Cbf16); a.ldc = ldc; a.Hmask = Hmask; a.ldh = ldh; a.scale = scale;
+    a.kmul = one_b ? 0 : 1; a.err = err;
+    a.act = act ? *act : ActEpi{};
+    const long long total = (long long)npairs * a.ntn;
+    const int cl = max_clusters(num_sms);
+    const unsigned grid = 2u * (unsigned)(total < cl ? total : cl);
+    const int drain = mode == 2 ? (a.act.drop ? kActDrop : kAct) : mode == 1 && Hmask ? kMask : Cbf16 ? kBf16 : kPlain;
+    auto go = [&](auto kernel) {
+        cudaError_t e = configure_kernel_once(reinterpret_cast<const void*>(kernel), SMEM_BYTES, false);
+        if (e != cudaSuccess) return e;
+        kernel<<<grid, THREADS, SMEM_BYTES, s>>>(*reinterpret_cast<const CUtensorMap*>(mapA), *reinterpret_cast<const CUtensorMap*>(mapB),
+                                                 *reinterpret_cast<const CUtensorMap*>(mapBlo), a);
+        ++g_kernel_launches;
+        return cudaGetLastError();
+    };
+#define GAD_DRAIN(D) case D: return passes > 1 ? go(gemm_rows_kernel<D, true>) : go(gemm_rows_kernel<D, false>)
+    switch (drain) {
+        GAD_DRAIN(kPlain);
+        GAD_DRAIN(kBf16);
+        GAD_DRAIN(kMask);
+        GAD_DRAIN(kAct);
+        GAD_DRAIN(kActDrop);
+    }
+#undef GAD_DRAIN
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace gad

@@ -1,0 +1,43 @@
+"""The paired tensor-core transforms at the edges of their tiles: rows that leave the second CTA of a pair empty, one row, full or
+ragged; reductions one value around a ring stage, columns around a tile, B resident or streamed, two or four lo tiles; replicas
+with parameters of their own; the ReLU mask, dropout and bfloat16 drains."""
+import numpy as np
+import pytest
+
+import __graft_entry__ as entry
+from conftest import small_random_case, rel_err
+from test_gpu_parity import make_pair, oracle_step, TOL
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    entry.build()
+
+
+@pytest.mark.parametrize("rows", [1, 127, 128, 129, 256, 257])
+@pytest.mark.parametrize("dims,kw", [
+    ((31, 17, 5), {}), ((33, 130, 16, 3), {}), ((700, 33, 2), {}), ((129, 256, 257, 4), dict(flags=4)),
+    ((300, 300, 64, 9), dict(flags=4, dropout=0.3)), ((64, 512, 40), dict(gemm_mode=1)), ((1433, 64, 40, 7), dict(gemm_mode=1, flags=4))])
+def test_row_and_column_edges(rows, dims, kw):
+    K = 3
+    case = small_random_case(rows, n=rows * K + 3, K=K, p=min(0.3, 4.0 / (rows * K)), halo=False)
+    tol = 5e-2 if kw.get("gemm_mode") else TOL
+    g, ref, _ = make_pair(case, dims, rows, lr=1e-3, **kw)   # (a longer step saturates the loss of a single row)
+    with g:
+        rng = np.random.default_rng(1)
+        if not kw.get("gemm_mode"):   # every replica its own parameters, before the first consensus makes them equal
+            for k in range(K):
+                theta = (ref.get_params(k) + 0.05 * rng.standard_normal(g.P)).astype(np.float32)
+                g.set_params(k, theta)
+                ref.set_params(k, theta)
+        for _ in range(2):
+            lg = g.train_epoch()
+            lr, _ = oracle_step(g, ref, tol)
+            assert np.max(np.abs(lg - lr)) <= (1e-4 if tol == TOL else 5e-2)
+        for l in range(1, len(dims)):
+            assert rel_err(g.get_activation(l), ref.activation(l)) <= tol
+        for k in range(K):
+            assert rel_err(g.get_grads(k), ref.get_grads(k)) <= tol
+            assert rel_err(g.get_params(k), ref.get_params(k)) <= tol

@@ -294,7 +294,7 @@ struct gad_ctx {
     cudaStream_t capture_stream = nullptr;   // epochs are captured on it, whatever stream they are launched on
     cudaStream_t copy_stream = nullptr;   // host -> device copies of gad_set_inputs
     cudaStream_t side_stream = nullptr;   // small kernels of an epoch that depend on little (operand split, zeta, bias gradients)
-    cudaEvent_t ev_fork = nullptr, ev_split = nullptr, ev_g1 = nullptr, ev_bias = nullptr, ev_join = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_g1 = nullptr, ev_bias = nullptr, ev_join = nullptr;
     cudaEvent_t ev_copied[2] = {nullptr, nullptr}, ev_gathered[2] = {nullptr, nullptr};
     int stage_idx = 0;              // staging pair the next gad_set_inputs uses
     bool hoist = false;             // keep A~ H^(0) across epochs (config flag bit 1)
@@ -406,12 +406,9 @@ int settle_now(gad_ctx* ctx) {
     return GAD_OK;
 }
 
-int forward_pass(gad_ctx* ctx, bool train, cudaStream_t ss) {
+// The operand copies of the weights that the tensor-core transforms read.
+int split_pass(gad_ctx* ctx) {
     const Plan& p = ctx->p;
-    float* Z = ctx->at<float>(p.o_G2);
-    const float* params = ctx->at<float>(p.o_params);
-    const int passes = ctx->cfg.gemm_mode == 0 ? 3 : 1;
-    const int64_t pstride = param_stride(ctx);
     if (ctx->use_tc) {
         std::vector<SplitLayer> sl((size_t)p.L);
         double weights = 0.0;
@@ -423,10 +420,18 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t ss) {
             weights += (plain ? 20.0 : 12.0) * y.fi * y.fo;
         }
         const int copies = ctx->same_params ? 1 : p.K;
-        GAD_RUN("split_weights", -1, weights * copies, 0.0, [&] { return launch_split_weights(params, pstride, copies, sl.data(), p.L, ss); });
+        GAD_RUN("split_weights", -1, weights * copies, 0.0, [&] { return launch_split_weights(ctx->at<float>(p.o_params), param_stride(ctx), copies, sl.data(), p.L, ctx->stream); });
     }
-    bool split_pending = ctx->use_tc && ss != ctx->stream;   // the first transform waits for the split operands
-    if (split_pending) GAD_CK(cudaEventRecord(ctx->ev_split, ss));
+    return GAD_OK;
+}
+
+// Every layer's forward step; split_pass comes before it.
+int forward_pass(gad_ctx* ctx, bool train) {
+    const Plan& p = ctx->p;
+    float* Z = ctx->at<float>(p.o_G2);
+    const float* params = ctx->at<float>(p.o_params);
+    const int passes = ctx->cfg.gemm_mode == 0 ? 3 : 1;
+    const int64_t pstride = param_stride(ctx);
     for (int l = 0; l < p.L; ++l) {
         const Layer& y = p.layers[l];
         Epilogue ep{params, pstride, y.b_int, ctx->at<int32_t>(p.o_sub_off), p.K, l < p.L - 1 ? 1 : 0,
@@ -439,7 +444,6 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t ss) {
                 if (l == 0) ctx->P_valid = true;
             }
             const ActEpi act = make_act(ep, 0);
-            if (split_pending) { GAD_CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_split, 0)); split_pending = false; }
             GAD_RUN("gemm_fwd", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
                 if (ctx->use_tc)
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 2, passes, y.fi, y.fo,
@@ -450,7 +454,6 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t ss) {
             });
             continue;
         }
-        if (split_pending) { GAD_CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_split, 0)); split_pending = false; }
         // reduced-precision mode: the transform writes the bfloat16 operand copy the aggregation gathers, and nothing else
         void* zb = ctx->use_tc ? bf16_of(ctx) : nullptr;
         GAD_RUN("gemm_fwd", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
@@ -471,8 +474,8 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t ss) {
 int zeta_pass(gad_ctx* ctx, cudaStream_t s) {
     const Plan& p = ctx->p;
     if (ctx->cfg.zeta_mode == 2 && !ctx->acts_valid) {   // asked for before any pass has run: an inference pass provides the activations
-        int rc = forward_pass(ctx, false, ctx->stream);
-        if (rc != GAD_OK) return rc;
+        int rc = split_pass(ctx);
+        if (rc != GAD_OK || (rc = forward_pass(ctx, false)) != GAD_OK) return rc;
     }
     if (ctx->cfg.zeta_mode == 1 && ctx->use_gram) {
         const double pairs = 128.0 * 128.0 * (double)p.gram_ptr[p.K];
@@ -733,7 +736,7 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
     ctx->hoist = (cfg->flags & 2) != 0;
     GAD_CK(cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking));
     GAD_CK(cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking));
-    for (cudaEvent_t* e : {&ctx->ev_fork, &ctx->ev_split, &ctx->ev_g1, &ctx->ev_bias, &ctx->ev_join})
+    for (cudaEvent_t* e : {&ctx->ev_fork, &ctx->ev_g1, &ctx->ev_bias, &ctx->ev_join})
         GAD_CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     for (int i = 0; i < 2; ++i) {
         GAD_CK(cudaEventCreateWithFlags(&ctx->ev_copied[i], cudaEventDisableTiming));
@@ -930,9 +933,11 @@ int gad_train_epoch_local(gad_ctx* ctx, float* loss_out) { return train_epoch(ct
 static int enqueue_epoch(gad_ctx* ctx, bool consensus) {
     const Plan& p = ctx->p;
     cudaStream_t ss = side_of(ctx);
-    int rc = hand_over(ctx, ctx->stream, ss, ctx->ev_fork);   // this epoch's side work follows everything enqueued so far
-    if (rc != GAD_OK) return rc;
-    if ((rc = forward_pass(ctx, true, ss)) != GAD_OK) return rc;
+    // The side work forks off behind the first kernel of the main sequence: as a second root of the graph it would come first, and
+    // the main sequence 10 us later.
+    int rc = split_pass(ctx);
+    if (rc != GAD_OK || (rc = hand_over(ctx, ctx->stream, ss, ctx->ev_fork)) != GAD_OK) return rc;
+    if ((rc = forward_pass(ctx, true)) != GAD_OK) return rc;
     // zeta beside the forward pass; with zeta_mode 2 it reads this pass's activations, so it follows it (beside the backward pass)
     if (ctx->cfg.zeta_mode == 2 && (rc = hand_over(ctx, ctx->stream, ss, ctx->ev_fork)) != GAD_OK) return rc;
     if (ss != ctx->stream && (rc = zeta_pass(ctx, ss)) != GAD_OK) return rc;
@@ -1039,8 +1044,8 @@ static int train_epoch(gad_ctx* ctx, float* loss_out, bool consensus) {
 int gad_forward(gad_ctx* ctx, float* logits_out) {
     if (!ctx || !logits_out) return GAD_ERR_ARG;
     const Plan& p = ctx->p;
-    int rc = forward_pass(ctx, false, ctx->stream);
-    if (rc != GAD_OK) return rc;
+    int rc = split_pass(ctx);
+    if (rc != GAD_OK || (rc = forward_pass(ctx, false)) != GAD_OK) return rc;
     const int C = p.dims[p.L];
     GAD_CK(cudaMemsetAsync(ctx->ws + p.o_stage, 0, 4 * (size_t)p.n * C, ctx->stream));
     GAD_CK(launch_scatter_core(ctx->H(p.L), p.ld[p.L], C, ctx->at<int32_t>(p.o_gid), ctx->at<RowSpan>(p.o_core_spans),
@@ -1365,7 +1370,7 @@ void gad_destroy(gad_ctx* ctx) {
     if (ctx->pinned) give_small_pinned(ctx->pinned, ctx->pinned_bytes);
     if (ctx->copy_stream) { cudaStreamSynchronize(ctx->copy_stream); cudaStreamDestroy(ctx->copy_stream); }
     if (ctx->side_stream) { cudaStreamSynchronize(ctx->side_stream); cudaStreamDestroy(ctx->side_stream); }
-    for (cudaEvent_t e : {ctx->ev_fork, ctx->ev_split, ctx->ev_g1, ctx->ev_bias, ctx->ev_join})
+    for (cudaEvent_t e : {ctx->ev_fork, ctx->ev_g1, ctx->ev_bias, ctx->ev_join})
         if (e) cudaEventDestroy(e);
     for (int i = 0; i < 2; ++i) {
         if (ctx->ev_copied[i]) cudaEventDestroy(ctx->ev_copied[i]);

@@ -61,6 +61,9 @@ struct Plan {
     size_t o_pair_tiles = 0;
     std::vector<RowSpan> tiles, chunks, core_spans;
     std::vector<int32_t> chunk_ptr;   // [K+1]
+    std::vector<RowSpan> zchunks;     // row chunks of the importance statistics, first chunk per subgraph [K+1]
+    std::vector<int32_t> zchunk_ptr;
+    size_t o_zchunks = 0, o_zchunk_ptr = 0;
     struct DwChunks { std::vector<RowSpan> spans; std::vector<int32_t> ptr; size_t o_spans = 0, o_ptr = 0; };
     std::vector<DwChunks> dw;         // [L] row chunks of each layer's weight gradient, their first chunk per subgraph [K+1]
     std::vector<int64_t> pair_ptr;    // [K+1] tiles of pairs per subgraph (zeta_mode 1 on the FP32 ALUs), else empty
@@ -78,6 +81,8 @@ struct Plan {
     std::vector<int32_t> nchunk_ptr;  // [K+1]
     size_t o_nchunks = 0, o_nchunk_ptr = 0, o_nw_partial = 0;
     size_t o_zeta_q = 0;              // [K] doubles: distance sums carried from layer to layer (zeta_mode 2)
+    size_t o_xbf16 = 0;               // [Np x ld_0] bfloat16 copy of the features, made when they are laid out (gemm_mode 1, layer 0 aggregating first)
+    size_t o_colsum = 0, o_cs_clusters = 0;   // column sums of the transforms' drains; first and last cluster per subgraph (one column tile)
     size_t o_bf16 = 0;                // [Np x widest SpMM operand] bfloat16 copy of the operand (gemm_mode 1), else unused
     size_t bytes = 0;
     // offsets into the workspace
@@ -139,6 +144,19 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
     const int64_t target = 592;
     int64_t R = round_up(std::max<int64_t>(1, (p.Np + target - 1) / target), 32);
     R = std::min<int64_t>(R, 16384);
+    // The importance statistics split their columns over CTAs as well: row chunks so that both together make about four CTAs per SM (each
+    // chunk's sums are read again when zeta is finished, and that kernel has one CTA per subgraph).
+    int32_t zcols = p.dims[0];
+    if (cfg->zeta_mode == 2)
+        for (int l = 0; l < p.L; ++l) zcols = std::max(zcols, p.dims[l]);
+    const int64_t ztarget = std::max<int64_t>(K, target / ((zcols + 127) / 128));
+    const int64_t Rz = std::max<int64_t>(32, round_up((p.Np + ztarget - 1) / ztarget, 32));
+    p.zchunk_ptr.assign(K + 1, 0);
+    for (int32_t k = 0; k < K; ++k) {
+        for (int64_t r = sub_off[k]; r < sub_off[k + 1]; r += Rz)
+            p.zchunks.push_back(RowSpan{(int32_t)r, (int32_t)std::min<int64_t>(Rz, sub_off[k + 1] - r), k, 0});
+        p.zchunk_ptr[k + 1] = (int32_t)p.zchunks.size();
+    }
     p.dw.resize(p.L);
     size_t dw_floats = 0;
     for (int l = 0; l < p.L; ++l) {
@@ -196,14 +214,19 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
     int32_t max_spmm_ld = 4;   // a layer's SpMMs run at its input width when it aggregates first, else at its output width
     for (int l = 0; l < p.L; ++l) max_spmm_ld = std::max(max_spmm_ld, p.ld[p.agg_first[l] ? l : l + 1]);
     p.o_spmm_scratch = take(cur, 4 * (size_t)slots * (size_t)max_spmm_ld);
-    if (cfg->gemm_mode == 1) p.o_bf16 = take(cur, 2 * Np * (size_t)max_spmm_ld);
+    if (cfg->gemm_mode == 1) {
+        p.o_bf16 = take(cur, 2 * Np * (size_t)max_spmm_ld);
+        if (p.agg_first[0]) p.o_xbf16 = take(cur, 2 * Np * (size_t)p.ld[0]);
+    }
+    p.o_colsum = take(cur, 4 * 8 * (size_t)(kMaxRowClusters + K) * (size_t)p.maxld); p.o_cs_clusters = take(cur, 8 * (size_t)K);
     p.o_G1 = take(cur, 4 * Np * (size_t)p.maxld); p.o_G2 = take(cur, 4 * Np * (size_t)p.maxld);
     p.o_params = take(cur, 4 * (size_t)K * (size_t)p.pstride); p.o_grads = take(cur, 4 * (size_t)K * (size_t)p.pstride);
     p.o_dw_partial = take(cur, 4 * dw_floats); p.o_cs_partial = take(cur, 4 * nc * (size_t)p.maxld);
     int32_t zeta_ld = p.ld[0];   // widest matrix the importance statistics run over: H^(0), or every layer's input (zeta_mode 2)
     if (cfg->zeta_mode == 2)
         for (int l = 0; l < p.L; ++l) zeta_ld = std::max(zeta_ld, p.ld[l]);
-    p.o_loss_partial = take(cur, 4 * nc); p.o_zeta_partial = take(cur, 8 * nc * 2 * (size_t)zeta_ld);
+    p.o_loss_partial = take(cur, 4 * nc); p.o_zeta_partial = take(cur, 8 * p.zchunks.size() * 2 * (size_t)zeta_ld);
+    p.o_zchunks = take(cur, sizeof(RowSpan) * p.zchunks.size()); p.o_zchunk_ptr = take(cur, 4 * (size_t)(K + 1));
     p.o_zeta_q = take(cur, 8 * (size_t)K);
     p.o_zeta = take(cur, 8 * (size_t)K); p.o_epoch = take(cur, 8);
     // what a waiting call reads lies together, so that it is one copy: losses and error words, zeta and the weights
@@ -366,6 +389,12 @@ int run(gad_ctx* ctx, const char* name, int layer, double bytes, double flops, F
 // Room for the bfloat16 copy of an aggregation's operand: the reduced-precision mode gathers from that copy.
 void* bf16_of(gad_ctx* ctx) { return ctx->cfg.gemm_mode == 1 ? (void*)(ctx->ws + ctx->p.o_bf16) : nullptr; }
 
+// The bfloat16 copy of the features for layer 0's aggregation.
+void* x_bf16(gad_ctx* ctx) { return ctx->p.o_xbf16 ? (void*)(ctx->ws + ctx->p.o_xbf16) : nullptr; }
+// Whether dPre^(l), the gradient at layer l's pre-activations, is wanted in bfloat16 alone: the reduced-precision mode, and nothing but the
+// backward aggregation reads it (`summed`: its producer sums its columns).
+bool dpre_bf16(const gad_ctx* ctx, int l, bool summed) { return ctx->cfg.gemm_mode == 1 && ctx->use_tc && !ctx->p.agg_first[l] && summed; }
+
 // Floats between the replicas' parameters as the kernels read them: copy 0 stands for all of them while they are equal.
 int64_t param_stride(const gad_ctx* ctx) { return ctx->same_params ? 0 : ctx->p.pstride; }
 
@@ -440,7 +469,10 @@ int forward_pass(gad_ctx* ctx, bool train) {
             // A~ (H W) = (A~ H) W: aggregate at the input width, finish the layer in the transform's epilogue
             if (!(l == 0 && ctx->hoist && ctx->P_valid)) {
                 GAD_RUN("spmm_fwd", l, spmm_bytes(p, y.fi), 2.0 * p.nnz * y.fi,
-                        [&] { return launch_spmm(ctx->A, ctx->H(l), y.ldi, ctx->at<float>(p.o_P[l]), y.ldi, y.fi, nullptr, bf16_of(ctx), false, ctx->stream); });
+                        [&] {
+                            void* xb = l == 0 ? x_bf16(ctx) : nullptr;
+                            return launch_spmm(ctx->A, ctx->H(l), y.ldi, ctx->at<float>(p.o_P[l]), y.ldi, y.fi, nullptr, xb ? xb : bf16_of(ctx), xb != nullptr, ctx->stream);
+                        });
                 if (l == 0) ctx->P_valid = true;
             }
             const ActEpi act = make_act(ep, 0);
@@ -506,8 +538,8 @@ int zeta_pass(gad_ctx* ctx, cudaStream_t s) {
     GAD_RUN("zeta", -1, 4.0 * p.Np * (cols + nl), 4.0 * p.Np * cols, [&] {
         for (int l = 0; l < nl; ++l) {
             const int phase = nl == 1 ? 0 : (l == 0 ? 1 : (l == nl - 1 ? 3 : 2));
-            cudaError_t e = launch_zeta(ctx->H(l), p.ld[l], p.dims[l], ctx->at<int32_t>(p.o_deg), ctx->at<RowSpan>(p.o_chunks),
-                                        (int)p.chunks.size(), ctx->at<int32_t>(p.o_chunk_ptr), ctx->at<int32_t>(p.o_sub_off), p.K,
+            cudaError_t e = launch_zeta(ctx->H(l), p.ld[l], p.dims[l], ctx->at<int32_t>(p.o_deg), ctx->at<RowSpan>(p.o_zchunks),
+                                        (int)p.zchunks.size(), ctx->at<int32_t>(p.o_zchunk_ptr), ctx->at<int32_t>(p.o_sub_off), p.K,
                                         ctx->at<int64_t>(p.o_deg_sum), ctx->at<int64_t>(p.o_deg_sq), ctx->cfg.beta,
                                         ctx->at<double>(p.o_zeta_partial), ctx->at<double>(p.o_zeta), ctx->at<double>(p.o_zeta_q), phase, s);
             if (e != cudaSuccess) return e;
@@ -530,6 +562,8 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
     const float scale = ctx->cfg.dropout > 0.f ? 1.f / (1.f - ctx->cfg.dropout) : 1.f;
     // whether this layer's dPre columns have been summed already: by the loss kernel, or by the layer above's fused narrow kernel
     bool bias_done = softmax_sums_columns(p.ld[p.L]);
+    bool in_bf16 = dpre_bf16(ctx, p.L - 1, bias_done);   // dPre of this layer is there as the bfloat16 operand copy only
+    const int npairs = (int)(p.pair_tiles.size() / 2);
     for (int l = p.L - 1; l >= 0; --l) {
         const Layer& y = p.layers[l];
         // the store of this layer's backward aggregation, and its entries
@@ -550,7 +584,8 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
         const bool agg_first = p.agg_first[l] != 0;   // then dW = (A~ H^(l))^T dPre, and dH^(l) = A~^T (dPre W^T)
         if (!agg_first)
             GAD_RUN("spmm_bwd", l, spmm_bytes(p, y.fo, nnz_b), 2.0 * nnz_b * y.fo,
-                    [&] { return launch_spmm(Ab, G1, y.ldo, G2, y.ldo, y.fo, nullptr, bf16_of(ctx), false, ctx->stream); });
+                    [&] { return launch_spmm(Ab, G1, y.ldo, G2, y.ldo, y.fo, nullptr, bf16_of(ctx), in_bf16, ctx->stream); });
+        in_bf16 = false;
         if (ctx->use_tc && p.narrow[l]) {
             // one pass over H^(l) and dZ gives both dW and dPre of the layer below (it writes G1: the column sums come first)
             if (ss != ctx->stream) GAD_CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_bias, 0));
@@ -604,17 +639,32 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
             continue;
         }
         if (l > 0 && ss != ctx->stream) GAD_CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_bias, 0));
-        if (l > 0)
-            GAD_RUN("gemm_dh", l, 4.0 * p.Np * (2.0 * y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
+        if (l == 0) break;
+        // the drain sums the columns of what it writes, dPre of the layer below: its bias gradient
+        const bool sums = ctx->use_tc && tc_rows_sums_columns(y.fi, npairs);
+        const bool out_bf16 = dpre_bf16(ctx, l - 1, sums);
+        GAD_RUN("gemm_dh", l, 4.0 * p.Np * (2.0 * y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
                 if (ctx->use_tc)
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 3], &ctx->maps[kMapsPerLayer * l + 4], &ctx->maps[kMapsPerLayer * l + 5], 1,
                                                ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G1, y.ldi, ctx->at<RowSpan>(p.o_pair_tiles),
                                                (int)(p.pair_tiles.size() / 2), ctx->H(l), y.ldi, scale, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
-                                               ctx->num_sms, ctx->stream, ctx->same_params);
+                                               ctx->num_sms, ctx->stream, ctx->same_params, out_bf16 ? bf16_of(ctx) : nullptr,
+                                               sums ? ctx->at<float>(p.o_colsum) : nullptr);
                 return launch_gemm_rows_simt(1, G2, y.ldo, y.fo, params, pstride, y.w_int, y.ldw, y.fi, G1, y.ldi,
                                              ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), ctx->H(l), y.ldi, scale, nullptr,
                                              ctx->stream);
             });
+        if (sums) {
+            int rc = hand_over(ctx, ctx->stream, ss, ctx->ev_g1);
+            if (rc != GAD_OK) return rc;
+            GAD_RUN("bias_sum", l - 1, 4.0 * 8 * (p.K + npairs) * y.fi, 1.0 * 8 * (p.K + npairs) * y.fi, [&] {
+                return launch_colsum_finish(ctx->at<float>(p.o_colsum), y.ldi, ctx->at<int2>(p.o_cs_clusters), p.K, grads, p.pstride,
+                                            p.layers[l - 1].b_int, ss);
+            });
+            if (ss != ctx->stream) GAD_CK(cudaEventRecord(ctx->ev_bias, ss));
+            bias_done = true;
+            in_bf16 = out_bf16;
+        }
     }
     return GAD_OK;
 }
@@ -818,11 +868,12 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
         (rc = upload(ctx, p.o_pair_ptr, p.pair_ptr)) || (rc = upload(ctx, p.o_gram_ptr, p.gram_ptr)) || (rc = upload(ctx, p.o_nchunks, p.nchunks)) ||
         (rc = upload(ctx, p.o_nchunk_ptr, p.nchunk_ptr)))
         return rc;
+    if ((rc = upload(ctx, p.o_zchunks, p.zchunks)) || (rc = upload(ctx, p.o_zchunk_ptr, p.zchunk_ptr))) return rc;
     for (const Plan::DwChunks& d : p.dw)
         if ((rc = upload(ctx, d.o_spans, d.spans)) || (rc = upload(ctx, d.o_ptr, d.ptr))) return rc;
     // features: graph order -> staging -> store-row order with zero pad columns
     GAD_CK(cudaMemcpyAsync(ctx->ws + p.o_stage, X, 4 * (size_t)g->n * p.dims[0], cudaMemcpyHostToDevice, ctx->stream));
-    GAD_CK(launch_gather_rows(ctx->at<float>(p.o_stage), p.dims[0], ctx->at<int32_t>(p.o_gid), p.Np, ctx->H(0), p.ld[0], ctx->stream));
+    GAD_CK(launch_gather_rows(ctx->at<float>(p.o_stage), p.dims[0], ctx->at<int32_t>(p.o_gid), p.Np, ctx->H(0), p.ld[0], x_bf16(ctx), ctx->stream));
     // parameters: one padded copy, which stands for all K while they are equal
     std::vector<float> ext((size_t)p.P);
     if (init_params) std::memcpy(ext.data(), init_params, sizeof(float) * (size_t)p.P);
@@ -852,6 +903,17 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
     }
     if (ctx->use_tc) {
         const int npairs = (int)(p.pair_tiles.size() / 2);
+        // the clusters of a transform with one column tile that meet each subgraph
+        std::vector<int2> meet((size_t)p.K, make_int2(1, 0));
+        const int64_t ncl = tc_rows_clusters(npairs, ctx->num_sms);
+        for (int64_t c = 0; c < ncl; ++c)
+            for (int64_t t = npairs * c / ncl; t < npairs * (c + 1) / ncl; ++t) {
+                int2& m = meet[(size_t)p.pair_tiles[(size_t)(2 * t)].k];
+                if (m.x > m.y) m.x = (int)c;
+                m.y = (int)c;
+            }
+        if ((rc = upload(ctx, p.o_cs_clusters, meet))) return rc;
+        GAD_CK(cudaStreamSynchronize(ctx->stream));   // (`meet` goes out of scope)
         ctx->maps.resize((size_t)kMapsPerLayer * p.L);
         bool ok = true;
         for (int l = 0; l < p.L && ok; ++l) {
@@ -946,7 +1008,8 @@ static int enqueue_epoch(gad_ctx* ctx, bool consensus) {
     GAD_RUN("softmax_xent", -1, 8.0 * p.Np * C, 0.0, [&] {
         return launch_softmax_xent(ctx->H(p.L), p.ld[p.L], C, ctx->at<int32_t>(p.o_label), ctx->at<uint8_t>(p.o_train),
                                    ctx->at<RowSpan>(p.o_chunks), (int)p.chunks.size(), ctx->at<float>(p.o_inv_ntrain),
-                                   ctx->at<float>(p.o_G1), ctx->at<float>(p.o_loss_partial), ctx->at<float>(p.o_cs_partial), p.maxld, ctx->stream);
+                                   ctx->at<float>(p.o_G1), ctx->at<float>(p.o_loss_partial), ctx->at<float>(p.o_cs_partial), p.maxld,
+                                   dpre_bf16(ctx, p.L - 1, softmax_sums_columns(p.ld[p.L])) ? bf16_of(ctx) : nullptr, ctx->stream);
     });
     // the sums over the chunks are needed at the end of the epoch only
     if ((rc = hand_over(ctx, ctx->stream, ss, ctx->ev_g1)) != GAD_OK) return rc;
@@ -981,7 +1044,11 @@ static bool graph_allowed(const gad_ctx* ctx) {
 }
 
 static void capture_epoch(gad_ctx* ctx, bool consensus, gad_ctx::EpochGraph& eg) {
-    if ((!ctx->capture_stream && cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess) ||
+    // The main sequence is captured at the highest priority and the side work at the lowest: a small kernel of the main sequence does not
+    // wait for the blocks of a large one beside it.
+    int least = 0, greatest = 0;
+    if ((!ctx->capture_stream && (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess ||
+                                  cudaStreamCreateWithPriority(&ctx->capture_stream, cudaStreamNonBlocking, greatest) != cudaSuccess)) ||
         cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         cudaGetLastError();
         eg.failed = true;
@@ -1229,7 +1296,7 @@ int gad_set_inputs(gad_ctx* ctx, const float* X, const int32_t* labels) {
     if (X) {
         GAD_RUN("gather_features", -1, 8.0 * p.Np * p.dims[0], 0.0, [&] {
             return launch_gather_rows(ctx->at<float>(o_x), p.dims[0], ctx->at<int32_t>(p.o_gid), p.Np, ctx->H(0), p.ld[0],
-                                      ctx->stream);
+                                      x_bf16(ctx), ctx->stream);
         });
         ctx->P_valid = false;   // A~ H^(0) is aggregated again by the next forward pass
     }

@@ -167,11 +167,15 @@ struct SplitLayers {
 cudaError_t launch_split_weights(const float* params, int64_t pstride, int K, const SplitLayer* layers, int L, cudaStream_t s);
 // pair_tiles: 2 npairs row tiles (at most 128 rows, or none), the two of a pair in the same subgraph; tc_rows_bn(n_cols, npairs) columns
 // per tile, half of them the rows of B's descriptor box.  one_b: the operand copies of replica 0 serve every subgraph.
-// Cbf16 (mode 0 only, may be null): the result goes there as bfloat16 [rows x ldc] INSTEAD of to C - the operand copy the
-// reduced-precision aggregation gathers, written by its producer.
+// Cbf16 (mode 0, or 1 with a mask; may be null): the result goes there as bfloat16 [rows x ldc] INSTEAD of to C - the operand copy the
+// reduced-precision aggregation gathers, written by its producer.  colsum (mode 1 with a mask, where tc_rows_sums_columns): the
+// column sums of the result, for launch_colsum_finish.
 cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols,
                                 float* C, int ldc, const RowSpan* pair_tiles, int npairs, const float* Hmask, int ldh, float scale,
-                                const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16 = nullptr);
+                                const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16 = nullptr, float* colsum = nullptr);
+bool tc_rows_sums_columns(int n_cols, int npairs);
+constexpr int kMaxRowClusters = 128;
+int tc_rows_clusters(long long ntiles, int num_sms);   // clusters of a launch: cluster c takes tiles [ntiles c / n, ntiles (c + 1) / n)
 
 // Tensor-core version of launch_gemm_tn_simt; mapH / mapZ are row-box descriptors (tc_tn_rows rows) of H^(l) and dZ.
 struct TnShape { int cg, ntm, ntn, bn; };   // CTAs per work unit, output tiles (of 128 cg rows and bn columns)
@@ -203,11 +207,16 @@ cudaError_t launch_colsum_chunks(const float* G, int ld, const RowSpan* chunks, 
                                  int64_t pstride_chunk, const int32_t* chunk_ptr, unsigned* counters, float* out,
                                  int64_t ostride, int64_t off, cudaStream_t s);
 
-// dlogits and per chunk the loss, and where softmax_sums_columns(ld) holds the column sums of dlogits (cs_partial).
+// out[k][off + j] = sum over the clusters first[k] .. last[k] that had tiles of subgraph k, and their eight row groups, of the column sums
+// a transform's drain has left (first > last: no rows).
+cudaError_t launch_colsum_finish(const float* colsum, int ld, const int2* clusters, int K, float* out, int64_t ostride, int64_t off, cudaStream_t s);
+
+// dlogits and per chunk the loss, and where softmax_sums_columns(ld) holds the column sums of dlogits (cs_partial); there dlogits_bf16 (may
+// be null) receives dlogits in bfloat16 instead.
 bool softmax_sums_columns(int ld);
 cudaError_t launch_softmax_xent(const float* logits, int ld, int C, const int32_t* label, const uint8_t* train,
                                 const RowSpan* chunks, int nchunks, const float* inv_ntrain, float* dlogits,
-                                float* loss_partial, float* cs_partial, int64_t pstride_chunk, cudaStream_t s);
+                                float* loss_partial, float* cs_partial, int64_t pstride_chunk, void* dlogits_bf16, cudaStream_t s);
 // loss[0..K-1] = mean loss of each subgraph, loss[K] = mean over all training rows, and with bias_ld > 0 out[k][off + j] = sum of
 // the column sums of subgraph k's chunks, j < bias_ld.
 cudaError_t launch_loss_finish(const float* loss_partial, const float* inv_ntrain, const int32_t* chunk_ptr, int K, float inv_total, float* loss,
@@ -263,7 +272,7 @@ cudaError_t launch_weights(const double* zeta, int K, int weighted, float* zeta_
 // to an input gradient that was aggregated after its transform).
 cudaError_t launch_relu_mask(float* G, const float* H, int ld, int64_t rows, float scale, cudaStream_t s);
 
-cudaError_t launch_gather_rows(const float* Xg, int F, const int32_t* gid, int64_t Np, float* H0, int ld,
+cudaError_t launch_gather_rows(const float* Xg, int F, const int32_t* gid, int64_t Np, float* H0, int ld, void* bf16_copy,
                                cudaStream_t s);
 cudaError_t launch_gather_labels(const int32_t* yg, const int32_t* gid, int64_t Np, int32_t* label, cudaStream_t s);
 cudaError_t launch_scatter_core(const float* logits, int ld, int C, const int32_t* gid, const RowSpan* core_spans,

@@ -31,6 +31,8 @@
 // peer at the cluster barrier, frees its tensor memory and returns.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "epilogue.cuh"
 #include "gad_internal.h"
 #include "tc_common.cuh"
@@ -43,7 +45,8 @@ constexpr int BK = 32;                                    // values of the reduc
 constexpr int A_BYTES = BM * BK * 4;                      // 16 KiB
 constexpr int MAX_STAGES = 8, MAX_LO = 4;
 constexpr int BAR_BYTES = 512;
-constexpr int DATA_BYTES = 232448 - 1024 - BAR_BYTES;     // 227 KiB less alignment and barriers
+constexpr int COLSUM_BYTES = 4 * 256 * 4;                 // column sums of the mask drain: 4 row quarters x 256 columns
+constexpr int DATA_BYTES = 232448 - 1024 - BAR_BYTES - COLSUM_BYTES;   // 227 KiB less alignment, barriers and column sums
 constexpr int SMEM_BYTES = 232448;
 constexpr int SPLIT_WARPS = 8, EPI_WARPS = 8, EPI_WARP0 = 2 + SPLIT_WARPS;
 constexpr int THREADS = 32 * (EPI_WARP0 + EPI_WARPS);
@@ -59,6 +62,8 @@ struct RowsArgs {
     const float* Hmask;
     int ldh;
     float scale;
+    float* colsum;            // masked drains: column sums of what is written (the bias gradient of the layer below), or null:
+                              // [(cluster + subgraph) * 8 + rank * 4 + row quarter][ldc] of every (cluster, subgraph) that meet
     int kmul;                 // 1: every subgraph has its own B; 0: one B for all (the replicas' parameters are equal)
     int32_t* err;
     ActEpi act;               // mode 2
@@ -67,7 +72,7 @@ struct RowsArgs {
 // What the drain does with a value: nothing (mode 0, or 1 without a mask), bfloat16 (mode 0), the ReLU mask and dropout scale (mode
 // 1), bias and ReLU (mode 2), those with dropout.  A template parameter, like the number of passes: as branches inside the unrolled
 // drain they made the kernel wait for instructions, 10.7 us per 128 x 256 tile.
-enum Drain { kPlain, kBf16, kMask, kAct, kActDrop };
+enum Drain { kPlain, kBf16, kMask, kMaskBf16, kAct, kActDrop };
 
 // Tile t of the launch: resident, column tile by column tile (B changes rarely); otherwise the column tiles of a row tile
 // follow each other (A comes from L2 the second time).
@@ -252,11 +257,28 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // In a 16 x 256-bit read lane t gets, of every 8 columns, columns 2 (t % 4) and the next one of rows t / 4 and t / 4 + 8.
         const int quarter = warp & 3, half = (warp - EPI_WARP0) >> 2;
         const int sub_r = lane >> 2, sub_c = 2 * (lane & 3);
+        constexpr bool masked = DRAIN == kMask || DRAIN == kMaskBf16, to_bf16 = DRAIN == kBf16 || DRAIN == kMaskBf16;
+        // This warp's column sums: the columns of its blocks, of its quarter of the rows; nobody else touches them.  They are written out
+        // when the subgraph changes and at the end: the tiles of a cluster are consecutive, so its subgraphs ascend and cluster +
+        // subgraph names the pair.
+        float* cs = reinterpret_cast<float*>(sm + DATA_BYTES + BAR_BYTES) + quarter * 256;
+        int cs_k = -1;
+        auto flush_colsum = [&](int next_k) {
+            __syncwarp();
+            for (int c0 = 32 * half; c0 < a.BN; c0 += 64) {
+                const int c = c0 + lane;
+                if (cs_k >= 0 && c < a.ldc && c < a.BN) a.colsum[((long long)(cl + cs_k) * 8 + (int)rank * 4 + quarter) * a.ldc + c] = cs[c];
+                cs[c] = 0.f;
+            }
+            __syncwarp();
+            cs_k = next_k;
+        };
         int acc = 0;
         uint32_t acc_phase = 0;
         for_tiles([&](int pair, int n, int, bool) {
             const RowSpan sp = a.tiles[2 * pair + (int)rank];
             const int n0 = n * a.BN;
+            if (masked && a.colsum && sp.k != cs_k) flush_colsum(sp.k);
             const int r0 = quarter * 32 + sub_r;                 // this lane's rows: r0 + 8 i
             float2 hm[4][4];
             auto fetch_mask = [&](int c0) {
@@ -275,7 +297,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const int ng = min(4, (min(a.BN - c0, a.ldc - n0 - c0) - sub_c + 7) >> 3);   // groups it has columns in
                 const long long at0 = ((long long)sp.row0 + r0) * a.ldc + nc;
                 float2 bias[4];
-                if (DRAIN == kMask) fetch_mask(c0);
+                if (masked) fetch_mask(c0);
                 if (DRAIN == kAct || DRAIN == kActDrop)
 #pragma unroll
                     for (int g = 0; g < 4; ++g) bias[g] = g < ng ? load_bias2(a.act, sp.k, nc + 8 * g) : make_float2(0.f, 0.f);
@@ -283,7 +305,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * a.BN + c0);
                 if (a.BN >= 32) tmem_ld_16x256b_x4(t0, v);
                 else tmem_ld_16x256b_x2(t0, v);
-                if (DRAIN == kMask) {
+                if (masked) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -291,6 +313,15 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             v[i][g].x = hm[i][g].x > 0.f ? v[i][g].x * a.scale : 0.f;
                             v[i][g].y = hm[i][g].y > 0.f ? v[i][g].y * a.scale : 0.f;
                         }
+                    if (a.colsum) {   // (rows and columns that do not exist are masked to zero)
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            float2 t = make_float2((v[0][g].x + v[1][g].x) + (v[2][g].x + v[3][g].x), (v[0][g].y + v[1][g].y) + (v[2][g].y + v[3][g].y));
+#pragma unroll
+                            for (int o = 4; o < 32; o <<= 1) { t.x += __shfl_xor_sync(0xffffffffu, t.x, o); t.y += __shfl_xor_sync(0xffffffffu, t.y, o); }
+                            if (lane < 4 && c0 + 8 * g < a.BN) { cs[c0 + 8 * g + sub_c] += t.x; cs[c0 + 8 * g + sub_c + 1] += t.y; }
+                        }
+                    }
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -310,7 +341,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             o.y = dropout_keep(key, nc + 8 * g + 1, a.act.thr) ? o.y * a.act.scale : 0.f;
                         }
                         if (g < ng) {
-                            if (DRAIN == kBf16) a.Cbf[(at + 8 * g) >> 1] = bf16_bits(o.x) | (bf16_bits(o.y) << 16);
+                            if (to_bf16) a.Cbf[(at + 8 * g) >> 1] = bf16_bits(o.x) | (bf16_bits(o.y) << 16);
                             else *reinterpret_cast<float2*>(a.C + at + 8 * g) = o;
                         }
                     }
@@ -322,6 +353,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             return true;
         });
+        if (masked && a.colsum) flush_colsum(-1);
     }
 
     // Tear-down.  After a time-out, give loads that may still be in flight a bounded chance to land before the shared memory is
@@ -386,21 +418,24 @@ int tc_rows_bn(int n_cols, int npairs) {
     return bn;
 }
 
+// The drain can sum columns when a tile holds all of them.
+bool tc_rows_sums_columns(int n_cols, int npairs) { return tc_rows_bn(n_cols, npairs) >= n_cols; }
+int tc_rows_clusters(long long ntiles, int num_sms) { return (int)std::min<long long>(ntiles, std::min(max_clusters(num_sms), kMaxRowClusters)); }
+
 cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols,
                                 float* C, int ldc, const RowSpan* pair_tiles, int npairs, const float* Hmask, int ldh, float scale,
-                                const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16) {
+                                const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16, float* colsum) {
     if (npairs <= 0) return cudaSuccess;
-    if ((mode == 2 && !act) || (Cbf16 && mode != 0)) return cudaErrorInvalidValue;
+    if ((mode == 2 && !act) || (Cbf16 && mode == 2) || (Cbf16 && mode == 1 && !Hmask)) return cudaErrorInvalidValue;
+    if (colsum && !(mode == 1 && Hmask && tc_rows_sums_columns(n_cols, npairs))) return cudaErrorInvalidValue;
     RowsArgs a;
     a.tiles = pair_tiles; a.npairs = npairs; a.BN = tc_rows_bn(n_cols, npairs); a.ntn = (ldc + a.BN - 1) / a.BN; a.Kd = Kd;
     rows_layout(a.BN, Kd, passes, a);
-    a.C = C; a.Cbf = reinterpret_cast<uint32_t*>(Cbf16); a.ldc = ldc; a.Hmask = Hmask; a.ldh = ldh; a.scale = scale;
+    a.C = C; a.Cbf = reinterpret_cast<uint32_t*>(Cbf16); a.ldc = ldc; a.Hmask = Hmask; a.ldh = ldh; a.scale = scale; a.colsum = colsum;
     a.kmul = one_b ? 0 : 1; a.err = err;
     a.act = act ? *act : ActEpi{};
-    const long long total = (long long)npairs * a.ntn;
-    const int cl = max_clusters(num_sms);
-    const unsigned grid = 2u * (unsigned)(total < cl ? total : cl);
-    const int drain = mode == 2 ? (a.act.drop ? kActDrop : kAct) : mode == 1 && Hmask ? kMask : Cbf16 ? kBf16 : kPlain;
+    const unsigned grid = 2u * (unsigned)tc_rows_clusters((long long)npairs * a.ntn, num_sms);
+    const int drain = mode == 2 ? (a.act.drop ? kActDrop : kAct) : mode == 1 && Hmask ? (Cbf16 ? kMaskBf16 : kMask) : Cbf16 ? kBf16 : kPlain;
     auto go = [&](auto kernel) {
         cudaError_t e = configure_kernel_once(reinterpret_cast<const void*>(kernel), SMEM_BYTES, false);
         if (e != cudaSuccess) return e;
@@ -414,6 +449,7 @@ cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* 
         GAD_DRAIN(kPlain);
         GAD_DRAIN(kBf16);
         GAD_DRAIN(kMask);
+        GAD_DRAIN(kMaskBf16);
         GAD_DRAIN(kAct);
         GAD_DRAIN(kActDrop);
     }

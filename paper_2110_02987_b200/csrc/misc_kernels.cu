@@ -5,6 +5,7 @@
 // reproducible.
 #include <math.h>
 
+#include "epilogue.cuh"
 #include "gad_internal.h"
 
 namespace gad {
@@ -46,11 +47,11 @@ __device__ __forceinline__ T segment_sum(const T* src, long long stride, long lo
     for (; c < e; ++c) s += __ldcg(src + (long long)c * stride + j);
     return s;
 }
-// Columns are handled 256 / nseg at a time; nseg = 256 / (columns rounded up to a power of two), at least 1.
-__device__ __forceinline__ int segments_for(int cols) {
+// Columns are handled T / nseg at a time by T threads; nseg = T / (columns rounded up to a power of two), at least 1.
+__device__ __forceinline__ int segments_for(int cols, int T = 256) {
     int p = 1;
-    while (p < cols && p < 256) p <<= 1;
-    return 256 / p;
+    while (p < cols && p < T) p <<= 1;
+    return T / p;
 }
 
 // What follows the loss kernel, beside the backward pass: the CTA of subgraph k adds up the column sums of its chunks' d logits
@@ -166,7 +167,8 @@ __global__ void __launch_bounds__(256) softmax_xent_kernel(const float* __restri
 }
 
 // Up to 128 classes: L lanes hold one row (a float4 each), 32/L rows per warp step, the row stays in registers.  The column sums of
-// d logits (the bias gradient of the last layer) come out of the same pass: per chunk into cs_partial.
+// d logits (the bias gradient of the last layer) come out of the same pass: per chunk into cs_partial.  dlogits_bf (may be null): d logits
+// go there in bfloat16 instead, the operand copy of the reduced-precision aggregation.
 template <int L>
 __global__ void __launch_bounds__(256) softmax_xent_small_kernel(const float* __restrict__ logits, int ld, int C,
                                                                  const int32_t* __restrict__ label,
@@ -174,7 +176,8 @@ __global__ void __launch_bounds__(256) softmax_xent_small_kernel(const float* __
                                                                  const RowSpan* __restrict__ chunks,
                                                                  const float* __restrict__ inv_ntrain,
                                                                  float* __restrict__ dlogits, float* __restrict__ loss_partial,
-                                                                 float* __restrict__ cs_partial, long long pstride_chunk) {
+                                                                 float* __restrict__ cs_partial, long long pstride_chunk,
+                                                                 uint2* __restrict__ dlogits_bf) {
     constexpr int RPW = 32 / L;
     __shared__ float wsum[8];
     __shared__ float4 csum[8][L];
@@ -199,16 +202,15 @@ __global__ void __launch_bounds__(256) softmax_xent_small_kernel(const float* __
         }
         return in;
     };
-    int r = warp * RPW + g;
-    RowIn cur = fetch(r);
-    for (; r < c.nrows; r += 8 * RPW) {
-        const RowIn nxt = fetch(r + 8 * RPW);
+    auto finish = [&](int r, const RowIn& cur) {
         const long long row = c.row0 + r;
         float4* gout = reinterpret_cast<float4*>(dlogits + row * ld);
         if (!cur.train) {
-            if (gl < ld4) gout[gl] = make_float4(0.f, 0.f, 0.f, 0.f);
-            cur = nxt;
-            continue;
+            if (gl < ld4) {
+                if (dlogits_bf) dlogits_bf[row * ld4 + gl] = make_uint2(0u, 0u);
+                else gout[gl] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            return;
         }
         float z[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
         if (gl < ld4) {
@@ -221,12 +223,12 @@ __global__ void __launch_bounds__(256) softmax_xent_small_kernel(const float* __
         float mx = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3]));
 #pragma unroll
         for (int o = L / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(gmask, mx, o, L));
-        float se = 0.f;
+        float se = 0.f, ex[4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) se += 4 * gl + t < C ? expf(z[t] - mx) : 0.f;
+        for (int t = 0; t < 4; ++t) { ex[t] = 4 * gl + t < C ? expf(z[t] - mx) : 0.f; se += ex[t]; }
 #pragma unroll
         for (int o = L / 2; o > 0; o >>= 1) se += __shfl_xor_sync(gmask, se, o, L);
-        const float lse = mx + logf(se);
+        const float lse = mx + logf(se), inv_se = 1.f / se;
         const int y = cur.y;
         const int yt = y & 3;
         const float mine = yt == 0 ? z[0] : (yt == 1 ? z[1] : (yt == 2 ? z[2] : z[3]));
@@ -237,12 +239,21 @@ __global__ void __launch_bounds__(256) softmax_xent_small_kernel(const float* __
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 const int j = 4 * gl + t;
-                o4[t] = j < C ? (expf(z[t] - lse) - (j == y ? 1.f : 0.f)) * inv : 0.f;
+                o4[t] = j < C ? (ex[t] * inv_se - (j == y ? 1.f : 0.f)) * inv : 0.f;
             }
-            gout[gl] = make_float4(o4[0], o4[1], o4[2], o4[3]);
+            if (dlogits_bf) dlogits_bf[row * ld4 + gl] = bf16_pack4(make_float4(o4[0], o4[1], o4[2], o4[3]));
+            else gout[gl] = make_float4(o4[0], o4[1], o4[2], o4[3]);
             cs.x += o4[0]; cs.y += o4[1]; cs.z += o4[2]; cs.w += o4[3];
         }
-        cur = nxt;
+    };
+    // Two rows per lane group at a time, and the next two on their way.
+    int r = warp * RPW + g;
+    RowIn a0 = fetch(r), a1 = fetch(r + 8 * RPW);
+    for (; r < c.nrows; r += 16 * RPW) {
+        const RowIn n0 = fetch(r + 16 * RPW), n1 = fetch(r + 24 * RPW);
+        finish(r, a0);
+        if (r + 8 * RPW < c.nrows) finish(r + 8 * RPW, a1);
+        a0 = n0; a1 = n1;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -269,10 +280,10 @@ __global__ void __launch_bounds__(256) softmax_xent_small_kernel(const float* __
 bool softmax_sums_columns(int ld) { return ld <= 128; }
 cudaError_t launch_softmax_xent(const float* logits, int ld, int C, const int32_t* label, const uint8_t* train,
                                 const RowSpan* chunks, int nchunks, const float* inv_ntrain, float* dlogits,
-                                float* loss_partial, float* cs_partial, int64_t pstride_chunk, cudaStream_t s) {
+                                float* loss_partial, float* cs_partial, int64_t pstride_chunk, void* dlogits_bf16, cudaStream_t s) {
     if (nchunks > 0) {
         const int ld4 = ld >> 2;
-#define GAD_SMALL(L) softmax_xent_small_kernel<L><<<(unsigned)nchunks, 256, 0, s>>>(logits, ld, C, label, train, chunks, inv_ntrain, dlogits, loss_partial, cs_partial, pstride_chunk)
+#define GAD_SMALL(L) softmax_xent_small_kernel<L><<<(unsigned)nchunks, 256, 0, s>>>(logits, ld, C, label, train, chunks, inv_ntrain, dlogits, loss_partial, cs_partial, pstride_chunk, reinterpret_cast<uint2*>(dlogits_bf16))
         if (ld4 <= 1) GAD_SMALL(1);
         else if (ld4 <= 2) GAD_SMALL(2);
         else if (ld4 <= 4) GAD_SMALL(4);
@@ -358,6 +369,32 @@ cudaError_t launch_colsum_chunks(const float* G, int ld, const RowSpan* chunks, 
     return cudaGetLastError();
 }
 
+__global__ void __launch_bounds__(256) colsum_finish_kernel(const float* __restrict__ colsum, int ld, const int2* __restrict__ clusters,
+                                                            float* __restrict__ out, long long ostride, long long off) {
+    __shared__ float seg_sm[256];
+    const int k = blockIdx.x;
+    const int2 r = clusters[k];
+    const int c0 = (r.x + k) * 8, c1 = (r.y + k + 1) * 8;   // rows of the partial sums
+    const int nseg = segments_for(ld), per = 256 / nseg;
+    const int jl = threadIdx.x % per, seg = threadIdx.x / per;
+    for (int j0 = 0; j0 < ld; j0 += per) {
+        const int j = j0 + jl;
+        seg_sm[threadIdx.x] = j < ld ? segment_sum(colsum, ld, j, c0, c1, seg, nseg) : 0.f;
+        __syncthreads();
+        if (seg == 0 && j < ld) {
+            float t = seg_sm[jl];
+            for (int q = 1; q < nseg; ++q) t += seg_sm[q * per + jl];
+            out[(long long)k * ostride + off + j] = t;
+        }
+        __syncthreads();
+    }
+}
+cudaError_t launch_colsum_finish(const float* colsum, int ld, const int2* clusters, int K, float* out, int64_t ostride, int64_t off, cudaStream_t s) {
+    colsum_finish_kernel<<<(unsigned)K, 256, 0, s>>>(colsum, ld, clusters, out, ostride, off);
+    ++g_kernel_launches;
+    return cudaGetLastError();
+}
+
 __global__ void reduce_chunks_kernel(const float* __restrict__ partial, long long pstride_chunk,
                                      const int32_t* __restrict__ chunk_ptr, float* __restrict__ out, long long ostride,
                                      long long off, long long len) {
@@ -395,12 +432,11 @@ cudaError_t launch_reduce_chunks(const float* partial, int64_t pstride_chunk, co
 // zeta_k = S_k / (D_k + beta) from the chunk sums of subgraph k, chunks added in order; one CTA per subgraph.
 // `phase` spreads one zeta over several matrices (the layers' inputs, zeta_mode 2): 0 = this matrix alone; 1 = the first
 // of several (its distance sum goes to q_acc[k]); 2 = a further one (added to q_acc[k]); 3 = the last one (added, then zeta).
-__global__ void __launch_bounds__(256) zeta_finish_kernel(const double* __restrict__ partial, int F, int ld, const int32_t* __restrict__ chunk_ptr,
+__global__ void __launch_bounds__(1024) zeta_finish_kernel(const double* __restrict__ partial, int F, int ld, const int32_t* __restrict__ chunk_ptr,
                                               const int32_t* __restrict__ sub_off, const int64_t* __restrict__ deg_sum,
                                               const int64_t* __restrict__ deg_sq, float beta, double* __restrict__ zeta,
                                               double* __restrict__ q_acc, int phase) {
-    __shared__ double red[256];
-    __shared__ double seg_a[256], seg_b[256];
+    __shared__ double seg_a[1024], seg_b[1024];
     const int k = blockIdx.x;
     const long long n = sub_off[k + 1] - sub_off[k];
     if (n == 0) return;   // zero since creation
@@ -410,7 +446,7 @@ __global__ void __launch_bounds__(256) zeta_finish_kernel(const double* __restri
     if (n > 0) {
         // segments of the chunk range in parallel, the segment sums then added in order, per feature
         const int c0 = chunk_ptr[k], c1 = chunk_ptr[k + 1];
-        const int nseg = segments_for(F), per = 256 / nseg;
+        const int nseg = segments_for(F, 1024), per = 1024 / nseg;
         const int fl = threadIdx.x % per, seg = threadIdx.x / per;
         for (int f0 = 0; f0 < F; f0 += per) {
             const int f = f0 + fl;
@@ -426,9 +462,10 @@ __global__ void __launch_bounds__(256) zeta_finish_kernel(const double* __restri
             __syncthreads();
         }
     }
+    double* red = seg_a;
     red[threadIdx.x] = q;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
+    for (int o = 512; o > 0; o >>= 1) {
         if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
         __syncthreads();
     }
@@ -503,7 +540,7 @@ cudaError_t launch_zeta(const float* X, int ld, int F, const int32_t* deg, const
                         float beta, double* partial, double* zeta, double* q_acc, int phase, cudaStream_t s) {
     if (nchunks > 0) {
         zeta_partial_kernel<<<dim3((unsigned)nchunks, (unsigned)((ld / 4 + 31) / 32)), 256, 0, s>>>(X, ld, deg, chunks, sub_off, deg_sum, partial);
-        zeta_finish_kernel<<<(unsigned)K, 256, 0, s>>>(partial, F, ld, chunk_ptr, sub_off, deg_sum, deg_sq, beta, zeta, q_acc, phase);
+        zeta_finish_kernel<<<(unsigned)K, 1024, 0, s>>>(partial, F, ld, chunk_ptr, sub_off, deg_sum, deg_sq, beta, zeta, q_acc, phase);
         g_kernel_launches += 2;
     }
     return cudaGetLastError();
@@ -671,15 +708,30 @@ cudaError_t launch_relu_mask(float* G, const float* H, int ld, int64_t rows, flo
 // ---------------------------------------------------------------------------------------------
 // Gathers between graph-node order and store-row order.
 // ---------------------------------------------------------------------------------------------
-__global__ void gather_rows_kernel(const float* __restrict__ Xg, int F, const int32_t* __restrict__ gid, long long Np,
-                                   float* __restrict__ H0, int ld) {
-    const long long row = blockIdx.x;
-    const float* src = Xg + (long long)gid[row] * F;
-    float* dst = H0 + row * ld;
-    for (int j = threadIdx.x; j < ld; j += blockDim.x) dst[j] = j < F ? src[j] : 0.f;
+// Four columns per thread (16 bytes where the rows of Xg allow it), and their bfloat16 copy where the reduced-precision aggregation will
+// gather it.  (One thread per column and a CTA per row: 63 us for 110 000 rows of 128.)
+template <bool VEC>
+__global__ void __launch_bounds__(256) gather_rows_kernel(const float* __restrict__ Xg, int F, const int32_t* __restrict__ gid, long long n4, int ld4,
+                                                          float4* __restrict__ H0, uint2* __restrict__ bf) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n4) return;
+    const long long row = i / ld4;
+    const int j = 4 * (int)(i % ld4);
+    const float* src = Xg + (long long)gid[row] * F + j;
+    float4 v;
+    if (VEC) v = *reinterpret_cast<const float4*>(src);
+    else v = make_float4(src[0], j + 1 < F ? src[1] : 0.f, j + 2 < F ? src[2] : 0.f, j + 3 < F ? src[3] : 0.f);
+    H0[i] = v;
+    if (bf) bf[i] = bf16_pack4(v);
 }
-cudaError_t launch_gather_rows(const float* Xg, int F, const int32_t* gid, int64_t Np, float* H0, int ld, cudaStream_t s) {
-    if (Np > 0) { gather_rows_kernel<<<(unsigned)Np, 128, 0, s>>>(Xg, F, gid, Np, H0, ld); ++g_kernel_launches; }
+cudaError_t launch_gather_rows(const float* Xg, int F, const int32_t* gid, int64_t Np, float* H0, int ld, void* bf16_copy, cudaStream_t s) {
+    const long long n4 = (long long)Np * (ld / 4);
+    if (n4 > 0) {
+        const unsigned grid = (unsigned)((n4 + 255) / 256);
+        if (F % 4 == 0) gather_rows_kernel<true><<<grid, 256, 0, s>>>(Xg, F, gid, n4, ld / 4, reinterpret_cast<float4*>(H0), reinterpret_cast<uint2*>(bf16_copy));
+        else gather_rows_kernel<false><<<grid, 256, 0, s>>>(Xg, F, gid, n4, ld / 4, reinterpret_cast<float4*>(H0), reinterpret_cast<uint2*>(bf16_copy));
+        ++g_kernel_launches;
+    }
     return cudaGetLastError();
 }
 __global__ void gather_labels_kernel(const int32_t* __restrict__ yg, const int32_t* __restrict__ gid, long long Np,

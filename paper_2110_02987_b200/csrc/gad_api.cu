@@ -15,6 +15,8 @@ namespace gad {
 
 std::atomic<int64_t> g_kernel_launches{0};
 
+PdlState& pdl_state() { static thread_local PdlState s; return s; }
+
 cudaError_t configure_kernel_once(const void* kernel, int smem_bytes, bool max_carveout) {
     static std::mutex lock;
     static std::set<std::pair<int, const void*>> done;   // (device, kernel)
@@ -407,13 +409,27 @@ double spmm_bytes(const Plan& p, int F, int64_t nnz = -1) { return 8.0 * (nnz < 
 // to a second stream and run beside the aggregation / transform sequence; events order them against it.  While
 // per-kernel timing is on everything stays on the context's stream, where the timing events are recorded.
 cudaStream_t side_of(gad_ctx* ctx) { return ctx->profiling ? ctx->stream : ctx->side_stream; }
+// `to` waits for the event; the kernel that follows there waits for everything in front of it.
+int wait_for(gad_ctx* ctx, cudaStream_t to, cudaEvent_t ev) {
+    GAD_CK(cudaStreamWaitEvent(to, ev, 0));
+    if (to == pdl_state().stream) pdl_state().direct = false;
+    return GAD_OK;
+}
 // Work enqueued on `to` after this call starts only when the work enqueued on `from` so far has finished.
 int hand_over(gad_ctx* ctx, cudaStream_t from, cudaStream_t to, cudaEvent_t ev) {
     if (from == to) return GAD_OK;
     GAD_CK(cudaEventRecord(ev, from));
-    GAD_CK(cudaStreamWaitEvent(to, ev, 0));
-    return GAD_OK;
+    return wait_for(ctx, to, ev);
 }
+
+// While it lives, the kernels of the main sequence may start before the one in front has finished (launch.cuh): not while they are timed,
+// and only on small stores, whose kernels last a few microseconds each (2000 rows: 71 -> 66 us an epoch, 2800 rows: 175 -> 160, 20 700:
+// 207 -> 200); on large ones the waiting blocks hold room that the kernels beside them would use (110 000 rows: 281 -> 291 us).
+constexpr int64_t kPdlRows = 48 << 10;
+struct PdlScope {
+    explicit PdlScope(gad_ctx* ctx) { pdl_state() = PdlState{ctx->stream, !ctx->profiling && ctx->p.Np <= kPdlRows, false}; }
+    ~PdlScope() { pdl_state() = PdlState{}; }
+};
 
 // After a consensus has been enqueued.
 void copies_made_equal(gad_ctx* ctx) {
@@ -588,7 +604,7 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
         in_bf16 = false;
         if (ctx->use_tc && p.narrow[l]) {
             // one pass over H^(l) and dZ gives both dW and dPre of the layer below (it writes G1: the column sums come first)
-            if (ss != ctx->stream) GAD_CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_bias, 0));
+            if (ss != ctx->stream) { int rcw = wait_for(ctx, ctx->stream, ctx->ev_bias); if (rcw != GAD_OK) return rcw; }
             // the chunk results hold db of layer l-1 and then dW of layer l, which is also their order in the parameter block
             const int64_t plen = (int64_t)y.ldi + (int64_t)y.fi * y.ldw;
             GAD_RUN("gemm_dwdh", l, 4.0 * p.Np * (2.0 * y.fi + y.fo) + 8.0 * p.K * y.fi * y.fo, 4.0 * p.Np * y.fi * y.fo, [&] {
@@ -631,14 +647,14 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
                 return launch_gemm_rows_simt(1, G1, y.ldo, y.fo, params, pstride, y.w_int, y.ldw, y.fi, G2, y.ldi,
                                              ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, nullptr, ctx->stream);
             });
-            if (ss != ctx->stream) GAD_CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_bias, 0));   // the column sums have read dPre
+            if (ss != ctx->stream) { int rcw = wait_for(ctx, ctx->stream, ctx->ev_bias); if (rcw != GAD_OK) return rcw; }   // the column sums have read dPre
             GAD_RUN("spmm_bwd", l, spmm_bytes(p, y.fi, nnz_b), 2.0 * nnz_b * y.fi,
                     [&] { return launch_spmm(Ab, G2, y.ldi, G1, y.ldi, y.fi, nullptr, bf16_of(ctx), false, ctx->stream); });
             GAD_RUN("relu_mask", l, 12.0 * p.Np * y.fi, 1.0 * p.Np * y.fi,
                     [&] { return launch_relu_mask(G1, ctx->H(l), y.ldi, p.Np, scale, ctx->stream); });
             continue;
         }
-        if (l > 0 && ss != ctx->stream) GAD_CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_bias, 0));
+        if (l > 0 && ss != ctx->stream) { int rcw = wait_for(ctx, ctx->stream, ctx->ev_bias); if (rcw != GAD_OK) return rcw; }
         if (l == 0) break;
         // the drain sums the columns of what it writes, dPre of the layer below: its bias gradient
         const bool sums = ctx->use_tc && tc_rows_sums_columns(y.fi, npairs);
@@ -995,6 +1011,7 @@ int gad_train_epoch_local(gad_ctx* ctx, float* loss_out) { return train_epoch(ct
 static int enqueue_epoch(gad_ctx* ctx, bool consensus) {
     const Plan& p = ctx->p;
     cudaStream_t ss = side_of(ctx);
+    const PdlScope pdl(ctx);
     // The side work forks off behind the first kernel of the main sequence: as a second root of the graph it would come first, and
     // the main sequence 10 us later.
     int rc = split_pass(ctx);
@@ -1111,8 +1128,11 @@ static int train_epoch(gad_ctx* ctx, float* loss_out, bool consensus) {
 int gad_forward(gad_ctx* ctx, float* logits_out) {
     if (!ctx || !logits_out) return GAD_ERR_ARG;
     const Plan& p = ctx->p;
-    int rc = split_pass(ctx);
-    if (rc != GAD_OK || (rc = forward_pass(ctx, false)) != GAD_OK) return rc;
+    int rc;
+    {
+        const PdlScope pdl(ctx);
+        if ((rc = split_pass(ctx)) != GAD_OK || (rc = forward_pass(ctx, false)) != GAD_OK) return rc;
+    }
     const int C = p.dims[p.L];
     GAD_CK(cudaMemsetAsync(ctx->ws + p.o_stage, 0, 4 * (size_t)p.n * C, ctx->stream));
     GAD_CK(launch_scatter_core(ctx->H(p.L), p.ld[p.L], C, ctx->at<int32_t>(p.o_gid), ctx->at<RowSpan>(p.o_core_spans),

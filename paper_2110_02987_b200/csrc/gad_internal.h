@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/gad.h"
+#include "launch.cuh"
 
 namespace gad {
 

@@ -110,6 +110,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     volatile uint32_t* abort_flag = tmem_slot + 1;
     const uint32_t tmem_cols = a.BN < 16 ? 32u : 2u * (uint32_t)a.BN;
 
+    pdl_next();
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (uniform, and known to be)
     if (threadIdx.x == 0) {
         for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
@@ -126,6 +127,9 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
 
+    // From here on operands are read (the tile list is nobody's output: what follows may have it already).  Every thread waits: each role
+    // reads or writes something of its own.
+    pdl_wait();
     // contiguous ranges of tiles: B changes as rarely as possible
     const int ntiles = a.npairs * a.ntn, ncl = gridDim.x >> 1, cl = blockIdx.x >> 1;
     const int t_begin = (int)((long long)ntiles * cl / ncl), t_end = (int)((long long)ntiles * (cl + 1) / ncl);
@@ -257,6 +261,10 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // In a 16 x 256-bit read lane t gets, of every 8 columns, columns 2 (t % 4) and the next one of rows t / 4 and t / 4 + 8.
         const int quarter = warp & 3, half = (warp - EPI_WARP0) >> 2;
         const int sub_r = lane >> 2, sub_c = 2 * (lane & 3);
+        const float* hmask = a.Hmask;
+        ActEpi act = a.act;
+        after_wait(hmask);
+        after_wait(act.params);
         constexpr bool masked = DRAIN == kMask || DRAIN == kMaskBf16, to_bf16 = DRAIN == kBf16 || DRAIN == kMaskBf16;
         // This warp's column sums: the columns of its blocks, of its quarter of the rows; nobody else touches them.  They are written out
         // when the subgraph changes and at the end: the tiles of a cluster are consecutive, so its subgraphs ascend and cluster +
@@ -283,7 +291,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             float2 hm[4][4];
             auto fetch_mask = [&](int c0) {
                 const int nc = n0 + c0 + sub_c, ng = min(4, (min(a.BN - c0, a.ldc - n0 - c0) - sub_c + 7) >> 3);
-                const float* h = a.Hmask + ((long long)sp.row0 + r0) * a.ldh + nc;
+                const float* h = hmask + ((long long)sp.row0 + r0) * a.ldh + nc;
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -300,7 +308,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if (masked) fetch_mask(c0);
                 if (DRAIN == kAct || DRAIN == kActDrop)
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) bias[g] = g < ng ? load_bias2(a.act, sp.k, nc + 8 * g) : make_float2(0.f, 0.f);
+                    for (int g = 0; g < 4; ++g) bias[g] = g < ng ? load_bias2(act, sp.k, nc + 8 * g) : make_float2(0.f, 0.f);
                 float2 v[4][4];                                  // [row r0 + 8 i][columns nc + 8 g]
                 const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * a.BN + c0);
                 if (a.BN >= 32) tmem_ld_16x256b_x4(t0, v);
@@ -439,10 +447,10 @@ cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* 
     auto go = [&](auto kernel) {
         cudaError_t e = configure_kernel_once(reinterpret_cast<const void*>(kernel), SMEM_BYTES, false);
         if (e != cudaSuccess) return e;
-        kernel<<<grid, THREADS, SMEM_BYTES, s>>>(*reinterpret_cast<const CUtensorMap*>(mapA), *reinterpret_cast<const CUtensorMap*>(mapB),
+        e = launch(kernel, dim3(grid), THREADS, SMEM_BYTES, s, *reinterpret_cast<const CUtensorMap*>(mapA), *reinterpret_cast<const CUtensorMap*>(mapB),
                                                  *reinterpret_cast<const CUtensorMap*>(mapBlo), a);
         ++g_kernel_launches;
-        return cudaGetLastError();
+        return e;
     };
 #define GAD_DRAIN(D) case D: return passes > 1 ? go(gemm_rows_kernel<D, true>) : go(gemm_rows_kernel<D, false>)
     switch (drain) {

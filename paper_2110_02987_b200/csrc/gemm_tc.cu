@@ -19,11 +19,14 @@ constexpr int BK = 32;   // values of an operand row per TMA box (128 bytes)
 // the plain layout, a 500 x 128 layer of 50 replicas took 39 us, bound by its 4-byte column writes).
 __global__ void __launch_bounds__(256) split_weights_kernel(const float* __restrict__ params, long long pstride, const SplitLayers ls) {
     __shared__ float th[32][33], tl[32][33];
+    pdl_next();
     const SplitLayer& y = ls.y[blockIdx.z];
     const int ntj = (y.ldw + 31) / 32, ntiles = ((y.fi + 31) / 32) * ntj;
     if ((int)blockIdx.x >= ntiles) return;
     const int i0 = ((int)blockIdx.x / ntj) * 32, j0 = ((int)blockIdx.x % ntj) * 32, k = blockIdx.y;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    pdl_wait();
+    after_wait(params);
     const float* W = params + (long long)k * pstride + y.w_int;
 #pragma unroll
     for (int r = 0; r < 32; r += 8) {
@@ -110,7 +113,7 @@ cudaError_t launch_split_weights(const float* params, int64_t pstride, int K, co
             const int t = ((ls.y[l].fi + 31) / 32) * ((ls.y[l].ldw + 31) / 32);
             tiles = tiles > t ? tiles : t;
         }
-        split_weights_kernel<<<dim3((unsigned)tiles, (unsigned)K, (unsigned)n), 256, 0, s>>>(params, pstride, ls);
+        launch(split_weights_kernel, dim3((unsigned)tiles, (unsigned)K, (unsigned)n), 256, 0, s, params, pstride, ls);
         ++g_kernel_launches;
     }
     return cudaGetLastError();

@@ -92,6 +92,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
     uint32_t acc_cols = 16;                                    // columns between the accumulators: BN rounded up to a power of two
     while (acc_cols < (uint32_t)a.BN) acc_cols <<= 1;
 
+    pdl_next();
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int groups = a.nlo == MAX_LO ? MAX_LO : 1;
     if (threadIdx.x == 0) {
@@ -114,6 +115,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
 
+    pdl_wait();   // from here on operands are read and results written
     const int tiles = a.ntm * a.ntn, ncl = gridDim.x / CG, cl = blockIdx.x / CG;
     const int u0 = (int)((long long)a.nunits * cl / ncl), u1 = (int)((long long)a.nunits * (cl + 1) / ncl);
     // calls f(chunk number, chunk, first output row of this CTA, first output column of the tile) until it returns false
@@ -321,13 +323,8 @@ cudaError_t launch_gemm_tn_tc(const void* mapH, const void* mapZ, int passes, in
     auto go = [&](auto kernel) {
         cudaError_t e = configure_kernel_once(reinterpret_cast<const void*>(kernel), SMEM_BYTES, false);
         if (e != cudaSuccess) return e;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((unsigned)(units * t.cg)); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)t.cg; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, kernel, *reinterpret_cast<const CUtensorMap*>(mapH), *reinterpret_cast<const CUtensorMap*>(mapZ), a);
+        e = launch_cluster(kernel, dim3((unsigned)(units * t.cg)), THREADS, SMEM_BYTES, (unsigned)t.cg, s, *reinterpret_cast<const CUtensorMap*>(mapH),
+                   *reinterpret_cast<const CUtensorMap*>(mapZ), a);
         ++g_kernel_launches;
         return e;
     };

@@ -128,9 +128,12 @@ __global__ void __launch_bounds__(256) softmax_xent_kernel(const float* __restri
                                                            const float* __restrict__ inv_ntrain,
                                                            float* __restrict__ dlogits, float* __restrict__ loss_partial) {
     __shared__ float wsum[8];
+    pdl_next();
     const RowSpan c = chunks[blockIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float inv = inv_ntrain[c.k];
+    pdl_wait();
+    after_wait(logits);
     float acc = 0.f;
     for (int r = warp; r < c.nrows; r += 8) {
         const long long row = c.row0 + r;
@@ -183,12 +186,16 @@ __global__ void __launch_bounds__(256) softmax_xent_small_kernel(const float* __
     __shared__ float4 csum[8][L];
     float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
     const RowSpan c = chunks[blockIdx.x];
+    pdl_next();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane / L, gl = lane & (L - 1);
     const unsigned gmask = L == 32 ? 0xffffffffu : (((1u << L) - 1u) << (lane & ~(L - 1)));
     const int ld4 = ld >> 2;
     const float inv = inv_ntrain[c.k];
     float acc = 0.f;
+    pdl_wait();
+    after_wait(logits);
+    after_wait(label);
     // the loads of a row (loss mask, label, logits) do not wait for one another, and the next row's are requested
     // before this row's are used
     struct RowIn { bool train; int y; float4 v; };
@@ -283,14 +290,14 @@ cudaError_t launch_softmax_xent(const float* logits, int ld, int C, const int32_
                                 float* loss_partial, float* cs_partial, int64_t pstride_chunk, void* dlogits_bf16, cudaStream_t s) {
     if (nchunks > 0) {
         const int ld4 = ld >> 2;
-#define GAD_SMALL(L) softmax_xent_small_kernel<L><<<(unsigned)nchunks, 256, 0, s>>>(logits, ld, C, label, train, chunks, inv_ntrain, dlogits, loss_partial, cs_partial, pstride_chunk, reinterpret_cast<uint2*>(dlogits_bf16))
+#define GAD_SMALL(L) launch(softmax_xent_small_kernel<L>, dim3((unsigned)nchunks), 256, 0, s, logits, ld, C, label, train, chunks, inv_ntrain, dlogits, loss_partial, cs_partial, pstride_chunk, reinterpret_cast<uint2*>(dlogits_bf16))
         if (ld4 <= 1) GAD_SMALL(1);
         else if (ld4 <= 2) GAD_SMALL(2);
         else if (ld4 <= 4) GAD_SMALL(4);
         else if (ld4 <= 8) GAD_SMALL(8);
         else if (ld4 <= 16) GAD_SMALL(16);
         else if (ld4 <= 32) GAD_SMALL(32);
-        else softmax_xent_kernel<<<(unsigned)nchunks, 256, 0, s>>>(logits, ld, C, label, train, chunks, inv_ntrain, dlogits, loss_partial);
+        else launch(softmax_xent_kernel, dim3((unsigned)nchunks), 256, 0, s, logits, ld, C, label, train, chunks, inv_ntrain, dlogits, loss_partial);
 #undef GAD_SMALL
         ++g_kernel_launches;
     }
@@ -398,9 +405,12 @@ cudaError_t launch_colsum_finish(const float* colsum, int ld, const int2* cluste
 __global__ void reduce_chunks_kernel(const float* __restrict__ partial, long long pstride_chunk,
                                      const int32_t* __restrict__ chunk_ptr, float* __restrict__ out, long long ostride,
                                      long long off, long long len) {
+    pdl_next();
     const int k = blockIdx.y;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= len) return;
+    pdl_wait();
+    after_wait(partial);
     float s = 0.f;
     const int c1 = chunk_ptr[k + 1];
     int c = chunk_ptr[k];
@@ -417,7 +427,7 @@ __global__ void reduce_chunks_kernel(const float* __restrict__ partial, long lon
 cudaError_t launch_reduce_chunks(const float* partial, int64_t pstride_chunk, const int32_t* chunk_ptr, int K, float* out,
                                  int64_t ostride, int64_t off, int64_t len, cudaStream_t s) {
     if (len > 0 && K > 0) {
-        reduce_chunks_kernel<<<dim3((unsigned)((len + 255) / 256), (unsigned)K), 256, 0, s>>>(partial, pstride_chunk, chunk_ptr, out,
+        launch(reduce_chunks_kernel, dim3((unsigned)((len + 255) / 256), (unsigned)K), 256, 0, s, partial, pstride_chunk, chunk_ptr, out,
                                                                                                ostride, off, len); ++g_kernel_launches; }
     return cudaGetLastError();
 }
@@ -602,6 +612,9 @@ __global__ void __launch_bounds__(256) sgd_consensus_kernel(float* params, long 
                                                             int32_t* words, long long* epoch, const float* report, float* report_to,
                                                             int nreport) {
     extern __shared__ float w_sm[];
+    pdl_wait();
+    after_wait(grads);
+    after_wait(zeta);
     const bool timed_out = words[1] != 0;   // a bounded wait ran out earlier in this epoch: keep the parameters as they are
     if (blockIdx.x == 0) {
         if (threadIdx.x == 0 && pstride_p != 0 && !timed_out) words[2] = 0;
@@ -621,7 +634,7 @@ cudaError_t launch_sgd_consensus(float* params, int64_t pstride_p, const float* 
     const long long len4 = len / 4;
     if (len4 > 0) {
         const int threads = len4 >= 148 * 256 * 4 ? 256 : 64;   // a small model is spread over more CTAs
-        sgd_consensus_kernel<<<(unsigned)((len4 + threads - 1) / threads), threads, (size_t)K * sizeof(float), s>>>(
+        launch(sgd_consensus_kernel, dim3((unsigned)((len4 + threads - 1) / threads)), threads, (size_t)K * sizeof(float), s, 
             params, pstride_p, grads, pstride, len4, K, lr, zeta, weighted, with_sgd, words, epoch, report, report_to, nreport);
         ++g_kernel_launches;
     }
@@ -688,8 +701,11 @@ cudaError_t launch_weights(const double* zeta, int K, int weighted, float* zeta_
 }
 
 __global__ void __launch_bounds__(256) relu_mask_kernel(float4* __restrict__ G, const float4* __restrict__ H, long long n4, float scale) {
+    pdl_next();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n4) return;
+    pdl_wait();
+    after_wait(H);
     float4 g = G[i];
     const float4 h = H[i];
     g.x = h.x > 0.f ? g.x * scale : 0.f; g.y = h.y > 0.f ? g.y * scale : 0.f;
@@ -699,7 +715,7 @@ __global__ void __launch_bounds__(256) relu_mask_kernel(float4* __restrict__ G, 
 cudaError_t launch_relu_mask(float* G, const float* H, int ld, int64_t rows, float scale, cudaStream_t s) {
     const long long n4 = (long long)rows * (ld / 4);
     if (n4 > 0) {
-        relu_mask_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, s>>>(reinterpret_cast<float4*>(G), reinterpret_cast<const float4*>(H), n4, scale);
+        launch(relu_mask_kernel, dim3((unsigned)((n4 + 255) / 256)), 256, 0, s, reinterpret_cast<float4*>(G), reinterpret_cast<const float4*>(H), n4, scale);
         ++g_kernel_launches;
     }
     return cudaGetLastError();

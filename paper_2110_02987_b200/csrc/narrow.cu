@@ -93,6 +93,7 @@ narrow_bwd_kernel(const float* __restrict__ H, int ldh, int fi, const float* __r
     const int slab = warp % nslab, rg = warp / nslab, nrg = kWarps / nslab;
     const int ldh4 = ldh >> 2, col4 = 32 * slab + lane, col = 4 * col4;
     const bool live = col4 < ldh4;
+    pdl_next();
     const int BR = block_rows(nslab);
     const int nblk = (ch.nrows + BR - 1) / BR;
     Ring ring;
@@ -108,6 +109,8 @@ narrow_bwd_kernel(const float* __restrict__ H, int ldh, int fi, const float* __r
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    pdl_wait();
+    after_wait(params);
     if (threadIdx.x == 0)
         for (int b = 0; b < min(kStages, nblk); ++b) ring.issue(b);
 
@@ -236,10 +239,10 @@ cudaError_t launch_narrow_bwd(const float* H, int ldh, int fi, const float* dZ, 
     auto go = [&](auto kernel) -> cudaError_t {
         cudaError_t e = prepare(kernel);
         if (e != cudaSuccess) return e;
-        kernel<<<(unsigned)nchunks, 32 * kWarps, smem, s>>>(H, ldh, fi, dZ, ldz, params, pstride, w_int, ldw, chunks, scale, dPre, partial,
-                                                            partial_stride, nslab, err);
+        e = launch(kernel, dim3((unsigned)nchunks), 32 * kWarps, smem, s, H, ldh, fi, dZ, ldz, params, pstride, w_int, ldw, chunks, scale, dPre, partial,
+                   partial_stride, nslab, err);
         ++g_kernel_launches;
-        return cudaGetLastError();
+        return e;
     };
     switch (nq) {
         case 1: return go(narrow_bwd_kernel<1>);

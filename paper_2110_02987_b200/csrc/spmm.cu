@@ -117,8 +117,9 @@ spmm_items_narrow_kernel(const uint2* __restrict__ ecv, const int4* __restrict__
     const int lane = threadIdx.x & 31, gl = lane & (GROUP - 1);
     const unsigned gmask = (GROUP == 32 ? 0xffffffffu : ((1u << GROUP) - 1u)) << (lane & ~(GROUP - 1));
     const long long idx = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / GROUP;
+    pdl_next();
     if (idx >= nitems) return;   // the whole group leaves together
-    const Item it = load_item(items, (int)idx, ecv);
+    const Item it = load_item(items, (int)idx, ecv);   // (the store and its work list are nobody's output)
     const uint2 pad = make_uint2((uint32_t)it.row, 0u);
     const char* zl = reinterpret_cast<const char*>(Z) + (long long)OpBytes<BF>::quad * min(gl, F4 - 1);   // lanes past the last column read it again
     const uint32_t ldzb = OpBytes<BF>::elem * (uint32_t)ldz;
@@ -129,6 +130,9 @@ spmm_items_narrow_kernel(const uint2* __restrict__ ecv, const int4* __restrict__
         const int e = gl + GROUP * i;
         next[i] = (e < NB && e < it.len) ? __ldg(it.ent + e) : pad;
     }
+    pdl_wait();
+    after_wait(zl);
+    after_wait(ep.act.params);
     for (int b = 0; b < it.len; b += NB) {
         uint2 mine[EPL];
 #pragma unroll
@@ -153,11 +157,15 @@ __global__ void __launch_bounds__(256) spmm_finish_kernel(const int4* __restrict
                                                           float* __restrict__ out, int ldo, int F4, EpiDev ep) {
     const int lane = threadIdx.x & 31;
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    pdl_next();
     if (i >= nfin || lane >= GROUP) return;
     const int4 f = fin[i];  // {row, first slot, slots, subgraph of the row}
     float4 acc[NV];
 #pragma unroll
     for (int j = 0; j < NV; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    pdl_wait();
+    after_wait(scratch);
+    after_wait(ep.act.params);
     // several slots are loaded together and added in slot order (a slot past the last one counts as zero)
     constexpr int Q = NV == 1 ? 16 : (NV == 2 ? 8 : (NV <= 4 ? 4 : 2));
     for (int p = 0; p < f.z; p += Q) {
@@ -275,6 +283,7 @@ spmm_items_kernel(const uint2* __restrict__ ecv, const int4* __restrict__ items,
     __shared__ __align__(16) uint2 stage_all[kItemWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int idx = blockIdx.x * kItemWarps + warp;
+    pdl_next();
     if (idx >= nitems) return;
     uint2* stage = stage_all[warp];
     const Item item = load_item(items, idx, ecv);
@@ -289,13 +298,17 @@ spmm_items_kernel(const uint2* __restrict__ ecv, const int4* __restrict__ items,
     for (int j = 0; j < NV; ++j) {
         // PAIR (F4 even): position j < NV / 2 is the lane's j-th run of eight bfloat16 columns (16 bytes)
         zl.off[j] = PAIR ? 16u * (uint32_t)min(lane + 32 * j, F4 / 2 - 1) : OpBytes<BF>::quad * (uint32_t)min(lane + 32 * j, F4 - 1);
-        zl.ptr[j] = zl.base + zl.off[j];
     }
     float4 acc[NV];
 #pragma unroll
     for (int j = 0; j < NV; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
 
     uint2 next = lane < len ? __ldg(ent + lane) : pad;
+    pdl_wait();
+    after_wait(zl.base);
+#pragma unroll
+    for (int j = 0; j < NV; ++j) zl.ptr[j] = zl.base + zl.off[j];
+    after_wait(ep.act.params);
     for (int b = 0; b < len; b += 32) {
         const uint2 mine = next;
         const int cnt = min(32, len - b);
@@ -331,29 +344,29 @@ static cudaError_t launch_rows(const SparseDev& A, const float* Z, int ldz, floa
                 // a bfloat16 operand of a whole number of 8-column runs: 16-byte loads, eight columns per lane and load
                 if (F4 % 2 == 0 && ldz % 8 == 0) {
                     paired = true;
-                    if (off32) spmm_items_kernel<NV, EPI, true, true, true><<<grid, 32 * kItemWarps, 0, s>>>(A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
-                    else spmm_items_kernel<NV, EPI, false, true, true><<<grid, 32 * kItemWarps, 0, s>>>(A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+                    if (off32) launch(spmm_items_kernel<NV, EPI, true, true, true>, dim3(grid), 32 * kItemWarps, 0, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+                    else launch(spmm_items_kernel<NV, EPI, false, true, true>, dim3(grid), 32 * kItemWarps, 0, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
                 }
             }
             if (!paired) {
-                if (off32) spmm_items_kernel<NV, EPI, true, BF, false><<<grid, 32 * kItemWarps, 0, s>>>(A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
-                else spmm_items_kernel<NV, EPI, false, BF, false><<<grid, 32 * kItemWarps, 0, s>>>(A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+                if (off32) launch(spmm_items_kernel<NV, EPI, true, BF, false>, dim3(grid), 32 * kItemWarps, 0, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+                else launch(spmm_items_kernel<NV, EPI, false, BF, false>, dim3(grid), 32 * kItemWarps, 0, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
             }
             ++g_kernel_launches;
         }
         if (A.nfin > 0) {
-            spmm_finish_kernel<NV, GROUP, EPI><<<(unsigned)((A.nfin + 7) / 8), 256, 0, s>>>(A.fin, A.nfin, A.scratch, out, ldo, F4, ep);
+            launch(spmm_finish_kernel<NV, GROUP, EPI>, dim3((unsigned)((A.nfin + 7) / 8)), 256, 0, s, A.fin, A.nfin, A.scratch, out, ldo, F4, ep);
             ++g_kernel_launches;
         }
         return cudaGetLastError();
     }
     if (A.nitems > 0) {
         const unsigned grid = (unsigned)(((long long)A.nitems * GROUP + 255) / 256);
-        spmm_items_narrow_kernel<GROUP, EPI, BF><<<grid, 256, 0, s>>>(A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+        launch(spmm_items_narrow_kernel<GROUP, EPI, BF>, dim3(grid), 256, 0, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
         ++g_kernel_launches;
     }
     if (A.nfin > 0) {
-        spmm_finish_kernel<NV, GROUP, EPI><<<(unsigned)((A.nfin + 7) / 8), 256, 0, s>>>(A.fin, A.nfin, A.scratch, out, ldo, F4, ep);
+        launch(spmm_finish_kernel<NV, GROUP, EPI>, dim3((unsigned)((A.nfin + 7) / 8)), 256, 0, s, A.fin, A.nfin, A.scratch, out, ldo, F4, ep);
         ++g_kernel_launches;
     }
     return cudaGetLastError();
@@ -418,8 +431,11 @@ cudaError_t launch_check_store(const SparseDev& A, long long nnz, long long slot
 
 // fp32 -> bfloat16 (round to nearest even; NaN stays NaN), four values per thread.
 __global__ void __launch_bounds__(256) to_bf16_kernel(const float4* __restrict__ in, uint2* __restrict__ out, long long n4) {
+    pdl_next();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n4) return;
+    pdl_wait();
+    after_wait(in);
     out[i] = bf16_pack4(in[i]);
 }
 
@@ -432,7 +448,7 @@ cudaError_t launch_spmm(const SparseDev& A, const float* Z, int ldz, float* out,
     const int F4_all = (int)(round_up(F, 4) / 4);
     if (bf16_scratch && !bf16_ready && A.nrows > 0) {
         const long long n4 = (long long)A.nrows * (ldz / 4);
-        to_bf16_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, s>>>(reinterpret_cast<const float4*>(Z), reinterpret_cast<uint2*>(bf16_scratch), n4);
+        launch(to_bf16_kernel, dim3((unsigned)((n4 + 255) / 256)), 256, 0, s, reinterpret_cast<const float4*>(Z), reinterpret_cast<uint2*>(bf16_scratch), n4);
         ++g_kernel_launches;
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -70,7 +70,7 @@ struct Plan {
     std::vector<DwChunks> dw;         // [L] row chunks of each layer's weight gradient, their first chunk per subgraph [K+1]
     std::vector<int64_t> pair_ptr;    // [K+1] tiles of pairs per subgraph (zeta_mode 1 on the FP32 ALUs), else empty
     size_t o_pair_ptr = 0, o_pair_partial = 0;
-    std::vector<int64_t> gram_ptr;    // [K+1] 128 x 128 tiles of pairs per subgraph (zeta_mode 1 on the tensor cores)
+    std::vector<int64_t> gram_ptr;    // [K+1] 256 x 256 tiles of pairs per subgraph (zeta_mode 1 on the tensor cores)
     size_t o_gram_ptr = 0, o_gram_partial = 0, o_norm2 = 0, o_xhi = 0, o_xlo = 0;
     bool pair_alu_ok = false;         // every subgraph is small enough for the FP32-ALU pairwise kernel
     std::vector<uint8_t> agg_first;   // [L] the layer aggregates before it transforms: sigma((A~ H^(l)) W + b)
@@ -526,7 +526,7 @@ int zeta_pass(gad_ctx* ctx, cudaStream_t s) {
         if (rc != GAD_OK || (rc = forward_pass(ctx, false)) != GAD_OK) return rc;
     }
     if (ctx->cfg.zeta_mode == 1 && ctx->use_gram) {
-        const double pairs = 128.0 * 128.0 * (double)p.gram_ptr[p.K];
+        const double pairs = 256.0 * 256.0 * (double)p.gram_ptr[p.K];
         GAD_RUN("zeta", -1, 4.0 * p.Np * (p.dims[0] + 2), 2.0 * pairs * p.dims[0], [&] {
             return launch_zeta_gram(&ctx->map_xhi, &ctx->map_xlo, ctx->H(0), p.ld[0], p.dims[0], p.Np, ctx->at<int32_t>(p.o_deg),
                                     ctx->at<int32_t>(p.o_sub_off), ctx->at<int64_t>(p.o_deg_sum), ctx->at<int64_t>(p.o_gram_ptr),
@@ -910,8 +910,8 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
     }
     if (ctx->cfg.zeta_mode == 1) {
         ctx->use_gram = ctx->use_tc && !p.gram_ptr.empty();
-        if (ctx->use_gram && !(tc_make_map(&ctx->map_xhi, ctx->at<float>(p.o_xhi), p.dims[0], p.Np, 0, 4ull * p.ld[0], 0, 128) &&
-                               tc_make_map(&ctx->map_xlo, ctx->at<float>(p.o_xlo), p.dims[0], p.Np, 0, 4ull * p.ld[0], 0, 128)))
+        if (ctx->use_gram && !(tc_make_map(&ctx->map_xhi, ctx->at<float>(p.o_xhi), p.dims[0], p.Np, 0, 4ull * p.ld[0], 0, zeta_gram_box_rows()) &&
+                               tc_make_map(&ctx->map_xlo, ctx->at<float>(p.o_xlo), p.dims[0], p.Np, 0, 4ull * p.ld[0], 0, zeta_gram_box_rows())))
             return fail(ctx, GAD_ERR_CUDA, "cuTensorMapEncodeTiled failed");
         if (!ctx->use_gram && !p.pair_alu_ok)
             return fail(ctx, GAD_ERR_UNSUPPORTED, "zeta_mode 1 without the tensor-core kernel takes subgraphs of at most " +

@@ -2,24 +2,31 @@
 //   zeta_k = sum over unordered pairs i < j of subgraph k of  p_i p_j / (|x_i - x_j|_2 + beta),
 // with the squared distances taken from a Gram matrix on the tensor cores:
 //   |x_i - x_j|^2 = |x_i|^2 + |x_j|^2 - 2 x_i . x_j .
-// The pairs of a subgraph are cut into tiles of 128 x 128 (i-block <= j-block).  A tile's inner products are one
-// tcgen05 accumulator: both operand tiles are rows of the feature matrix (K-major, loaded by TMA with the 128-byte
-// swizzle).  The features are split once per call into TF32-exact hi and lo = x - hi copies (a streaming kernel that
-// also takes the squared norms), and the product is accumulated as hi.hi + hi.lo + lo.hi in fp32 in tensor memory -
-// the error-compensated product of the layer transforms, here with both operands split ahead of time because the
-// drain below needs the SM's issue slots.  While the MMA warp fills the second accumulator, sixteen warps read the
-// first one back (tcgen05.ld), turn every inner product into a distance and add p_j / (d + beta) over the pairs
-// i < j inside the subgraph (approximate square root and reciprocal, relative error 2^-23 each: far inside the
-// 2e-6 the result is held to, and the errors of different pairs do not add up coherently).
+// The pairs of a subgraph are cut into tiles of 256 x 256 (i-block <= j-block).  A tile's inner products are one tcgen05 accumulator of a
+// pair of CTAs: each CTA holds 128 rows of the i-block and half of the j-block (rows of the feature matrix, K-major, loaded by TMA with the
+// 128-byte swizzle) and receives 128 x 256 products.  The features are split once per call into TF32-exact hi and lo = x - hi copies (a
+// streaming kernel that also takes the squared norms), and the product is accumulated as hi.hi + hi.lo + lo.hi in fp32 in tensor memory -
+// the error-compensated product of the layer transforms, here with both operands split ahead of time because the drain below needs the
+// SM's issue slots.  What bounds it is the tensor pipe; in 128 x 128 tiles of one CTA it was shared memory, read for A and B at the rate
+// of the MMAs and written by TMA on top (8 x 6560 rows of 128: 300 us, now 182; of 32: 245, now 140).
+//
+// While the MMA warp fills the second accumulator, sixteen warps read the first one back (tcgen05.ld), turn every inner product into a
+// distance and add p_j / (d + beta) over the pairs i < j inside the subgraph.  Two pairs share a reciprocal, p / x + q / y = (p y + q x) /
+// (x y): with a square root and half a reciprocal per pair the special-function unit (16 a cycle and SM) keeps up with the MMAs from 64
+// features on.  (Approximate square root and reciprocal, relative error 2^-23 each: far inside the 2e-6 the result is held to, and the
+// errors of different pairs do not add up coherently.)
 //
 // Cancellation: for two rows that are close compared with their norms the Gram form loses digits, so a pair whose
-// squared distance comes out below 5 % of |x_i|^2 + |x_j|^2 is recomputed from the differences x_if - x_jf
+// squared distance comes out below 5 % of |x_i|^2 + |x_j|^2 is computed from the differences x_if - x_jf
 // themselves (plain loads, FP32 ALU).  On generic features that never happens; on features that are all alike it is
 // every pair, which then costs what the FP32 tile kernel of zeta_pair.cu costs.
 //
-// Order of the sum: persistent CTAs take the tiles t = blockIdx.x, blockIdx.x + gridDim.x, ... (ascending, subgraph
-// by subgraph); every draining warp keeps one fp64 running sum per subgraph and writes it to its own slot; a second
-// kernel adds the slots in slot order.  For a given number of CTAs the result does not depend on scheduling.
+// Order of the sum: every cluster takes a contiguous range of tiles (ascending, subgraph by subgraph; the i-block stays in L2); every
+// draining warp keeps one fp64 running sum per subgraph and writes it to its own slot; a second kernel adds the slots of the clusters
+// whose ranges meet the subgraph in slot order.  For a given number of clusters the result does not depend on scheduling.
+#include <algorithm>
+#include <atomic>
+
 #include "gad_internal.h"
 #include "tc_common.cuh"
 
@@ -27,18 +34,21 @@ namespace gad {
 
 namespace {
 
-constexpr int GT = 128;                                   // rows of a tile side (M and N of the MMA)
+constexpr int GT = 256;                                   // rows of a tile side
+constexpr int GH = 128;                                   // rows of a tile a CTA has of A (M of the pair's MMA is twice that)
+constexpr int GBOX = 64;                                  // rows of a TMA box
 constexpr int GBK = 32;                                   // features per ring stage
-constexpr int G_TILE_BYTES = GT * GBK * 4;                // 16 KiB
+constexpr int G_TILE_BYTES = GH * GBK * 4;                // 16 KiB
+constexpr int G_BOX_BYTES = GBOX * GBK * 4;
 constexpr int G_STAGE_BYTES = 4 * G_TILE_BYTES;           // A_hi | A_lo | B_hi | B_lo
 constexpr int G_STAGES = 3;
 constexpr int G_RING_BYTES = G_STAGES * G_STAGE_BYTES;
-constexpr int G_EPI_WARPS = 16;                           // four per quarter of the tensor-memory lanes, one block of 32 columns each
+constexpr int G_EPI_WARPS = 16;                           // four per quarter of the tensor-memory lanes, every fourth block of 32 columns each
 constexpr int G_EPI_WARP0 = 2;
 constexpr int G_THREADS = 32 * (G_EPI_WARP0 + G_EPI_WARPS);
 constexpr int G_COL_BYTES = G_EPI_WARPS * 32 * 8;         // per draining warp: (p_j, |x_j|^2) of its 32 columns
 constexpr int G_SMEM_BYTES = G_RING_BYTES + 1024 + 256 + G_COL_BYTES;
-constexpr int G_TMEM_COLS = 2 * GT;                       // two accumulators of 128 columns
+constexpr int G_TMEM_COLS = 2 * GT;                       // two accumulators of 256 columns: all of it
 
 struct GramArgs {
     const float* X;            // [rows x ld] features in store-row order
@@ -49,37 +59,53 @@ struct GramArgs {
     const int64_t* deg_sum;
     const int64_t* tile_ptr;   // [K+1] first tile of every subgraph
     int K;
-    long long ntiles;
+    long long ntiles;          // tiles x parts
+    int parts;                 // column parts of a tile, each taken on its own: 1, or 2 of 128 columns
     float beta;
-    double* partial;           // [gridDim.x][G_EPI_WARPS][K]
+    double* partial;           // [gridDim.x][G_EPI_WARPS][K], slots of subgraphs the cluster does not meet unwritten
     int32_t* err;
 };
 
-struct TilePos { int k, r0, n, i0, j0; };
+// Contiguous share of cluster c out of n.
+__host__ __device__ __forceinline__ long long share(long long ntiles, int c, int n) { return ntiles * c / n; }
 
-// Tile t of the list: subgraph k (largest k with tile_ptr[k] <= t), then (bi, bj), bi <= bj, from the position inside
-// the row-major list of the upper triangle of T x T blocks.
-__device__ __forceinline__ TilePos tile_pos(const GramArgs& a, long long t) {
-    int lo = 0, hi = a.K;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (a.tile_ptr[mid] <= t) lo = mid; else hi = mid;
+// A position in the list of (tile, part): subgraph by subgraph, the upper triangle of its T x T blocks row by row.
+struct TilePos {
+    int k, r0, n, T, bi, bj, part;
+    __device__ __forceinline__ void open(const GramArgs& a, int k_) {
+        k = k_;
+        r0 = a.sub_off[k];
+        n = a.sub_off[k + 1] - r0;
+        T = (n + GT - 1) / GT;
     }
-    TilePos p;
-    p.k = lo;
-    p.r0 = a.sub_off[lo];
-    p.n = a.sub_off[lo + 1] - p.r0;
-    const long long T = (p.n + GT - 1) / GT;
-    const long long q = t - a.tile_ptr[lo];
-    long long bi = (long long)(((double)(2 * T + 1) - sqrt((double)(2 * T + 1) * (double)(2 * T + 1) - 8.0 * (double)q)) * 0.5);
-    bi = max(0ll, min(bi, T - 1));
-    while (bi > 0 && bi * T - bi * (bi - 1) / 2 > q) --bi;                      // rows before bi hold bi T - bi (bi - 1) / 2 tiles
-    while (bi + 1 < T && (bi + 1) * T - (bi + 1) * bi / 2 <= q) ++bi;
-    const long long bj = bi + (q - (bi * T - bi * (bi - 1) / 2));
-    p.i0 = (int)bi * GT;
-    p.j0 = (int)bj * GT;
-    return p;
-}
+    __device__ __forceinline__ TilePos(const GramArgs& a, long long tp) {
+        part = (int)(tp % a.parts);
+        const long long t = tp / a.parts;
+        int lo = 0, hi = a.K;                              // the largest k with tile_ptr[k] <= t
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (a.tile_ptr[mid] <= t) lo = mid; else hi = mid;
+        }
+        open(a, lo);
+        long long q = t - a.tile_ptr[lo];
+        bi = 0;
+        while (bi + 1 < T && q >= T - bi) { q -= T - bi; ++bi; }
+        bj = bi + (int)q;
+    }
+    __device__ __forceinline__ void next(const GramArgs& a) {
+        if (++part < a.parts) return;
+        part = 0;
+        if (++bj < T) return;
+        bj = ++bi;
+        if (bi < T) return;
+        bi = bj = 0;
+        int nk = k + 1;
+        while (nk < a.K - 1 && a.tile_ptr[nk + 1] == a.tile_ptr[nk]) ++nk;   // (subgraphs without rows have no tiles)
+        if (nk < a.K) open(a, nk);
+    }
+    __device__ __forceinline__ int i0() const { return bi * GT; }
+    __device__ __forceinline__ int j0(const GramArgs& a) const { return bj * GT + part * (GT / a.parts); }
+};
 
 __device__ __forceinline__ float sqrt_approx(float x) {
     float y;
@@ -92,108 +118,167 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 
-__global__ void __launch_bounds__(G_THREADS, 1)
+// p_j / (d_ij + beta) summed over 16 columns j of one row i.  EACH: only the columns first .. last - 1, and without the pairs that have to be
+// taken from the differences; those are reported in `close` either way.
+template <bool EACH>
+__device__ __forceinline__ float gram_terms(const uint32_t (&v)[16], const float2* cols, float ni, float beta, int first, int last, bool& close) {
+    float part = 0.f, p0 = 0.f, x0 = 0.f;
+#pragma unroll
+    for (int jj = 0; jj < 16; ++jj) {
+        float2 c = cols[jj];                                   // (p_j, |x_j|^2), one broadcast load
+        const float s2 = ni + c.y;
+        float d2 = fmaf(-2.f, __uint_as_float(v[jj]), s2);
+        bool near = d2 < 0.05f * s2;
+        if (EACH) {
+            const bool valid = jj >= first && jj < last;
+            const bool counts = valid && !near;
+            near = near && valid;
+            c.x = counts ? c.x : 0.f;
+            d2 = counts ? d2 : 1.f;
+        }
+        close |= near;
+        const float x = sqrt_approx(d2) + beta;
+        if (jj & 1) part = fmaf(fmaf(p0, x, c.x * x0), rcp_approx(x0 * x), part);
+        p0 = c.x; x0 = x;
+    }
+    return part;
+}
+
+__device__ __noinline__ float distance2(const float4* x, const float4* y, int n4) {
+    float s = 0.f;
+    for (int f = 0; f < n4; ++f) {       // pad columns are zero
+        const float4 u = __ldg(x + f), w = __ldg(y + f);
+        const float dx = u.x - w.x, dy = u.y - w.y, dz = u.z - w.z, dw = u.w - w.w;
+        s = fmaf(dx, dx, s); s = fmaf(dy, dy, s); s = fmaf(dz, dz, s); s = fmaf(dw, dw, s);
+    }
+    return s;
+}
+
+// This warp's 32 tensor-memory lanes x 16 columns, complete on return: lane t receives its own lane's.
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+          "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(addr)
+        : "memory");
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(G_THREADS, 1)
 zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant__ CUtensorMap tmLo, const GramArgs a) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
-    const uint32_t pad = ((raw_addr + 1023u) & ~1023u) - raw_addr;
-    uint8_t* sm = smem_raw + pad;                 // 1024-byte aligned: the 128B swizzle pattern repeats every 1024 bytes
+    const uint32_t pad = ((raw_addr + 1023u) & ~1023u) - raw_addr;   // the same in both CTAs (the 128B swizzle repeats every 1024 bytes)
+    uint8_t* sm = smem_raw + pad;
     const uint32_t sm_addr = raw_addr + pad;
+    const uint32_t rank = cluster_rank();
     const uint32_t bars = sm_addr + G_RING_BYTES;
     auto full = [&](int s) { return bars + 8u * s; };
     auto empty = [&](int s) { return bars + 8u * (G_STAGES + s); };
-    auto tfull = [&](int i) { return bars + 8u * (2 * G_STAGES + i); };
-    auto tempty = [&](int i) { return bars + 8u * (2 * G_STAGES + 2 + i); };
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + G_RING_BYTES + 8 * (2 * G_STAGES + 4));
+    auto pfull = [&](int s) { return bars + 8u * (2 * G_STAGES + s); };      // leader: the other CTA's stage is full
+    auto tfull = [&](int i) { return bars + 8u * (3 * G_STAGES + i); };
+    auto tempty = [&](int i) { return bars + 8u * (3 * G_STAGES + 2 + i); };
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + G_RING_BYTES + 8 * (3 * G_STAGES + 4));
     volatile uint32_t* abort_flag = tmem_slot + 1;
     float2* col_sm = reinterpret_cast<float2*>(sm + G_RING_BYTES + 256);   // [G_EPI_WARPS][32]
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < G_STAGES; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(tfull(i), 1); mbar_init(tempty(i), G_EPI_WARPS); }
+        for (int s = 0; s < G_STAGES; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); mbar_init(pfull(s), 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(tfull(i), 1); mbar_init(tempty(i), 2 * G_EPI_WARPS); }
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(G_TMEM_COLS) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    if (warp == 0) tmem_alloc2(smem_u32(tmem_slot), G_TMEM_COLS);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    cluster_sync();           // the peer's barriers exist before anything arrives at them
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
 
-    const int nkb = (a.F + GBK - 1) / GBK;
+    const int nkb = (a.F + GBK - 1) / GBK, width = GT / a.parts;
+    const int ncl = gridDim.x >> 1, cl = blockIdx.x >> 1;
+    const long long t_begin = share(a.ntiles, cl, ncl), t_end = share(a.ntiles, cl + 1, ncl);
 
     if (warp == 0 && lane == 0) {
-        // ---------------- TMA producer: hi and lo of the two row blocks of the tile, 32 features at a time ----------------
+        // ---------------- TMA producer: hi and lo of this CTA's rows of the two blocks of the tile, 32 features at a time ----------------
         int stage = 0;
         uint32_t phase = 0;
         bool ok = true;
-        for (long long t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
-            const TilePos p = tile_pos(a, t);
+        TilePos p(a, t_begin);
+        for (long long t = t_begin; t < t_end && ok; ++t, p.next(a)) {
+            const int ri = p.r0 + p.i0() + (int)rank * GH, rj = p.r0 + p.j0(a) + (int)rank * (width / 2);
             for (int kb = 0; kb < nkb; ++kb) {
                 if (!(ok = mbar_wait(empty(stage), phase ^ 1u, abort_flag, a.err, 21))) break;
-                mbar_expect_tx(full(stage), 4u * G_TILE_BYTES);
+                mbar_expect_tx(full(stage), 2u * G_TILE_BYTES + 2u * (uint32_t)(width / 2) * (GBK * 4));
                 const uint32_t base = sm_addr + stage * G_STAGE_BYTES;
-                tma_load_2d(base, &tmHi, kb * GBK, p.r0 + p.i0, full(stage));
-                tma_load_2d(base + G_TILE_BYTES, &tmLo, kb * GBK, p.r0 + p.i0, full(stage));
-                tma_load_2d(base + 2 * G_TILE_BYTES, &tmHi, kb * GBK, p.r0 + p.j0, full(stage));
-                tma_load_2d(base + 3 * G_TILE_BYTES, &tmLo, kb * GBK, p.r0 + p.j0, full(stage));
+                for (int b = 0; b < GH / GBOX; ++b) {
+                    tma_load_2d(base + b * G_BOX_BYTES, &tmHi, kb * GBK, ri + b * GBOX, full(stage));
+                    tma_load_2d(base + G_TILE_BYTES + b * G_BOX_BYTES, &tmLo, kb * GBK, ri + b * GBOX, full(stage));
+                }
+                for (int b = 0; b < width / 2 / GBOX; ++b) {
+                    tma_load_2d(base + 2 * G_TILE_BYTES + b * G_BOX_BYTES, &tmHi, kb * GBK, rj + b * GBOX, full(stage));
+                    tma_load_2d(base + 3 * G_TILE_BYTES + b * G_BOX_BYTES, &tmLo, kb * GBK, rj + b * GBOX, full(stage));
+                }
                 if (++stage == G_STAGES) { stage = 0; phase ^= 1u; }
             }
         }
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer ----------------
+    } else if (warp == 1 && rank == 1) {
+        // ---------------- the other CTA's stages: the leader is told of each ----------------
+        int stage = 0;
+        uint32_t phase = 0;
+        for (long long i = (t_end - t_begin) * nkb; i > 0 && lane == 0; --i) {
+            if (!mbar_wait(full(stage), phase, abort_flag, a.err, 24)) break;
+            mbar_arrive_leader(pfull(stage));
+            if (++stage == G_STAGES) { stage = 0; phase ^= 1u; }
+        }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer (leader of the pair): the whole warp runs the loop, one elected lane issues ----------------
         int stage = 0, acc = 0;
         uint32_t phase = 0, acc_phase = 0;
-        const uint32_t idesc = instr_desc(GT);
+        const uint32_t idesc = instr_desc(width, 2 * GH);
         bool ok = true;
-        for (long long t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
-            if (!(ok = mbar_wait(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 22))) break;
+        for (long long t = t_begin; t < t_end && ok; ++t) {
+            if (!(ok = __all_sync(0xffffffffu, mbar_wait(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 22)))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t d = tmem_base + (uint32_t)(acc * GT);
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!(ok = mbar_wait(full(stage), phase, abort_flag, a.err, 23))) break;
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait(full(stage), phase, abort_flag, a.err, 23) &&
+                                                       mbar_wait(pfull(stage), phase, abort_flag, a.err, 25)))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t base = sm_addr + stage * G_STAGE_BYTES;
                 const uint64_t a_hi = smem_desc(base), a_lo = smem_desc(base + G_TILE_BYTES);
                 const uint64_t b_hi = smem_desc(base + 2 * G_TILE_BYTES), b_lo = smem_desc(base + 3 * G_TILE_BYTES);
                 const int nks = min(GBK / 8, (a.F - kb * GBK + 7) / 8);
-                if (nks == GBK / 8) {
+                if (elect_one()) {
+                    // 8 TF32 values = 32 bytes = 2 descriptor units along K
 #pragma unroll
-                    for (int ks = 0; ks < GBK / 8; ++ks) {           // 8 TF32 values = 32 bytes = 2 descriptor units along K
-                        mma_tf32(d, a_hi + 2 * ks, b_hi + 2 * ks, idesc, ks == 0 ? (kb != 0 ? 1u : 0u) : 1u);
-                        mma_tf32(d, a_hi + 2 * ks, b_lo + 2 * ks, idesc, 1u);
-                        mma_tf32(d, a_lo + 2 * ks, b_hi + 2 * ks, idesc, 1u);
-                    }
-                } else {
-                    for (int ks = 0; ks < nks; ++ks) {
-                        const uint64_t adv = (uint64_t)(2 * ks);
-                        mma_tf32(d, a_hi + adv, b_hi + adv, idesc, (kb | ks) != 0 ? 1u : 0u);
-                        mma_tf32(d, a_hi + adv, b_lo + adv, idesc, 1u);
-                        mma_tf32(d, a_lo + adv, b_hi + adv, idesc, 1u);
-                    }
+                    for (int ks = 0; ks < GBK / 8; ++ks)
+                        if (ks < nks) {
+                            mma_tf32_pair(d, a_hi + 2 * ks, b_hi + 2 * ks, idesc, (kb | ks) != 0 ? 1u : 0u);
+                            mma_tf32_pair(d, a_hi + 2 * ks, b_lo + 2 * ks, idesc, 1u);
+                            mma_tf32_pair(d, a_lo + 2 * ks, b_hi + 2 * ks, idesc, 1u);
+                        }
+                    mma_commit2(empty(stage));                    // in both CTAs
+                    if (kb == nkb - 1) mma_commit2(tfull(acc));
                 }
-                mma_commit(empty(stage));
+                __syncwarp();
                 if (++stage == G_STAGES) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) break;
-            mma_commit(tfull(acc));
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
     } else if (warp >= G_EPI_WARP0) {
         // ---------------- drain: inner products -> distances -> weighted sum over the pairs i < j ----------------
-        // this warp may read tensor-memory lanes 32q .. 32q+31 (tile rows i); of the four warps of a quarter each takes
-        // one block of 32 columns (tile columns j)
-        const int ew = warp - G_EPI_WARP0, q = warp & 3, c0 = 32 * (ew >> 2);
+        // this warp may read tensor-memory lanes 32q .. 32q+31 (this CTA's rows i of the tile); of the four warps of a quarter each takes
+        // every fourth block of 32 columns (tile columns j)
+        const int ew = warp - G_EPI_WARP0, q = warp & 3;
         float2* cols = col_sm + ew * 32;
-        int acc = 0;
+        int acc = 0, cur_k = -1;
         uint32_t acc_phase = 0;
-        bool ok = true;
+        bool ok = true, uniform = false;
         double sum = 0.0;
-        int cur_k = -1;
+        float invD = 0.f;
         double* slot = a.partial + ((long long)blockIdx.x * G_EPI_WARPS + ew) * a.K;
         auto flush = [&]() {
             if (cur_k < 0) return;
@@ -202,88 +287,69 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
             if (lane == 0) slot[cur_k] = sum;
             sum = 0.0;
         };
-        for (long long t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
-            const TilePos p = tile_pos(a, t);
-            if (p.k != cur_k) { flush(); cur_k = p.k; }
-            const bool uniform = a.deg_sum[p.k] == 0;
-            const float invD = (float)(1.0 / (uniform ? (double)p.n : (double)a.deg_sum[p.k]));
-            const int i = p.i0 + q * 32 + lane;                       // this thread's row of the tile, inside the subgraph
+        TilePos p(a, t_begin);
+        for (long long t = t_begin; t < t_end; ++t, p.next(a)) {
+            if (p.k != cur_k) {
+                flush();
+                cur_k = p.k;
+                uniform = a.deg_sum[p.k] == 0;
+                invD = (float)(1.0 / (uniform ? (double)p.n : (double)a.deg_sum[p.k]));
+            }
+            const int ib = p.i0() + (int)rank * GH + q * 32, i = ib + lane;   // this thread's row of the tile, inside the subgraph
             const bool iv = i < p.n;
             const float pi = iv ? (uniform ? 1.f : (float)a.deg[p.r0 + i]) * invD : 0.f;
             const float ni = iv ? a.norm2[p.r0 + i] : 0.f;
-            {
-                const int jl = p.j0 + c0 + lane;                      // the column this lane looks up for the warp
-                const bool jlv = jl < p.n;
-                __syncwarp();                                         // the previous tile's columns have been read
-                cols[lane] = make_float2(jlv ? (uniform ? 1.f : (float)a.deg[p.r0 + jl]) * invD : 0.f, jlv ? a.norm2[p.r0 + jl] : 0.f);
-                __syncwarp();
-            }
             if (!(ok = __all_sync(0xffffffffu, mbar_wait(tfull(acc), acc_phase, abort_flag, a.err, 26)))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            uint32_t v[32];
-            tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * GT + c0), v);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            // the accumulator block is in registers: hand the accumulator back before the arithmetic
+            float part = 0.f;
+            for (int c0 = 32 * (ew >> 2); c0 < width; c0 += 128) {
+                const int jb = p.j0(a) + c0;
+                if (jb + 31 <= ib || jb >= p.n || ib >= p.n) continue;        // no pair i < j of the subgraph in this block
+                __syncwarp();                                                // the previous block's columns have been read
+                {
+                    const int jl = jb + lane;                                // the column this lane looks up for the warp
+                    const bool jlv = jl < p.n;
+                    cols[lane] = make_float2(jlv ? (uniform ? 1.f : (float)a.deg[p.r0 + jl]) * invD : 0.f, jlv ? a.norm2[p.r0 + jl] : 0.f);
+                }
+                __syncwarp();
+                const float4* xi = reinterpret_cast<const float4*>(a.X + (long long)(p.r0 + min(i, p.n - 1)) * a.ld);
+                for (int h = 0; h < 32; h += 16) {                           // (32 at a time do not fit the registers)
+                    uint32_t v[16];
+                    tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * GT + c0 + h), v);
+                    // every pair of the block counts, or the columns [first, last) of this row do
+                    const bool whole = ib + 31 < jb + h && ib + 31 < p.n && jb + h + 15 < p.n;
+                    const int first = i + 1 - jb - h, last = iv ? min(16, p.n - jb - h) : 0;
+                    bool close = false;
+                    float blk = 0.f;
+                    if (whole) blk = gram_terms<false>(v, cols + h, ni, a.beta, 0, 16, close);
+                    if (!whole || __any_sync(0xffffffffu, close)) {
+                        close = false;
+                        blk = gram_terms<true>(v, cols + h, ni, a.beta, first, last, close);
+                        if (close) {   // rows close to each other compared with their norms: those pairs from the differences themselves
+#pragma unroll
+                            for (int jj = 0; jj < 16; ++jj) {                // (unrolled: the accumulator block stays in registers)
+                                const float2 c = cols[h + jj];
+                                const float s2 = ni + c.y;
+                                const float d2 = fmaf(-2.f, __uint_as_float(v[jj]), s2);
+                                if (jj >= first && jj < last && d2 < 0.05f * s2)
+                                    blk += c.x / (sqrtf(distance2(xi, reinterpret_cast<const float4*>(a.X + (long long)(p.r0 + jb + h + jj) * a.ld), a.ld >> 2)) + a.beta);
+                            }
+                        }
+                    }
+                    part += blk;
+                }
+            }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(tempty(acc));
+            if (lane == 0) mbar_arrive_leader(tempty(acc));
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
-
-            // every pair of the block counts (a tile off the diagonal and wholly inside the subgraph), or each is tested
-            const bool whole = p.i0 != p.j0 && p.i0 + GT <= p.n && p.j0 + GT <= p.n;
-            float part = 0.f;
-            bool close = false;
-            if (whole) {
-#pragma unroll
-                for (int jj = 0; jj < 32; ++jj) {
-                    const float2 c = cols[jj];                         // (p_j, |x_j|^2), one broadcast load
-                    const float s2 = ni + c.y;
-                    const float d2 = fmaf(-2.f, __uint_as_float(v[jj]), s2);
-                    close |= d2 < 0.05f * s2;
-                    part = fmaf(c.x, rcp_approx(sqrt_approx(fmaxf(d2, 0.f)) + a.beta), part);
-                }
-            } else {
-#pragma unroll
-                for (int jj = 0; jj < 32; ++jj) {
-                    const float2 c = cols[jj];
-                    const int j = p.j0 + c0 + jj;
-                    const bool valid = iv && j < p.n && i < j;
-                    const float s2 = ni + c.y;
-                    const float d2 = fmaf(-2.f, __uint_as_float(v[jj]), s2);
-                    close |= valid && d2 < 0.05f * s2;
-                    const float term = c.x * rcp_approx(sqrt_approx(fmaxf(d2, 0.f)) + a.beta);
-                    part += valid ? term : 0.f;
-                }
-            }
-            if (__any_sync(0xffffffffu, close)) {
-                // rows close to each other compared with their norms: those pairs again, from the differences themselves
-                const float4* xi = reinterpret_cast<const float4*>(a.X + (long long)(p.r0 + min(i, p.n - 1)) * a.ld);
-#pragma unroll
-                for (int jj = 0; jj < 32; ++jj) {                      // (unrolled: the accumulator block stays in registers)
-                    const float2 c = cols[jj];
-                    const int j = p.j0 + c0 + jj;
-                    const bool valid = iv && j < p.n && i < j;
-                    const float s2 = ni + c.y;
-                    const float d2 = fmaf(-2.f, __uint_as_float(v[jj]), s2);
-                    if (valid && d2 < 0.05f * s2) {
-                        const float4* xj = reinterpret_cast<const float4*>(a.X + (long long)(p.r0 + j) * a.ld);
-                        float s = 0.f;
-                        for (int f4 = 0; f4 < (a.ld >> 2); ++f4) {       // pad columns are zero
-                            const float4 u = __ldg(xi + f4), w = __ldg(xj + f4);
-                            const float dx = u.x - w.x, dy = u.y - w.y, dz = u.z - w.z, dw = u.w - w.w;
-                            s = fmaf(dx, dx, s); s = fmaf(dy, dy, s); s = fmaf(dz, dz, s); s = fmaf(dw, dw, s);
-                        }
-                        part += c.x / (sqrtf(s) + a.beta) - c.x * rcp_approx(sqrt_approx(fmaxf(d2, 0.f)) + a.beta);
-                    }
-                }
-            }
             sum += (double)(pi * part);
         }
         if (ok) flush();
     }
 
-    // Tear-down.  After a time-out, give loads that may still be in flight a bounded chance to land before the
-    // shared memory is released.
+    // Tear-down.  After a time-out, give loads that may still be in flight a bounded chance to land before the shared memory is
+    // released.  Neither CTA leaves while the other may still read its operands or arrive at its barriers.
     __syncthreads();
     if (*abort_flag && threadIdx.x == 0)
         for (int s = 0; s < G_STAGES; ++s)
@@ -291,9 +357,10 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
                 if (mbar_try_wait(full(s), 0) || mbar_try_wait(full(s), 1)) break;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    cluster_sync();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(G_TMEM_COLS) : "memory");
+        tmem_dealloc2(tmem_base, G_TMEM_COLS);
     }
 }
 
@@ -324,24 +391,50 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict
     if (lane == 0) norm2[r] = s;
 }
 
-// zeta_k = the slots of subgraph k added in slot order (one warp per subgraph).
-__global__ void zeta_gram_finish_kernel(const double* __restrict__ partial, int nslots, int K, double* __restrict__ zeta) {
-    const int k = blockIdx.x, lane = threadIdx.x;
+// zeta_k = the slots of the clusters that meet subgraph k added in slot order (one CTA per subgraph; a warp adds every eighth slot).
+__global__ void __launch_bounds__(256) zeta_gram_finish_kernel(const double* __restrict__ partial, const int64_t* __restrict__ tile_ptr, long long ntiles,
+                                                               int parts, int ncl, int K, double* __restrict__ zeta) {
+    __shared__ double warp_sum[8];
+    const int k = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long t0 = tile_ptr[k] * parts, t1 = tile_ptr[k + 1] * parts;
     double s = 0.0;
-    for (int i = lane; i < nslots; i += 32) s += partial[(long long)i * K + k];
+    for (int c = w; c < ncl; c += 8)
+        if (share(ntiles, c, ncl) < t1 && share(ntiles, c + 1, ncl) > t0) s += partial[((long long)c * 2 * G_EPI_WARPS + lane) * K + k];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) zeta[k] = s;
+    if (lane == 0) warp_sum[w] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < 8; ++i) s += warp_sum[i];
+        zeta[k] = s;
+    }
+}
+static_assert(2 * G_EPI_WARPS == 32, "a warp reads the slots of a cluster");
+
+// Clusters of two CTAs that fit the GPU at once (a cluster stays inside a GPC).
+int gram_clusters(int num_sms) {
+    static std::atomic<int> known{0};
+    int c = known.load();
+    if (c > 0) return c;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(num_sms & ~1)); cfg.blockDim = dim3(G_THREADS); cfg.dynamicSmemBytes = G_SMEM_BYTES; cfg.attrs = attr; cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&c, zeta_gram_kernel, &cfg) != cudaSuccess || c < 1) { cudaGetLastError(); c = num_sms / 2; }
+    known.store(c);
+    return c;
 }
 
 }  // namespace
 
-// Tiles of a subgraph of `rows` rows: T (T + 1) / 2 with T = ceil(rows / 128).
+// Tiles of a subgraph of `rows` rows: T (T + 1) / 2 with T = ceil(rows / 256).
 int64_t zeta_gram_tiles(int64_t rows) {
     const int64_t T = (rows + GT - 1) / GT;
     return T * (T + 1) / 2;
 }
 int64_t zeta_gram_partials(int num_sms, int K) { return (int64_t)num_sms * G_EPI_WARPS * K; }
+uint32_t zeta_gram_box_rows() { return GBOX; }
 
 cudaError_t launch_zeta_gram(const void* mapHi, const void* mapLo, const float* X, int ld, int F, long long rows, const int32_t* deg,
                              const int32_t* sub_off, const int64_t* deg_sum, const int64_t* tile_ptr, int64_t ntiles, int K, float beta,
@@ -351,18 +444,22 @@ cudaError_t launch_zeta_gram(const void* mapHi, const void* mapLo, const float* 
     if (e != cudaSuccess) return e;
     split_rows_kernel<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(X, ld, rows, Xhi, Xlo, norm2);
     ++g_kernel_launches;
-    e = cudaMemsetAsync(partial, 0, sizeof(double) * (size_t)zeta_gram_partials(num_sms, K), s);
-    if (e != cudaSuccess) return e;
-    if (ntiles > 0) {
-        GramArgs a;
-        a.X = X; a.ld = ld; a.F = F; a.norm2 = norm2; a.deg = deg; a.sub_off = sub_off; a.deg_sum = deg_sum; a.tile_ptr = tile_ptr;
-        a.K = K; a.ntiles = ntiles; a.beta = beta; a.partial = partial; a.err = err;
-        const unsigned grid = (unsigned)(ntiles < num_sms ? ntiles : num_sms);
-        zeta_gram_kernel<<<grid, G_THREADS, G_SMEM_BYTES, s>>>(*reinterpret_cast<const CUtensorMap*>(mapHi),
-                                                               *reinterpret_cast<const CUtensorMap*>(mapLo), a);
+    GramArgs a;
+    a.X = X; a.ld = ld; a.F = F; a.norm2 = norm2; a.deg = deg; a.sub_off = sub_off; a.deg_sum = deg_sum; a.tile_ptr = tile_ptr;
+    a.K = K; a.beta = beta; a.partial = partial; a.err = err;
+    // Tiles of 256 columns keep the tensor pipe busy.  Tiles of 128 read A twice as often and wait for shared memory, a quarter longer
+    // per column, but where there are few tiles they share them out better.
+    const int64_t most = std::max(1, std::min(gram_clusters(num_sms), num_sms / 2));
+    const auto turns = [&](int64_t n) { return (n + most - 1) / most; };
+    a.parts = 5 * turns(2 * ntiles) < 8 * turns(ntiles) ? 2 : 1;
+    a.ntiles = ntiles * a.parts;
+    const int ncl = (int)std::min<int64_t>(a.ntiles, most);
+    if (ncl > 0) {
+        zeta_gram_kernel<<<2 * ncl, G_THREADS, G_SMEM_BYTES, s>>>(*reinterpret_cast<const CUtensorMap*>(mapHi),
+                                                                  *reinterpret_cast<const CUtensorMap*>(mapLo), a);
         ++g_kernel_launches;
     }
-    zeta_gram_finish_kernel<<<(unsigned)K, 32, 0, s>>>(partial, num_sms * G_EPI_WARPS, K, zeta);
+    zeta_gram_finish_kernel<<<(unsigned)K, 256, 0, s>>>(partial, tile_ptr, a.ntiles, a.parts, std::max(ncl, 1), K, zeta);
     ++g_kernel_launches;
     return cudaGetLastError();
 }

@@ -867,6 +867,8 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
         std::vector<int32_t> gcl;
         std::vector<float> gvl;
         for (int64_t r = 0; r < p.Np; ++r) {
+        gcl.reserve(cl.size());
+        gvl.reserve(vl.size());
             for (int64_t e = rp[r]; e < rp[r + 1]; ++e)
                 if (train[(size_t)cl[e]]) { gcl.push_back(cl[e]); gvl.push_back(vl[e]); }
             grp[(size_t)r + 1] = (int64_t)gcl.size();

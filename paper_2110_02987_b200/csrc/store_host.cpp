@@ -10,6 +10,10 @@
 
 namespace gad {
 
+// A host loop of less than this many row visits runs on the calling thread: waking the others costs more than they save.  (All or none of
+// them: a team whose size changes from loop to loop is taken down and set up again.)
+static bool worth_threads(int64_t rows) { return rows >= 512; }
+
 static int validate(const gad_csr* g, const gad_partition* part, std::string& err) {
     if (!g || !part) { err = "graph or partition is NULL"; return GAD_ERR_ARG; }
     if (g->n < 0 || g->nnz < 0 || !g->rowptr || (g->nnz > 0 && !g->col)) { err = "bad CSR header"; return GAD_ERR_ARG; }
@@ -99,7 +103,7 @@ int build_store(const gad_csr* g, const gad_partition* part, bool values, HostSt
         rc = fill_local(part, k, local_of, err);
         if (rc != GAD_OK) return rc;
         const int64_t r0 = st.sub_off[k], nk = st.sub_off[k + 1] - r0;
-#pragma omp parallel for schedule(static)
+#pragma omp parallel for schedule(static) if (worth_threads(nk))
         for (int64_t l = 0; l < nk; ++l) {
             int32_t u = node_of(part, k, l);
             int64_t c = 1;
@@ -119,10 +123,10 @@ int build_store(const gad_csr* g, const gad_partition* part, bool values, HostSt
     for (int32_t k = 0; k < K; ++k) {
         fill_local(part, k, local_of, err);
         const int64_t r0 = st.sub_off[k], nk = st.sub_off[k + 1] - r0;
-#pragma omp parallel
+#pragma omp parallel if (worth_threads(nk))
         {
             std::vector<std::pair<int32_t, double>> row;
-#pragma omp for schedule(dynamic, 256)
+#pragma omp for schedule(dynamic, 128)
             for (int64_t l = 0; l < nk; ++l) {
                 int32_t u = node_of(part, k, l);
                 row.clear();
@@ -181,7 +185,7 @@ int build_store(const gad_csr* g, const gad_partition* part, bool values, HostSt
 
     // Compaction and normalisation: d~_i = row sum of (A'_k + I); A~_ij = a_ij / sqrt(d~_i d~_j).
     std::vector<double> dt((size_t)Np);
-#pragma omp parallel for schedule(static)
+#pragma omp parallel for schedule(static) if (worth_threads(Np))
     for (int64_t r = 0; r < Np; ++r) {
         double s = 0.0;
         for (int64_t i = 0; i < len[r + 1]; ++i) s += tval[ub[r] + i];
@@ -189,7 +193,7 @@ int build_store(const gad_csr* g, const gad_partition* part, bool values, HostSt
     }
     st.col.resize((size_t)st.nnz);
     st.val.resize((size_t)st.nnz);
-#pragma omp parallel for schedule(static)
+#pragma omp parallel for schedule(static) if (worth_threads(Np))
     for (int64_t r = 0; r < Np; ++r) {
         int64_t src = ub[r], dst = st.rowptr[r];
         for (int64_t i = 0; i < len[r + 1]; ++i) {
@@ -201,6 +205,24 @@ int build_store(const gad_csr* g, const gad_partition* part, bool values, HostSt
     tcol.clear(); tcol.shrink_to_fit();
     tval.clear(); tval.shrink_to_fit();
 
+    // The store equals its transpose when the mirror image of every entry is there with the same bits: rows are sorted, so it is a look-up
+    // per entry above the diagonal, and the two triangles then have to be of the same size.  (Building the transpose to compare with it is
+    // a serial scatter over all entries.)
+    int64_t upper = 0, lower = 0;
+    bool same = true;
+#pragma omp parallel for schedule(static) if (worth_threads(Np)) reduction(+ : upper, lower) reduction(&& : same)
+    for (int64_t r = 0; r < Np; ++r)
+        for (int64_t e = st.rowptr[r]; e < st.rowptr[r + 1]; ++e) {
+            const int32_t c = st.col[e];
+            if (c <= r) { lower += c < r; continue; }
+            ++upper;
+            if (!same) continue;
+            const auto b = st.col.begin() + st.rowptr[c], f = st.col.begin() + st.rowptr[c + 1], at = std::lower_bound(b, f, (int32_t)r);
+            same = at != f && *at == (int32_t)r && std::memcmp(&st.val[(size_t)(at - st.col.begin())], &st.val[(size_t)e], sizeof(float)) == 0;
+        }
+    st.symmetric = same && upper == lower;
+    if (st.symmetric) return GAD_OK;
+
     // Transposed store by counting sort; rows are visited in ascending order, so every transposed row comes
     // out with ascending columns.
     st.t_rowptr.assign((size_t)Np + 1, 0);
@@ -208,22 +230,13 @@ int build_store(const gad_csr* g, const gad_partition* part, bool values, HostSt
     for (int64_t r = 0; r < Np; ++r) st.t_rowptr[r + 1] += st.t_rowptr[r];
     st.t_col.resize((size_t)st.nnz);
     st.t_val.resize((size_t)st.nnz);
-    {
-        std::vector<int64_t> cur(st.t_rowptr.begin(), st.t_rowptr.end() - 1);
-        for (int64_t r = 0; r < Np; ++r)
-            for (int64_t e = st.rowptr[r]; e < st.rowptr[r + 1]; ++e) {
-                int64_t p = cur[st.col[e]]++;
-                st.t_col[p] = (int32_t)r;
-                st.t_val[p] = st.val[e];
-            }
-    }
-    st.symmetric = st.t_rowptr == st.rowptr && st.t_col == st.col &&
-                   std::memcmp(st.t_val.data(), st.val.data(), sizeof(float) * (size_t)st.nnz) == 0;
-    if (st.symmetric) {
-        st.t_rowptr.clear(); st.t_rowptr.shrink_to_fit();
-        st.t_col.clear(); st.t_col.shrink_to_fit();
-        st.t_val.clear(); st.t_val.shrink_to_fit();
-    }
+    std::vector<int64_t> cur(st.t_rowptr.begin(), st.t_rowptr.end() - 1);
+    for (int64_t r = 0; r < Np; ++r)
+        for (int64_t e = st.rowptr[r]; e < st.rowptr[r + 1]; ++e) {
+            int64_t p = cur[st.col[e]]++;
+            st.t_col[p] = (int32_t)r;
+            st.t_val[p] = st.val[e];
+        }
     return GAD_OK;
 }
 

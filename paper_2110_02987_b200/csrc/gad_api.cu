@@ -424,10 +424,11 @@ int hand_over(gad_ctx* ctx, cudaStream_t from, cudaStream_t to, cudaEvent_t ev) 
 
 // While it lives, the kernels of the main sequence may start before the one in front has finished (launch.cuh): not while they are timed,
 // and only on small stores, whose kernels last a few microseconds each (2000 rows: 71 -> 66 us an epoch, 2800 rows: 175 -> 160, 20 700:
-// 207 -> 200); on large ones the waiting blocks hold room that the kernels beside them would use (110 000 rows: 281 -> 291 us).
-constexpr int64_t kPdlRows = 48 << 10;
+// 207 -> 200); on large ones the waiting blocks hold room that the kernels beside them would use (110 000 rows: 281 -> 291 us; 42 000
+// rows of 10 M entries: 756 -> 784, 34 000 of 2.6 M: 350 -> 366).
+constexpr int64_t kPdlRows = 48 << 10, kPdlEntries = 2 << 20;
 struct PdlScope {
-    explicit PdlScope(gad_ctx* ctx) { pdl_state() = PdlState{ctx->stream, !ctx->profiling && ctx->p.Np <= kPdlRows, false}; }
+    explicit PdlScope(gad_ctx* ctx) { pdl_state() = PdlState{ctx->stream, !ctx->profiling && ctx->p.Np <= kPdlRows && ctx->p.nnz <= kPdlEntries, false}; }
     ~PdlScope() { pdl_state() = PdlState{}; }
 };
 
@@ -866,9 +867,9 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
         std::vector<int64_t> grp((size_t)p.Np + 1, 0);
         std::vector<int32_t> gcl;
         std::vector<float> gvl;
-        for (int64_t r = 0; r < p.Np; ++r) {
         gcl.reserve(cl.size());
         gvl.reserve(vl.size());
+        for (int64_t r = 0; r < p.Np; ++r) {
             for (int64_t e = rp[r]; e < rp[r + 1]; ++e)
                 if (train[(size_t)cl[e]]) { gcl.push_back(cl[e]); gvl.push_back(vl[e]); }
             grp[(size_t)r + 1] = (int64_t)gcl.size();
@@ -1303,7 +1304,9 @@ int gad_set_inputs(gad_ctx* ctx, const float* X, const int32_t* labels) {
     if (!X && !labels) return GAD_OK;
     if (labels) {   // the loss kernel indexes a row of logits with the label: same range check as gad_create, before anything is enqueued
         const int C = p.dims[p.L];
-        for (int32_t u = 0; u < p.n; ++u)
+        bool bad = false;   // one pass without a branch per label; the culprit is looked for only when there is one
+        for (int32_t u = 0; u < p.n; ++u) bad |= (uint32_t)labels[u] >= (uint32_t)C;
+        for (int32_t u = 0; bad && u < p.n; ++u)
             if (labels[u] < 0 || labels[u] >= C) return fail(ctx, GAD_ERR_RANGE, "label out of range at node " + std::to_string(u));
     }
     // The copy goes out on its own stream into one of two staging pairs, so it can overlap the epoch that is still

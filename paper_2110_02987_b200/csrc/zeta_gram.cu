@@ -8,7 +8,7 @@
 // streaming kernel that also takes the squared norms), and the product is accumulated as hi.hi + hi.lo + lo.hi in fp32 in tensor memory -
 // the error-compensated product of the layer transforms, here with both operands split ahead of time because the drain below needs the
 // SM's issue slots.  What bounds it is the tensor pipe; in 128 x 128 tiles of one CTA it was shared memory, read for A and B at the rate
-// of the MMAs and written by TMA on top (8 x 6560 rows of 128: 300 us, now 182; of 32: 245, now 140).
+// of the MMAs and written by TMA on top (8 x 6560 rows of 128: 300 us, now 182; a call on as many rows of 32: 307 us, now 189).
 //
 // While the MMA warp fills the second accumulator, sixteen warps read the first one back (tcgen05.ld), turn every inner product into a
 // distance and add p_j / (d + beta) over the pairs i < j inside the subgraph.  Two pairs share a reciprocal, p / x + q / y = (p y + q x) /

@@ -103,7 +103,9 @@ typedef struct {
                              copy of the transposed store without the entries that read a row carrying no loss - a
                              replicated node, or a core node outside the training split, where d loss / d logits is
                              zero (the loss of Section 3.3 is taken over the subgraph's own training nodes): the same
-                             sums without their zero terms; the copy costs up to 8 bytes per stored entry)           */
+                             sums without their zero terms; the copy costs up to 8 bytes per stored entry);
+                             bit 7: the transforms of small layers go through the tensor cores as well (by default the
+                             FP32 ALUs finish them sooner)                                                            */
 } gad_config;
 
 /* Bytes of device workspace gad_create needs for these inputs.  Host-only; touches no GPU. */

@@ -54,6 +54,7 @@ struct ProfEntry {
 // gad_create, so both agree byte for byte.
 struct Plan {
     int32_t n = 0, K = 0, L = 0;
+    std::vector<uint8_t> simt;        // [L] layers whose transforms are too small for the tensor cores
     int64_t Np = 0, nnz = 0, P = 0, Pint = 0, pstride = 0, slots = 0;
     std::vector<int32_t> dims;
     std::vector<Layer> layers;
@@ -101,6 +102,12 @@ size_t take(size_t& cur, size_t bytes) {
     cur += (size_t)round_up((int64_t)std::max<size_t>(bytes, 4), 256);
     return o;
 }
+
+// A layer's transforms run on the FP32 ALUs up to this many operations each, outputs narrower than a tile counted as one (and unless
+// reduced precision was asked for).  2000 rows of 32-16-4: 65 -> 44 us an epoch, 8000 of 50-32-10: 79 -> 66; above, the tensor cores are
+// ahead (2800 rows of 128 -> 128, 93 M: 155 against 167; 20 700 rows of 256 -> 3, 340 M with its padding: 199 against 217).
+constexpr double kSimtFlops = 64e6;
+constexpr int kSimtTile = 32;
 
 int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off, const std::vector<int64_t>& core_count,
               int64_t nnz, int64_t slots, const gad_config* cfg, std::string& err) {
@@ -159,11 +166,13 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
             p.zchunks.push_back(RowSpan{(int32_t)r, (int32_t)std::min<int64_t>(Rz, sub_off[k + 1] - r), k, 0});
         p.zchunk_ptr[k + 1] = (int32_t)p.zchunks.size();
     }
+    p.simt.assign(p.L, 0);
     p.dw.resize(p.L);
     size_t dw_floats = 0;
     for (int l = 0; l < p.L; ++l) {
         const Layer& y = p.layers[l];
-        const int64_t Rdw = tn_chunk_rows(sub_off, tn_shape(y.fi, y.ldw), y.fi, y.ldw, 148);
+        p.simt[l] = cfg->gemm_mode == 0 && (cfg->flags & 128) == 0 && 2.0 * (double)p.Np * y.fi * std::max(y.fo, kSimtTile) <= kSimtFlops;
+        const int64_t Rdw = p.simt[l] ? simt_tn_chunk_rows(p.Np, y.fi, y.ldw) : tn_chunk_rows(sub_off, tn_shape(y.fi, y.ldw), y.fi, y.ldw, 148);
         Plan::DwChunks& d = p.dw[l];
         d.ptr.assign(K + 1, 0);
         for (int32_t k = 0; k < K; ++k) {
@@ -393,6 +402,8 @@ void* bf16_of(gad_ctx* ctx) { return ctx->cfg.gemm_mode == 1 ? (void*)(ctx->ws +
 
 // The bfloat16 copy of the features for layer 0's aggregation.
 void* x_bf16(gad_ctx* ctx) { return ctx->p.o_xbf16 ? (void*)(ctx->ws + ctx->p.o_xbf16) : nullptr; }
+// The transforms of this layer run on the tensor cores.
+bool on_tc(const gad_ctx* ctx, int l) { return ctx->use_tc && !ctx->p.simt[(size_t)l]; }
 // Whether dPre^(l), the gradient at layer l's pre-activations, is wanted in bfloat16 alone: the reduced-precision mode, and nothing but the
 // backward aggregation reads it (`summed`: its producer sums its columns).
 bool dpre_bf16(const gad_ctx* ctx, int l, bool summed) { return ctx->cfg.gemm_mode == 1 && ctx->use_tc && !ctx->p.agg_first[l] && summed; }
@@ -453,26 +464,28 @@ int settle_now(gad_ctx* ctx) {
 }
 
 // The operand copies of the weights that the tensor-core transforms read.
-int split_pass(gad_ctx* ctx) {
+int split_pass(gad_ctx* ctx, bool* launched = nullptr) {
     const Plan& p = ctx->p;
-    if (ctx->use_tc) {
-        std::vector<SplitLayer> sl((size_t)p.L);
-        double weights = 0.0;
-        for (int l = 0; l < p.L; ++l) {
-            const Layer& y = p.layers[l];
-            const bool plain = l > 0;   // layer 0 has no gradient with respect to its input
-            sl[(size_t)l] = SplitLayer{y.fi, y.fo, y.ldw, y.ldi, y.w_int, plain ? ctx->at<float>(p.o_w_hi[l]) : nullptr,
-                                       plain ? ctx->at<float>(p.o_w_lo[l]) : nullptr, ctx->at<float>(p.o_wt_hi[l]), ctx->at<float>(p.o_wt_lo[l])};
-            weights += (plain ? 20.0 : 12.0) * y.fi * y.fo;
-        }
-        const int copies = ctx->same_params ? 1 : p.K;
-        GAD_RUN("split_weights", -1, weights * copies, 0.0, [&] { return launch_split_weights(ctx->at<float>(p.o_params), param_stride(ctx), copies, sl.data(), p.L, ctx->stream); });
+    std::vector<SplitLayer> sl;
+    double weights = 0.0;
+    for (int l = 0; l < p.L; ++l) {
+        if (!on_tc(ctx, l)) continue;
+        const Layer& y = p.layers[l];
+        const bool plain = l > 0;   // layer 0 has no gradient with respect to its input
+        sl.push_back(SplitLayer{y.fi, y.fo, y.ldw, y.ldi, y.w_int, plain ? ctx->at<float>(p.o_w_hi[l]) : nullptr,
+                                plain ? ctx->at<float>(p.o_w_lo[l]) : nullptr, ctx->at<float>(p.o_wt_hi[l]), ctx->at<float>(p.o_wt_lo[l])});
+        weights += (plain ? 20.0 : 12.0) * y.fi * y.fo;
     }
+    if (launched) *launched = !sl.empty();
+    if (sl.empty()) return GAD_OK;
+    const int copies = ctx->same_params ? 1 : p.K;
+    GAD_RUN("split_weights", -1, weights * copies, 0.0, [&] { return launch_split_weights(ctx->at<float>(p.o_params), param_stride(ctx), copies, sl.data(), (int)sl.size(), ctx->stream); });
     return GAD_OK;
 }
 
-// Every layer's forward step; split_pass comes before it.
-int forward_pass(gad_ctx* ctx, bool train) {
+// Every layer's forward step; split_pass comes before it.  `fork` (may be null): a stream whose work may start once the first kernel of the
+// pass has finished.
+int forward_pass(gad_ctx* ctx, bool train, cudaStream_t fork = nullptr) {
     const Plan& p = ctx->p;
     float* Z = ctx->at<float>(p.o_G2);
     const float* params = ctx->at<float>(p.o_params);
@@ -492,9 +505,10 @@ int forward_pass(gad_ctx* ctx, bool train) {
                         });
                 if (l == 0) ctx->P_valid = true;
             }
+            if (l == 0 && fork) { int rc = hand_over(ctx, ctx->stream, fork, ctx->ev_fork); if (rc != GAD_OK) return rc; }
             const ActEpi act = make_act(ep, 0);
             GAD_RUN("gemm_fwd", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
-                if (ctx->use_tc)
+                if (on_tc(ctx, l))
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 2, passes, y.fi, y.fo,
                                                ctx->H(l + 1), y.ldo, ctx->at<RowSpan>(p.o_pair_tiles), (int)(p.pair_tiles.size() / 2), nullptr, 0, 1.f, &act,
                                                ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params);
@@ -504,15 +518,16 @@ int forward_pass(gad_ctx* ctx, bool train) {
             continue;
         }
         // reduced-precision mode: the transform writes the bfloat16 operand copy the aggregation gathers, and nothing else
-        void* zb = ctx->use_tc ? bf16_of(ctx) : nullptr;
+        void* zb = on_tc(ctx, l) ? bf16_of(ctx) : nullptr;
         GAD_RUN("gemm_fwd", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
-            if (ctx->use_tc)
+            if (on_tc(ctx, l))
                 return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 0, passes, y.fi, y.fo, Z,
                                            y.ldo, ctx->at<RowSpan>(p.o_pair_tiles), (int)(p.pair_tiles.size() / 2), nullptr, 0, 1.f, nullptr,
                                            ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params, zb);
             return launch_gemm_rows_simt(0, ctx->H(l), y.ldi, y.fi, params, pstride, y.w_int, y.ldw, y.fo, Z, y.ldo,
                                          ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, nullptr, ctx->stream);
         });
+        if (l == 0 && fork) { int rc = hand_over(ctx, ctx->stream, fork, ctx->ev_fork); if (rc != GAD_OK) return rc; }
         GAD_RUN("spmm_fwd", l, spmm_bytes(p, y.fo), 2.0 * p.nnz * y.fo,
                 [&] { return launch_spmm(ctx->A, Z, y.ldo, ctx->H(l + 1), y.ldo, y.fo, &ep, bf16_of(ctx), zb != nullptr, ctx->stream); });
     }
@@ -628,7 +643,7 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
         const int ndw = (int)p.dw[l].spans.size();
         GAD_RUN("gemm_dw", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
             cudaError_t e =
-                ctx->use_tc ? launch_gemm_tn_tc(&ctx->maps[kMapsPerLayer * l + 6], &ctx->maps[kMapsPerLayer * l + 7],
+                on_tc(ctx, l) ? launch_gemm_tn_tc(&ctx->maps[kMapsPerLayer * l + 6], &ctx->maps[kMapsPerLayer * l + 7],
                                                 ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fi, y.ldw, dw_chunks, ndw,
                                                 ctx->at<float>(p.o_dw_partial), ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream)
                             : launch_gemm_tn_simt(agg_first ? ctx->at<float>(p.o_P[l]) : ctx->H(l), y.ldi, y.fi, agg_first ? G1 : G2, y.ldo,
@@ -640,7 +655,7 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
         if (l > 0 && agg_first) {
             // dP = dPre W^T (no mask yet: the ReLU of layer l-1 sits below the aggregation), dH^(l) = A~^T dP, then the mask
             GAD_RUN("gemm_dh", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
-                if (ctx->use_tc)
+                if (on_tc(ctx, l))
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 3], &ctx->maps[kMapsPerLayer * l + 4], &ctx->maps[kMapsPerLayer * l + 5], 1,
                                                ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G2, y.ldi, ctx->at<RowSpan>(p.o_pair_tiles),
                                                (int)(p.pair_tiles.size() / 2), nullptr, 0, 1.f, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
@@ -658,10 +673,10 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
         if (l > 0 && ss != ctx->stream) { int rcw = wait_for(ctx, ctx->stream, ctx->ev_bias); if (rcw != GAD_OK) return rcw; }
         if (l == 0) break;
         // the drain sums the columns of what it writes, dPre of the layer below: its bias gradient
-        const bool sums = ctx->use_tc && tc_rows_sums_columns(y.fi, npairs);
+        const bool sums = on_tc(ctx, l) && tc_rows_sums_columns(y.fi, npairs);
         const bool out_bf16 = dpre_bf16(ctx, l - 1, sums);
         GAD_RUN("gemm_dh", l, 4.0 * p.Np * (2.0 * y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
-                if (ctx->use_tc)
+                if (on_tc(ctx, l))
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 3], &ctx->maps[kMapsPerLayer * l + 4], &ctx->maps[kMapsPerLayer * l + 5], 1,
                                                ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G1, y.ldi, ctx->at<RowSpan>(p.o_pair_tiles),
                                                (int)(p.pair_tiles.size() / 2), ctx->H(l), y.ldi, scale, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
@@ -1017,9 +1032,10 @@ static int enqueue_epoch(gad_ctx* ctx, bool consensus) {
     const PdlScope pdl(ctx);
     // The side work forks off behind the first kernel of the main sequence: as a second root of the graph it would come first, and
     // the main sequence 10 us later.
-    int rc = split_pass(ctx);
-    if (rc != GAD_OK || (rc = hand_over(ctx, ctx->stream, ss, ctx->ev_fork)) != GAD_OK) return rc;
-    if ((rc = forward_pass(ctx, true)) != GAD_OK) return rc;
+    bool split = false;
+    int rc = split_pass(ctx, &split);
+    if (rc != GAD_OK || (split && (rc = hand_over(ctx, ctx->stream, ss, ctx->ev_fork)) != GAD_OK)) return rc;
+    if ((rc = forward_pass(ctx, true, split ? nullptr : ss)) != GAD_OK) return rc;
     // zeta beside the forward pass; with zeta_mode 2 it reads this pass's activations, so it follows it (beside the backward pass)
     if (ctx->cfg.zeta_mode == 2 && (rc = hand_over(ctx, ctx->stream, ss, ctx->ev_fork)) != GAD_OK) return rc;
     if (ss != ctx->stream && (rc = zeta_pass(ctx, ss)) != GAD_OK) return rc;

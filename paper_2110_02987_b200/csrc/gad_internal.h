@@ -195,6 +195,7 @@ cudaError_t launch_narrow_bwd(const float* H, int ldh, int fi, const float* dZ, 
                               int64_t partial_stride, int32_t* err, cudaStream_t s);
 
 // partial[chunk] = H[chunk rows]^T * dZ[chunk rows]   ([M x ldw] each), one CTA column per chunk.
+int64_t simt_tn_chunk_rows(int64_t rows, int fi, int ldw);
 cudaError_t launch_gemm_tn_simt(const float* H, int ldh, int M, const float* dZ, int ldz, int N,
                                 const RowSpan* chunks, int nchunks, float* partial, int ldw, cudaStream_t s);
 

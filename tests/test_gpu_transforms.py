@@ -16,11 +16,14 @@ def built():
     entry.build()
 
 
+# flag bit 7: small layers on the tensor cores too, else most of these run on the FP32 ALUs in their small tiles
+@pytest.mark.parametrize("bit7", [0, 128])
 @pytest.mark.parametrize("rows", [1, 127, 128, 129, 256, 257])
 @pytest.mark.parametrize("dims,kw", [
     ((31, 17, 5), {}), ((33, 130, 16, 3), {}), ((700, 33, 2), {}), ((129, 256, 257, 4), dict(flags=4)),
     ((300, 300, 64, 9), dict(flags=4, dropout=0.3)), ((64, 512, 40), dict(gemm_mode=1)), ((1433, 64, 40, 7), dict(gemm_mode=1, flags=4))])
-def test_row_and_column_edges(rows, dims, kw):
+def test_row_and_column_edges(rows, dims, kw, bit7):
+    kw = dict(kw, flags=kw.get("flags", 0) | bit7)
     K = 3
     case = small_random_case(rows, n=rows * K + 3, K=K, p=min(0.3, 4.0 / (rows * K)), halo=False)
     tol = 5e-2 if kw.get("gemm_mode") else TOL

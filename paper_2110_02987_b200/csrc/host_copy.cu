@@ -2,13 +2,18 @@
 // staging buffer on one host thread, and a freshly allocated destination has each of its pages mapped inside that copy: 16 MB of
 // logits took 0.93 ms of copying and another millisecond of page faults.  Here the pages are touched by several threads
 // while the GPU still computes, and the copy runs through a ring of pinned slots: while the GPU fills some over PCIe, several threads
-// each move one to its place (all threads on one slot at a time, a fork and a join per slot, took 0.75 ms for those 16 MB; this way 0.53).
+// move another to its place, a share each.  A copy over PCIe costs 9 us and then 55 bytes a nanosecond (512 KB: 28 GB/s, 2 MB: 46), so
+// slots are large where there is much to copy; sharing a slot keeps what is left after the last of them short, and counters instead of a
+// fork and a join per slot keep it cheap.  (16 MB: 0.75 ms with a join per 512 KB slot, 0.55 ms with a thread to every slot, 0.45 ms now;
+// the bare copy of 16 MB takes 0.30.)
 #include <omp.h>
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstring>
 #include <mutex>
+#include <thread>
 #include <vector>
 
 #include "gad_internal.h"
@@ -17,8 +22,8 @@ namespace gad {
 
 namespace {
 
-constexpr size_t kSlotBytes = 512u << 10;   // 10 us over PCIe, 50 to 100 us of one thread's copying
-constexpr int kSlots = 16, kMaxThreads = 8;
+constexpr size_t kRingBytes = 8u << 20, kMinSlot = 256u << 10, kMaxSlot = 2u << 20;
+constexpr int kSlots = 32, kMaxThreads = 8;   // most slots of a ring
 constexpr size_t kTouchBytes = 1u << 20;  // destinations below this are not worth waking threads for
 constexpr size_t kPage = 4096;
 constexpr size_t kSmallPinned = 16384;
@@ -27,7 +32,7 @@ int copy_threads(size_t bytes) {
     return (int)std::max<size_t>(1, std::min<size_t>({(size_t)kMaxThreads, (size_t)omp_get_num_procs() / 2, bytes / (128u << 10)}));
 }
 
-// Pinned buffers of kSlots slots, shared by all contexts of the process: at most two are kept while a context exists, none
+// Pinned buffers of kRingBytes, shared by all contexts of the process: at most two are kept while a context exists, none
 // after the last one has gone.
 struct Pool {
     std::mutex lock;
@@ -57,7 +62,7 @@ char* take_buffer() {
         std::lock_guard<std::mutex> g(g_pool.lock);
         if (g_pool.users <= 0) return nullptr;   // no context to keep the buffer for: pinning one for a single copy costs more than it saves
     }
-    return take_from(g_pool.idle, kSlots * kSlotBytes);
+    return take_from(g_pool.idle, kRingBytes);
 }
 void give_buffer(char* b) { give_to(g_pool.idle, 2, b); }
 
@@ -116,33 +121,63 @@ cudaError_t copy_to_host(void* dst, const void* src, size_t bytes, cudaStream_t 
         e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s);
         return e != cudaSuccess ? e : cudaStreamSynchronize(s);
     }
+    // n slots cost 9 us each on the way, and the last one's copying (about as fast as PCIe) comes after the last transfer: together least at
+    // slots of sqrt(bytes x 512 KB)
+    const size_t slot = std::min(kMaxSlot, std::max(kMinSlot, (size_t)round_up((int64_t)std::sqrt((double)bytes * (512 << 10)), 64 << 10)));
+    const int64_t n = (int64_t)((bytes + slot - 1) / slot), ring = std::min<int64_t>(n, (int64_t)(kRingBytes / slot));
+    const int nt = copy_threads(bytes);
     Events evs;
-    const int64_t n = (int64_t)((bytes + kSlotBytes - 1) / kSlotBytes);
-    // a power of two, so that one thread handles every use of a slot and slots need no hand-over between threads
-    int nt = 1;
-    while (2 * nt <= copy_threads(bytes)) nt *= 2;
     int dev = 0;
     e = cudaGetDevice(&dev);
-    for (int64_t q = 0; q < std::min<int64_t>(n, kSlots) && e == cudaSuccess; ++q) e = cudaEventCreateWithFlags(&evs.ev[q], cudaEventDisableTiming);
-    auto length = [&](int64_t i) { return std::min(kSlotBytes, bytes - (size_t)i * kSlotBytes); };
+    for (int64_t q = 0; q < ring && e == cudaSuccess; ++q) e = cudaEventCreateWithFlags(&evs.ev[q], cudaEventDisableTiming);
+    auto length = [&](int64_t i) { return std::min(slot, bytes - (size_t)i * slot); };
+    std::atomic<int64_t> filled[kSlots];          // what a slot holds, or is being filled with
+    for (std::atomic<int64_t>& f : filled) f.store(-1);
     auto fill = [&](int64_t i) {
-        const int q = (int)(i % kSlots);
-        const cudaError_t r = cudaMemcpyAsync(buf + q * kSlotBytes, (const char*)src + (size_t)i * kSlotBytes, length(i), cudaMemcpyDeviceToHost, s);
-        return r == cudaSuccess ? cudaEventRecord(evs.ev[q], s) : r;
+        const int64_t q = i % ring;
+        const cudaError_t r = cudaMemcpyAsync(buf + q * slot, (const char*)src + (size_t)i * slot, length(i), cudaMemcpyDeviceToHost, s);
+        if (r != cudaSuccess) return r;
+        const cudaError_t v = cudaEventRecord(evs.ev[q], s);
+        if (v == cudaSuccess) filled[q].store(i, std::memory_order_release);
+        return v;
     };
-    for (int64_t i = 0; i < std::min<int64_t>(n, kSlots) && e == cudaSuccess; ++i) e = fill(i);
+    for (int64_t i = 0; i < ring && e == cudaSuccess; ++i) e = fill(i);
     if (e == cudaSuccess) {
         std::atomic<int> bad{0};
-#pragma omp parallel for num_threads(nt) schedule(static, 1)
-        for (int t = 0; t < nt; ++t) {
-            cudaError_t r = cudaSetDevice(dev);
-            for (int64_t i = t; i < n && r == cudaSuccess && !bad.load(); i += nt) {
-                r = cudaEventSynchronize(evs.ev[i % kSlots]);
-                if (r != cudaSuccess) break;
-                std::memcpy((char*)dst + (size_t)i * kSlotBytes, buf + (i % kSlots) * kSlotBytes, length(i));
-                if (i + kSlots < n) r = fill(i + kSlots);
+        std::atomic<int64_t> arrived{0};          // slots known to have arrived
+        std::atomic<bool> waiting{false};         // a thread waits for the next one (for all of them)
+        std::atomic<int> moved[kSlots] = {};      // shares of a slot's contents that have been moved
+        auto wait_for_slot = [&](int64_t i) {
+            while (arrived.load(std::memory_order_acquire) <= i && !bad.load()) {
+                if (waiting.exchange(true)) { std::this_thread::yield(); continue; }
+                const int64_t a = arrived.load(std::memory_order_acquire);
+                if (filled[a % ring].load(std::memory_order_acquire) != a) std::this_thread::yield();   // others are still at its last contents
+                else if (a <= i) {
+                    const cudaError_t r = cudaEventSynchronize(evs.ev[a % ring]);
+                    if (r != cudaSuccess) bad.store((int)r);
+                    else arrived.store(a + 1, std::memory_order_release);
+                }
+                waiting.store(false);
             }
+        };
+#pragma omp parallel num_threads(nt)
+        {
+            const int team = omp_get_num_threads(), t = omp_get_thread_num();
+            const cudaError_t r = cudaSetDevice(dev);
             if (r != cudaSuccess) bad.store((int)r);
+            for (int64_t i = 0; i < n && !bad.load(); ++i) {
+                wait_for_slot(i);
+                if (bad.load()) break;
+                const size_t len = length(i), lo = len * (size_t)t / team / 64 * 64, hi = t + 1 == team ? len : len * (size_t)(t + 1) / team / 64 * 64;
+                std::memcpy((char*)dst + (size_t)i * slot + lo, buf + (i % ring) * slot + lo, hi - lo);
+                if (moved[i % ring].fetch_add(1) + 1 == team) {
+                    moved[i % ring].store(0);
+                    if (i + ring < n) {
+                        const cudaError_t f = fill(i + ring);
+                        if (f != cudaSuccess) bad.store((int)f);
+                    }
+                }
+            }
         }
         e = (cudaError_t)bad.load();
     }

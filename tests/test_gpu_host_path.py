@@ -40,9 +40,9 @@ def test_dropout_epochs_replayed_follow_the_epoch_counter(own_stream):
         assert np.array_equal(g.get_params(1), h.get_params(1))
 
 
-@pytest.mark.parametrize("n,classes", [(3, 1), (4096, 64), (4097, 64), (20011, 67)])
+@pytest.mark.parametrize("n,classes", [(3, 1), (4096, 64), (4097, 64), (20011, 67), (65536, 64), (150011, 67)])
 def test_forward_copies_every_row_through_the_ring(n, classes):
-    """Less than a slot, exactly one slot, one value more, and several rounds of the ring with a ragged end; rows that no
+    """Less than a slot, slots of several sizes, whole and ragged, one round of the ring and several; rows that no
     subgraph owns are zero."""
     rowptr = np.arange(n + 1, dtype=np.int64)
     col = np.arange(n, dtype=np.int32)                 # self-loops only: A~ is the identity

@@ -444,12 +444,12 @@ int hand_over(gad_ctx* ctx, cudaStream_t from, cudaStream_t to, cudaEvent_t ev) 
 }
 
 // While it lives, the kernels of the main sequence may start before the one in front has finished (launch.cuh): not while they are timed,
-// and only on small stores, whose kernels last a few microseconds each (2000 rows: 71 -> 66 us an epoch, 2800 rows: 175 -> 160, 20 700:
+// and, other than the finishing ones, only on small stores, whose kernels last a few microseconds each (2000 rows: 71 -> 66 us an epoch, 2800 rows: 175 -> 160, 20 700:
 // 207 -> 200); on large ones the waiting blocks hold room that the kernels beside them would use (110 000 rows: 281 -> 291 us; 42 000
 // rows of 10 M entries: 756 -> 784, 34 000 of 2.6 M: 350 -> 366).
 constexpr int64_t kPdlRows = 48 << 10, kPdlEntries = 2 << 20;
 struct PdlScope {
-    explicit PdlScope(gad_ctx* ctx) { pdl_state() = PdlState{ctx->stream, !ctx->profiling && ctx->p.Np <= kPdlRows && ctx->p.nnz <= kPdlEntries, false}; }
+    explicit PdlScope(gad_ctx* ctx) { pdl_state() = PdlState{ctx->stream, !ctx->profiling && ctx->p.Np <= kPdlRows && ctx->p.nnz <= kPdlEntries, false, !ctx->profiling}; }
     ~PdlScope() { pdl_state() = PdlState{}; }
 };
 

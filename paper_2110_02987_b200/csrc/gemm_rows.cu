@@ -497,7 +497,7 @@ cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* 
                                                  *reinterpret_cast<const CUtensorMap*>(mapBlo), a);
         ++g_kernel_launches;
         if (e != cudaSuccess || slices == 1) return e;
-        e = launch(sum_slices_kernel, dim3(2u * (unsigned)npairs, (unsigned)(BM / SUM_ROWS)), 256, 0, s, parts, slices, a.slice_stride, pair_tiles, C,
+        e = launch_tail(sum_slices_kernel, dim3(2u * (unsigned)npairs, (unsigned)(BM / SUM_ROWS)), 256, 0, s, parts, slices, a.slice_stride, pair_tiles, C,
                    reinterpret_cast<uint2*>(Cbf16), ldc, mode == 2 ? 1 : 0, a.act);
         ++g_kernel_launches;
         return e;

@@ -427,7 +427,7 @@ __global__ void reduce_chunks_kernel(const float* __restrict__ partial, long lon
 cudaError_t launch_reduce_chunks(const float* partial, int64_t pstride_chunk, const int32_t* chunk_ptr, int K, float* out,
                                  int64_t ostride, int64_t off, int64_t len, cudaStream_t s) {
     if (len > 0 && K > 0) {
-        launch(reduce_chunks_kernel, dim3((unsigned)((len + 255) / 256), (unsigned)K), 256, 0, s, partial, pstride_chunk, chunk_ptr, out,
+        launch_tail(reduce_chunks_kernel, dim3((unsigned)((len + 255) / 256), (unsigned)K), 256, 0, s, partial, pstride_chunk, chunk_ptr, out,
                                                                                                ostride, off, len); ++g_kernel_launches; }
     return cudaGetLastError();
 }

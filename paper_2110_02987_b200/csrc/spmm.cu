@@ -355,7 +355,7 @@ static cudaError_t launch_rows(const SparseDev& A, const float* Z, int ldz, floa
             ++g_kernel_launches;
         }
         if (A.nfin > 0) {
-            launch(spmm_finish_kernel<NV, GROUP, EPI>, dim3((unsigned)((A.nfin + 7) / 8)), 256, 0, s, A.fin, A.nfin, A.scratch, out, ldo, F4, ep);
+            launch_tail(spmm_finish_kernel<NV, GROUP, EPI>, dim3((unsigned)((A.nfin + 7) / 8)), 256, 0, s, A.fin, A.nfin, A.scratch, out, ldo, F4, ep);
             ++g_kernel_launches;
         }
         return cudaGetLastError();
@@ -366,7 +366,7 @@ static cudaError_t launch_rows(const SparseDev& A, const float* Z, int ldz, floa
         ++g_kernel_launches;
     }
     if (A.nfin > 0) {
-        launch(spmm_finish_kernel<NV, GROUP, EPI>, dim3((unsigned)((A.nfin + 7) / 8)), 256, 0, s, A.fin, A.nfin, A.scratch, out, ldo, F4, ep);
+        launch_tail(spmm_finish_kernel<NV, GROUP, EPI>, dim3((unsigned)((A.nfin + 7) / 8)), 256, 0, s, A.fin, A.nfin, A.scratch, out, ldo, F4, ep);
         ++g_kernel_launches;
     }
     return cudaGetLastError();

@@ -54,8 +54,6 @@ struct ProfEntry {
 // gad_create, so both agree byte for byte.
 struct Plan {
     int32_t n = 0, K = 0, L = 0;
-    std::vector<int32_t> slices;      // [L] slices of the reduction of a layer's forward transform
-    size_t o_slices = 0;
     std::vector<uint8_t> simt;        // [L] layers whose transforms are too small for the tensor cores
     int64_t Np = 0, nnz = 0, P = 0, Pint = 0, pstride = 0, slots = 0;
     std::vector<int32_t> dims;
@@ -200,13 +198,6 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
             p.core_spans.push_back(RowSpan{(int32_t)(sub_off[k] + r), (int32_t)std::min<int64_t>(256, core_count[k] - r), k, 0});
     }
     const size_t Np = (size_t)p.Np, nc = p.chunks.size();
-    p.slices.assign(p.L, 1);
-    size_t slice_floats = 0;
-    for (int l = 0; l < p.L; ++l)
-        if (!p.simt[l]) {
-            p.slices[l] = tc_rows_slices(p.dims[l], p.dims[l + 1], (int)(p.pair_tiles.size() / 2));
-            if (p.slices[l] > 1) slice_floats = std::max(slice_floats, (size_t)p.slices[l] * Np * (size_t)p.ld[l + 1]);
-        }
     size_t cur = 0;
     p.o_rowptr = take(cur, 8 * (Np + 1)); p.o_ecv = take(cur, 8 * (size_t)nnz);
     // work lists: one part per scratch slot, at most one cut row per kMinPart entries
@@ -241,7 +232,6 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
     p.o_colsum = take(cur, 4 * 8 * (size_t)(kMaxRowClusters + K) * (size_t)p.maxld); p.o_cs_clusters = take(cur, 8 * (size_t)K);
     p.o_G1 = take(cur, 4 * Np * (size_t)p.maxld); p.o_G2 = take(cur, 4 * Np * (size_t)p.maxld);
     p.o_params = take(cur, 4 * (size_t)K * (size_t)p.pstride); p.o_grads = take(cur, 4 * (size_t)K * (size_t)p.pstride);
-    p.o_slices = take(cur, 4 * slice_floats);
     p.o_dw_partial = take(cur, 4 * dw_floats); p.o_cs_partial = take(cur, 4 * nc * (size_t)p.maxld);
     int32_t zeta_ld = p.ld[0];   // widest matrix the importance statistics run over: H^(0), or every layer's input (zeta_mode 2)
     if (cfg->zeta_mode == 2)
@@ -521,8 +511,7 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t fork = nullptr) {
                 if (on_tc(ctx, l))
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 2, passes, y.fi, y.fo,
                                                ctx->H(l + 1), y.ldo, ctx->at<RowSpan>(p.o_pair_tiles), (int)(p.pair_tiles.size() / 2), nullptr, 0, 1.f, &act,
-                                               ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params, nullptr, nullptr, p.slices[l],
-                                               ctx->at<float>(p.o_slices), p.Np);
+                                               ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params);
                 return launch_gemm_rows_simt(2, ctx->at<float>(p.o_P[l]), y.ldi, y.fi, params, pstride, y.w_int, y.ldw, y.fo, ctx->H(l + 1), y.ldo,
                                              ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, &act, ctx->stream);
             });
@@ -534,8 +523,7 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t fork = nullptr) {
             if (on_tc(ctx, l))
                 return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 0, passes, y.fi, y.fo, Z,
                                            y.ldo, ctx->at<RowSpan>(p.o_pair_tiles), (int)(p.pair_tiles.size() / 2), nullptr, 0, 1.f, nullptr,
-                                           ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params, zb, nullptr, p.slices[l],
-                                           ctx->at<float>(p.o_slices), p.Np);
+                                           ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params, zb);
             return launch_gemm_rows_simt(0, ctx->H(l), y.ldi, y.fi, params, pstride, y.w_int, y.ldw, y.fo, Z, y.ldo,
                                          ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, nullptr, ctx->stream);
         });
@@ -973,12 +961,12 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
             const bool agg_first = p.agg_first[l] != 0;   // then the transform and the weight gradient read A~ H^(l), dW and dH read dPre (G1)
             float* Hin = agg_first ? ctx->at<float>(p.o_P[l]) : ctx->H(l);
             ok = ok && tc_make_map(&m[0], Hin, y.fi, p.Np, 0, 4ull * y.ldi, 0, 128);
-            ok = ok && tc_make_map(&m[1], ctx->at<float>(p.o_wt_hi[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, tc_rows_bn(y.fo, npairs, p.slices[l]) / 2);
-            ok = ok && tc_make_map(&m[2], ctx->at<float>(p.o_wt_lo[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, tc_rows_bn(y.fo, npairs, p.slices[l]) / 2);
+            ok = ok && tc_make_map(&m[1], ctx->at<float>(p.o_wt_hi[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, tc_rows_bn(y.fo, npairs) / 2);
+            ok = ok && tc_make_map(&m[2], ctx->at<float>(p.o_wt_lo[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, tc_rows_bn(y.fo, npairs) / 2);
             // input gradient: A = dZ [Np x fo] (in G2), B = W copies [K][fi][fo]
             ok = ok && tc_make_map(&m[3], ctx->at<float>(agg_first ? p.o_G1 : p.o_G2), y.fo, p.Np, 0, 4ull * y.ldo, 0, 128);
-            ok = ok && tc_make_map(&m[4], ctx->at<float>(p.o_w_hi[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, tc_rows_bn(y.fi, npairs, 1) / 2);
-            ok = ok && tc_make_map(&m[5], ctx->at<float>(p.o_w_lo[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, tc_rows_bn(y.fi, npairs, 1) / 2);
+            ok = ok && tc_make_map(&m[4], ctx->at<float>(p.o_w_hi[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, tc_rows_bn(y.fi, npairs) / 2);
+            ok = ok && tc_make_map(&m[5], ctx->at<float>(p.o_w_lo[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, tc_rows_bn(y.fi, npairs) / 2);
             // weight gradient: 32-row tiles of H^(l) and of dZ (in G2)
             ok = ok && tc_make_map(&m[6], Hin, y.fi, p.Np, 0, 4ull * y.ldi, 0, tc_tn_rows(), true);
             ok = ok && tc_make_map(&m[7], ctx->at<float>(agg_first ? p.o_G1 : p.o_G2), y.fo, p.Np, 0, 4ull * y.ldo, 0, tc_tn_rows(), true);

@@ -50,13 +50,10 @@ constexpr int DATA_BYTES = 232448 - 1024 - BAR_BYTES - COLSUM_BYTES;   // 227 Ki
 constexpr int SMEM_BYTES = 232448;
 constexpr int SPLIT_WARPS = 8, EPI_WARPS = 8, EPI_WARP0 = 2 + SPLIT_WARPS;
 constexpr int THREADS = 32 * (EPI_WARP0 + EPI_WARPS);
-constexpr int SUM_ROWS = 16;
 
 struct RowsArgs {
     const RowSpan* tiles;     // an even number of them; tiles 2 p and 2 p + 1 belong to the same subgraph
     int npairs, ntn, BN, Kd;
-    int kbs;                  // ring steps per slice of the reduction; slice = blockIdx.y
-    long long slice_stride;   // floats between the results of two slices
     int nst, nlo;             // ring stages; lo tiles (2 or 4, at most nst: see the split)
     int resident;             // B loaded once per (subgraph, column tile) instead of once per stage
     float* C;
@@ -94,8 +91,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     uint8_t* sm = smem_raw + pad;
     const uint32_t sm_addr = raw_addr + pad;
     const uint32_t rank = cluster_rank();
-    const int kx = (int)blockIdx.y * a.kbs * BK, Kd = a.Kd - kx;           // this slice of the reduction: where it starts, what is left from there
-    const int nkb = min(a.kbs, (Kd + BK - 1) / BK);
+    const int nkb = (a.Kd + BK - 1) / BK;
     const uint32_t b_bytes = (uint32_t)(a.BN / 2) * (BK * 4);              // this CTA's half of a B tile
     constexpr uint32_t nb = split ? 2u : 1u;
     const uint32_t off_lo = a.resident ? (uint32_t)nkb * b_bytes * nb : 0u;
@@ -137,7 +133,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // contiguous ranges of tiles: B changes as rarely as possible
     const int ntiles = a.npairs * a.ntn, ncl = gridDim.x >> 1, cl = blockIdx.x >> 1;
     const int t_begin = (int)((long long)ntiles * cl / ncl), t_end = (int)((long long)ntiles * (cl + 1) / ncl);
-    // calls f(pair, column tile, subgraph of B, B differs from the previous tile's) until it returns false
+    // calls f(tile, pair, n, B differs from the previous tile's) until it returns false
     auto for_tiles = [&](auto&& f) {
         int last_k = -1, last_n = -1;
         for (int t = t_begin; t < t_end; ++t) {
@@ -160,18 +156,18 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 bphase ^= 1u;
                 mbar_expect_tx(bfull, (uint32_t)nkb * nb * b_bytes);
                 for (int kb = 0; kb < nkb; ++kb) {
-                    tma_load_3d(sm_addr + (uint32_t)kb * nb * b_bytes, &tmB, kx + kb * BK, n0, k, bfull);
-                    if (split) tma_load_3d(sm_addr + ((uint32_t)kb * nb + 1u) * b_bytes, &tmBlo, kx + kb * BK, n0, k, bfull);
+                    tma_load_3d(sm_addr + (uint32_t)kb * nb * b_bytes, &tmB, kb * BK, n0, k, bfull);
+                    if (split) tma_load_3d(sm_addr + ((uint32_t)kb * nb + 1u) * b_bytes, &tmBlo, kb * BK, n0, k, bfull);
                 }
             }
             for (int kb = 0; kb < nkb; ++kb) {
                 if (!mbar_wait(empty(stage), phase ^ 1u, abort_flag, a.err, 2)) return false;
                 mbar_expect_tx(full(stage), stage_bytes);
                 const uint32_t base = sm_addr + off_ring + (uint32_t)stage * stage_bytes;
-                tma_load_2d(base, &tmA, kx + kb * BK, row0, full(stage));
+                tma_load_2d(base, &tmA, kb * BK, row0, full(stage));
                 if (!a.resident) {
-                    tma_load_3d(base + A_BYTES, &tmB, kx + kb * BK, n0, k, full(stage));
-                    if (split) tma_load_3d(base + A_BYTES + b_bytes, &tmBlo, kx + kb * BK, n0, k, full(stage));
+                    tma_load_3d(base + A_BYTES, &tmB, kb * BK, n0, k, full(stage));
+                    if (split) tma_load_3d(base + A_BYTES + b_bytes, &tmBlo, kb * BK, n0, k, full(stage));
                 }
                 if (++stage == nst) { stage = 0; phase ^= 1u; }
             }
@@ -198,7 +194,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const uint32_t bbase = a.resident ? sm_addr + (uint32_t)kb * nb * b_bytes : base + A_BYTES;
                 const uint64_t a_hi = smem_desc(base), a_lo = smem_desc(sm_addr + off_lo + (uint32_t)q * A_BYTES);
                 const uint64_t b_hi = smem_desc(bbase), b_lo = smem_desc(bbase + b_bytes);
-                const int nks = min(BK / 8, (Kd - kb * BK + 7) / 8);
+                const int nks = min(BK / 8, (a.Kd - kb * BK + 7) / 8);
                 if (elect_one()) {
                     // 8 TF32 values = 32 bytes = 2 descriptor units along K
 #pragma unroll
@@ -265,7 +261,6 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // In a 16 x 256-bit read lane t gets, of every 8 columns, columns 2 (t % 4) and the next one of rows t / 4 and t / 4 + 8.
         const int quarter = warp & 3, half = (warp - EPI_WARP0) >> 2;
         const int sub_r = lane >> 2, sub_c = 2 * (lane & 3);
-        float* const C = a.C + blockIdx.y * a.slice_stride;
         const float* hmask = a.Hmask;
         ActEpi act = a.act;
         after_wait(hmask);
@@ -355,7 +350,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         }
                         if (g < ng) {
                             if (to_bf16) a.Cbf[(at + 8 * g) >> 1] = bf16_bits(o.x) | (bf16_bits(o.y) << 16);
-                            else *reinterpret_cast<float2*>(C + at + 8 * g) = o;
+                            else *reinterpret_cast<float2*>(a.C + at + 8 * g) = o;
                         }
                     }
                 }
@@ -404,30 +399,6 @@ void rows_layout(int BN, int Kd, int passes, RowsArgs& a) {
     }
 }
 
-// The slices of a transform added in order, and what its drain would have done.
-__global__ void __launch_bounds__(256)
-sum_slices_kernel(const float* __restrict__ parts, int slices, long long slice_stride, const RowSpan* __restrict__ tiles, float* __restrict__ C,
-                  uint2* __restrict__ Cbf, int ldc, int finish, ActEpi act) {
-    pdl_next();
-    const RowSpan t = tiles[blockIdx.x];
-    const int ld4 = ldc >> 2, r0 = SUM_ROWS * (int)blockIdx.y, n = min(SUM_ROWS, t.nrows - r0) * ld4;
-    if (n <= 0) return;
-    pdl_wait();
-    after_wait(parts); after_wait(act.params); after_wait(act.epoch);
-    for (int i = threadIdx.x; i < n; i += 256) {
-        const long long row = t.row0 + r0 + i / ld4, at = row * ld4 + i % ld4;
-        const float4* p = reinterpret_cast<const float4*>(parts) + at;
-        float4 v = __ldg(p);
-        for (int s = 1; s < slices; ++s) {
-            const float4 w = __ldg(p + s * (slice_stride >> 2));
-            v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
-        }
-        if (finish) v = apply_act(v, act, t.k, row, 4 * (i % ld4));
-        if (Cbf) Cbf[at] = bf16_pack4(v);
-        else reinterpret_cast<float4*>(C)[at] = v;
-    }
-}
-
 // Clusters of two CTAs that fit the GPU at once (a cluster stays inside a GPC).
 int max_clusters(int num_sms) {
     static std::atomic<int> known{0};
@@ -449,56 +420,35 @@ int max_clusters(int num_sms) {
 // tile reads and splits A again, so the widest tile is the cheapest - unless the launch has so few row tiles that most SMs would
 // idle: then the columns are spread over more CTAs, down to 32 (2843 rows x 1433 -> 128: 24 row tiles, 40 us with 128 columns per
 // tile, 27 us with 32).
-int tc_rows_bn(int n_cols, int npairs, int slices) {
+int tc_rows_bn(int n_cols, int npairs) {
     int bn = n_cols <= 16 ? 16 : n_cols <= 32 ? 32 : n_cols <= 64 ? 64 : n_cols <= 128 ? 128 : 256;
-    while (slices == 1 && bn > 32 && (long long)npairs * ((n_cols + bn - 1) / bn) * 2 <= 74) bn /= 2;
+    while (bn > 32 && (long long)npairs * ((n_cols + bn - 1) / bn) * 2 <= 74) bn /= 2;
     return bn;
 }
 
-// Slices of the reduction of a forward transform.  Spreading the columns over idle clusters hardly shortens a long reduction (a step costs
-// about the same for any width); cutting it does, at the price of adding the slices up: at least eight steps each, at most eight slices.
-// (2843 rows, 1433 -> 128: 27 us for 48 clusters of 32 columns, 17 us for 72 of a sixth of the reduction, sum included; 3000 rows, 1200 ->
-// 16: 11 us less.)  Wider outputs keep the columns: their steps do take longer and the slices are larger (2500 x 900 -> 256: 4 us more).
-int tc_rows_slices(int Kd, int n_cols, int npairs) {
-    if (n_cols > 128) return 1;
-    const int bn = tc_rows_bn(n_cols, npairs, 2), nkb = (Kd + BK - 1) / BK;
-    const long long tiles = (long long)npairs * ((n_cols + bn - 1) / bn);
-    const int want = (int)std::min<long long>(std::min(8, nkb / 8), tiles > 0 ? 74 / tiles : 1);
-    if (want < 2) return 1;
-    const int kbs = (nkb + want - 1) / want;
-    return (nkb + kbs - 1) / kbs;
-}
-
 // The drain can sum columns when a tile holds all of them.
-bool tc_rows_sums_columns(int n_cols, int npairs) { return tc_rows_bn(n_cols, npairs, 1) >= n_cols; }
+bool tc_rows_sums_columns(int n_cols, int npairs) { return tc_rows_bn(n_cols, npairs) >= n_cols; }
 int tc_rows_clusters(long long ntiles, int num_sms) { return (int)std::min<long long>(ntiles, std::min(max_clusters(num_sms), kMaxRowClusters)); }
 
 cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols,
                                 float* C, int ldc, const RowSpan* pair_tiles, int npairs, const float* Hmask, int ldh, float scale,
-                                const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16, float* colsum, int slices,
-                                float* parts, int64_t rows) {
+                                const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16, float* colsum) {
     if (npairs <= 0) return cudaSuccess;
     if ((mode == 2 && !act) || (Cbf16 && mode == 2) || (Cbf16 && mode == 1 && !Hmask)) return cudaErrorInvalidValue;
     if (colsum && !(mode == 1 && Hmask && tc_rows_sums_columns(n_cols, npairs))) return cudaErrorInvalidValue;
-    if (slices > 1 && (mode == 1 || !parts)) return cudaErrorInvalidValue;
     RowsArgs a;
-    a.tiles = pair_tiles; a.npairs = npairs; a.BN = tc_rows_bn(n_cols, npairs, slices); a.ntn = (ldc + a.BN - 1) / a.BN; a.Kd = Kd;
-    a.kbs = ((Kd + BK - 1) / BK + slices - 1) / slices; a.slice_stride = slices > 1 ? (long long)rows * ldc : 0;
-    rows_layout(a.BN, std::min(Kd, a.kbs * BK), passes, a);
-    a.C = slices > 1 ? parts : C; a.Cbf = reinterpret_cast<uint32_t*>(Cbf16); a.ldc = ldc; a.Hmask = Hmask; a.ldh = ldh; a.scale = scale; a.colsum = colsum;
+    a.tiles = pair_tiles; a.npairs = npairs; a.BN = tc_rows_bn(n_cols, npairs); a.ntn = (ldc + a.BN - 1) / a.BN; a.Kd = Kd;
+    rows_layout(a.BN, Kd, passes, a);
+    a.C = C; a.Cbf = reinterpret_cast<uint32_t*>(Cbf16); a.ldc = ldc; a.Hmask = Hmask; a.ldh = ldh; a.scale = scale; a.colsum = colsum;
     a.kmul = one_b ? 0 : 1; a.err = err;
     a.act = act ? *act : ActEpi{};
-    const dim3 grid(2u * (unsigned)tc_rows_clusters((long long)npairs * a.ntn, num_sms), (unsigned)slices);
-    const int drain = slices > 1 ? kPlain : mode == 2 ? (a.act.drop ? kActDrop : kAct) : mode == 1 && Hmask ? (Cbf16 ? kMaskBf16 : kMask) : Cbf16 ? kBf16 : kPlain;
+    const unsigned grid = 2u * (unsigned)tc_rows_clusters((long long)npairs * a.ntn, num_sms);
+    const int drain = mode == 2 ? (a.act.drop ? kActDrop : kAct) : mode == 1 && Hmask ? (Cbf16 ? kMaskBf16 : kMask) : Cbf16 ? kBf16 : kPlain;
     auto go = [&](auto kernel) {
         cudaError_t e = configure_kernel_once(reinterpret_cast<const void*>(kernel), SMEM_BYTES, false);
         if (e != cudaSuccess) return e;
-        e = launch(kernel, grid, THREADS, SMEM_BYTES, s, *reinterpret_cast<const CUtensorMap*>(mapA), *reinterpret_cast<const CUtensorMap*>(mapB),
+        e = launch(kernel, dim3(grid), THREADS, SMEM_BYTES, s, *reinterpret_cast<const CUtensorMap*>(mapA), *reinterpret_cast<const CUtensorMap*>(mapB),
                                                  *reinterpret_cast<const CUtensorMap*>(mapBlo), a);
-        ++g_kernel_launches;
-        if (e != cudaSuccess || slices == 1) return e;
-        e = launch_tail(sum_slices_kernel, dim3(2u * (unsigned)npairs, (unsigned)(BM / SUM_ROWS)), 256, 0, s, parts, slices, a.slice_stride, pair_tiles, C,
-                   reinterpret_cast<uint2*>(Cbf16), ldc, mode == 2 ? 1 : 0, a.act);
         ++g_kernel_launches;
         return e;
     };

@@ -282,7 +282,7 @@ cudaError_t launch_scatter_core(const float* logits, int ld, int C, const int32_
                                 int nspans, float* out, cudaStream_t s);
 
 // host_copy.cu: `bytes` of device memory into the caller's memory through pinned slots, complete on return; the pages of
-// a pageable destination touched ahead of it (they are overwritten by the copy); contexts that may copy, + 1 / - 1.
+// a pageable destination touched ahead of it, their contents kept; contexts that may copy, + 1 / - 1.
 cudaError_t copy_to_host(void* dst, const void* src, size_t bytes, cudaStream_t s);
 void host_prefault(void* dst, size_t bytes);
 void host_copy_user(int delta);

@@ -485,14 +485,14 @@ int plan_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int
     if (g->nnz < 0 || g->rowptr[0] != 0) { err = "rowptr must start at 0 and nnz must not be negative"; return GAD_ERR_ARG; }
     if (!cfg->graph_resident) {
         int bad = 0;
-#pragma omp parallel for schedule(static) reduction(| : bad) num_threads(8) if (g->n > (1 << 16))
+#pragma omp parallel for schedule(static) reduction(| : bad) if (g->n > (1 << 16))
         for (int32_t v = 0; v < g->n; ++v) bad |= g->rowptr[v + 1] < g->rowptr[v];
         if (bad) { err = "rowptr decreases"; return GAD_ERR_UNSORTED; }
     }
     if (g->rowptr[g->n] != g->nnz) { err = "rowptr[n] differs from nnz"; return GAD_ERR_ARG; }
     if (!cfg->graph_resident) {
         int bad = 0;
-#pragma omp parallel for schedule(static) reduction(| : bad) num_threads(8) if (g->nnz > (1 << 16))
+#pragma omp parallel for schedule(static) reduction(| : bad) if (g->nnz > (1 << 16))
         for (int64_t e = 0; e < g->nnz; ++e) bad |= g->col[e] < 0 || g->col[e] >= g->n;
         if (bad) { err = "column out of range"; return GAD_ERR_RANGE; }
     }
@@ -500,7 +500,7 @@ int plan_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int
         if (core_ptr[k + 1] < core_ptr[k]) { err = "core_ptr decreases"; return GAD_ERR_UNSORTED; }
     p.max_walks.assign((size_t)K, 0);
     int bad = 0;
-#pragma omp parallel for schedule(dynamic) reduction(| : bad) num_threads(8) if (core_ptr[K] - core_ptr[0] > (1 << 15))
+#pragma omp parallel for schedule(dynamic) reduction(| : bad) if (core_ptr[K] - core_ptr[0] > (1 << 15))
     for (int32_t k = 0; k < K; ++k) {
         int64_t deg = 0;
         for (int64_t t = core_ptr[k]; t < core_ptr[k + 1]; ++t) {

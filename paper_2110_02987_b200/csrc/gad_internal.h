@@ -14,6 +14,10 @@
 
 namespace gad {
 
+// Host loops run on OpenMP's default team or on the calling thread alone, never on a team of another size: a smaller one takes the threads
+// it does not need down, and the next full one sets them up again (16 threads: a region of the same team 2 us, the first full one after
+// a region of 2 / 4 / 8 threads 310 / 260 / 150 us).
+
 inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
 // Kernels launched by this library in this process (every <<<>>> adds one; contexts on several host threads share it).

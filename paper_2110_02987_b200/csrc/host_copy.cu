@@ -23,11 +23,12 @@ namespace gad {
 namespace {
 
 constexpr size_t kRingBytes = 8u << 20, kMinSlot = 256u << 10, kMaxSlot = 2u << 20;
-constexpr int kSlots = 32, kMaxThreads = 8;   // most slots of a ring
+constexpr int kSlots = 32, kMaxThreads = 8;   // most slots of a ring; most threads that copy
 constexpr size_t kTouchBytes = 1u << 20;  // destinations below this are not worth waking threads for
 constexpr size_t kPage = 4096;
 constexpr size_t kSmallPinned = 16384;
 
+// Threads that take part.  They belong to the team of all host loops of the library (gad_internal.h); the others of it leave at once.
 int copy_threads(size_t bytes) {
     return (int)std::max<size_t>(1, std::min<size_t>({(size_t)kMaxThreads, (size_t)omp_get_num_procs() / 2, bytes / (128u << 10)}));
 }
@@ -110,9 +111,13 @@ void host_prefault(void* dst, size_t bytes) {
     if (bytes < kTouchBytes || !is_pageable(dst)) return;
     char* d = (char*)dst;
     const int64_t n = (int64_t)(bytes / kPage);
-#pragma omp parallel for num_threads(copy_threads(bytes)) schedule(static)
-    for (int64_t i = 0; i < n; ++i)   // adding nothing is a write as far as the page is concerned, and leaves what is there: the copy may never come
-        __atomic_fetch_add(d + (size_t)i * kPage, 0, __ATOMIC_RELAXED);
+    const int nt = copy_threads(bytes);
+#pragma omp parallel if (nt > 1)
+    {
+        const int team = std::min(nt, omp_get_num_threads()), t = omp_get_thread_num();
+        // adding nothing is a write as far as the page is concerned, and leaves what is there: the copy may never come
+        for (int64_t i = n * t / team; t < team && i < n * (t + 1) / team; ++i) __atomic_fetch_add(d + (size_t)i * kPage, 0, __ATOMIC_RELAXED);
+    }
 }
 
 cudaError_t copy_to_host(void* dst, const void* src, size_t bytes, cudaStream_t s) {
@@ -161,12 +166,12 @@ cudaError_t copy_to_host(void* dst, const void* src, size_t bytes, cudaStream_t 
                 waiting.store(false);
             }
         };
-#pragma omp parallel num_threads(nt)
+#pragma omp parallel if (nt > 1)
         {
-            const int team = omp_get_num_threads(), t = omp_get_thread_num();
-            const cudaError_t r = cudaSetDevice(dev);
+            const int team = std::min(nt, omp_get_num_threads()), t = omp_get_thread_num();
+            const cudaError_t r = t < team ? cudaSetDevice(dev) : cudaSuccess;
             if (r != cudaSuccess) bad.store((int)r);
-            for (int64_t i = 0; i < n && !bad.load(); ++i) {
+            for (int64_t i = 0; t < team && i < n && !bad.load(); ++i) {
                 wait_for_slot(i);
                 if (bad.load()) break;
                 const size_t len = length(i), lo = len * (size_t)t / team / 64 * 64, hi = t + 1 == team ? len : len * (size_t)(t + 1) / team / 64 * 64;

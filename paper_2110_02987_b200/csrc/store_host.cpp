@@ -10,8 +10,7 @@
 
 namespace gad {
 
-// A host loop of less than this many row visits runs on the calling thread: waking the others costs more than they save.  (All or none of
-// them: a team whose size changes from loop to loop is taken down and set up again.)
+// A host loop of less than this many row visits runs on the calling thread: waking the others costs more than they save.
 static bool worth_threads(int64_t rows) { return rows >= 512; }
 
 static int validate(const gad_csr* g, const gad_partition* part, std::string& err) {

@@ -341,8 +341,12 @@ int gad_launch_count(int64_t* launches);
  * gad_create). */
 const char* gad_last_error(const gad_ctx* ctx);
 
-/* Frees the context.  Frees nothing the caller allocated (workspace, stream). */
+/* Frees the context.  Frees nothing the caller allocated (workspace, stream).  Its pinned host memory is kept for the next
+ * context: at most 16 blocks of 16 KB and two of 8 MB in a process. */
 void gad_destroy(gad_ctx* ctx);
+
+/* Frees the pinned host memory that the library keeps and no context or call is using. */
+int gad_release_pinned(void);
 
 #ifdef __cplusplus
 }

@@ -27,7 +27,7 @@ SYMBOLS = (
     "gad_profile_reset", "gad_profile_count", "gad_profile_read", "gad_subgraph_weights_static", "gad_launch_count",
     "gad_last_error", "gad_destroy", "gad_train_epoch_local", "gad_consensus_floats", "gad_consensus_partial",
     "gad_consensus_apply", "gad_export_params", "gad_get_train_counts", "gad_augment_workspace_bytes", "gad_augment",
-    "gad_augment_last_error", "gad_debug_expire_wait", "gad_default_params", "gad_check_store",
+    "gad_augment_last_error", "gad_debug_expire_wait", "gad_default_params", "gad_check_store", "gad_release_pinned",
 )
 
 
@@ -413,6 +413,13 @@ def launch_count() -> int:
     if rc != GAD_OK:
         raise GadError(rc)
     return int(n.value)
+
+
+def release_pinned():
+    """gad_release_pinned: frees the pinned host memory the library keeps for later contexts."""
+    rc = load().gad_release_pinned()
+    if rc != GAD_OK:
+        raise GadError(rc)
 
 
 class _AugmentConfig(C.Structure):

@@ -317,8 +317,8 @@ struct gad_ctx {
     bool profiling = false;
     std::vector<ProfEntry> prof;
     std::vector<float> host_block;  // staging for parameter pack / unpack
-    char* pinned = nullptr;         // pinned host memory the small results of waiting calls land in (pinned_bytes)
-    size_t pinned_bytes = 0;
+    Pinned pinned_block;
+    char* pinned = nullptr;         // pinned host memory the small results of waiting calls land in
     float* published = nullptr;     // second half of it: losses and error words as the last kernel of an epoch leaves them
     // The replicas' parameters are equal (after creation and every consensus) until gad_set_params gives one its own: copy 0 then
     // stands for all of them and the others are stale.  `unsettled`: a consensus over differing copies has been enqueued and
@@ -833,8 +833,8 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
     ctx->cfg.dims = ctx->p.dims.data();
     const Plan& p = ctx->p;
     const size_t report_bytes = (size_t)round_up((int64_t)std::max(p.o_flags + 16 - p.o_loss, 8 * (size_t)p.K), 128);
-    ctx->pinned_bytes = 2 * report_bytes;
-    if (!(ctx->pinned = take_small_pinned(ctx->pinned_bytes))) return fail(ctx, GAD_ERR_OOM, "no pinned host memory");
+    ctx->pinned_block = take_small_pinned(2 * report_bytes);
+    if (!(ctx->pinned = ctx->pinned_block.p)) return fail(ctx, GAD_ERR_OOM, "no pinned host memory");
     ctx->published = reinterpret_cast<float*>(ctx->pinned + report_bytes);
     if (workspace_bytes < p.bytes) return fail(ctx, GAD_ERR_OOM, "workspace smaller than gad_workspace_bytes");
     const int C = p.dims[p.L];
@@ -1468,6 +1468,11 @@ int gad_launch_count(int64_t* launches) {
 
 const char* gad_last_error(const gad_ctx* ctx) { return ctx ? ctx->err.c_str() : g_last_error.c_str(); }
 
+int gad_release_pinned(void) {
+    release_pinned();
+    return GAD_OK;
+}
+
 void gad_destroy(gad_ctx* ctx) {
     if (!ctx) return;
     for (auto& eg : ctx->graphs)
@@ -1475,7 +1480,7 @@ void gad_destroy(gad_ctx* ctx) {
     for (auto& e : ctx->prof)
         for (auto& pr : e.pending) { cudaEventDestroy(pr.first); cudaEventDestroy(pr.second); }
     if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
-    if (ctx->pinned) give_small_pinned(ctx->pinned, ctx->pinned_bytes);
+    if (ctx->pinned) give_small_pinned(ctx->pinned_block);
     if (ctx->copy_stream) { cudaStreamSynchronize(ctx->copy_stream); cudaStreamDestroy(ctx->copy_stream); }
     if (ctx->side_stream) { cudaStreamSynchronize(ctx->side_stream); cudaStreamDestroy(ctx->side_stream); }
     for (cudaEvent_t e : {ctx->ev_fork, ctx->ev_g1, ctx->ev_bias, ctx->ev_join})

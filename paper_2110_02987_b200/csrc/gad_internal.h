@@ -290,7 +290,9 @@ cudaError_t launch_scatter_core(const float* logits, int ld, int C, const int32_
 cudaError_t copy_to_host(void* dst, const void* src, size_t bytes, cudaStream_t s);
 void host_prefault(void* dst, size_t bytes);
 void host_copy_user(int delta);
-char* take_small_pinned(size_t bytes);
-void give_small_pinned(char* b, size_t bytes);
+struct Pinned { char* p = nullptr; size_t bytes = 0; unsigned long long id = 0; };
+Pinned take_small_pinned(size_t bytes);   // p null: none to be had
+void give_small_pinned(const Pinned& m);
+void release_pinned();   // frees the pinned memory that lies idle
 
 }  // namespace gad

@@ -6,6 +6,7 @@
 // slots are large where there is much to copy; sharing a slot keeps what is left after the last of them short, and counters instead of a
 // fork and a join per slot keep it cheap.  (16 MB: 0.75 ms with a join per 512 KB slot, 0.55 ms with a thread to every slot, 0.45 ms now;
 // the bare copy of 16 MB takes 0.30.)
+#include <cuda.h>
 #include <omp.h>
 
 #include <algorithm>
@@ -33,39 +34,62 @@ int copy_threads(size_t bytes) {
     return (int)std::max<size_t>(1, std::min<size_t>({(size_t)kMaxThreads, (size_t)omp_get_num_procs() / 2, bytes / (128u << 10)}));
 }
 
-// Pinned buffers of kRingBytes, shared by all contexts of the process: at most two are kept while a context exists, none
-// after the last one has gone.
+// Pinned memory that lies idle, for all contexts of the process: at most two rings and sixteen small blocks.  It stays when the last
+// context goes (pinning 16 KB took 1.0 to 2.3 ms and 8 MB 4 to 6, freeing them 0.4 and 1.3, each wait for the device included: a program
+// with one context at a time paid that in every one) until gad_release_pinned or the end of the process.
+struct Block { char* p; unsigned long long id; };   // id: the driver's of this very allocation
 struct Pool {
     std::mutex lock;
     int users = 0;
-    std::vector<char*> idle, idle_small;
+    std::vector<Block> idle, idle_small;
 } g_pool;
 
-// One buffer of `bytes` from the idle ones, or a new one (null if there is none to be had).
-char* take_from(std::vector<char*>& idle, size_t bytes) {
-    {
-        std::lock_guard<std::mutex> g(g_pool.lock);
-        if (!idle.empty()) { char* b = idle.back(); idle.pop_back(); return b; }
-    }
-    void* b = nullptr;
-    if (cudaHostAlloc(&b, bytes, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    return (char*)b;
+// The driver's identifier of the allocation at p, which no other one ever gets; 0 if there is none.
+unsigned long long allocation_id(const void* p) {
+    typedef CUresult (*GetAttributeFn)(void*, CUpointer_attribute, CUdeviceptr);
+    static const GetAttributeFn get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPoint("cuPointerGetAttribute", &f, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess;
+        if (!ok) cudaGetLastError();
+        return ok ? (GetAttributeFn)f : nullptr;
+    }();
+    unsigned long long id = 0;
+    return get && get(&id, CU_POINTER_ATTRIBUTE_BUFFER_ID, (CUdeviceptr)p) == CUDA_SUCCESS ? id : 0;
 }
-void give_to(std::vector<char*>& idle, size_t most, char* b) {
-    {
-        std::lock_guard<std::mutex> g(g_pool.lock);
-        if (g_pool.users > 0 && idle.size() < most) { idle.push_back(b); return; }
+
+// One block of `bytes` from the idle ones, or a new one (null if there is none to be had).  An idle block that is no longer what it was
+// (the device has been reset since) is forgotten, not freed.
+Block take_from(std::vector<Block>& idle, size_t bytes) {
+    for (;;) {
+        Block b{nullptr, 0};
+        {
+            std::lock_guard<std::mutex> g(g_pool.lock);
+            if (idle.empty()) break;
+            b = idle.back();
+            idle.pop_back();
+        }
+        if (allocation_id(b.p) == b.id) return b;
     }
-    cudaFreeHost(b);
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, bytes, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return {nullptr, 0}; }
+    return {(char*)p, allocation_id(p)};
 }
-char* take_buffer() {
+void give_to(std::vector<Block>& idle, size_t most, Block b) {
+    if (b.id) {
+        std::lock_guard<std::mutex> g(g_pool.lock);
+        if (idle.size() < most) { idle.push_back(b); return; }
+    }
+    cudaFreeHost(b.p);
+}
+Block take_buffer() {
     {
         std::lock_guard<std::mutex> g(g_pool.lock);
-        if (g_pool.users <= 0) return nullptr;   // no context to keep the buffer for: pinning one for a single copy costs more than it saves
+        if (g_pool.users <= 0 && g_pool.idle.empty()) return {nullptr, 0};   // no context: pinning a ring for a single copy costs more than it saves
     }
     return take_from(g_pool.idle, kRingBytes);
 }
-void give_buffer(char* b) { give_to(g_pool.idle, 2, b); }
+void give_buffer(Block b) { give_to(g_pool.idle, 2, b); }
 
 bool is_pageable(const void* p) {
     cudaPointerAttributes a;
@@ -81,30 +105,32 @@ struct Events {
 }  // namespace
 
 void host_copy_user(int delta) {
-    std::vector<char*> drop;
-    {
-        std::lock_guard<std::mutex> g(g_pool.lock);
-        g_pool.users += delta;
-        if (g_pool.users <= 0) {
-            drop.swap(g_pool.idle);
-            drop.insert(drop.end(), g_pool.idle_small.begin(), g_pool.idle_small.end());
-            g_pool.idle_small.clear();
-        }
-    }
-    for (char* b : drop) cudaFreeHost(b);
+    std::lock_guard<std::mutex> g(g_pool.lock);
+    g_pool.users += delta;
 }
 
-// Pinned memory for a context's small results.  Allocating pinned memory costs about a millisecond and waits for the device, so
-// blocks of the common size are kept (at most 16) for the next context.
-char* take_small_pinned(size_t bytes) {
-    if (bytes <= kSmallPinned) return take_from(g_pool.idle_small, kSmallPinned);
-    void* b = nullptr;
-    if (cudaHostAlloc(&b, bytes, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    return (char*)b;
+void release_pinned() {
+    std::vector<Block> drop;
+    {
+        std::lock_guard<std::mutex> g(g_pool.lock);
+        drop.swap(g_pool.idle);
+        drop.insert(drop.end(), g_pool.idle_small.begin(), g_pool.idle_small.end());
+        g_pool.idle_small.clear();
+    }
+    for (const Block& b : drop)
+        if (allocation_id(b.p) == b.id) cudaFreeHost(b.p);
 }
-void give_small_pinned(char* b, size_t bytes) {
-    if (bytes <= kSmallPinned) give_to(g_pool.idle_small, 16, b);
-    else cudaFreeHost(b);
+
+// Pinned memory for a context's small results.
+Pinned take_small_pinned(size_t bytes) {
+    if (bytes <= kSmallPinned) { const Block b = take_from(g_pool.idle_small, kSmallPinned); return {b.p, bytes, b.id}; }
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, bytes, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); p = nullptr; }
+    return {(char*)p, bytes, 0};
+}
+void give_small_pinned(const Pinned& m) {
+    if (m.bytes <= kSmallPinned) give_to(g_pool.idle_small, 16, {m.p, m.id});
+    else cudaFreeHost(m.p);
 }
 
 void host_prefault(void* dst, size_t bytes) {
@@ -122,7 +148,8 @@ void host_prefault(void* dst, size_t bytes) {
 
 cudaError_t copy_to_host(void* dst, const void* src, size_t bytes, cudaStream_t s) {
     cudaError_t e;
-    char* buf = bytes > 0 && is_pageable(dst) ? take_buffer() : nullptr;
+    const Block ring_block = bytes > 0 && is_pageable(dst) ? take_buffer() : Block{nullptr, 0};
+    char* buf = ring_block.p;
     if (!buf) {   // pinned destination, or no ring: one plain copy
         e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s);
         return e != cudaSuccess ? e : cudaStreamSynchronize(s);
@@ -188,7 +215,7 @@ cudaError_t copy_to_host(void* dst, const void* src, size_t bytes, cudaStream_t 
         e = (cudaError_t)bad.load();
     }
     if (e != cudaSuccess) cudaStreamSynchronize(s);   // nothing may still be writing into the buffer when it goes back
-    give_buffer(buf);
+    give_buffer(ring_block);
     return e;
 }
 

@@ -1,0 +1,48 @@
+"""Host memory that outlives a context: pinned blocks are kept for the next one and can be given back."""
+import time
+
+import numpy as np
+import pytest
+
+import __graft_entry__ as entry
+from conftest import small_random_case
+from paper_2110_02987_b200 import binding
+from test_gpu_parity import make_pair
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    entry.build()
+
+
+def test_a_context_after_the_last_one_pins_nothing_anew():
+    """One context at a time: the first result of each is copied through memory that is pinned already (pinning the ring takes
+    4 ms or more, the whole call a tenth of one)."""
+    case = small_random_case(5, n=300, K=3, p=0.03)
+    first = []
+    for _ in range(7):
+        g, _, _ = make_pair(case, (20, 24, 6), 5)
+        with g:
+            t0 = time.perf_counter()
+            g.forward()
+            first.append(time.perf_counter() - t0)
+    assert min(first[1:]) < 1.5e-3, first
+
+
+def test_release_pinned_leaves_live_contexts_alone():
+    case = small_random_case(6, n=300, K=3, p=0.03)
+    g, ref, _ = make_pair(case, (20, 24, 6), 6)
+    with g:
+        for _ in range(3):
+            binding.release_pinned()
+            lg, lr = g.train_epoch(), ref.train_epoch()
+            assert np.max(np.abs(lg - lr)) <= 1e-4
+            a = g.forward()
+            binding.release_pinned()
+            assert np.array_equal(a, g.forward())
+    binding.release_pinned()
+    g, ref, _ = make_pair(case, (20, 24, 6), 6)
+    with g:
+        assert np.max(np.abs(g.train_epoch() - ref.train_epoch())) <= 1e-4

@@ -921,10 +921,10 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
     {
         int dev = 0;
         GAD_CK(cudaGetDevice(&dev));
-        cudaDeviceProp prop;
-        GAD_CK(cudaGetDeviceProperties(&prop, dev));
-        ctx->num_sms = prop.multiProcessorCount;
-        ctx->use_tc = (cfg->flags & 1) == 0 && prop.major == 10 && p.Np > 0;
+        int major = 0;   // (the whole of cudaGetDeviceProperties takes 2.5 ms and more)
+        GAD_CK(cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, dev));
+        GAD_CK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
+        ctx->use_tc = (cfg->flags & 1) == 0 && major == 10 && p.Np > 0;
     }
     if (ctx->cfg.zeta_mode == 1) {
         ctx->use_gram = ctx->use_tc && !p.gram_ptr.empty();

@@ -5,7 +5,8 @@ import numpy as np
 import pytest
 
 import __graft_entry__ as entry
-from conftest import small_random_case
+import paper_2110_02987_b200 as pkg
+from conftest import flat, small_random_case
 from paper_2110_02987_b200 import binding
 from test_gpu_parity import make_pair
 
@@ -15,6 +16,21 @@ pytestmark = pytest.mark.gpu
 @pytest.fixture(scope="module", autouse=True)
 def built():
     entry.build()
+
+
+def test_a_small_context_is_created_at_once():
+    """Streams, events and a store of 300 nodes take 0.5 ms; asking the driver for all properties of the device took 2.5 and more, and
+    pinning another one."""
+    case = small_random_case(7, n=300, K=3, p=0.03)
+    n, rowptr, col, w, core, halos = case
+    X, y, split = np.zeros((n, 20), np.float32), np.zeros(n, np.int32), np.zeros(n, np.uint8)
+    took = []
+    for _ in range(7):
+        t0 = time.perf_counter()
+        g = pkg.Gad(n, rowptr, col, *flat(core), *flat(halos), X, y, split, (20, 24, 6))
+        took.append(time.perf_counter() - t0)
+        g.close()
+    assert min(took[1:]) < 1.7e-3, took
 
 
 def test_a_context_after_the_last_one_pins_nothing_anew():

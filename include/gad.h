@@ -317,7 +317,8 @@ typedef struct {
     uint64_t seed;
     int32_t graph_resident; /* 0: copy g to the device; 1: the caller vouches that an earlier gad_augment call with   *
                              * this very workspace and the same g (n, nnz, rowptr, col unchanged) left it there:  *
-                             * the copy is skipped (the graph sits at the start of the workspace)                   */
+                             * the copy is skipped (the graph sits at the start of the workspace).  The arrays are   *
+                             * checked all the same, the columns while the GPU works                                 */
 } gad_augment_config;
 
 /* Bytes of device workspace gad_augment needs.  Host-only. */

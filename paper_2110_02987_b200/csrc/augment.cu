@@ -66,6 +66,7 @@ struct SubDesc {
     int64_t core0, ncore;   // its part of the batch's core list
     int64_t key0;           // first ranking key
     int64_t top0, top_cap;  // first row, and rows, of the leading walks' sequences; the buffer of gathered keys is kTopSlack times that
+    int64_t max_walks;      // there is room for: cap times the core set's degree sum, which no count of walks exceeds on the same graph
     int32_t sub, pad;       // number of the subgraph: its random stream
 };
 struct SubState {
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__(256) walk_count_kernel(const int64_t* __restri
                                                          int32_t* __restrict__ count, int32_t* __restrict__ node, int64_t plane) {
     const SubDesc d = desc[blockIdx.y];
     const SubState& s = state[blockIdx.y];
-    const int64_t nB = s.nB, j1 = extra ? s.nwalks : (int64_t)s.n0;
+    const int64_t nB = s.nB, j1 = extra ? s.nwalks : min((int64_t)s.n0, d.max_walks);
     const uint8_t* in = inside + (int64_t)blockIdx.y * n;
     int32_t* cnt = count + (int64_t)blockIdx.y * n;
     int32_t seq[kMaxSteps + 1];
@@ -264,17 +265,17 @@ __global__ void __launch_bounds__(256) count_stats_kernel(const int32_t* __restr
 }
 // Number of walks from the Monte-Carlo error equation, sigma / mean of the visit frequencies from the integer sums.  Every
 // operation is rounded on its own, as on the host.
-__global__ void decide_walks_kernel(SubState* __restrict__ state, int G, double zc_over_E, int cap) {
+__global__ void decide_walks_kernel(SubState* __restrict__ state, const SubDesc* __restrict__ desc, int G, double zc_over_E, int cap) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= G) return;
     SubState& s = state[g];
-    const long long n0 = (long long)s.n0;
+    const long long n0 = min((long long)s.n0, (long long)desc[g].max_walks);
     long long want = 0;
     if (s.m > 0) {
         const double ratio = __dadd_rn(__ddiv_rn(__dmul_rn((double)s.m, (double)s.s2), __dmul_rn((double)s.s1, (double)s.s1)), -1.0);
         if (ratio > 0.0) want = (long long)ceil(__dmul_rn(__dmul_rn(zc_over_E, zc_over_E), ratio));
     }
-    const long long most = (long long)cap * n0;
+    const long long most = min((long long)cap * n0, (long long)desc[g].max_walks);
     s.nwalks = max(n0, min(want, most));
     if (s.nwalks > n0) { s.m = 0; s.s1 = 0; s.s2 = 0; }   // counted again over all walks
 }
@@ -475,27 +476,28 @@ BatchLayout batch_layout(const AugPlan& p, size_t base, int64_t n, const int64_t
 constexpr size_t kBatchNodeBytes = 256u << 20;    // visit counts, inside and boundary maps, 6 bytes per node and subgraph
 constexpr int64_t kBatchWalkBytes = 1ll << 30;    // a ranking key (8 bytes) and steps + 1 nodes per walk
 
+int check_columns(const gad_csr* g, std::string& err) {
+    int bad = 0;
+#pragma omp parallel for schedule(static) reduction(| : bad) if (g->nnz > (1 << 16))
+    for (int64_t e = 0; e < g->nnz; ++e) bad |= g->col[e] < 0 || g->col[e] >= g->n;
+    if (bad) { err = "column out of range"; return GAD_ERR_RANGE; }
+    return GAD_OK;
+}
+
+// `columns`: check them here; else the caller does (check_columns).
 int plan_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int32_t* core_nodes, const gad_augment_config* cfg, AugPlan& p,
-                 std::string& err) {
+                 std::string& err, bool columns) {
     if (!g || !g->rowptr || (g->nnz > 0 && !g->col) || g->n < 0 || K < 1 || !core_ptr || !cfg) { err = "bad arguments"; return GAD_ERR_ARG; }
     if (cfg->steps < 1 || cfg->steps > kMaxSteps) { err = "steps must be 1 .. 8"; return GAD_ERR_ARG; }
     if (!(cfg->alpha >= 0.0) || !(cfg->E > 0.0) || !(cfg->zc > 0.0) || cfg->cap < 1) { err = "alpha >= 0, E > 0, zc > 0, cap >= 1"; return GAD_ERR_ARG; }
-    // the kernels index rowptr, col and the per-node arrays with the caller's values: check the whole CSR here, on the host.
-    // With graph_resident the caller vouches that this very graph went through here before.
+    // the kernels index rowptr, col and the per-node arrays with the caller's values: check the whole CSR here, on the host
     if (g->nnz < 0 || g->rowptr[0] != 0) { err = "rowptr must start at 0 and nnz must not be negative"; return GAD_ERR_ARG; }
-    if (!cfg->graph_resident) {
-        int bad = 0;
-#pragma omp parallel for schedule(static) reduction(| : bad) if (g->n > (1 << 16))
-        for (int32_t v = 0; v < g->n; ++v) bad |= g->rowptr[v + 1] < g->rowptr[v];
-        if (bad) { err = "rowptr decreases"; return GAD_ERR_UNSORTED; }
-    }
+    int down = 0;
+#pragma omp parallel for schedule(static) reduction(| : down) if (g->n > (1 << 16))
+    for (int32_t v = 0; v < g->n; ++v) down |= g->rowptr[v + 1] < g->rowptr[v];
+    if (down) { err = "rowptr decreases"; return GAD_ERR_UNSORTED; }
     if (g->rowptr[g->n] != g->nnz) { err = "rowptr[n] differs from nnz"; return GAD_ERR_ARG; }
-    if (!cfg->graph_resident) {
-        int bad = 0;
-#pragma omp parallel for schedule(static) reduction(| : bad) if (g->nnz > (1 << 16))
-        for (int64_t e = 0; e < g->nnz; ++e) bad |= g->col[e] < 0 || g->col[e] >= g->n;
-        if (bad) { err = "column out of range"; return GAD_ERR_RANGE; }
-    }
+    if (columns) { int rc = check_columns(g, err); if (rc != GAD_OK) return rc; }
     for (int32_t k = 0; k < K; ++k)
         if (core_ptr[k + 1] < core_ptr[k]) { err = "core_ptr decreases"; return GAD_ERR_UNSORTED; }
     p.max_walks.assign((size_t)K, 0);
@@ -556,7 +558,7 @@ int gad_augment_workspace_bytes(const gad_csr* g, int32_t K, const int64_t* core
     if (!bytes) return GAD_ERR_ARG;
     AugPlan p;
     std::string err;
-    int rc = plan_augment(g, K, core_ptr, core_nodes, cfg, p, err);
+    int rc = plan_augment(g, K, core_ptr, core_nodes, cfg, p, err, true);
     if (rc != GAD_OK) return aug_fail(rc, err);
     *bytes = p.bytes;
     return GAD_OK;
@@ -568,7 +570,10 @@ int gad_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int3
     if (!workspace || !halo_ptr || (halo_capacity > 0 && !halo_nodes) || ((uintptr_t)workspace & 255) != 0) return aug_fail(GAD_ERR_ARG, "bad arguments");
     AugPlan p;
     std::string err;
-    int rc = plan_augment(g, K, core_ptr, core_nodes, cfg, p, err);
+    // A graph that is on the device already had its columns checked on the way there; the kernels read that copy, so the caller's columns, which
+    // the host reads after them, are checked while they run.
+    bool unchecked = cfg && cfg->graph_resident != 0;
+    int rc = plan_augment(g, K, core_ptr, core_nodes, cfg, p, err, !unchecked);
     if (rc != GAD_OK) return aug_fail(rc, err);
     if (workspace_bytes < p.bytes) return aug_fail(GAD_ERR_OOM, "workspace smaller than gad_augment_workspace_bytes");
     cudaStream_t s = (cudaStream_t)stream_;
@@ -596,7 +601,7 @@ int gad_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int3
         for (int32_t k = k0; k < k1; ++k) {
             SubDesc& d = desc[(size_t)(k - k0)];
             d.core0 = core_ptr[k] - core_ptr[k0]; d.ncore = core_ptr[k + 1] - core_ptr[k];
-            d.key0 = key0; d.top0 = top0; d.top_cap = leading_walks(p.max_walks[(size_t)k], cfg->alpha, d.ncore); d.sub = k; d.pad = 0;
+            d.key0 = key0; d.top0 = top0; d.top_cap = leading_walks(p.max_walks[(size_t)k], cfg->alpha, d.ncore); d.max_walks = p.max_walks[(size_t)k]; d.sub = k; d.pad = 0;
             key0 += p.max_walks[(size_t)k]; top0 += d.top_cap;
             most_walks = std::max(most_walks, p.max_walks[(size_t)k]);
         }
@@ -624,7 +629,7 @@ int gad_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int3
         for (int extra = 0; extra < 2; ++extra) {   // the first batch of walks, then what the error equation asks for on top
             AUG_LAUNCH(walk_count_kernel, walk_grid, 256, d_rowptr, d_col, d_B, d_inside, n, d_desc, d_state, cfg->seed, extra, steps, d_count, d_node, L.nkeys);
             AUG_LAUNCH(count_stats_kernel, node_grid, 256, d_count, n, d_state, extra);
-            if (!extra) AUG_LAUNCH(decide_walks_kernel, (unsigned)((G + 127) / 128), 128, d_state, G, cfg->zc / cfg->E, cfg->cap);
+            if (!extra) AUG_LAUNCH(decide_walks_kernel, (unsigned)((G + 127) / 128), 128, d_state, d_desc, G, cfg->zc / cfg->E, cfg->cap);
         }
         AUG_LAUNCH(decide_lead_kernel, (unsigned)((G + 127) / 128), 128, d_state, d_desc, G, cfg->alpha, steps);
         AUG_LAUNCH(walk_key_kernel, walk_grid, 256, n, d_desc, d_state, steps, d_count, d_node, L.nkeys, d_key, 0);
@@ -638,6 +643,11 @@ int gad_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int3
         AUG_LAUNCH(key_gather_kernel, walk_grid, 256, d_key, d_desc, d_state, d_top);
         AUG_LAUNCH(lead_walks_kernel, grid(64, std::max<int64_t>(1, kTopSlack * L.ntop / G), 16), 256, d_desc, d_state, steps, d_node, L.nkeys, d_top, d_seq);
         AUG_CK(cudaGetLastError());
+        if (unchecked && (rc = check_columns(g, err)) != GAD_OK) {
+            cudaStreamSynchronize(s);   // the kernels are done with the workspace when the call returns
+            return aug_fail(rc, err);
+        }
+        unchecked = false;
         back.resize(L.o_seq - L.o_state + 4 * (size_t)L.ntop * (size_t)(steps + 1));
         AUG_CK(copy_to_host(back.data(), ws + L.o_state, back.size(), s));
         const SubState* state = (const SubState*)back.data();
@@ -646,7 +656,7 @@ int gad_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int3
             const int gi = k - k0;
             const SubState& st = state[gi];
             if (walks_out) walks_out[k] = st.nwalks;
-            if (st.nwalks > p.max_walks[(size_t)k]) return aug_fail(GAD_ERR_OOM, "more walks than planned");
+            if ((int64_t)st.n0 > p.max_walks[(size_t)k] / cfg->cap) return aug_fail(GAD_ERR_ARG, "the graph on the device is not the caller's (graph_resident)");
             if ((int64_t)st.got < st.lead || (int64_t)st.got > kTopSlack * desc[(size_t)gi].top_cap) return aug_fail(GAD_ERR_CUDA, "selection of the leading walks came out with the wrong count");
             const int64_t first = out;
             auto offer = [&](int32_t v) {   // false: the caller's list is full

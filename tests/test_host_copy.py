@@ -59,3 +59,26 @@ for f in (augment, store, touch, store, touch, augment):
 """ % (os.path.dirname(os.path.dirname(os.path.abspath(__file__))), os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", code], env=dict(os.environ, OMP_NUM_THREADS="3"), capture_output=True, text=True)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("resident", [0, 1])
+def test_augment_checks_the_graph_whether_or_not_it_is_on_the_device(resident):
+    from paper_2110_02987_b200 import binding as b
+    L = pkg.load()
+    n = 50
+    rowptr, col = np.arange(n + 1, dtype=np.int64), np.arange(n, dtype=np.int32)
+    cp = np.array([0, n], np.int64)
+    nodes = np.arange(n, dtype=np.int32)
+
+    def ws():
+        csr = b.gad_csr(n, n, b._ptr(rowptr, C.c_int64), b._ptr(col, C.c_int32), None)
+        out = C.c_size_t(0)
+        cfg = b._AugmentConfig(2, 4, 0.01, 0.05, 1.96, 0, resident)
+        return L.gad_augment_workspace_bytes(C.byref(csr), C.c_int32(1), b._ptr(cp, C.c_int64), b._ptr(nodes, C.c_int32), C.byref(cfg), C.byref(out))
+
+    assert ws() == 0
+    col[7] = n
+    assert ws() == -2
+    col[7] = 7
+    rowptr[9] = 12
+    assert ws() == -3

@@ -342,7 +342,7 @@ int gad_launch_count(int64_t* launches);
  * gad_create). */
 const char* gad_last_error(const gad_ctx* ctx);
 
-/* Frees the context.  Frees nothing the caller allocated (workspace, stream).  Its pinned host memory is kept for the next
+/* Waits for the context's work and frees the context.  Frees nothing the caller allocated (workspace, stream).  Its pinned host memory is kept for the next
  * context: at most 16 blocks of 16 KB and two of 8 MB in a process. */
 void gad_destroy(gad_ctx* ctx);
 

@@ -1475,6 +1475,10 @@ int gad_release_pinned(void) {
 
 void gad_destroy(gad_ctx* ctx) {
     if (!ctx) return;
+    // Epochs that nobody has waited for still write their losses into this context's pinned block and use the caller's workspace: the one goes to the next
+    // context, the other wherever the caller wants it.
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) cudaStreamSynchronize(ctx->stream);
     for (auto& eg : ctx->graphs)
         if (eg.exec) cudaGraphExecDestroy(eg.exec);
     for (auto& e : ctx->prof)

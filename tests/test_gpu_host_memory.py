@@ -62,3 +62,17 @@ def test_release_pinned_leaves_live_contexts_alone():
     g, ref, _ = make_pair(case, (20, 24, 6), 6)
     with g:
         assert np.max(np.abs(g.train_epoch() - ref.train_epoch())) <= 1e-4
+
+
+def test_a_context_waits_for_its_epochs_before_it_goes():
+    """Its pinned block is the next context's and its workspace the caller's again: no epoch may still be writing there."""
+    import torch
+    from gad_synth import make_workload
+    s = torch.cuda.Stream()
+    g = pkg.from_workload(make_workload("c2", scale=0.2), None, stream=s)
+    g.train_epoch()
+    for _ in range(300):
+        g.train_epoch(wait=False)
+    assert not s.query()        # (some ten milliseconds of epochs are on their way)
+    g.close()
+    assert s.query()

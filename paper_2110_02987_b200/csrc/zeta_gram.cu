@@ -118,9 +118,15 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 
+// Whether a pair has to be taken from the differences (true also where the Gram form has overflowed).
+__device__ __forceinline__ bool near_pair(float d2, float s2) { return !(d2 >= 0.05f * s2); }
+// Within these bounds of beta and of both squared norms the product of two denominators (distances up to 2^62, plus beta) neither
+// overflows nor underflows.
+constexpr float kLeastBeta = 0x1p-60f, kMostBeta = 0x1p60f, kMostNorm2 = 0x1p122f;
+
 // p_j / (d_ij + beta) summed over 16 columns j of one row i.  EACH: only the columns first .. last - 1, and without the pairs that have to be
-// taken from the differences; those are reported in `close` either way.
-template <bool EACH>
+// taken from the differences; those are reported in `close` either way.  PAIRED: two pairs share a reciprocal.
+template <bool EACH, bool PAIRED>
 __device__ __forceinline__ float gram_terms(const uint32_t (&v)[16], const float2* cols, float ni, float beta, int first, int last, bool& close) {
     float part = 0.f, p0 = 0.f, x0 = 0.f;
 #pragma unroll
@@ -128,7 +134,7 @@ __device__ __forceinline__ float gram_terms(const uint32_t (&v)[16], const float
         float2 c = cols[jj];                                   // (p_j, |x_j|^2), one broadcast load
         const float s2 = ni + c.y;
         float d2 = fmaf(-2.f, __uint_as_float(v[jj]), s2);
-        bool near = d2 < 0.05f * s2;
+        bool near = near_pair(d2, s2);
         if (EACH) {
             const bool valid = jj >= first && jj < last;
             const bool counts = valid && !near;
@@ -138,7 +144,8 @@ __device__ __forceinline__ float gram_terms(const uint32_t (&v)[16], const float
         }
         close |= near;
         const float x = sqrt_approx(d2) + beta;
-        if (jj & 1) part = fmaf(fmaf(p0, x, c.x * x0), rcp_approx(x0 * x), part);
+        if (!PAIRED) part = fmaf(c.x, rcp_approx(x), part);
+        else if (jj & 1) part = fmaf(fmaf(p0, x, c.x * x0), rcp_approx(x0 * x), part);
         p0 = c.x; x0 = x;
     }
     return part;
@@ -279,6 +286,7 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
         bool ok = true, uniform = false;
         double sum = 0.0;
         float invD = 0.f;
+        const bool beta_ok = a.beta >= kLeastBeta && a.beta <= kMostBeta;
         double* slot = a.partial + ((long long)blockIdx.x * G_EPI_WARPS + ew) * a.K;
         auto flush = [&]() {
             if (cur_k < 0) return;
@@ -306,12 +314,12 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
                 const int jb = p.j0(a) + c0;
                 if (jb + 31 <= ib || jb >= p.n || ib >= p.n) continue;        // no pair i < j of the subgraph in this block
                 __syncwarp();                                                // the previous block's columns have been read
-                {
-                    const int jl = jb + lane;                                // the column this lane looks up for the warp
-                    const bool jlv = jl < p.n;
-                    cols[lane] = make_float2(jlv ? (uniform ? 1.f : (float)a.deg[p.r0 + jl]) * invD : 0.f, jlv ? a.norm2[p.r0 + jl] : 0.f);
-                }
+                const int jl = jb + lane;                                    // the column this lane looks up for the warp
+                const bool jlv = jl < p.n;
+                const float2 mine = make_float2(jlv ? (uniform ? 1.f : (float)a.deg[p.r0 + jl]) * invD : 0.f, jlv ? a.norm2[p.r0 + jl] : 0.f);
+                cols[lane] = mine;
                 __syncwarp();
+                const bool plain = beta_ok && __all_sync(0xffffffffu, fmaxf(ni, mine.y) <= kMostNorm2);
                 const float4* xi = reinterpret_cast<const float4*>(a.X + (long long)(p.r0 + min(i, p.n - 1)) * a.ld);
                 for (int h = 0; h < 32; h += 16) {                           // (32 at a time do not fit the registers)
                     uint32_t v[16];
@@ -321,17 +329,17 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
                     const int first = i + 1 - jb - h, last = iv ? min(16, p.n - jb - h) : 0;
                     bool close = false;
                     float blk = 0.f;
-                    if (whole) blk = gram_terms<false>(v, cols + h, ni, a.beta, 0, 16, close);
-                    if (!whole || __any_sync(0xffffffffu, close)) {
+                    if (whole && plain) blk = gram_terms<false, true>(v, cols + h, ni, a.beta, 0, 16, close);
+                    if (!whole || !plain || __any_sync(0xffffffffu, close)) {
                         close = false;
-                        blk = gram_terms<true>(v, cols + h, ni, a.beta, first, last, close);
+                        blk = plain ? gram_terms<true, true>(v, cols + h, ni, a.beta, first, last, close) : gram_terms<true, false>(v, cols + h, ni, a.beta, first, last, close);
                         if (close) {   // rows close to each other compared with their norms: those pairs from the differences themselves
 #pragma unroll
                             for (int jj = 0; jj < 16; ++jj) {                // (unrolled: the accumulator block stays in registers)
                                 const float2 c = cols[h + jj];
                                 const float s2 = ni + c.y;
                                 const float d2 = fmaf(-2.f, __uint_as_float(v[jj]), s2);
-                                if (jj >= first && jj < last && d2 < 0.05f * s2)
+                                if (jj >= first && jj < last && near_pair(d2, s2))
                                     blk += c.x / (sqrtf(distance2(xi, reinterpret_cast<const float4*>(a.X + (long long)(p.r0 + jb + h + jj) * a.ld), a.ld >> 2)) + a.beta);
                             }
                         }

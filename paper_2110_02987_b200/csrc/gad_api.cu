@@ -647,7 +647,7 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
                                                 ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fi, y.ldw, dw_chunks, ndw,
                                                 ctx->at<float>(p.o_dw_partial), ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream)
                             : launch_gemm_tn_simt(agg_first ? ctx->at<float>(p.o_P[l]) : ctx->H(l), y.ldi, y.fi, agg_first ? G1 : G2, y.ldo,
-                                                  y.fo, dw_chunks, ndw, ctx->at<float>(p.o_dw_partial), y.ldw, ctx->stream);
+                                                  y.fo, dw_chunks, ndw, p.simt[(size_t)l] != 0, ctx->at<float>(p.o_dw_partial), y.ldw, ctx->stream);
             if (e != cudaSuccess) return e;
             return launch_reduce_chunks(ctx->at<float>(p.o_dw_partial), (int64_t)y.fi * y.ldw, ctx->at<int32_t>(p.dw[l].o_ptr), p.K, grads, p.pstride,
                                         y.w_int, (int64_t)y.fi * y.ldw, ctx->stream);

@@ -198,10 +198,11 @@ cudaError_t launch_narrow_bwd(const float* H, int ldh, int fi, const float* dZ, 
                               int64_t w_int, int ldw, const RowSpan* chunks, int nchunks, float scale, float* dPre, float* partial,
                               int64_t partial_stride, int32_t* err, cudaStream_t s);
 
-// partial[chunk] = H[chunk rows]^T * dZ[chunk rows]   ([M x ldw] each), one CTA column per chunk.
+// partial[chunk] = H[chunk rows]^T * dZ[chunk rows]   ([M x ldw] each), one CTA column per chunk.  small_chunks: they are of
+// simt_tn_chunk_rows.
 int64_t simt_tn_chunk_rows(int64_t rows, int fi, int ldw);
 cudaError_t launch_gemm_tn_simt(const float* H, int ldh, int M, const float* dZ, int ldz, int N,
-                                const RowSpan* chunks, int nchunks, float* partial, int ldw, cudaStream_t s);
+                                const RowSpan* chunks, int nchunks, bool small_chunks, float* partial, int ldw, cudaStream_t s);
 
 // out[k][off + i] = sum over the chunks of subgraph k, in chunk order, of partial[chunk][i], i < len.
 cudaError_t launch_reduce_chunks(const float* partial, int64_t pstride_chunk, const int32_t* chunk_ptr, int K,

@@ -342,10 +342,12 @@ int64_t simt_tn_chunk_rows(int64_t rows, int fi, int ldw) {
 }
 
 cudaError_t launch_gemm_tn_simt(const float* H, int ldh, int M, const float* dZ, int ldz, int N, const RowSpan* chunks,
-                                int nchunks, float* partial, int ldw, cudaStream_t s) {
+                                int nchunks, bool small_chunks, float* partial, int ldw, cudaStream_t s) {
     if (nchunks <= 0) return cudaSuccess;
     const long long pstride_chunk = (long long)M * ldw;
-    if ((long long)nchunks * ((M + 127) / 128) * ((ldw + 63) / 64) < 148) {
+    // Chunks of simt_tn_chunk_rows make about two blocks of 32 x 32 outputs for every SM, however many rows there are; a 128-row tile over such a
+    // chunk is mostly padding.
+    if (small_chunks || (long long)nchunks * ((M + 127) / 128) * ((ldw + 63) / 64) < 148) {
         const int ntm = (M + ST - 1) / ST, ntn = (ldw + ST - 1) / ST;
         launch(small_tn_kernel, dim3((unsigned)(ntm * ntn), (unsigned)nchunks), S_THREADS, 0, s, H, ldh, M, dZ, ldz, chunks, partial, pstride_chunk, ldw, ntn);
         ++g_kernel_launches;

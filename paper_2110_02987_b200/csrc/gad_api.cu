@@ -104,8 +104,11 @@ size_t take(size_t& cur, size_t bytes) {
 }
 
 // A layer's transforms run on the FP32 ALUs up to this many operations each, outputs narrower than a tile counted as one (and unless
-// reduced precision was asked for).  2000 rows of 32-16-4: 65 -> 44 us an epoch, 8000 of 50-32-10: 79 -> 66; above, the tensor cores are
-// ahead (2800 rows of 128 -> 128, 93 M: 155 against 167; 20 700 rows of 256 -> 3, 340 M with its padding: 199 against 217).
+// reduced precision was asked for).  Both sides below the line, ALUs / tensor cores, us an epoch: 2100 rows of 32-16-4 31 / 51, 36 750 of
+// 24-16-4 55 / 79, 94 500 of 8-8-4 82 / 113, 9460 of 100-32-32-8 67 / 87, 7350 in 50 subgraphs of 64-64-64-8 83 / 96; where only the last
+// of the layers is below it: 47 250 of 30-20-6 82 / 85, 21 000 in 50 subgraphs of 40-40-40-5 119 / 120, 2840 of 300-128-7 59 / 57.  Above it the
+// net decides: 63 000 of 16-16-4 (64.5 M) 68 / 96 and 31 500 of 32-32-32 62 / 79, but 21 000 in 50 subgraphs of 40-40-40-5 123 / 120 with
+// all its layers on the ALUs, and from 128 M on 8400 of 96-96-12 74 / 57.
 constexpr double kSimtFlops = 64e6;
 constexpr int kSimtTile = 32;
 

@@ -60,4 +60,13 @@ cudaError_t launch_tail(void (*kernel)(P...), dim3 grid, unsigned block, size_t 
     return launch_cluster(kernel, grid, block, smem, 1, true, s, std::forward<Args>(args)...);
 }
 
+// A kernel of one or two blocks for every SM, each with work for several microseconds, does not come up early: its blocks would go where
+// the kernel in front leaves room first, eight to sixteen on an SM, and the other SMs would have none (weight gradient of 20 x 6 over
+// 47 250 rows: 17 us, spread over all SMs 6).
+template <class... P, class... Args>
+cudaError_t launch_spread(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, Args&&... args) {
+    if (s == pdl_state().stream) pdl_state().direct = false;
+    return launch(kernel, grid, block, smem, s, std::forward<Args>(args)...);
+}
+
 }  // namespace gad

@@ -184,11 +184,11 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         for_tiles([&](int, int, int, bool new_b) {
             if (a.resident && new_b && !first && elect_one()) mma_commit2(bempty);   // every MMA on the previous B has been issued
             first = false;
-            if (!__all_sync(0xffffffffu, mbar_wait(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 3))) return false;
+            if (!__all_sync(0xffffffffu, mbar_wait<true>(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 3))) return false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t d = tmem_base + (uint32_t)(acc * a.BN);
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!__all_sync(0xffffffffu, mbar_wait(xfull(q), qphase, abort_flag, a.err, 4))) return false;
+                if (!__all_sync(0xffffffffu, mbar_wait<true>(xfull(q), qphase, abort_flag, a.err, 4))) return false;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t base = sm_addr + off_ring + (uint32_t)stage * stage_bytes;
                 const uint32_t bbase = a.resident ? sm_addr + (uint32_t)kb * nb * b_bytes : base + A_BYTES;
@@ -357,7 +357,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive_leader(tempty(acc));
+            if (lane == 0) mbar_arrive_leader_drained(tempty(acc));
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             return true;
         });

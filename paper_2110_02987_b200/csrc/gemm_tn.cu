@@ -64,6 +64,11 @@ __device__ __forceinline__ void arrive_any(uint32_t bar) {
     if constexpr (CG == 2) mbar_arrive_leader(bar);
     else mbar_arrive(bar);
 }
+template <int CG>
+__device__ __forceinline__ void arrive_drained(uint32_t bar) {
+    if constexpr (CG == 2) mbar_arrive_leader_drained(bar);
+    else mbar_arrive(bar);
+}
 
 // CG: CTAs that work together on a unit (1, or 2 = a cluster).
 template <int CG, bool split>
@@ -150,11 +155,11 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
         const uint32_t idesc = instr_desc(a.BN, CG * BM) | (1u << 15) | (1u << 16);   // A and B MN-major
         for_units([&](int, const RowSpan c, int, int) {
             const int nkb = (c.nrows + TBK - 1) / TBK;
-            if (!__all_sync(0xffffffffu, mbar_wait(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 12))) return false;
+            if (!__all_sync(0xffffffffu, mbar_wait<CG == 2>(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 12))) return false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t d = tmem_base + (uint32_t)acc * acc_cols;
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!__all_sync(0xffffffffu, mbar_wait(xfull(q), qphase, abort_flag, a.err, 13))) return false;
+                if (!__all_sync(0xffffffffu, mbar_wait<CG == 2>(xfull(q), qphase, abort_flag, a.err, 13))) return false;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t base = sm_addr + off_ring + (uint32_t)stage * stage_bytes, lo = sm_addr + (uint32_t)q * stage_bytes;
                 const uint64_t a_hi = smem_desc_mn(base), b_hi = smem_desc_mn(base + A_BLOCKS * BLOCK_BYTES);
@@ -247,7 +252,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) arrive_any<CG>(tempty(acc));
+            if (lane == 0) arrive_drained<CG>(tempty(acc));
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             return true;
         });

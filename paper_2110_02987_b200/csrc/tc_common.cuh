@@ -36,11 +36,26 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// The same at cluster scope, for a barrier that the other CTA of a pair arrives at.
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.b32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 // Bounded wait.  Returns false when the wait ran out or another role of this CTA has given up.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, int32_t* err, int code,
                                           uint32_t limit = WAIT_LIMIT) {
     for (uint32_t i = 0; i < limit; ++i) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) return true;
         if (*abort_flag) return false;
     }
     *abort_flag = 1u;
@@ -106,15 +121,30 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
 }
-// Arrives at the leader's barrier of this offset.  (Without a .release.cluster: that waits for every earlier store of the thread to
-// be visible, global ones included, and cost 1500 cycles an arrival.  What the leader reads after it are shared-memory writes
-// ordered by the proxy fence before the arrival, and tensor memory ordered by tcgen05.fence.)
+// Arrives at the leader's barrier of this offset, in the form every arrival has that names no scope: a release at the scope of the CTA.  For what
+// the leader's own threads wrote that is what the PTX memory model asks for.  For operands the other CTA wrote it is not: the model wants a release at
+// cluster scope, and nothing in it says that the MMA then reads them.  What is relied on is the hardware: the pair's MMA reads each CTA's operands in that CTA's
+// own shared memory, and the writer's fence.proxy.async has completed its writes there before the arrival is sent.  It is the usual form for
+// operands that a pair's second CTA transforms.  With .release.cluster an arrival takes 1500 cycles, whether or not the thread has stored anything else:
+// epochs took 5 to 23 % longer (163 -> 172, 200 -> 246, 907 -> 962, 1689 -> 1873 us), and with one thread of the other CTA passing the
+// arrivals on at cluster scope 7 to 17 %.
 __device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
     asm volatile(
         "{\n"
         ".reg .b32 r;\n"
         "mapa.shared::cluster.u32 r, %0, 0;\n"
         "mbarrier.arrive.shared::cluster.b64 _, [r];\n"
+        "}\n" ::"r"(bar)
+        : "memory");
+}
+// The same for an arrival that publishes no memory: this warp has read its tensor memory (tcgen05.wait::ld), and tcgen05.fence on either side of a
+// relaxed arrival at cluster scope orders that against the MMAs that overwrite it.
+__device__ __forceinline__ void mbar_arrive_leader_drained(uint32_t bar) {
+    asm volatile(
+        "{\n"
+        ".reg .b32 r;\n"
+        "mapa.shared::cluster.u32 r, %0, 0;\n"
+        "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [r];\n"
         "}\n" ::"r"(bar)
         : "memory");
 }

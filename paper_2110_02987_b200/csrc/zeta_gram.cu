@@ -247,12 +247,12 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
         const uint32_t idesc = instr_desc(width, 2 * GH);
         bool ok = true;
         for (long long t = t_begin; t < t_end && ok; ++t) {
-            if (!(ok = __all_sync(0xffffffffu, mbar_wait(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 22)))) break;
+            if (!(ok = __all_sync(0xffffffffu, mbar_wait<true>(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 22)))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t d = tmem_base + (uint32_t)(acc * GT);
             for (int kb = 0; kb < nkb; ++kb) {
                 if (!(ok = __all_sync(0xffffffffu, mbar_wait(full(stage), phase, abort_flag, a.err, 23) &&
-                                                       mbar_wait(pfull(stage), phase, abort_flag, a.err, 25)))) break;
+                                                       mbar_wait<true>(pfull(stage), phase, abort_flag, a.err, 25)))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t base = sm_addr + stage * G_STAGE_BYTES;
                 const uint64_t a_hi = smem_desc(base), a_lo = smem_desc(base + G_TILE_BYTES);
@@ -349,7 +349,7 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive_leader(tempty(acc));
+            if (lane == 0) mbar_arrive_leader_drained(tempty(acc));
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             sum += (double)(pi * part);
         }

@@ -36,6 +36,17 @@ cudaError_t configure_kernel_once(const void* kernel, int smem_bytes, bool max_c
     return cudaSuccess;
 }
 
+int max_active_pairs(const void* kernel, unsigned threads, size_t smem_bytes, int num_sms) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(num_sms & ~1)); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem_bytes; cfg.attrs = attr; cfg.numAttrs = 1;
+    int c = 0;
+    if (cudaOccupancyMaxActiveClusters(&c, kernel, &cfg) != cudaSuccess || c < 1) { cudaGetLastError(); c = num_sms / 2; }
+    return c;
+}
+
 }  // namespace gad
 
 // TMA descriptors kept per layer: forward A, B_hi, B_lo; input-gradient A, B_hi, B_lo; weight-gradient H, dZ.
@@ -77,7 +88,7 @@ struct Plan {
     std::vector<uint8_t> agg_first;   // [L] the layer aggregates before it transforms: sigma((A~ H^(l)) W + b)
     std::vector<size_t> o_P;          // [L] A~ H^(l)  [Np x ld_l] of those layers
     size_t o_epoch = 0;               // device epoch counter (indexes the dropout mask)
-    size_t o_counters = 0;            // arrival counters: [loss | K column sums | K zeta]
+    size_t o_counters = 0;            // arrival counters: [K column sums | K zeta]
     // layers l >= 1 of at most 16 output columns take the streaming FP32 kernel on the way back (flag bit 2 switches it off)
     std::vector<uint8_t> narrow;      // [L]
     std::vector<RowSpan> nchunks;     // their row chunks: about three CTAs per SM, never across subgraphs
@@ -255,7 +266,7 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
         p.o_w_hi[l] = take(cur, 4 * (size_t)K * y.fi * y.ldw); p.o_w_lo[l] = take(cur, 4 * (size_t)K * y.fi * y.ldw);
         p.o_wt_hi[l] = take(cur, 4 * (size_t)K * y.fo * y.ldi); p.o_wt_lo[l] = take(cur, 4 * (size_t)K * y.fo * y.ldi);
     }
-    p.o_counters = take(cur, 4 * (size_t)(1 + 2 * K));
+    p.o_counters = take(cur, 8 * (size_t)K);
     p.o_P.assign(p.L, 0);
     for (int l = 0; l < p.L; ++l)
         if (p.agg_first[l]) p.o_P[l] = take(cur, 4 * Np * (size_t)p.ld[l]);
@@ -327,7 +338,7 @@ struct gad_ctx {
     // stands for all of them and the others are stale.  `unsettled`: a consensus over differing copies has been enqueued and
     // nothing has waited for it since; should a bounded wait have run out it left them as they were (error word 2 tells).
     bool same_params = true, unsettled = false;
-    bool epoch_dirty = false;       // the device counter differs from `epoch` (gad_set_epoch, epochs without dropout)
+    bool epoch_dirty = false;       // the device counter differs from `epoch` (after gad_set_epoch)
     cudaStream_t capture_stream = nullptr;   // epochs are captured on it, whatever stream they are launched on
     cudaStream_t copy_stream = nullptr;   // host -> device copies of gad_set_inputs
     cudaStream_t side_stream = nullptr;   // small kernels of an epoch that depend on little (operand split, zeta, bias gradients)
@@ -560,7 +571,7 @@ int zeta_pass(gad_ctx* ctx, cudaStream_t s) {
         GAD_RUN("zeta", -1, 4.0 * p.Np * (p.dims[0] + 1), 3.0 * pairs * p.dims[0], [&] {
             return launch_zeta_pair(ctx->H(0), p.ld[0], p.dims[0], ctx->at<int32_t>(p.o_deg), ctx->at<int32_t>(p.o_sub_off),
                                     ctx->at<int64_t>(p.o_deg_sum), ctx->at<int64_t>(p.o_pair_ptr), p.pair_ptr[p.K], p.K, ctx->cfg.beta,
-                                    ctx->at<double>(p.o_pair_partial), ctx->at<unsigned>(p.o_counters) + 1 + p.K,
+                                    ctx->at<double>(p.o_pair_partial), ctx->at<unsigned>(p.o_counters) + p.K,
                                     ctx->at<double>(p.o_zeta), s);
         });
         return GAD_OK;
@@ -611,7 +622,7 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
             if (rc != GAD_OK) return rc;
             GAD_RUN("bias_grad", l, 4.0 * p.Np * y.fo, 1.0 * p.Np * y.fo, [&] {
                 return launch_colsum_chunks(G1, y.ldo, chunks, nc, ctx->at<float>(p.o_cs_partial), p.maxld, chunk_ptr,
-                                            ctx->at<unsigned>(p.o_counters) + 1, grads, p.pstride, y.b_int, ss);
+                                            ctx->at<unsigned>(p.o_counters), grads, p.pstride, y.b_int, ss);
             });
             if (ss != ctx->stream) GAD_CK(cudaEventRecord(ctx->ev_bias, ss));
         }
@@ -979,7 +990,7 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
     GAD_CK(cudaMemsetAsync(ctx->ws + p.o_loss, 0, 4 * (size_t)(p.K + 1), ctx->stream));
     GAD_CK(cudaMemsetAsync(ctx->ws + p.o_epoch, 0, 8, ctx->stream));
     GAD_CK(cudaMemsetAsync(ctx->ws + p.o_zeta, 0, 8 * (size_t)p.K, ctx->stream));   // empty subgraphs keep zeta = 0
-    GAD_CK(cudaMemsetAsync(ctx->ws + p.o_counters, 0, 4 * (size_t)(1 + 2 * p.K), ctx->stream));
+    GAD_CK(cudaMemsetAsync(ctx->ws + p.o_counters, 0, 8 * (size_t)p.K, ctx->stream));
     GAD_CK(cudaStreamSynchronize(ctx->stream));
     guard.ok = true;
     *out = ctx;

@@ -27,6 +27,9 @@ extern std::atomic<int64_t> g_kernel_launches;
 // memory and, with `max_carveout`, for the largest shared-memory share of the SM.  Safe from several host threads.
 cudaError_t configure_kernel_once(const void* kernel, int smem_bytes, bool max_carveout);
 
+// Clusters of two CTAs of a kernel that fit the GPU at once (a cluster stays inside a GPC).
+int max_active_pairs(const void* kernel, unsigned threads, size_t smem_bytes, int num_sms);
+
 // ---------------------------------------------------------------------------------------------
 // Host-side result of building the block-diagonal store (create-time, not on the timed path).
 // ---------------------------------------------------------------------------------------------

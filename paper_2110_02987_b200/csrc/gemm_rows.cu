@@ -288,16 +288,6 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             const int n0 = n * a.BN;
             if (masked && a.colsum && sp.k != cs_k) flush_colsum(sp.k);
             const int r0 = quarter * 32 + sub_r;                 // this lane's rows: r0 + 8 i
-            float2 hm[4][4];
-            auto fetch_mask = [&](int c0) {
-                const int nc = n0 + c0 + sub_c, ng = min(4, (min(a.BN - c0, a.ldc - n0 - c0) - sub_c + 7) >> 3);
-                const float* h = hmask + ((long long)sp.row0 + r0) * a.ldh + nc;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int g = 0; g < 4; ++g)
-                        hm[i][g] = r0 + 8 * i < sp.nrows && g < ng ? __ldg(reinterpret_cast<const float2*>(h + 8 * i * a.ldh + 8 * g)) : make_float2(0.f, 0.f);
-            };
             if (!__all_sync(0xffffffffu, mbar_wait(tfull(acc), acc_phase, abort_flag, a.err, 8))) return false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             for (int c0 = 32 * half; c0 < a.BN && n0 + c0 < a.ldc; c0 += 64) {
@@ -305,7 +295,15 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const int ng = min(4, (min(a.BN - c0, a.ldc - n0 - c0) - sub_c + 7) >> 3);   // groups it has columns in
                 const long long at0 = ((long long)sp.row0 + r0) * a.ldc + nc;
                 float2 bias[4];
-                if (masked) fetch_mask(c0);
+                float2 hm[4][4];
+                if (masked) {
+                    const float* h = hmask + ((long long)sp.row0 + r0) * a.ldh + nc;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int g = 0; g < 4; ++g)
+                            hm[i][g] = r0 + 8 * i < sp.nrows && g < ng ? __ldg(reinterpret_cast<const float2*>(h + 8 * i * a.ldh + 8 * g)) : make_float2(0.f, 0.f);
+                }
                 if (DRAIN == kAct || DRAIN == kActDrop)
 #pragma unroll
                     for (int g = 0; g < 4; ++g) bias[g] = g < ng ? load_bias2(act, sp.k, nc + 8 * g) : make_float2(0.f, 0.f);
@@ -399,19 +397,10 @@ void rows_layout(int BN, int Kd, int passes, RowsArgs& a) {
     }
 }
 
-// Clusters of two CTAs that fit the GPU at once (a cluster stays inside a GPC).
 int max_clusters(int num_sms) {
     static std::atomic<int> known{0};
-    int c = known.load();
-    if (c > 0) return c;
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)num_sms); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = SMEM_BYTES; cfg.attrs = attr; cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&c, gemm_rows_kernel<kPlain, true>, &cfg) != cudaSuccess || c < 1) { cudaGetLastError(); c = num_sms / 2; }
-    known.store(c);
-    return c;
+    if (known.load() <= 0) known.store(max_active_pairs(reinterpret_cast<const void*>(gemm_rows_kernel<kPlain, true>), THREADS, SMEM_BYTES, num_sms));
+    return known.load();
 }
 
 }  // namespace

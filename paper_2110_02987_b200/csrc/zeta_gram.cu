@@ -419,19 +419,10 @@ __global__ void __launch_bounds__(256) zeta_gram_finish_kernel(const double* __r
 }
 static_assert(2 * G_EPI_WARPS == 32, "a warp reads the slots of a cluster");
 
-// Clusters of two CTAs that fit the GPU at once (a cluster stays inside a GPC).
 int gram_clusters(int num_sms) {
     static std::atomic<int> known{0};
-    int c = known.load();
-    if (c > 0) return c;
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)(num_sms & ~1)); cfg.blockDim = dim3(G_THREADS); cfg.dynamicSmemBytes = G_SMEM_BYTES; cfg.attrs = attr; cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&c, zeta_gram_kernel, &cfg) != cudaSuccess || c < 1) { cudaGetLastError(); c = num_sms / 2; }
-    known.store(c);
-    return c;
+    if (known.load() <= 0) known.store(max_active_pairs(reinterpret_cast<const void*>(zeta_gram_kernel), G_THREADS, G_SMEM_BYTES, num_sms));
+    return known.load();
 }
 
 }  // namespace

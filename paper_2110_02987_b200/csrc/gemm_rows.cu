@@ -23,9 +23,9 @@
 //     sectors go to global memory straight from the registers;
 //   - the ring of loaded tiles is separate from the two lo tiles, so that most of the space holds loads in flight (short
 //     reductions are a chain of TMA latency, split and MMA).
-// Before this kernel (one CTA per tile, B streamed, drain through shared memory) and with it, 525 000 rows: 100 -> 256 281 -> 165 us,
-// 256 -> 256 325 -> 282 us (the three passes alone: 252 us at the TF32 rate), 256 -> 47 167 -> 130 us; 110 000 rows, 128 -> 128:
-// 43 -> 29 us; 2843 rows, 1433 -> 128: 40 -> 27 us.
+// Before this kernel (one CTA per tile, B streamed, drain through shared memory) and with it, event times inside an epoch under the power cap,
+// 525 000 rows: 100 -> 256 300 -> 187 us, 256 -> 256 346 -> 305 us (tensor pipe active 72 - 77 % of the time), 256 -> 47 181 -> 153 us; 110 000 rows,
+// 128 -> 128: 48 -> 33 us; 2843 rows, 1433 -> 128, on its own: 40 -> 27 us.
 // Roles of a CTA: warp 0 issues TMA loads, warps 2-9 split the A tile and tell the pair's leader, warp 1 of the leader
 // issues the MMAs, warps 10-17 drain.  Every mbarrier wait is bounded: on a time-out the CTA raises an error word, stops, meets its
 // peer at the cluster barrier, frees its tensor memory and returns.

@@ -5,14 +5,15 @@
 // and one MMA (K = 8) consumes 8 rows.  fp32 accuracy as in gemm_rows.cu; both operands are activations here, so both get a lo tile
 // in shared memory, and rows past the end of a chunk are zeroed there.
 //
-// What bounds it is shared-memory bandwidth, then HBM.  For 256 x 256 outputs a CTA on its own moves 288 KB per 32 rows (operand reads
+// What bounds it is the tensor pipe for 256 x 256 outputs, shared-memory bandwidth for narrower ones, then HBM.  For 256 x 256 outputs a CTA on its own moves 288 KB per 32 rows (operand reads
 // 144, TMA 48, split 96: 2300 cycles at 128 B) where the tensor pipe needs 1536.  With CTAs working in pairs (cta_group::2: each
 // has 128 of the H columns and half of the dZ columns) it is 192 KB, which is 1536 cycles too; layers of at most 128 input columns
 // have nothing to share and use one CTA.  The ring of loaded tiles is separate from the lo tiles, as in gemm_rows.cu, so that five or more
 // stages hold loads in flight instead of three; CTAs are persistent and have two accumulators, so that a work unit (a chunk of rows and an
 // output tile) drains while the next one is multiplied.
-// Before (one CTA per chunk and tile, three-stage ring, both orders of split and drain in sequence) and now, 525 000 rows: 256 x 256 438 ->
-// 267 us, 256 x 47 194 -> 132 us, 100 x 256 224 -> 225 us; 60 000 rows, 602 x 256: 180 -> 96 us.
+// Before (one CTA per chunk and tile, three-stage ring, both orders of split and drain in sequence) and now, event times inside an epoch
+// under the power cap, 525 000 rows: 256 x 256 470 -> 291 us (tensor pipe active 81 % of the time), 256 x 47 215 -> 147 us, 100 x 256 243 -> 224 us; 63 000
+// rows, 602 x 256: 196 -> 114 us.
 #include <cuda.h>
 
 #include <algorithm>

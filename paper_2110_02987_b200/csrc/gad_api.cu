@@ -1489,10 +1489,11 @@ int gad_release_pinned(void) {
 
 void gad_destroy(gad_ctx* ctx) {
     if (!ctx) return;
-    // Epochs that nobody has waited for still write their losses into this context's pinned block and use the caller's workspace: the one goes to the next
-    // context, the other wherever the caller wants it.
+    // Epochs that nobody has waited for still write their losses into this context's pinned block and use the caller's workspace: the one
+    // goes to the next context, the other wherever the caller wants it.  (A stream that is being captured has nothing of this to wait for.)
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(ctx->stream, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) cudaStreamSynchronize(ctx->stream);
+    if (cudaStreamIsCapturing(ctx->stream, &capturing) != cudaSuccess) cudaGetLastError();
+    else if (capturing == cudaStreamCaptureStatusNone) cudaStreamSynchronize(ctx->stream);
     for (auto& eg : ctx->graphs)
         if (eg.exec) cudaGraphExecDestroy(eg.exec);
     for (auto& e : ctx->prof)

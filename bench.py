@@ -244,8 +244,9 @@ def cpu_baseline(w, theta, budget_s=20.0):
 
 
 def consensus_point(K, D, steps, hbm_peak):
-    """Update + weighted consensus over K copies of one D x D layer: the kernel's time inside an epoch (SGD step and
-    consensus, 12 K P bytes) and inside gad_consensus (consensus alone, 8 K P bytes) by per-kernel CUDA events."""
+    """Update + weighted consensus over K replicas of one D x D layer, equal as they are from the first consensus on (one copy stands for all): the
+    kernel's time inside an epoch (SGD step and consensus: K gradient sets and the copy in, the copy out, 4 (K + 2) P bytes) and inside
+    gad_consensus (8 P bytes) by per-kernel CUDA events."""
     from gad_synth.graphs import sbm_graph
     from gad_synth.partition import contiguous_partition, one_hop_halo
     from gad_synth import glorot_params
@@ -285,8 +286,8 @@ def consensus_point(K, D, steps, hbm_peak):
     line = {"micro": "consensus", "K": K, "layer": "%d-%d" % (D, D), "P": P, "bytes_per_copy_set": 4 * K * P,
             "sgd_consensus_in_epoch": {"ms": ms_in, "bytes": e["bytes_per_launch"], "GBps": e["bytes_per_launch"] / ms_in / 1e6,
                                        "frac": e["bytes_per_launch"] / ms_in / 1e6 / hbm_peak},
-            "gad_consensus": {"ms": ms_alone, "bytes": 8.0 * K * P, "GBps": 8.0 * K * P / ms_alone / 1e6,
-                              "frac": 8.0 * K * P / ms_alone / 1e6 / hbm_peak},
+            "gad_consensus": {"ms": ms_alone, "bytes": c["bytes_per_launch"], "GBps": c["bytes_per_launch"] / ms_alone / 1e6,
+                              "frac": c["bytes_per_launch"] / ms_alone / 1e6 / hbm_peak},
             "zeta": {"ms": ms_zeta, "bytes": z["bytes_per_launch"], "GBps": z["bytes_per_launch"] / ms_zeta / 1e6},
             "peak": hbm_peak, "unit": "GB/s"}
     g.destroy()
@@ -676,7 +677,7 @@ def main():
         "kernel": top["name"], "bound": "hbm", "achieved": top["bytes_per_launch"] / (avg_ms * 1e-3) / 1e9,
         "peak": hbm_peak, "unit": "GB/s", "peak_source": peak_kind, "avg_launch_ms": avg_ms,
         "share_of_step": top["total_ms"] / total_prof if total_prof > 0 else None,
-        "traffic": NCU_TRAFFIC.get((args.workload, top["name"])),
+        "traffic": NCU_TRAFFIC.get((args.workload, top["name"])) if args.gemm_mode == 0 and args.flags == 0 else None,
     }
     roofline["frac"] = roofline["achieved"] / hbm_peak
     if top["name"].startswith("spmm"):

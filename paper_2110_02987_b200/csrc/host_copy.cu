@@ -137,12 +137,11 @@ void host_prefault(void* dst, size_t bytes) {
     if (bytes < kTouchBytes || !is_pageable(dst)) return;
     char* d = (char*)dst;
     const int64_t n = (int64_t)(bytes / kPage);
-    const int nt = copy_threads(bytes);
-#pragma omp parallel if (nt > 1)
+#pragma omp parallel if (copy_threads(bytes) > 1)
     {
-        const int team = std::min(nt, omp_get_num_threads()), t = omp_get_thread_num();
+        const int team = omp_get_num_threads(), t = omp_get_thread_num();
         // adding nothing is a write as far as the page is concerned, and leaves what is there: the copy may never come
-        for (int64_t i = n * t / team; t < team && i < n * (t + 1) / team; ++i) __atomic_fetch_add(d + (size_t)i * kPage, 0, __ATOMIC_RELAXED);
+        for (int64_t i = n * t / team; i < n * (t + 1) / team; ++i) __atomic_fetch_add(d + (size_t)i * kPage, 0, __ATOMIC_RELAXED);
     }
 }
 

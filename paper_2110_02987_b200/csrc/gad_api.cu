@@ -168,12 +168,15 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
     int64_t R = round_up(std::max<int64_t>(1, (p.Np + target - 1) / target), 32);
     R = std::min<int64_t>(R, 16384);
     // The importance statistics split their columns over CTAs as well: row chunks so that both together make about four CTAs per SM (each
-    // chunk's sums are read again when zeta is finished, and that kernel has one CTA per subgraph).
+    // chunk's sums are read again when zeta is finished, and that kernel has one CTA per subgraph), and no more than that where the subgraphs allow
+    // it: four is what an SM holds, and the CTAs left over would run by themselves (K = 64, 1 M rows of 256: 640 CTAs 255 us, 512 204; K = 50, 200 000 rows of 256: 600 70, 500 56).
     int32_t zcols = p.dims[0];
     if (cfg->zeta_mode == 2)
         for (int l = 0; l < p.L; ++l) zcols = std::max(zcols, p.dims[l]);
     const int64_t ztarget = std::max<int64_t>(K, target / ((zcols + 127) / 128));
-    const int64_t Rz = std::max<int64_t>(32, round_up((p.Np + ztarget - 1) / ztarget, 32));
+    int64_t Rz = std::max<int64_t>(32, round_up((p.Np + ztarget - 1) / ztarget, 32));
+    auto zcount = [&](int64_t R) { int64_t c = 0; for (int32_t k = 0; k < K; ++k) c += (sub_off[k + 1] - sub_off[k] + R - 1) / R; return c; };
+    for (const int64_t first = Rz; zcount(Rz) > ztarget && Rz < 2 * first;) Rz += std::max<int64_t>(32, round_up(first / 32, 32));
     p.zchunk_ptr.assign(K + 1, 0);
     for (int32_t k = 0; k < K; ++k) {
         for (int64_t r = sub_off[k]; r < sub_off[k + 1]; r += Rz)

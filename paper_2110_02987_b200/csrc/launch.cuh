@@ -27,11 +27,20 @@ template <class P> __device__ __forceinline__ void after_wait(P& p) {
 struct PdlState { cudaStream_t stream = nullptr; bool on = false, direct = false, tails = false; };   // tails: those of launch_tail only
 PdlState& pdl_state();   // of this thread
 
+// How much shared memory an SM sets aside while it runs a kernel (the rest of its 256 KB is L1) is changed only when the SM is empty, and a
+// kernel that does not ask runs with what the SM has been cut for.  Where blocks of a small kernel beside the aggregation had come up on
+// SMs still cut for a transform (227 KB), the whole aggregation behind them ran with the L1 that leaves, which holds fewer operand rows
+// in flight than its warps ask for (8 x 7800 rows of 265 entries, 256 wide: 807 us beside the importance statistics, 609 on its own, now 633).
+// So these kernels ask: the aggregation for what its blocks need (16 of 2 KB), the importance statistics for four blocks of 17 KB.
+// Not where the kernels of the main sequence overlap: each change then waits for an SM that the overlap keeps busy (2708 rows: 163 -> 166 us an epoch).
+constexpr unsigned kGatherSharedKB = 32, kZetaSharedKB = 100;
+
 template <class... P, class... Args>
-cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, unsigned cluster, bool tail, cudaStream_t s, Args&&... args) {
+cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, unsigned cluster, bool tail, unsigned shared_kb, cudaStream_t s,
+                           Args&&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     cfg.attrs = attr;
     if (cluster > 1) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
@@ -47,17 +56,27 @@ cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, unsigned block, size
         }
         st.direct = true;
     }
+    if (shared_kb && !st.on) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[cfg.numAttrs].val.sharedMemCarveout = 100 * shared_kb / 228;   // percent; rounded up to a size there is
+        ++cfg.numAttrs;
+    }
     return cudaLaunchKernelEx(&cfg, kernel, P(std::forward<Args>(args))...);
 }
 template <class... P, class... Args>
 cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, Args&&... args) {
-    return launch_cluster(kernel, grid, block, smem, 1, false, s, std::forward<Args>(args)...);
+    return launch_cluster(kernel, grid, block, smem, 1, false, 0, s, std::forward<Args>(args)...);
+}
+// The same for a kernel that asks for a share of the SM's memory (kGatherSharedKB, kZetaSharedKB).
+template <class... P, class... Args>
+cudaError_t launch_share(void (*kernel)(P...), dim3 grid, unsigned block, unsigned shared_kb, cudaStream_t s, Args&&... args) {
+    return launch_cluster(kernel, grid, block, 0, 1, false, shared_kb, s, std::forward<Args>(args)...);
 }
 // A small kernel that only finishes what the one in front has left (rows cut into parts, sums of chunks): its blocks find room beside the
 // last ones in front on a store of any size (89 250 rows in 50 subgraphs: 912 -> 903 us an epoch; 70 000 of 60-60-60-5: 362 -> 356).
 template <class... P, class... Args>
 cudaError_t launch_tail(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, Args&&... args) {
-    return launch_cluster(kernel, grid, block, smem, 1, true, s, std::forward<Args>(args)...);
+    return launch_cluster(kernel, grid, block, smem, 1, true, 0, s, std::forward<Args>(args)...);
 }
 
 // A kernel of one or two blocks for every SM, each with work for several microseconds, does not come up early: its blocks would go where

@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(256) colsum_finish_kernel(const float* __restr
     }
 }
 cudaError_t launch_colsum_finish(const float* colsum, int ld, const int2* clusters, int K, float* out, int64_t ostride, int64_t off, cudaStream_t s) {
-    colsum_finish_kernel<<<(unsigned)K, 256, 0, s>>>(colsum, ld, clusters, out, ostride, off);
+    launch_share(colsum_finish_kernel, dim3((unsigned)K), 256, kGatherSharedKB, s, colsum, ld, clusters, out, ostride, off);
     ++g_kernel_launches;
     return cudaGetLastError();
 }
@@ -549,8 +549,8 @@ cudaError_t launch_zeta(const float* X, int ld, int F, const int32_t* deg, const
                         const int32_t* chunk_ptr, const int32_t* sub_off, int K, const int64_t* deg_sum, const int64_t* deg_sq,
                         float beta, double* partial, double* zeta, double* q_acc, int phase, cudaStream_t s) {
     if (nchunks > 0) {
-        zeta_partial_kernel<<<dim3((unsigned)nchunks, (unsigned)((ld / 4 + 31) / 32)), 256, 0, s>>>(X, ld, deg, chunks, sub_off, deg_sum, partial);
-        zeta_finish_kernel<<<(unsigned)K, 1024, 0, s>>>(partial, F, ld, chunk_ptr, sub_off, deg_sum, deg_sq, beta, zeta, q_acc, phase);
+        launch_share(zeta_partial_kernel, dim3((unsigned)nchunks, (unsigned)((ld / 4 + 31) / 32)), 256, kZetaSharedKB, s, X, ld, deg, chunks, sub_off, deg_sum, partial);
+        launch_share(zeta_finish_kernel, dim3((unsigned)K), 1024, kZetaSharedKB, s, partial, F, ld, chunk_ptr, sub_off, deg_sum, deg_sq, beta, zeta, q_acc, phase);
         g_kernel_launches += 2;
     }
     return cudaGetLastError();

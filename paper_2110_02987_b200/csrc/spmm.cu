@@ -344,13 +344,13 @@ static cudaError_t launch_rows(const SparseDev& A, const float* Z, int ldz, floa
                 // a bfloat16 operand of a whole number of 8-column runs: 16-byte loads, eight columns per lane and load
                 if (F4 % 2 == 0 && ldz % 8 == 0) {
                     paired = true;
-                    if (off32) launch(spmm_items_kernel<NV, EPI, true, true, true>, dim3(grid), 32 * kItemWarps, 0, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
-                    else launch(spmm_items_kernel<NV, EPI, false, true, true>, dim3(grid), 32 * kItemWarps, 0, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+                    if (off32) launch_share(spmm_items_kernel<NV, EPI, true, true, true>, dim3(grid), 32 * kItemWarps, kGatherSharedKB, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+                    else launch_share(spmm_items_kernel<NV, EPI, false, true, true>, dim3(grid), 32 * kItemWarps, kGatherSharedKB, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
                 }
             }
             if (!paired) {
-                if (off32) launch(spmm_items_kernel<NV, EPI, true, BF, false>, dim3(grid), 32 * kItemWarps, 0, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
-                else launch(spmm_items_kernel<NV, EPI, false, BF, false>, dim3(grid), 32 * kItemWarps, 0, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+                if (off32) launch_share(spmm_items_kernel<NV, EPI, true, BF, false>, dim3(grid), 32 * kItemWarps, kGatherSharedKB, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+                else launch_share(spmm_items_kernel<NV, EPI, false, BF, false>, dim3(grid), 32 * kItemWarps, kGatherSharedKB, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
             }
             ++g_kernel_launches;
         }
@@ -362,7 +362,7 @@ static cudaError_t launch_rows(const SparseDev& A, const float* Z, int ldz, floa
     }
     if (A.nitems > 0) {
         const unsigned grid = (unsigned)(((long long)A.nitems * GROUP + 255) / 256);
-        launch(spmm_items_narrow_kernel<GROUP, EPI, BF>, dim3(grid), 256, 0, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+        launch_share(spmm_items_narrow_kernel<GROUP, EPI, BF>, dim3(grid), 256, kGatherSharedKB, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
         ++g_kernel_launches;
     }
     if (A.nfin > 0) {

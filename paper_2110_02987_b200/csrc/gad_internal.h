@@ -82,7 +82,7 @@ struct SparseDev {
     const int64_t* rowptr = nullptr;  // [Np+1] (kept for the accessors; the kernels read the work list)
     const uint2* ecv = nullptr;       // [nnz] packed (column, value bits)
     const int4* fin = nullptr;        // rows made of several parts
-    const int4* items = nullptr;      // parts and uncut rows together, longest first
+    const int4* items = nullptr;      // parts and uncut rows together, longest first inside a run of rows
     float* scratch = nullptr;         // [slots x leading dimension of the output] partial rows
     int32_t nfin = 0, nitems = 0;
     int64_t nrows = 0;                // rows (and columns) of the store

@@ -3,7 +3,7 @@
 // the transposed store it is the backward aggregation dZ = A~^T dPre.
 //
 // Work list: every row, or every part of a row too long for one item, is an item {row, position of its first
-// entry, entries, scratch slot}; items are grouped by subgraph and sorted longest first inside one.  Operands wider
+// entry, entries, scratch slot}; items are grouped by subgraph and, inside one, by runs of rows, longest first in each.  Operands wider
 // than 64 columns take a warp per item, narrower ones a group of 4, 8 or 16 lanes per item; every lane owns 16
 // bytes of each operand row it gathers.  The parts of a cut row go to scratch slots and a second kernel adds them
 // in part order, so results never depend on scheduling.

@@ -81,7 +81,12 @@ __device__ __forceinline__ void tile_of(const RowsArgs& a, int t, int& pair, int
     else { pair = t / a.ntn; n = t % a.ntn; }
 }
 
-template <int DRAIN, bool split>
+// How A reaches the tensor cores: as loaded (one pass); its lo part beside it in shared memory; or both parts through tensor memory.
+enum Form { kOnePass, kSharedLo, kTensorMem };
+constexpr int SLOTS = 4, SLOT_COLS = 2 * BK;   // tensor-memory slots of a 128 x 32 step of A: 32 columns of hi, 32 of lo
+constexpr uint32_t TMEM_COLS = 512;
+
+template <int DRAIN, int FORM>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBlo,
                  const RowsArgs a) {
@@ -93,9 +98,10 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const uint32_t rank = cluster_rank();
     const int nkb = (a.Kd + BK - 1) / BK;
     const uint32_t b_bytes = (uint32_t)(a.BN / 2) * (BK * 4);              // this CTA's half of a B tile
+    constexpr bool split = FORM != kOnePass;
     constexpr uint32_t nb = split ? 2u : 1u;
     const uint32_t off_lo = a.resident ? (uint32_t)nkb * b_bytes * nb : 0u;
-    const uint32_t off_ring = off_lo + (split ? (uint32_t)a.nlo * A_BYTES : 0u);
+    const uint32_t off_ring = off_lo + (FORM == kSharedLo ? (uint32_t)a.nlo * A_BYTES : 0u);
     const uint32_t stage_bytes = (uint32_t)A_BYTES + (a.resident ? 0u : nb * b_bytes);
     const int nst = a.nst;
     const uint32_t bars = sm_addr + DATA_BYTES;
@@ -108,13 +114,15 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const uint32_t bfull = bars + 8u * (2 * MAX_STAGES + 2 * MAX_LO + 4), bempty = bfull + 8u;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + DATA_BYTES + 8 * (2 * MAX_STAGES + 2 * MAX_LO + 6));
     volatile uint32_t* abort_flag = tmem_slot + 1;
-    const uint32_t tmem_cols = a.BN < 16 ? 32u : 2u * (uint32_t)a.BN;
+    const uint32_t tmem_cols = FORM == kTensorMem ? TMEM_COLS : 2u * (uint32_t)a.BN;
+    // groups of splitting warps that take steps in turn (kTensorMem: a group has a warp for every quarter of the lanes)
+    const int groups = FORM == kTensorMem ? SPLIT_WARPS / 4 : a.nlo == MAX_LO ? MAX_LO : 1;
 
     pdl_next();
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (uniform, and known to be)
     if (threadIdx.x == 0) {
-        for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
-        for (int q = 0; q < MAX_LO; ++q) { mbar_init(xfull(q), 2 * SPLIT_WARPS / (a.nlo == MAX_LO ? MAX_LO : 1)); mbar_init(loempty(q), 1); }
+        for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), FORM == kTensorMem && a.resident ? SPLIT_WARPS / groups : 1); }
+        for (int q = 0; q < MAX_LO; ++q) { mbar_init(xfull(q), 2 * SPLIT_WARPS / groups); mbar_init(loempty(q), 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(tfull(i), 1); mbar_init(tempty(i), 2 * EPI_WARPS); }
         mbar_init(bfull, 1); mbar_init(bempty, 1);
         *abort_flag = 0u;
@@ -193,6 +201,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const uint32_t base = sm_addr + off_ring + (uint32_t)stage * stage_bytes;
                 const uint32_t bbase = a.resident ? sm_addr + (uint32_t)kb * nb * b_bytes : base + A_BYTES;
                 const uint64_t a_hi = smem_desc(base), a_lo = smem_desc(sm_addr + off_lo + (uint32_t)q * A_BYTES);
+                const uint32_t a_tm = tmem_base + TMEM_COLS - SLOTS * SLOT_COLS + (uint32_t)(q * SLOT_COLS);
                 const uint64_t b_hi = smem_desc(bbase), b_lo = smem_desc(bbase + b_bytes);
                 const int nks = min(BK / 8, (a.Kd - kb * BK + 7) / 8);
                 if (elect_one()) {
@@ -200,6 +209,12 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
                     for (int ks = 0; ks < BK / 8; ++ks) {
                         if (ks < nks) {
+                            if constexpr (FORM == kTensorMem) {
+                                mma_tf32_pair_ts(d, a_tm + 8 * ks, b_hi + 2 * ks, idesc, (kb | ks) != 0 ? 1u : 0u);
+                                mma_tf32_pair_ts(d, a_tm + 8 * ks, b_lo + 2 * ks, idesc, 1u);
+                                mma_tf32_pair_ts(d, a_tm + BK + 8 * ks, b_hi + 2 * ks, idesc, 1u);
+                                continue;
+                            }
                             mma_tf32_pair(d, a_hi + 2 * ks, b_hi + 2 * ks, idesc, (kb | ks) != 0 ? 1u : 0u);
                             if (split) {
                                 mma_tf32_pair(d, a_hi + 2 * ks, b_lo + 2 * ks, idesc, 1u);
@@ -207,8 +222,9 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             }
                         }
                     }
-                    mma_commit2(empty(stage));     // the stage may be refilled, and the lo tile rewritten, in both CTAs once these MMAs
-                    mma_commit2(loempty(q));       // have read them
+                    // the stage may be refilled, and the lo tile rewritten, in both CTAs once these MMAs have read them
+                    if (FORM != kTensorMem || !a.resident) mma_commit2(empty(stage));
+                    mma_commit2(loempty(q));
                     if (kb == nkb - 1) mma_commit2(tfull(acc));   // accumulator complete, in both CTAs
                 }
                 __syncwarp();
@@ -224,7 +240,8 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // that take turns: what a step costs is then mostly waiting - for the barriers, the proxy fence and the arrival - so four
         // steps are in hand at a time.  (A group's wait for a ring stage is unambiguous because nlo <= nst: once its own previous
         // step has been multiplied, so has the step before in that stage.)
-        const int groups = a.nlo == MAX_LO ? MAX_LO : 1, gw = SPLIT_WARPS / groups, group = (warp - 2) / gw, tt = threadIdx.x - 64 - 32 * gw * group;
+        const int gw = SPLIT_WARPS / groups, group = (warp - 2) / gw, tt = threadIdx.x - 64 - 32 * gw * group;
+        const int row = 32 * (warp & 3) + lane;       // kTensorMem: this thread's row of the tile, in its warp's quarter of the lanes
         int stage = 0, q = 0;
         uint32_t phase = 0, qphase = 0, bphase = 0;
         for_tiles([&](int, int, int, bool new_b) {
@@ -234,9 +251,32 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 bphase ^= 1u;
             }
             for (int kb = 0; kb < nkb; ++kb) {
-                if (groups == 1 || q == group) {
+                if (groups == 1 || (q & (groups - 1)) == group) {
                     if (!__all_sync(0xffffffffu, mbar_wait(loempty(q), qphase ^ 1u, abort_flag, a.err, 6))) return false;
                     if (!__all_sync(0xffffffffu, mbar_wait(full(stage), phase, abort_flag, a.err, 7))) return false;
+                    if constexpr (FORM == kTensorMem) {
+                        // (the 16-byte pieces of a row are swizzled by the row; eight neighbouring lanes cover all banks)
+                        const uint8_t* src = sm + off_ring + (uint32_t)stage * stage_bytes + row * (4 * BK);
+                        float hi[BK], lo[BK];
+#pragma unroll
+                        for (int j = 0; j < BK / 4; ++j) {
+                            const float4 v = *reinterpret_cast<const float4*>(src + ((j ^ (row & 7)) << 4));
+                            hi[4 * j] = v.x; hi[4 * j + 1] = v.y; hi[4 * j + 2] = v.z; hi[4 * j + 3] = v.w;
+                        }
+#pragma unroll
+                        for (int i = 0; i < BK; ++i) lo[i] = tf32_rest(hi[i]);
+                        const uint32_t dst = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + TMEM_COLS - SLOTS * SLOT_COLS + (uint32_t)(q * SLOT_COLS);
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");   // the MMAs that read the slot have completed
+                        tmem_st_32x32b_x32(dst, hi);
+                        tmem_st_32x32b_x32(dst + BK, lo);
+                        tmem_wait_st();
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) {
+                            if (a.resident) mbar_arrive(empty(stage));   // nobody else reads the stage
+                            mbar_arrive_leader_tmem(xfull(q));
+                        }
+                    } else {
                     if (split) {
                         const float4* hi = reinterpret_cast<const float4*>(sm + off_ring + (uint32_t)stage * stage_bytes);
                         float4* lo = reinterpret_cast<float4*>(sm + off_lo + (uint32_t)q * A_BYTES);
@@ -249,6 +289,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tensor-core reads
                     __syncwarp();
                     if (lane == 0) mbar_arrive_leader(xfull(q));
+                    }
                 }
                 if (++q == a.nlo) { q = 0; qphase ^= 1u; }
                 if (++stage == nst) { stage = 0; phase ^= 1u; }
@@ -309,8 +350,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     for (int g = 0; g < 4; ++g) bias[g] = g < ng ? load_bias2(act, sp.k, nc + 8 * g) : make_float2(0.f, 0.f);
                 float2 v[4][4];                                  // [row r0 + 8 i][columns nc + 8 g]
                 const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * a.BN + c0);
-                if (a.BN >= 32) tmem_ld_16x256b_x4(t0, v);
-                else tmem_ld_16x256b_x2(t0, v);
+                tmem_ld_16x256b_x4(t0, v);
                 if (masked) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
@@ -355,7 +395,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive_leader_drained(tempty(acc));
+            if (lane == 0) mbar_arrive_leader_tmem(tempty(acc));
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             return true;
         });
@@ -382,11 +422,23 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
 namespace {
 
+// Which form a launch takes.  Through tensor memory A costs shared memory one write and one read where a lo tile beside it costs six times its
+// size (written and read by the split, read by three MMAs); with 256 columns a tile's two accumulators fill the tensor memory.
+int form_for(int BN, int passes) { return passes <= 1 ? kOnePass : BN <= 128 ? kTensorMem : kSharedLo; }
+
 // Where the data of a CTA goes: four lo tiles if at least as many ring stages fit beside them, else two; B resident if at least
 // three ring stages fit beside it.
-void rows_layout(int BN, int Kd, int passes, RowsArgs& a) {
+void rows_layout(int BN, int Kd, int form, RowsArgs& a) {
+    const int passes = form == kOnePass ? 1 : 3;
     const int nkb = (Kd + BK - 1) / BK, nb = passes > 1 ? 2 : 1;
     const int b_bytes = BN / 2 * (BK * 4);
+    if (form == kTensorMem) {   // as many stages as there are slots, at least (see the split)
+        const long long room_a = (long long)DATA_BYTES - (long long)nkb * nb * b_bytes;
+        a.nlo = SLOTS;
+        a.resident = room_a >= SLOTS * A_BYTES ? 1 : 0;
+        a.nst = (int)std::min<long long>(MAX_STAGES, a.resident ? room_a / A_BYTES : DATA_BYTES / (A_BYTES + nb * b_bytes));
+        return;
+    }
     for (a.nlo = 4;; a.nlo = 2) {
         const long long room = (long long)DATA_BYTES - (passes > 1 ? a.nlo * A_BYTES : 0), room_a = room - (long long)nkb * nb * b_bytes;
         a.resident = room_a >= (a.nlo > 3 ? a.nlo : 3) * A_BYTES ? 1 : 0;
@@ -399,7 +451,7 @@ void rows_layout(int BN, int Kd, int passes, RowsArgs& a) {
 
 int max_clusters(int num_sms) {
     static std::atomic<int> known{0};
-    if (known.load() <= 0) known.store(max_active_pairs(reinterpret_cast<const void*>(gemm_rows_kernel<kPlain, true>), THREADS, SMEM_BYTES, num_sms));
+    if (known.load() <= 0) known.store(max_active_pairs(reinterpret_cast<const void*>(gemm_rows_kernel<kPlain, kSharedLo>), THREADS, SMEM_BYTES, num_sms));
     return known.load();
 }
 
@@ -410,7 +462,7 @@ int max_clusters(int num_sms) {
 // idle: then the columns are spread over more CTAs, down to 32 (2843 rows x 1433 -> 128: 24 row tiles, 40 us with 128 columns per
 // tile, 27 us with 32).
 int tc_rows_bn(int n_cols, int npairs) {
-    int bn = n_cols <= 16 ? 16 : n_cols <= 32 ? 32 : n_cols <= 64 ? 64 : n_cols <= 128 ? 128 : 256;
+    int bn = n_cols <= 32 ? 32 : n_cols <= 64 ? 64 : n_cols <= 128 ? 128 : 256;
     while (bn > 32 && (long long)npairs * ((n_cols + bn - 1) / bn) * 2 <= 74) bn /= 2;
     return bn;
 }
@@ -427,7 +479,8 @@ cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* 
     if (colsum && !(mode == 1 && Hmask && tc_rows_sums_columns(n_cols, npairs))) return cudaErrorInvalidValue;
     RowsArgs a;
     a.tiles = pair_tiles; a.npairs = npairs; a.BN = tc_rows_bn(n_cols, npairs); a.ntn = (ldc + a.BN - 1) / a.BN; a.Kd = Kd;
-    rows_layout(a.BN, Kd, passes, a);
+    const int form = form_for(a.BN, passes);
+    rows_layout(a.BN, Kd, form, a);
     a.C = C; a.Cbf = reinterpret_cast<uint32_t*>(Cbf16); a.ldc = ldc; a.Hmask = Hmask; a.ldh = ldh; a.scale = scale; a.colsum = colsum;
     a.kmul = one_b ? 0 : 1; a.err = err;
     a.act = act ? *act : ActEpi{};
@@ -441,14 +494,14 @@ cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* 
         ++g_kernel_launches;
         return e;
     };
-#define GAD_DRAIN(D) case D: return passes > 1 ? go(gemm_rows_kernel<D, true>) : go(gemm_rows_kernel<D, false>)
+#define GAD_DRAIN(D) case D: return form == kTensorMem ? go(gemm_rows_kernel<D, kTensorMem>) : form == kSharedLo ? go(gemm_rows_kernel<D, kSharedLo>) : go(gemm_rows_kernel<D, kOnePass>)
     switch (drain) {
         GAD_DRAIN(kPlain);
-        GAD_DRAIN(kBf16);
         GAD_DRAIN(kMask);
-        GAD_DRAIN(kMaskBf16);
         GAD_DRAIN(kAct);
         GAD_DRAIN(kActDrop);
+        case kBf16: if (form == kOnePass) return go(gemm_rows_kernel<kBf16, kOnePass>); break;   // the reduced-precision mode's
+        case kMaskBf16: if (form == kOnePass) return go(gemm_rows_kernel<kMaskBf16, kOnePass>); break;
     }
 #undef GAD_DRAIN
     return cudaErrorInvalidValue;

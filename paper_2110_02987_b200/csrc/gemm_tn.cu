@@ -67,7 +67,7 @@ __device__ __forceinline__ void arrive_any(uint32_t bar) {
 }
 template <int CG>
 __device__ __forceinline__ void arrive_drained(uint32_t bar) {
-    if constexpr (CG == 2) mbar_arrive_leader_drained(bar);
+    if constexpr (CG == 2) mbar_arrive_leader_tmem(bar);
     else mbar_arrive(bar);
 }
 

@@ -137,9 +137,9 @@ __device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
         "}\n" ::"r"(bar)
         : "memory");
 }
-// The same for an arrival that publishes no memory: this warp has read its tensor memory (tcgen05.wait::ld), and tcgen05.fence on either side of a
-// relaxed arrival at cluster scope orders that against the MMAs that overwrite it.
-__device__ __forceinline__ void mbar_arrive_leader_drained(uint32_t bar) {
+// The same for an arrival that publishes no memory: this warp has read or written its tensor memory (tcgen05.wait::ld, ::st), and tcgen05.fence on
+// either side of a relaxed arrival at cluster scope orders that against the MMAs that overwrite or read it.
+__device__ __forceinline__ void mbar_arrive_leader_tmem(uint32_t bar) {
     asm volatile(
         "{\n"
         ".reg .b32 r;\n"
@@ -165,6 +165,28 @@ __device__ __forceinline__ void mma_tf32_pair(uint32_t tmem_d, uint64_t adesc, u
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// The same with A in tensor memory: row i of each CTA's 128 rows in lane i, a value of the reduction per column.
+__device__ __forceinline__ void mma_tf32_pair_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "setp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::2.kind::tf32 [%0], [%1], %2, %3, p;\n"
+        "}\n" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// One value per lane into each of 32 columns of this warp's 32 tensor-memory lanes.
+__device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t addr, const float (&v)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, "
+        "%22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(addr),
+        "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]),
+        "f"(v[13]), "f"(v[14]), "f"(v[15]), "f"(v[16]), "f"(v[17]), "f"(v[18]), "f"(v[19]), "f"(v[20]), "f"(v[21]), "f"(v[22]), "f"(v[23]), "f"(v[24]),
+        "f"(v[25]), "f"(v[26]), "f"(v[27]), "f"(v[28]), "f"(v[29]), "f"(v[30]), "f"(v[31])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // One arrival at the barrier of this offset in both CTAs once the MMAs issued so far have completed.
 __device__ __forceinline__ void mma_commit2(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((uint16_t)3)

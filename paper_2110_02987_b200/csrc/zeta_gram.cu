@@ -349,7 +349,7 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive_leader_drained(tempty(acc));
+            if (lane == 0) mbar_arrive_leader_tmem(tempty(acc));
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             sum += (double)(pi * part);
         }

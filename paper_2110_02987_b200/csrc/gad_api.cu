@@ -86,6 +86,7 @@ struct Plan {
     size_t o_gram_ptr = 0, o_gram_partial = 0, o_norm2 = 0, o_xhi = 0, o_xlo = 0;
     bool pair_alu_ok = false;         // every subgraph is small enough for the FP32-ALU pairwise kernel
     std::vector<uint8_t> agg_first;   // [L] the layer aggregates before it transforms: sigma((A~ H^(l)) W + b)
+    std::vector<size_t> o_bits;       // [L] which values of H^(l) are above zero, a bit each, for the layers whose way back masks with them; else 0
     std::vector<size_t> o_P;          // [L] A~ H^(l)  [Np x ld_l] of those layers
     size_t o_epoch = 0;               // device epoch counter (indexes the dropout mask)
     size_t o_counters = 0;            // arrival counters: [K column sums | K zeta]
@@ -274,10 +275,13 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
     for (int l = 0; l < p.L; ++l)
         if (p.agg_first[l]) p.o_P[l] = take(cur, 4 * Np * (size_t)p.ld[l]);
     p.narrow.assign(p.L, 0);
+    p.o_bits.assign(p.L, 0);
     int64_t narrow_partial = 0;
     for (int l = 0; l < p.L; ++l) {
         const Layer& y = p.layers[l];
         p.narrow[l] = (cfg->flags & 5) == 0 && l > 0 && !p.agg_first[l] && narrow_supported(y.ldi, y.ldo);
+        // the forward transform of such a layer leaves them, the one back through it masks with them
+        if (l > 0 && (cfg->flags & 1) == 0 && !p.simt[l] && !p.agg_first[l] && !p.narrow[l]) p.o_bits[l] = take(cur, 4 * Np * (size_t)bit_words_of(y.ldi));
         if (p.narrow[l]) narrow_partial = std::max(narrow_partial, (int64_t)y.fi * y.ldw + y.ldi);
     }
     if (narrow_partial > 0) {
@@ -361,6 +365,7 @@ struct gad_ctx {
     std::vector<TMap> maps;         // per layer: forward A, B_hi, B_lo; input-gradient A, B_hi, B_lo
 
     template <class T> T* at(size_t off) const { return reinterpret_cast<T*>(ws + off); }
+    uint32_t* bits(int l) const { return use_tc && p.o_bits[(size_t)l] ? at<uint32_t>(p.o_bits[(size_t)l]) : nullptr; }
     float* H(int l) const { return at<float>(p.o_H[l]); }
 };
 
@@ -539,7 +544,7 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t fork = nullptr) {
         GAD_RUN("gemm_fwd", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
             if (on_tc(ctx, l))
                 return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 0, passes, y.fi, y.fo, Z,
-                                           y.ldo, ctx->at<RowSpan>(p.o_pair_tiles), (int)(p.pair_tiles.size() / 2), nullptr, 0, 1.f, nullptr,
+                                           y.ldo, ctx->at<RowSpan>(p.o_pair_tiles), (int)(p.pair_tiles.size() / 2), train ? ctx->bits(l) : nullptr, bit_words_of(y.ldi), 1.f, nullptr,
                                            ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params, zb);
             return launch_gemm_rows_simt(0, ctx->H(l), y.ldi, y.fi, params, pstride, y.w_int, y.ldw, y.fo, Z, y.ldo,
                                          ctx->at<RowSpan>(p.o_tiles), (int)p.tiles.size(), nullptr, 0, 1.f, nullptr, ctx->stream);
@@ -696,7 +701,7 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
                 if (on_tc(ctx, l))
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 3], &ctx->maps[kMapsPerLayer * l + 4], &ctx->maps[kMapsPerLayer * l + 5], 1,
                                                ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G1, y.ldi, ctx->at<RowSpan>(p.o_pair_tiles),
-                                               (int)(p.pair_tiles.size() / 2), ctx->H(l), y.ldi, scale, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
+                                               (int)(p.pair_tiles.size() / 2), ctx->bits(l), bit_words_of(y.ldi), scale, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
                                                ctx->num_sms, ctx->stream, ctx->same_params, out_bf16 ? bf16_of(ctx) : nullptr,
                                                sums ? ctx->at<float>(p.o_colsum) : nullptr);
                 return launch_gemm_rows_simt(1, G2, y.ldo, y.fo, params, pstride, y.w_int, y.ldw, y.fi, G1, y.ldi,

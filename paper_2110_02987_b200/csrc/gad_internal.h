@@ -174,13 +174,15 @@ struct SplitLayers {
 };
 cudaError_t launch_split_weights(const float* params, int64_t pstride, int K, const SplitLayer* layers, int L, cudaStream_t s);
 // pair_tiles: 2 npairs row tiles (at most 128 rows, or none), the two of a pair in the same subgraph; tc_rows_bn(n_cols, npairs) columns
-// per tile, half of them the rows of B's descriptor box.  one_b: the operand copies of replica 0 serve every subgraph.
+// per tile, half of them the rows of B's descriptor box.  bits: with mode 0 (may be null) the transform leaves there which values of A are above
+// zero, bit c % 32 of word c / 32 of a row of bit_words words; mode 1 masks with such bits (null: no mask), 1/32 of the bytes of the activations.  one_b: the operand copies of replica 0 serve every subgraph.
 // Cbf16 (mode 0, or 1 with a mask; may be null): the result goes there as bfloat16 [rows x ldc] INSTEAD of to C - the operand copy the
 // reduced-precision aggregation gathers, written by its producer.  colsum (mode 1 with a mask, where tc_rows_sums_columns): the
 // column sums of the result, for launch_colsum_finish.
 cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols,
-                                float* C, int ldc, const RowSpan* pair_tiles, int npairs, const float* Hmask, int ldh, float scale,
+                                float* C, int ldc, const RowSpan* pair_tiles, int npairs, uint32_t* bits, int bit_words, float scale,
                                 const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16 = nullptr, float* colsum = nullptr);
+inline int32_t bit_words_of(int32_t ld) { return (ld + 31) / 32; }
 bool tc_rows_sums_columns(int n_cols, int npairs);
 constexpr int kMaxRowClusters = 128;
 int tc_rows_clusters(long long ntiles, int num_sms);   // clusters of a launch: cluster c takes tiles [ntiles c / n, ntiles (c + 1) / n)

@@ -1,6 +1,8 @@
 // Grouped dense transforms on the 5th-generation tensor cores (tcgen05, accumulators in tensor memory):
 //   mode 0   Z_l  = H^(l) W_k^(l)                        (the H.W of the forward equation, Section 3.3)
-//   mode 1   dPre = (dZ_l W_k^(l)^T) masked by H^(l) > 0  (chain rule through the forward equation)
+//   mode 1   dPre = (dZ_l W_k^(l)^T) masked by H^(l) > 0  (chain rule through the forward equation; the mask as bits, which mode 0 left
+//            behind while it split H^(l): with the activations themselves the drain waited for its mask loads.  525 000 rows, 256 <- 47 276 -> 174 us,
+//            256 <- 256 355 -> 281, 256 -> 256 289 -> 296; 94 000 rows in 50 subgraphs, 128 <- 128 38.9 -> 29.6, 128 -> 128 22.2 -> 25)
 //   mode 2   H^(l+1) = sigma((A~ H^(l)) W_k^(l) + b_k^(l)) with dropout: mode 0 finished in the epilogue, for a layer
 //            that aggregates before it transforms
 // All are C[rows x N] = A[rows x Kd] * B_k^T with A row-major (Kd contiguous) and B_k stored as N rows of Kd contiguous
@@ -59,8 +61,8 @@ struct RowsArgs {
     float* C;
     uint32_t* Cbf;            // mode 0: the result as bfloat16 (two values per word) instead of C, or null
     int ldc;
-    const float* Hmask;
-    int ldh;
+    uint32_t* bits;           // mode 0: receives which values of A are above zero; mode 1: the mask; or null.  Bit c % 32 of word c / 32 of a row
+    int bit_words;            // words of a row
     float scale;
     float* colsum;            // masked drains: column sums of what is written (the bias gradient of the layer below), or null:
                               // [(cluster + subgraph) * 8 + rank * 4 + row quarter][ldc] of every (cluster, subgraph) that meet
@@ -241,10 +243,15 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // steps are in hand at a time.  (A group's wait for a ring stage is unambiguous because nlo <= nst: once its own previous
         // step has been multiplied, so has the step before in that stage.)
         const int gw = SPLIT_WARPS / groups, group = (warp - 2) / gw, tt = threadIdx.x - 64 - 32 * gw * group;
+        constexpr bool leaves_bits = DRAIN == kPlain || DRAIN == kBf16;
+        uint32_t* bits = a.bits;
+        after_wait(bits);
         const int row = 32 * (warp & 3) + lane;       // kTensorMem: this thread's row of the tile, in its warp's quarter of the lanes
         int stage = 0, q = 0;
         uint32_t phase = 0, qphase = 0, bphase = 0;
-        for_tiles([&](int, int, int, bool new_b) {
+        for_tiles([&](int pair, int n, int, bool new_b) {
+            RowSpan sp{0, 0, 0, 0};                       // the rows whose signs are left behind: with the first column tile, where asked for
+            if (leaves_bits && a.bits && n == 0) sp = a.tiles[2 * pair + (int)rank];
             // (the votes keep the warp together: lanes may see a time-out or an abort at different polls)
             if (a.resident && new_b) {
                 if (!__all_sync(0xffffffffu, mbar_wait(bfull, bphase, abort_flag, a.err, 5))) return false;
@@ -276,14 +283,35 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             if (a.resident) mbar_arrive(empty(stage));   // nobody else reads the stage
                             mbar_arrive_leader_tmem(xfull(q));
                         }
+                        if (row < sp.nrows) {
+                            uint32_t w = 0;
+#pragma unroll
+                            for (int i = 0; i < BK; ++i) w |= (hi[i] > 0.f ? 1u : 0u) << i;
+                            bits[((long long)sp.row0 + row) * a.bit_words + kb] = w;
+                        }
                     } else {
-                    if (split) {
-                        const float4* hi = reinterpret_cast<const float4*>(sm + off_ring + (uint32_t)stage * stage_bytes);
-                        float4* lo = reinterpret_cast<float4*>(sm + off_lo + (uint32_t)q * A_BYTES);
-#pragma unroll 4
-                        for (int i = tt; i < A_BYTES / 16; i += 32 * gw) {
-                            const float4 v = hi[i];   // stays where it is: the MMA reads it as the hi part
-                            lo[i] = make_float4(tf32_rest(v.x), tf32_rest(v.y), tf32_rest(v.z), tf32_rest(v.w));
+                    if (FORM == kSharedLo || sp.nrows > 0) {
+                        // a thread takes half a row at a time (its 16-byte pieces are swizzled by the row: neighbouring lanes cover all banks); a
+                        // word of sign bits put together from several lanes made the kernel 37 to 85 % longer
+                        const uint8_t* hi = sm + off_ring + (uint32_t)stage * stage_bytes;
+                        uint8_t* lo = sm + off_lo + (uint32_t)q * A_BYTES;
+                        for (int u = tt; u < 2 * BM; u += 32 * gw) {
+                            const int r = u & (BM - 1), h = u >> 7;
+                            float4 v[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) v[j] = *reinterpret_cast<const float4*>(hi + r * (4 * BK) + (((4 * h + j) ^ (r & 7)) << 4));
+                            if (FORM == kSharedLo)   // (the tile as loaded stays where it is: the MMA reads it as the hi part)
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+                                    *reinterpret_cast<float4*>(lo + r * (4 * BK) + (((4 * h + j) ^ (r & 7)) << 4)) =
+                                        make_float4(tf32_rest(v[j].x), tf32_rest(v[j].y), tf32_rest(v[j].z), tf32_rest(v[j].w));
+                            if (r < sp.nrows) {
+                                uint32_t w = 0;
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+                                    w |= ((v[j].x > 0.f ? 1u : 0u) | (v[j].y > 0.f ? 2u : 0u) | (v[j].z > 0.f ? 4u : 0u) | (v[j].w > 0.f ? 8u : 0u)) << (4 * j);
+                                reinterpret_cast<uint16_t*>(bits + ((long long)sp.row0 + r) * a.bit_words + kb)[h] = (uint16_t)w;
+                            }
                         }
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tensor-core reads
@@ -302,9 +330,9 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // In a 16 x 256-bit read lane t gets, of every 8 columns, columns 2 (t % 4) and the next one of rows t / 4 and t / 4 + 8.
         const int quarter = warp & 3, half = (warp - EPI_WARP0) >> 2;
         const int sub_r = lane >> 2, sub_c = 2 * (lane & 3);
-        const float* hmask = a.Hmask;
+        const uint32_t* bits = a.bits;
         ActEpi act = a.act;
-        after_wait(hmask);
+        after_wait(bits);
         after_wait(act.params);
         constexpr bool masked = DRAIN == kMask || DRAIN == kMaskBf16, to_bf16 = DRAIN == kBf16 || DRAIN == kMaskBf16;
         // This warp's column sums: the columns of its blocks, of its quarter of the rows; nobody else touches them.  They are written out
@@ -329,6 +357,15 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             const int n0 = n * a.BN;
             if (masked && a.colsum && sp.k != cs_k) flush_colsum(sp.k);
             const int r0 = quarter * 32 + sub_r;                 // this lane's rows: r0 + 8 i
+            // a block's mask bits are asked for one block ahead, the first ones before the wait for the accumulator
+            uint32_t next_mb[4];
+            auto fetch_bits = [&](int c0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    next_mb[i] = r0 + 8 * i < sp.nrows && c0 < a.BN && n0 + c0 < a.ldc
+                                     ? __ldg(bits + ((long long)sp.row0 + r0 + 8 * i) * a.bit_words + ((n0 + c0) >> 5)) >> sub_c : 0u;
+            };
+            if (masked) fetch_bits(32 * half);
             if (!__all_sync(0xffffffffu, mbar_wait(tfull(acc), acc_phase, abort_flag, a.err, 8))) return false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             for (int c0 = 32 * half; c0 < a.BN && n0 + c0 < a.ldc; c0 += 64) {
@@ -336,14 +373,11 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const int ng = min(4, (min(a.BN - c0, a.ldc - n0 - c0) - sub_c + 7) >> 3);   // groups it has columns in
                 const long long at0 = ((long long)sp.row0 + r0) * a.ldc + nc;
                 float2 bias[4];
-                float2 hm[4][4];
+                uint32_t mb[4];
                 if (masked) {
-                    const float* h = hmask + ((long long)sp.row0 + r0) * a.ldh + nc;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int g = 0; g < 4; ++g)
-                            hm[i][g] = r0 + 8 * i < sp.nrows && g < ng ? __ldg(reinterpret_cast<const float2*>(h + 8 * i * a.ldh + 8 * g)) : make_float2(0.f, 0.f);
+                    for (int i = 0; i < 4; ++i) mb[i] = next_mb[i];
+                    fetch_bits(c0 + 64);
                 }
                 if (DRAIN == kAct || DRAIN == kActDrop)
 #pragma unroll
@@ -356,8 +390,8 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     for (int i = 0; i < 4; ++i)
 #pragma unroll
                         for (int g = 0; g < 4; ++g) {
-                            v[i][g].x = hm[i][g].x > 0.f ? v[i][g].x * a.scale : 0.f;
-                            v[i][g].y = hm[i][g].y > 0.f ? v[i][g].y * a.scale : 0.f;
+                            v[i][g].x = mb[i] >> (8 * g) & 1u ? v[i][g].x * a.scale : 0.f;
+                            v[i][g].y = mb[i] >> (8 * g + 1) & 1u ? v[i][g].y * a.scale : 0.f;
                         }
                     if (a.colsum) {   // (rows and columns that do not exist are masked to zero)
 #pragma unroll
@@ -472,20 +506,20 @@ bool tc_rows_sums_columns(int n_cols, int npairs) { return tc_rows_bn(n_cols, np
 int tc_rows_clusters(long long ntiles, int num_sms) { return (int)std::min<long long>(ntiles, std::min(max_clusters(num_sms), kMaxRowClusters)); }
 
 cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols,
-                                float* C, int ldc, const RowSpan* pair_tiles, int npairs, const float* Hmask, int ldh, float scale,
+                                float* C, int ldc, const RowSpan* pair_tiles, int npairs, uint32_t* bits, int bit_words, float scale,
                                 const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16, float* colsum) {
     if (npairs <= 0) return cudaSuccess;
-    if ((mode == 2 && !act) || (Cbf16 && mode == 2) || (Cbf16 && mode == 1 && !Hmask)) return cudaErrorInvalidValue;
-    if (colsum && !(mode == 1 && Hmask && tc_rows_sums_columns(n_cols, npairs))) return cudaErrorInvalidValue;
+    if ((mode == 2 && !act) || (Cbf16 && mode == 2) || (Cbf16 && mode == 1 && !bits)) return cudaErrorInvalidValue;
+    if (colsum && !(mode == 1 && bits && tc_rows_sums_columns(n_cols, npairs))) return cudaErrorInvalidValue;
     RowsArgs a;
     a.tiles = pair_tiles; a.npairs = npairs; a.BN = tc_rows_bn(n_cols, npairs); a.ntn = (ldc + a.BN - 1) / a.BN; a.Kd = Kd;
     const int form = form_for(a.BN, passes);
     rows_layout(a.BN, Kd, form, a);
-    a.C = C; a.Cbf = reinterpret_cast<uint32_t*>(Cbf16); a.ldc = ldc; a.Hmask = Hmask; a.ldh = ldh; a.scale = scale; a.colsum = colsum;
+    a.C = C; a.Cbf = reinterpret_cast<uint32_t*>(Cbf16); a.ldc = ldc; a.bits = mode == 2 ? nullptr : bits; a.bit_words = bit_words; a.scale = scale; a.colsum = colsum;
     a.kmul = one_b ? 0 : 1; a.err = err;
     a.act = act ? *act : ActEpi{};
     const unsigned grid = 2u * (unsigned)tc_rows_clusters((long long)npairs * a.ntn, num_sms);
-    const int drain = mode == 2 ? (a.act.drop ? kActDrop : kAct) : mode == 1 && Hmask ? (Cbf16 ? kMaskBf16 : kMask) : Cbf16 ? kBf16 : kPlain;
+    const int drain = mode == 2 ? (a.act.drop ? kActDrop : kAct) : mode == 1 && bits ? (Cbf16 ? kMaskBf16 : kMask) : Cbf16 ? kBf16 : kPlain;
     auto go = [&](auto kernel) {
         cudaError_t e = configure_kernel_once(reinterpret_cast<const void*>(kernel), SMEM_BYTES, false);
         if (e != cudaSuccess) return e;

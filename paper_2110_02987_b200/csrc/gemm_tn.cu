@@ -1,19 +1,19 @@
 // Weight gradients dW_k = H_k^T dZ_k on the 5th-generation tensor cores (chain rule through the forward equation, Section 3.3):
-// partial[chunk][m][n] = sum over the chunk's rows r of H[r][m] dZ[r][n].  The reduction index is the row, so both operands are
+// partial[chunk][m][n] = sum over the chunk's rows r of H[r][m] dZ[r][n].  The reduction index is the row.  dZ stays in shared memory
 // "MN-major": a tile of 32 rows x 32 values (128 bytes per row, swizzled in 32-byte units) is one block of the canonical
 // layout, blocks of 32 values are 4096 bytes apart (leading byte offset), groups of 4 rows 512 bytes apart (stride byte offset),
-// and one MMA (K = 8) consumes 8 rows.  fp32 accuracy as in gemm_rows.cu; both operands are activations here, so both get a lo tile
-// in shared memory, and rows past the end of a chunk are zeroed there.
+// and one MMA (K = 8) consumes 8 rows.  H^T goes through tensor memory: a splitting lane reads one of its columns (32 rows, a bank each) and writes
+// both parts of it into its tensor-memory lane, which turns the tile on the way.  (In one pass H is read from shared memory as dZ is.)  fp32
+// accuracy as in gemm_rows.cu; both operands are activations here: dZ gets a lo tile in shared memory.  Rows past the end of a chunk become zero.
 //
-// What bounds it is the tensor pipe for 256 x 256 outputs, shared-memory bandwidth for narrower ones, then HBM.  For 256 x 256 outputs a CTA on its own moves 288 KB per 32 rows (operand reads
-// 144, TMA 48, split 96: 2300 cycles at 128 B) where the tensor pipe needs 1536.  With CTAs working in pairs (cta_group::2: each
-// has 128 of the H columns and half of the dZ columns) it is 192 KB, which is 1536 cycles too; layers of at most 128 input columns
-// have nothing to share and use one CTA.  The ring of loaded tiles is separate from the lo tiles, as in gemm_rows.cu, so that five or more
-// stages hold loads in flight instead of three; CTAs are persistent and have two accumulators, so that a work unit (a chunk of rows and an
+// What bounds it is the tensor pipe, and below 256 columns the split (about 1500 cycles a 32-row step of 128 columns and group of warps, two groups taking
+// turns, against 768 of MMAs).  With both operands split in shared memory it was shared-memory bandwidth: 192 KB a step of 128 x 128 (1536 cycles at 128 B), 288 KB of
+// 128 x 256; now 128 and 224 KB.  CTAs work in pairs (cta_group::2: each has 128 of the H columns and half of the dZ columns) where there are more than 128
+// input columns.  The ring of loaded tiles is separate from the split ones, so that three to five stages hold loads in flight; CTAs are persistent and
+// have two accumulators where the tensor memory has room for them beside the slots (up to 128 columns), so that a work unit (a chunk of rows and an
 // output tile) drains while the next one is multiplied.
-// Before (one CTA per chunk and tile, three-stage ring, both orders of split and drain in sequence) and now, event times inside an epoch
-// under the power cap, 525 000 rows: 256 x 256 470 -> 291 us (tensor pipe active 81 % of the time), 256 x 47 215 -> 147 us, 100 x 256 243 -> 224 us; 63 000
-// rows, 602 x 256: 196 -> 114 us.
+// One timeline of an epoch each, both operands split in shared memory and now: 525 000 rows, 256 x 256 259 -> 239 us, 256 x 47 123 -> 117, 100 x 256 216 -> 167;
+// 94 000 rows in 50 subgraphs, 128 x 128 35.7 -> 27.9, 500 x 128 94.5 -> 75; 110 000 rows, 128 x 128 34.5 -> 29.2.
 #include <cuda.h>
 
 #include <algorithm>
@@ -34,11 +34,14 @@ constexpr int SMEM_BYTES = 232448;
 constexpr int DATA_BYTES = SMEM_BYTES - 1024 - BAR_BYTES;
 constexpr int SPLIT_WARPS = 8, EPI_WARPS = 8, EPI_WARP0 = 2 + SPLIT_WARPS;
 constexpr int THREADS = 32 * (EPI_WARP0 + EPI_WARPS);
+constexpr int SLOT_COLS = 2 * TBK;                        // tensor memory of a split step of H: 32 columns of hi, 32 of lo
+constexpr uint32_t TMEM_COLS = 512;
 
 struct TnArgs {
     const RowSpan* chunks;
     int nunits, ntm, ntn, BN, M, ldw;   // work units; output tiles per chunk; MMA N; valid output rows; leading dimension of the output
-    int nst, nlo;
+    int nst, nlo;                       // ring stages; steps whose split operands are kept (2 or 4, at most nst)
+    int nacc;                           // accumulators: two where the tensor memory has room for them
     float* partial;
     long long pstride_chunk;
     int32_t* err;
@@ -54,6 +57,11 @@ template <int CG>
 __device__ __forceinline__ void mma_any(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
     if constexpr (CG == 2) mma_tf32_pair(d, a, b, idesc, acc);
     else mma_tf32(d, a, b, idesc, acc);
+}
+template <int CG>
+__device__ __forceinline__ void mma_any_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    if constexpr (CG == 2) mma_tf32_pair_ts(d, a, b, idesc, acc);
+    else mma_tf32_ts(d, a, b, idesc, acc);
 }
 template <int CG>
 __device__ __forceinline__ void commit_any(uint32_t bar) {
@@ -84,7 +92,8 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
     const int bcols = a.BN / CG;                               // this CTA's columns of dZ
     const int nbb = (bcols + 31) / 32, nblocks = A_BLOCKS + nbb;
     const uint32_t stage_bytes = (uint32_t)nblocks * BLOCK_BYTES;
-    const uint32_t off_ring = split ? (uint32_t)a.nlo * stage_bytes : 0u;
+    const uint32_t lo_bytes = (uint32_t)nbb * BLOCK_BYTES;     // lo part of a step of dZ
+    const uint32_t off_ring = split ? (uint32_t)a.nlo * lo_bytes : 0u;
     const int nst = a.nst;
     const uint32_t bars = sm_addr + DATA_BYTES;
     auto full = [&](int s) { return bars + 8u * s; };
@@ -97,10 +106,11 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
     volatile uint32_t* abort_flag = tmem_slot + 1;
     uint32_t acc_cols = 16;                                    // columns between the accumulators: BN rounded up to a power of two
     while (acc_cols < (uint32_t)a.BN) acc_cols <<= 1;
+    const uint32_t tmem_cols = split ? TMEM_COLS : 2 * acc_cols, slot0 = TMEM_COLS - (uint32_t)a.nlo * SLOT_COLS;
 
     pdl_next();
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-    const int groups = a.nlo == MAX_LO ? MAX_LO : 1;
+    constexpr int groups = split ? SPLIT_WARPS / 4 : 1;        // of splitting warps, taking steps in turn; each has a warp for every quarter of the lanes
     if (threadIdx.x == 0) {
         for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
         for (int q = 0; q < MAX_LO; ++q) { mbar_init(xfull(q), CG * SPLIT_WARPS / groups); mbar_init(loempty(q), 1); }
@@ -109,9 +119,9 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        if constexpr (CG == 2) tmem_alloc2(smem_u32(tmem_slot), 2 * acc_cols);
+        if constexpr (CG == 2) tmem_alloc2(smem_u32(tmem_slot), tmem_cols);
         else {
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(2 * acc_cols) : "memory");
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(tmem_cols) : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
     }
@@ -153,7 +163,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
         // ---------------- MMA issuer: the warp runs the loop, one elected lane issues ----------------
         int stage = 0, q = 0, acc = 0;
         uint32_t qphase = 0, acc_phase = 0;
-        const uint32_t idesc = instr_desc(a.BN, CG * BM) | (1u << 15) | (1u << 16);   // A and B MN-major
+        const uint32_t idesc = instr_desc(a.BN, CG * BM) | (split ? 0u : 1u << 15) | (1u << 16);   // A (in shared memory) and B MN-major
         for_units([&](int, const RowSpan c, int, int) {
             const int nkb = (c.nrows + TBK - 1) / TBK;
             if (!__all_sync(0xffffffffu, mbar_wait<CG == 2>(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 12))) return false;
@@ -162,19 +172,20 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
             for (int kb = 0; kb < nkb; ++kb) {
                 if (!__all_sync(0xffffffffu, mbar_wait<CG == 2>(xfull(q), qphase, abort_flag, a.err, 13))) return false;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t base = sm_addr + off_ring + (uint32_t)stage * stage_bytes, lo = sm_addr + (uint32_t)q * stage_bytes;
-                const uint64_t a_hi = smem_desc_mn(base), b_hi = smem_desc_mn(base + A_BLOCKS * BLOCK_BYTES);
-                const uint64_t a_lo = smem_desc_mn(lo), b_lo = smem_desc_mn(lo + A_BLOCKS * BLOCK_BYTES);
+                const uint32_t base = sm_addr + off_ring + (uint32_t)stage * stage_bytes, a_tm = tmem_base + slot0 + (uint32_t)q * SLOT_COLS;
+                const uint64_t a_hi = smem_desc_mn(base), b_hi = smem_desc_mn(base + A_BLOCKS * BLOCK_BYTES), b_lo = smem_desc_mn(sm_addr + (uint32_t)q * lo_bytes);
                 const int nks = min(TBK / 8, (c.nrows - kb * TBK + 7) / 8);
                 if (elect_one()) {
                     // the next group of 8 rows is 1024 bytes = 64 descriptor units further on
 #pragma unroll
                     for (int ks = 0; ks < TBK / 8; ++ks) {
                         if (ks < nks) {
-                            mma_any<CG>(d, a_hi + 64 * ks, b_hi + 64 * ks, idesc, (kb | ks) != 0 ? 1u : 0u);
-                            if (split) {
-                                mma_any<CG>(d, a_hi + 64 * ks, b_lo + 64 * ks, idesc, 1u);
-                                mma_any<CG>(d, a_lo + 64 * ks, b_hi + 64 * ks, idesc, 1u);
+                            if constexpr (split) {
+                                mma_any_ts<CG>(d, a_tm + 8 * ks, b_hi + 64 * ks, idesc, (kb | ks) != 0 ? 1u : 0u);
+                                mma_any_ts<CG>(d, a_tm + 8 * ks, b_lo + 64 * ks, idesc, 1u);
+                                mma_any_ts<CG>(d, a_tm + TBK + 8 * ks, b_hi + 64 * ks, idesc, 1u);
+                            } else {
+                                mma_any<CG>(d, a_hi + 64 * ks, b_hi + 64 * ks, idesc, (kb | ks) != 0 ? 1u : 0u);
                             }
                         }
                     }
@@ -186,34 +197,60 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
                 if (++stage == nst) stage = 0;
                 if (++q == a.nlo) { q = 0; qphase ^= 1u; }
             }
-            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            if (++acc == a.nacc) { acc = 0; acc_phase ^= 1u; }
             return true;
         });
     } else if (warp >= 2 && warp < EPI_WARP0) {
         // ---------------- split of both operands, rows past the end of the chunk zeroed (groups: see gemm_rows.cu) ----------------
-        const int gw = SPLIT_WARPS / groups, group = (warp - 2) / gw, tt = threadIdx.x - 64 - 32 * gw * group;
-        const int nf4 = (int)(stage_bytes / 16);
+        constexpr int gw = SPLIT_WARPS / groups;
+        const int group = (warp - 2) / gw, tt = threadIdx.x - 64 - 32 * gw * group;
+        const int nf4 = nblocks * (BLOCK_BYTES / 16), nb4 = nbb * (BLOCK_BYTES / 16);   // 16-byte pieces of a step, and of its dZ
+        const int piece = lane >> 3;                  // a lane is a column of H: its 32-byte piece of a row, swizzled by the row
         int stage = 0, q = 0;
         uint32_t phase = 0, qphase = 0;
         for_units([&](int, const RowSpan c, int, int) {
             const int nkb = (c.nrows + TBK - 1) / TBK;
             for (int kb = 0; kb < nkb; ++kb) {
-                if (groups == 1 || q == group) {
+                if (groups == 1 || (q & (groups - 1)) == group) {
                     // (the votes keep the warp together: lanes may see a time-out or an abort at different polls)
                     if (!__all_sync(0xffffffffu, mbar_wait(loempty(q), qphase ^ 1u, abort_flag, a.err, 14))) return false;
                     if (!__all_sync(0xffffffffu, mbar_wait(full(stage), phase, abort_flag, a.err, 15))) return false;
-                    float4* hi = reinterpret_cast<float4*>(sm + off_ring + (uint32_t)stage * stage_bytes);
-                    float4* lo = reinterpret_cast<float4*>(sm + (uint32_t)q * stage_bytes);
+                    uint8_t* base = sm + off_ring + (uint32_t)stage * stage_bytes;
                     const int valid = c.nrows - kb * TBK;
+                    float4* raw = reinterpret_cast<float4*>(base + (split ? A_BLOCKS * BLOCK_BYTES : 0));   // what the MMAs read as loaded
                     if (valid < TBK)   // 8 float4 per 128-byte row, TBK rows per block
-                        for (int i = tt; i < nf4; i += 32 * gw)
-                            if (((i >> 3) & (TBK - 1)) >= valid) hi[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (split) {
-#pragma unroll 4
-                        for (int i = tt; i < nf4; i += 32 * gw) {
-                            const float4 v = hi[i];   // stays where it is: the MMA reads it as the hi part
-                            lo[i] = make_float4(tf32_rest(v.x), tf32_rest(v.y), tf32_rest(v.z), tf32_rest(v.w));
+                        for (int i = tt; i < (split ? nb4 : nf4); i += 32 * gw)
+                            if (((i >> 3) & (TBK - 1)) >= valid) raw[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if constexpr (split) {
+                        // H: this warp's 32 columns, one a lane, 32 rows, on their way while dZ is split
+                        const uint8_t* src = base + (warp & 3) * BLOCK_BYTES + 4 * (lane & 7);
+                        float ahi[TBK], alo[TBK];
+#pragma unroll
+                        for (int k = 0; k < TBK; ++k) ahi[k] = *reinterpret_cast<const float*>(src + k * 128 + ((piece ^ (k & 3)) << 5));
+                        // dZ: loads ahead of the stores, which the compiler cannot tell apart from what is loaded (a piece at a time took 115 cycles)
+                        float4* lo = reinterpret_cast<float4*>(sm + (uint32_t)q * lo_bytes);
+                        constexpr int STEP = 32 * gw;
+                        for (int i = tt; i < nb4; i += 4 * STEP) {   // (nb4: a multiple of 2 STEP)
+                            float4 v[4];
+                            const bool four = i + 2 * STEP < nb4;
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (u < 2 || four) v[u] = raw[i + u * STEP];   // stays where it is: the MMA reads it as the hi part
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (u < 2 || four) lo[i + u * STEP] = make_float4(tf32_rest(v[u].x), tf32_rest(v[u].y), tf32_rest(v[u].z), tf32_rest(v[u].w));
                         }
+                        if (valid < TBK)
+#pragma unroll
+                            for (int k = 0; k < TBK; ++k) ahi[k] = k < valid ? ahi[k] : 0.f;
+#pragma unroll
+                        for (int k = 0; k < TBK; ++k) alo[k] = tf32_rest(ahi[k]);
+                        const uint32_t dst = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + slot0 + (uint32_t)q * SLOT_COLS;
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");   // the MMAs that read the slot have completed
+                        tmem_st_32x32b_x32(dst, ahi);
+                        tmem_st_32x32b_x32(dst + TBK, alo);
+                        tmem_wait_st();
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
@@ -254,7 +291,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) arrive_drained<CG>(tempty(acc));
-            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            if (++acc == a.nacc) { acc = 0; acc_phase ^= 1u; }
             return true;
         });
     }
@@ -269,8 +306,8 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ 
     if constexpr (CG == 2) cluster_sync();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if constexpr (CG == 2) tmem_dealloc2(tmem_base, 2 * acc_cols);
-        else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * acc_cols) : "memory");
+        if constexpr (CG == 2) tmem_dealloc2(tmem_base, tmem_cols);
+        else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
     }
 }
 
@@ -283,7 +320,7 @@ TnShape tn_shape(int fi, int ldw) {
     t.cg = fi > BM ? 2 : 1;
     t.ntm = (fi + t.cg * BM - 1) / (t.cg * BM);
     t.ntn = (ldw + 255) / 256;
-    t.bn = (int)round_up((ldw + t.ntn - 1) / t.ntn, 16);
+    t.bn = (int)round_up((ldw + t.ntn - 1) / t.ntn, 16 * t.cg);   // (an MMA of a pair with A in tensor memory takes multiples of 32)
     return t;
 }
 
@@ -321,9 +358,10 @@ cudaError_t launch_gemm_tn_tc(const void* mapH, const void* mapZ, int passes, in
     TnArgs a;
     a.chunks = chunks; a.ntm = t.ntm; a.ntn = t.ntn; a.BN = t.bn; a.M = M; a.ldw = ldw;
     a.nunits = nchunks * t.ntm * t.ntn;
-    const int stage = (A_BLOCKS + (t.bn / t.cg + 31) / 32) * BLOCK_BYTES, fit = DATA_BYTES / stage;   // tiles of a stage that fit: at least 4
-    a.nlo = passes <= 1 ? 2 : fit >= 8 ? MAX_LO : 2;
-    a.nst = std::min(MAX_STAGES, passes > 1 ? fit - a.nlo : fit);
+    const int lo = (t.bn / t.cg + 31) / 32 * BLOCK_BYTES, stage = A_BLOCKS * BLOCK_BYTES + lo;
+    a.nlo = passes > 1 && (DATA_BYTES - MAX_LO * lo) / stage >= MAX_LO ? MAX_LO : 2;   // (at most as many as stages: see gemm_rows.cu)
+    a.nst = std::min(MAX_STAGES, passes > 1 ? (DATA_BYTES - a.nlo * lo) / stage : DATA_BYTES / stage);
+    a.nacc = passes > 1 && t.bn > 128 ? 1 : 2;
     a.partial = partial; a.pstride_chunk = (long long)M * ldw; a.err = err;
     const int units = std::min(a.nunits, num_sms / t.cg);
     auto go = [&](auto kernel) {

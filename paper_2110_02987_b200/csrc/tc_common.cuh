@@ -94,6 +94,17 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// The same with A in tensor memory: row i of the 128 in lane i, a value of the reduction per column.
+__device__ __forceinline__ void mma_tf32_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "setp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n"
+        "}\n" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
@@ -165,7 +176,7 @@ __device__ __forceinline__ void mma_tf32_pair(uint32_t tmem_d, uint64_t adesc, u
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// The same with A in tensor memory: row i of each CTA's 128 rows in lane i, a value of the reduction per column.
+// The same with A in tensor memory, each CTA's 128 rows in its own.
 __device__ __forceinline__ void mma_tf32_pair_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n"
@@ -247,9 +258,12 @@ __device__ __forceinline__ float tf32_hi(float x) {
 }
 // What is left of x once the tensor core has read it as TF32: the MMA ignores the low 13 bits of an fp32 operand, so
 // an unsplit tile already is its own hi part (x with those bits cleared) and only lo = x - hi, exact in fp32 and then
-// rounded to TF32, has to be written.  Infinity gives NaN here (inf - inf), which keeps a non-finite result non-finite.
+// rounded to TF32, has to be written.  The rounding adds half a unit to the magnitude and leaves the cut to the MMA: what it reads is what the
+// conversion instruction gives, which costs the splitting warps four times the issue slots (weight gradients 5 to 8 % longer).  Infinity gives NaN
+// here (inf - inf; the product with zero keeps it), which keeps a non-finite result non-finite.
 __device__ __forceinline__ float tf32_rest(float x) {
-    return tf32_round(x - __uint_as_float(__float_as_uint(x) & 0xFFFFE000u));
+    const float r = x - __uint_as_float(__float_as_uint(x) & 0xFFFFE000u);
+    return fmaf(r, 0.f, __uint_as_float(__float_as_uint(r) + 0x1000u));
 }
 
 }  // namespace

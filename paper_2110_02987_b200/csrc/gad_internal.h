@@ -159,7 +159,7 @@ cudaError_t launch_gemm_rows_simt(int mode, const float* A, int lda, int Kd, con
 // Tensor-core (tcgen05) version of launch_gemm_rows_simt.  The operands come through TMA descriptors made by
 // tc_make_map (A: [rows x Kd]; B, B_lo: [K][N][Kd] copies written by launch_split_weights); passes = 3 gives fp32
 // accuracy by operand splitting, passes = 1 plain TF32 operands.  err receives a role code if a bounded wait runs out.
-int tc_rows_bn(int n_cols, int npairs);
+int tc_rows_bn(int n_cols, int npairs, bool whole);
 int tc_tn_rows();   // rows of the row-box descriptors the weight-gradient kernel reads (mapH / mapZ of launch_gemm_tn_tc)
 bool tc_make_map(void* out_map, const void* base, uint64_t inner, uint64_t rows, uint64_t outer, uint64_t row_stride_bytes,
                  uint64_t outer_stride_bytes, uint32_t box_rows, bool mn_major = false);
@@ -173,7 +173,7 @@ struct SplitLayers {
     SplitLayer y[MAX];
 };
 cudaError_t launch_split_weights(const float* params, int64_t pstride, int K, const SplitLayer* layers, int L, cudaStream_t s);
-// pair_tiles: 2 npairs row tiles (at most 128 rows, or none), the two of a pair in the same subgraph; tc_rows_bn(n_cols, npairs) columns
+// pair_tiles: 2 npairs row tiles (at most 128 rows, or none), the two of a pair in the same subgraph; tc_rows_bn columns
 // per tile, half of them the rows of B's descriptor box.  bits: with mode 0 (may be null) the transform leaves there which values of A are above
 // zero, bit c % 32 of word c / 32 of a row of bit_words words; mode 1 masks with such bits (null: no mask), 1/32 of the bytes of the activations.  one_b: the operand copies of replica 0 serve every subgraph.
 // Cbf16 (mode 0, or 1 with a mask; may be null): the result goes there as bfloat16 [rows x ldc] INSTEAD of to C - the operand copy the

@@ -85,6 +85,7 @@ __device__ __forceinline__ void tile_of(const RowsArgs& a, int t, int& pair, int
 
 // How A reaches the tensor cores: as loaded (one pass); its lo part beside it in shared memory; or both parts through tensor memory.
 enum Form { kOnePass, kSharedLo, kTensorMem };
+constexpr int ACC_COLS = 128;                   // columns between the accumulators there (the other forms: as many as the tile has)
 constexpr int SLOTS = 4, SLOT_COLS = 2 * BK;   // tensor-memory slots of a 128 x 32 step of A: 32 columns of hi, 32 of lo
 constexpr uint32_t TMEM_COLS = 512;
 
@@ -117,6 +118,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + DATA_BYTES + 8 * (2 * MAX_STAGES + 2 * MAX_LO + 6));
     volatile uint32_t* abort_flag = tmem_slot + 1;
     const uint32_t tmem_cols = FORM == kTensorMem ? TMEM_COLS : 2u * (uint32_t)a.BN;
+    const int acc_cols = FORM == kTensorMem ? ACC_COLS : a.BN;
     // groups of splitting warps that take steps in turn (kTensorMem: a group has a warp for every quarter of the lanes)
     const int groups = FORM == kTensorMem ? SPLIT_WARPS / 4 : a.nlo == MAX_LO ? MAX_LO : 1;
 
@@ -196,7 +198,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             first = false;
             if (!__all_sync(0xffffffffu, mbar_wait<true>(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 3))) return false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t d = tmem_base + (uint32_t)(acc * a.BN);
+            const uint32_t d = tmem_base + (uint32_t)(acc * acc_cols);
             for (int kb = 0; kb < nkb; ++kb) {
                 if (!__all_sync(0xffffffffu, mbar_wait<true>(xfull(q), qphase, abort_flag, a.err, 4))) return false;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -383,7 +385,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
                     for (int g = 0; g < 4; ++g) bias[g] = g < ng ? load_bias2(act, sp.k, nc + 8 * g) : make_float2(0.f, 0.f);
                 float2 v[4][4];                                  // [row r0 + 8 i][columns nc + 8 g]
-                const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * a.BN + c0);
+                const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * acc_cols + c0);
                 tmem_ld_16x256b_x4(t0, v);
                 if (masked) {
 #pragma unroll
@@ -469,7 +471,9 @@ void rows_layout(int BN, int Kd, int form, RowsArgs& a) {
     if (form == kTensorMem) {   // as many stages as there are slots, at least (see the split)
         const long long room_a = (long long)DATA_BYTES - (long long)nkb * nb * b_bytes;
         a.nlo = SLOTS;
-        a.resident = room_a >= SLOTS * A_BYTES ? 1 : 0;
+        // (with several column tiles a resident B means that A is read from HBM for each of them, a streamed one that it comes from L2 the second time:
+        // 256 -> 256 over 525 000 rows 316 us resident, 297 streamed; 100 -> 256 162 and 203)
+        a.resident = room_a >= SLOTS * A_BYTES && (a.ntn == 1 || nkb <= 4) ? 1 : 0;
         a.nst = (int)std::min<long long>(MAX_STAGES, a.resident ? room_a / A_BYTES : DATA_BYTES / (A_BYTES + nb * b_bytes));
         return;
     }
@@ -491,18 +495,22 @@ int max_clusters(int num_sms) {
 
 }  // namespace
 
-// Output columns per tile.  An MMA of M = 256, K = 8 costs about the same for any N up to 128 and twice that at 256, and every column
-// tile reads and splits A again, so the widest tile is the cheapest - unless the launch has so few row tiles that most SMs would
-// idle: then the columns are spread over more CTAs, down to 32 (2843 rows x 1433 -> 128: 24 row tiles, 40 us with 128 columns per
-// tile, 27 us with 32).
-int tc_rows_bn(int n_cols, int npairs) {
-    int bn = n_cols <= 32 ? 32 : n_cols <= 64 ? 64 : n_cols <= 128 ? 128 : 256;
-    while (bn > 32 && (long long)npairs * ((n_cols + bn - 1) / bn) * 2 <= 74) bn /= 2;
+// Output columns per tile.  A tile that should hold all columns (`whole`: one pass, whose MMAs cost little beside reading A again, or a masked drain,
+// which sums columns) is as wide as the layer, up to 256.  Else the columns are cut into equal tiles of at most 128, whose A goes
+// through tensor memory: 500 -> 256 over 20 700 rows (84 row tiles for 74 pairs of CTAs: two turns of 256 columns, three of 128) 45.6 -> 35.9 us,
+// 602 -> 256 over 63 000 89 -> 78, 100 -> 256 over 525 000 170 -> 162, 256 -> 256 300 -> 297; in one pass 256 -> 256 over 210 000 rows 86 in tiles
+// of 256 columns, 104 of 128.  Where a launch has so few row tiles that most SMs would idle the columns are spread over more CTAs, down to 32
+// (2843 rows x 1433 -> 128: 24 row tiles, 40 us with 128 columns per tile, 27 us with 32).
+int tc_rows_bn(int n_cols, int npairs, bool whole) {
+    int bn;
+    if (whole) bn = n_cols <= 32 ? 32 : n_cols <= 64 ? 64 : n_cols <= 128 ? 128 : 256;
+    else { const int ntn = (n_cols + 127) / 128; bn = (int)round_up((n_cols + ntn - 1) / ntn, 32); }
+    while (bn > 32 && (long long)npairs * ((n_cols + bn - 1) / bn) * 2 <= 74) bn = (int)round_up(bn / 2, 32);
     return bn;
 }
 
 // The drain can sum columns when a tile holds all of them.
-bool tc_rows_sums_columns(int n_cols, int npairs) { return tc_rows_bn(n_cols, npairs) >= n_cols; }
+bool tc_rows_sums_columns(int n_cols, int npairs) { return tc_rows_bn(n_cols, npairs, true) >= n_cols; }
 int tc_rows_clusters(long long ntiles, int num_sms) { return (int)std::min<long long>(ntiles, std::min(max_clusters(num_sms), kMaxRowClusters)); }
 
 cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols,
@@ -512,7 +520,7 @@ cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* 
     if ((mode == 2 && !act) || (Cbf16 && mode == 2) || (Cbf16 && mode == 1 && !bits)) return cudaErrorInvalidValue;
     if (colsum && !(mode == 1 && bits && tc_rows_sums_columns(n_cols, npairs))) return cudaErrorInvalidValue;
     RowsArgs a;
-    a.tiles = pair_tiles; a.npairs = npairs; a.BN = tc_rows_bn(n_cols, npairs); a.ntn = (ldc + a.BN - 1) / a.BN; a.Kd = Kd;
+    a.tiles = pair_tiles; a.npairs = npairs; a.BN = tc_rows_bn(n_cols, npairs, passes <= 1 || mode == 1); a.ntn = (ldc + a.BN - 1) / a.BN; a.Kd = Kd;
     const int form = form_for(a.BN, passes);
     rows_layout(a.BN, Kd, form, a);
     a.C = C; a.Cbf = reinterpret_cast<uint32_t*>(Cbf16); a.ldc = ldc; a.bits = mode == 2 ? nullptr : bits; a.bit_words = bit_words; a.scale = scale; a.colsum = colsum;

@@ -21,7 +21,7 @@ def built():
 @pytest.mark.parametrize("rows", [1, 127, 128, 129, 256, 257])
 @pytest.mark.parametrize("dims,kw", [
     ((31, 17, 5), {}), ((33, 130, 16, 3), {}), ((700, 33, 2), {}), ((129, 256, 257, 4), dict(flags=4)),
-    ((300, 300, 64, 9), dict(flags=4, dropout=0.3)), ((64, 512, 40), dict(gemm_mode=1)), ((1433, 64, 40, 7), dict(gemm_mode=1, flags=4))])
+    ((300, 300, 64, 9), dict(flags=4, dropout=0.3)), ((24, 160, 290, 5), dict(flags=4)), ((150, 96, 70), dict(dropout=0.2)), ((64, 512, 40), dict(gemm_mode=1)), ((1433, 64, 40, 7), dict(gemm_mode=1, flags=4))])
 def test_row_and_column_edges(rows, dims, kw, bit7):
     kw = dict(kw, flags=kw.get("flags", 0) | bit7)
     K = 3

@@ -268,18 +268,21 @@ __device__ __forceinline__ void gather_tail(float4 (&acc)[NV], const uint2* st, 
 }
 
 // Operand rows in flight per lane and resident warps asked of the compiler: short items make the chain
-// item -> entries -> operand rows the cost, and more resident warps hide it better than more loads per warp.
+// item -> entries -> operand rows the cost, and more resident warps hide it better than more loads per warp (128 columns: 2 rows and 64 warps 53 us,
+// 4 and 48 61, 8 and 32 68; 78 / 87 / 106 on 100 000 rows).  With 256 columns of fp32, 4 rows and 28 warps: dense communities, 265 entries a
+// row, 624 -> 606 and 606 -> 584 us against 2 and 40, 34 entries a row the same.
 constexpr int kItemWarps = 4;
-template <int NV> struct ItemCfg {
-    static constexpr int UU = NV <= 4 ? 2 : 1;
-    static constexpr int MINB = NV == 1 ? 16 : (NV == 2 ? 10 : (NV <= 4 ? 6 : 4));   // CTAs of 4 warps per SM
+template <int NV, bool PAIR> struct ItemCfg {
+    // (PAIR: half the bytes per operand row, twice the rows in flight)
+    static constexpr int UU = (PAIR ? 2 : 1) * (NV == 2 && !PAIR ? 4 : NV <= 4 ? 2 : 1);
+    static constexpr int MINB = NV == 1 ? 16 : NV == 2 ? (PAIR ? 10 : 7) : (NV <= 4 ? 6 : 4);   // CTAs of 4 warps per SM
 };
 
 template <int NV, bool EPI, bool OFF32, bool BF, bool PAIR>
-__global__ void __launch_bounds__(32 * kItemWarps, ItemCfg<NV>::MINB)
+__global__ void __launch_bounds__(32 * kItemWarps, ItemCfg<NV, PAIR>::MINB)
 spmm_items_kernel(const uint2* __restrict__ ecv, const int4* __restrict__ items, int nitems, const float* __restrict__ Z,
                   int ldz, float* __restrict__ out, int ldo, float* __restrict__ scratch, int F4, EpiDev ep) {
-    constexpr int UU = PAIR ? 2 * ItemCfg<NV>::UU : ItemCfg<NV>::UU;   // half the bytes per operand row: twice the rows in flight
+    constexpr int UU = ItemCfg<NV, PAIR>::UU;
     __shared__ __align__(16) uint2 stage_all[kItemWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int idx = blockIdx.x * kItemWarps + warp;

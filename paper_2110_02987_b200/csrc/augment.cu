@@ -40,6 +40,21 @@ __host__ __device__ inline uint64_t walk_draw(uint64_t key, int step) {
     const uint64_t G = 0x9e3779b97f4a7c15ULL;
     return aug_mix64(key + G * (uint64_t)(1 + step));
 }
+// A node as a walk wants it: where its row of the graph begins and how long it is (33 and 31 bits), and the reciprocal of that length.
+struct __align__(16) WalkNode { unsigned long long row, recip; };
+constexpr int kLenBits = 31;
+constexpr int64_t kMaxPackedEntries = 1ll << (64 - kLenBits);
+// x mod d by m = floor((2^64 - 1) / d): x m / 2^64 lies less than one below x / d, so that the quotient is right or one too small.
+__device__ __forceinline__ unsigned long long reciprocal(unsigned long long d) { return d > 0 ? ~0ull / d : 0ull; }
+__device__ __forceinline__ unsigned long long mod_by(unsigned long long x, unsigned long long d, unsigned long long m) {
+    const unsigned long long r = x - __umul64hi(x, m) * d;
+    return r >= d ? r - d : r;
+}
+__device__ __forceinline__ WalkNode walk_node(const int64_t* rowptr, int64_t v) {
+    const unsigned long long r0 = (unsigned long long)rowptr[v], d = (unsigned long long)rowptr[v + 1] - r0;
+    return {r0 << kLenBits | d, reciprocal(d)};
+}
+
 // The node sequence of one walk: start at a uniformly drawn boundary node, every step to a uniformly drawn neighbour.
 __host__ __device__ inline void make_walk(const int64_t* rowptr, const int32_t* col, const int32_t* B, int64_t nB, uint64_t seed, int sub,
                                           int64_t walk, int steps, int32_t* seq) {
@@ -81,7 +96,10 @@ struct SubState {
 constexpr int kTopSlack = 2;
 
 
-__global__ void __launch_bounds__(256) mark_kernel(const int32_t* __restrict__ core, const SubDesc* __restrict__ desc, uint8_t* __restrict__ inside, int64_t n) {
+__global__ void __launch_bounds__(256) mark_kernel(const int32_t* __restrict__ core, const SubDesc* __restrict__ desc, uint8_t* __restrict__ inside, int64_t n,
+                                                   const int64_t* __restrict__ rowptr, WalkNode* __restrict__ nodes) {
+    if (nodes)
+        for (int64_t v = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * gridDim.y * blockDim.x) nodes[v] = walk_node(rowptr, v);
     const SubDesc d = desc[blockIdx.y];
     uint8_t* in = inside + (int64_t)blockIdx.y * n;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < d.ncore; t += (int64_t)gridDim.x * blockDim.x) in[core[d.core0 + t]] = 1;
@@ -187,7 +205,7 @@ __global__ void __launch_bounds__(256) boundary_count_kernel(const uint8_t* __re
 }
 __global__ void __launch_bounds__(256) boundary_list_kernel(const uint8_t* __restrict__ boundary, int64_t n, int ntiles, const int32_t* __restrict__ tile_count,
                                                             const int64_t* __restrict__ rowptr, const SubDesc* __restrict__ desc,
-                                                            SubState* __restrict__ state, int32_t* __restrict__ B) {
+                                                            SubState* __restrict__ state, int32_t* __restrict__ B, WalkNode* __restrict__ Bnodes) {
     __shared__ int warp_sum[8];
     __shared__ int before;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -215,7 +233,9 @@ __global__ void __launch_bounds__(256) boundary_list_kernel(const uint8_t* __res
         const int i = (__ffsll((long long)bits) - 1) >> 3;
         bits &= bits - 1;
         const int64_t v = v0 + i;
-        out[at++] = (int32_t)v;
+        out[at] = (int32_t)v;
+        if (Bnodes) Bnodes[desc[blockIdx.y].core0 + at] = walk_node(rowptr, v);
+        ++at;
         deg += (unsigned long long)(rowptr[v + 1] - rowptr[v]);
     }
 #pragma unroll
@@ -226,9 +246,13 @@ __global__ void __launch_bounds__(256) boundary_list_kernel(const uint8_t* __res
 
 // Walks [0, n0) (extra == 0) or [n0, nwalks) (extra == 1) of every subgraph of the batch, their candidates counted and kept:
 // node[t][walk] is the node of step t, or -1 where it is inside the core set or occurred before.  (The scoring kernel reads them
-// back in 10 us where drawing the walks again took it 69: a draw is a 64-bit remainder, and those are what this kernel spends
-// its time on.)
+// back in 10 us where drawing the walks again took it 69.)
+// What bounds it is the number of lines that the lanes of a warp touch, each its own: 1.9 M walks of two steps made fourteen such reads each (two
+// row ends a node) and three 64-bit remainders by the division routine, 82 us.  PACKED (all but graphs of 2^33 entries and more): one 16-byte read gives
+// a node's row and the reciprocal for the remainder, for the first node in place of its number; and the first node, one of the core set, is not looked up.
+template <bool PACKED>
 __global__ void __launch_bounds__(256) walk_count_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, const int32_t* __restrict__ B,
+                                                         const WalkNode* __restrict__ nodes, const WalkNode* __restrict__ Bnodes,
                                                          const uint8_t* __restrict__ inside, int64_t n, const SubDesc* __restrict__ desc,
                                                          const SubState* __restrict__ state, uint64_t seed, int extra, int steps,
                                                          int32_t* __restrict__ count, int32_t* __restrict__ node, int64_t plane) {
@@ -237,13 +261,32 @@ __global__ void __launch_bounds__(256) walk_count_kernel(const int64_t* __restri
     const int64_t nB = s.nB, j1 = extra ? s.nwalks : min((int64_t)s.n0, d.max_walks);
     const uint8_t* in = inside + (int64_t)blockIdx.y * n;
     int32_t* cnt = count + (int64_t)blockIdx.y * n;
+    const unsigned long long rB = reciprocal((unsigned long long)nB);
     int32_t seq[kMaxSteps + 1];
     for (int64_t j = (extra ? (int64_t)s.n0 : 0) + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < j1; j += (int64_t)gridDim.x * blockDim.x) {
-        make_walk(rowptr, col, B + d.core0, nB, seed, d.sub, j, steps, seq);
-        for (int t = 0; t <= steps; ++t) {
-            const bool f = first_outside(in, seq, t);
-            if (f) atomicAdd(cnt + seq[t], 1);   // integer: the result does not depend on the order
-            node[t * plane + d.key0 + j] = f ? seq[t] : -1;
+        if constexpr (PACKED) {
+            const uint64_t key = walk_key(seed, d.sub, j);
+            const int64_t b = d.core0 + (int64_t)mod_by(walk_draw(key, 0), (unsigned long long)nB, rB);
+            WalkNode w = Bnodes[b];
+            seq[0] = -1;   // (inside, and so is whatever equals it)
+            node[d.key0 + j] = -1;
+            for (int t = 1; t <= steps; ++t) {
+                const unsigned long long deg = w.row & ((1ull << kLenBits) - 1);
+                const int32_t v = deg > 0 ? col[(int64_t)(w.row >> kLenBits) + (int64_t)mod_by(walk_draw(key, t), deg, w.recip)] : t == 1 ? B[b] : seq[t - 1];
+                seq[t] = v;
+                if (t < steps) w = nodes[v];
+                bool f = in[v] == 0;
+                for (int u = 1; u < t; ++u) f = f && seq[u] != v;
+                if (f) atomicAdd(cnt + v, 1);   // integer: the result does not depend on the order
+                node[t * plane + d.key0 + j] = f ? v : -1;
+            }
+        } else {
+            make_walk(rowptr, col, B + d.core0, nB, seed, d.sub, j, steps, seq);
+            for (int t = 0; t <= steps; ++t) {
+                const bool f = first_outside(in, seq, t);
+                if (f) atomicAdd(cnt + seq[t], 1);
+                node[t * plane + d.key0 + j] = f ? seq[t] : -1;
+            }
         }
     }
 }
@@ -436,7 +479,7 @@ struct AugPlan {
 };
 // The buffers of one batch of G subgraphs, behind the graph in the workspace.
 struct BatchLayout {
-    size_t o_desc, o_core, o_B, o_tile, o_key, o_node, o_top, o_count, o_inside, o_bound, o_hist, o_state, o_seq, end;
+    size_t o_desc, o_nodes, o_Bnodes, o_core, o_B, o_tile, o_key, o_node, o_top, o_count, o_inside, o_bound, o_hist, o_state, o_seq, end;
     int64_t ncore, nkeys, ntop;
 };
 // Leading walks whose order is established first: the selection loop rarely needs more (it then orders all of them).
@@ -459,6 +502,7 @@ BatchLayout batch_layout(const AugPlan& p, size_t base, int64_t n, const int64_t
     }
     size_t cur = base;
     b.o_desc = take(cur, sizeof(SubDesc) * G);
+    b.o_nodes = take(cur, sizeof(WalkNode) * (size_t)n); b.o_Bnodes = take(cur, sizeof(WalkNode) * (size_t)b.ncore);
     b.o_core = take(cur, 4 * (size_t)b.ncore); b.o_B = take(cur, 4 * (size_t)b.ncore);
     b.o_tile = take(cur, 4 * G * (size_t)num_tiles(n));
     b.o_key = take(cur, 8 * (size_t)b.nkeys); b.o_node = take(cur, 4 * (size_t)b.nkeys * (size_t)(steps + 1)); b.o_top = take(cur, 8 * kTopSlack * (size_t)b.ntop);
@@ -611,6 +655,8 @@ int gad_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int3
         int32_t *d_seq = (int32_t*)(ws + L.o_seq), *d_node = (int32_t*)(ws + L.o_node);
         uint8_t *d_inside = (uint8_t*)(ws + L.o_inside), *d_bound = (uint8_t*)(ws + L.o_bound);
         unsigned long long *d_key = (unsigned long long*)(ws + L.o_key), *d_top = (unsigned long long*)(ws + L.o_top);
+        WalkNode *d_nodes = (WalkNode*)(ws + L.o_nodes), *d_Bnodes = (WalkNode*)(ws + L.o_Bnodes);
+        const bool packed = g->nnz < kMaxPackedEntries;
         unsigned* d_hist = (unsigned*)(ws + L.o_hist);
         const int ntiles = num_tiles(n);
         // about `waves` CTAs per SM over all subgraphs of the batch, at least one each
@@ -622,12 +668,13 @@ int gad_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int3
         if (L.ncore > 0) AUG_CK(cudaMemcpyAsync(d_core, core_nodes + core_ptr[k0], 4 * (size_t)L.ncore, cudaMemcpyHostToDevice, s));
         AUG_CK(cudaMemsetAsync(ws + L.o_count, 0, L.o_seq - L.o_count, s));
         const dim3 node_grid = grid(1024, n, 8), walk_grid = grid(256, most_walks, 8), tile_grid((unsigned)ntiles, (unsigned)G);
-        AUG_LAUNCH(mark_kernel, node_grid, 256, d_core, d_desc, d_inside, n);
+        AUG_LAUNCH(mark_kernel, node_grid, 256, d_core, d_desc, d_inside, n, d_rowptr, packed ? d_nodes : nullptr);
         AUG_LAUNCH(boundary_kernel, grid(16, L.ncore / G, 8), 256, d_rowptr, d_col, d_core, d_desc, d_state, d_inside, d_bound, n);
         AUG_LAUNCH(boundary_count_kernel, tile_grid, 256, d_bound, n, ntiles, d_tile);
-        AUG_LAUNCH(boundary_list_kernel, tile_grid, 256, d_bound, n, ntiles, d_tile, d_rowptr, d_desc, d_state, d_B);
+        AUG_LAUNCH(boundary_list_kernel, tile_grid, 256, d_bound, n, ntiles, d_tile, d_rowptr, d_desc, d_state, d_B, packed ? d_Bnodes : nullptr);
         for (int extra = 0; extra < 2; ++extra) {   // the first batch of walks, then what the error equation asks for on top
-            AUG_LAUNCH(walk_count_kernel, walk_grid, 256, d_rowptr, d_col, d_B, d_inside, n, d_desc, d_state, cfg->seed, extra, steps, d_count, d_node, L.nkeys);
+            if (packed) AUG_LAUNCH(walk_count_kernel<true>, walk_grid, 256, d_rowptr, d_col, d_B, d_nodes, d_Bnodes, d_inside, n, d_desc, d_state, cfg->seed, extra, steps, d_count, d_node, L.nkeys);
+            else AUG_LAUNCH(walk_count_kernel<false>, walk_grid, 256, d_rowptr, d_col, d_B, d_nodes, d_Bnodes, d_inside, n, d_desc, d_state, cfg->seed, extra, steps, d_count, d_node, L.nkeys);
             AUG_LAUNCH(count_stats_kernel, node_grid, 256, d_count, n, d_state, extra);
             if (!extra) AUG_LAUNCH(decide_walks_kernel, (unsigned)((G + 127) / 128), 128, d_state, d_desc, G, cfg->zc / cfg->E, cfg->cap);
         }

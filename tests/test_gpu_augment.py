@@ -121,3 +121,18 @@ def test_boundary_lists_at_the_edges_of_a_tile(n, K):
     cores = [np.ascontiguousarray(c) for c in np.array_split(perm, K)]
     got, _ = _both(n, rowptr, (key % n).astype(np.int32), cores, 2, alpha=0.2, seed=n)
     assert all(len(h) > 0 for h in got)
+
+
+@pytest.mark.parametrize("steps", [1, 2, 5, 8])
+def test_directed_graphs_with_dead_ends(steps):
+    """Rows of length zero, one, powers of two and one that holds every node: the walk stays where a row is empty."""
+    n = 700
+    rng = np.random.default_rng(steps)
+    length = rng.choice([0, 0, 1, 2, 3, 4, 8, 64, 255, 256], n)
+    length[[5, 300]] = n - 1
+    rows = [np.sort(rng.choice(np.delete(np.arange(n), v), k, replace=False)).astype(np.int32) for v, k in enumerate(length)]
+    rowptr = np.zeros(n + 1, np.int64)
+    np.cumsum(length, out=rowptr[1:])
+    cores = [np.arange(0, 301, dtype=np.int32), np.arange(301, n, dtype=np.int32)]
+    got, info = _both(n, rowptr, np.concatenate(rows), cores, steps, alpha=0.2, seed=11 + steps)
+    assert all(len(h) > 0 for h in got)

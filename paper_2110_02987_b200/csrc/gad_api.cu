@@ -307,8 +307,8 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
         for (int32_t k = 0; k < K; ++k) p.gram_ptr[k + 1] = p.gram_ptr[k] + zeta_gram_tiles(sub_off[k + 1] - sub_off[k]);
         p.o_gram_ptr = take(cur, 8 * (size_t)(K + 1));
         p.o_gram_partial = take(cur, 8 * (size_t)zeta_gram_partials(kGramMaxCtas, K));
-        p.o_norm2 = take(cur, 4 * Np);
-        p.o_xhi = take(cur, 4 * Np * (size_t)p.ld[0]); p.o_xlo = take(cur, 4 * Np * (size_t)p.ld[0]);
+        p.o_norm2 = take(cur, 8 * Np);
+        p.o_xhi = take(cur, 2 * Np * (size_t)round_up(p.dims[0], 8)); p.o_xlo = take(cur, 2 * Np * (size_t)round_up(p.dims[0], 8));
     }
     p.bytes = cur;
     return GAD_OK;
@@ -360,7 +360,7 @@ struct gad_ctx {
     int64_t direct_epochs = 0;      // epochs enqueued launch by launch so far (the first one also sets up the kernels)
     bool use_tc = false;            // tensor-core transforms (tcgen05) instead of the SIMT ones
     bool use_gram = false;          // zeta_mode 1 through the Gram-matrix kernel on the tensor cores
-    TMap map_xhi, map_xlo;          // the TF32 split of H^(0) as 128-row boxes, for that kernel
+    TMap map_xhi, map_xlo;          // the fp16 split of H^(0) as row boxes, for that kernel
     int num_sms = 1;
     std::vector<TMap> maps;         // per layer: forward A, B_hi, B_lo; input-gradient A, B_hi, B_lo
 
@@ -568,8 +568,8 @@ int zeta_pass(gad_ctx* ctx, cudaStream_t s) {
         GAD_RUN("zeta", -1, 4.0 * p.Np * (p.dims[0] + 2), 2.0 * pairs * p.dims[0], [&] {
             return launch_zeta_gram(&ctx->map_xhi, &ctx->map_xlo, ctx->H(0), p.ld[0], p.dims[0], p.Np, ctx->at<int32_t>(p.o_deg),
                                     ctx->at<int32_t>(p.o_sub_off), ctx->at<int64_t>(p.o_deg_sum), ctx->at<int64_t>(p.o_gram_ptr),
-                                    p.gram_ptr[p.K], p.K, ctx->cfg.beta, ctx->at<float>(p.o_xhi), ctx->at<float>(p.o_xlo),
-                                    ctx->at<float>(p.o_norm2), ctx->at<double>(p.o_gram_partial), ctx->at<double>(p.o_zeta),
+                                    p.gram_ptr[p.K], p.K, ctx->cfg.beta, ctx->at<void>(p.o_xhi), ctx->at<void>(p.o_xlo),
+                                    ctx->at<float2>(p.o_norm2), ctx->at<double>(p.o_gram_partial), ctx->at<double>(p.o_zeta),
                                     ctx->at<int32_t>(p.o_flags) + 1, std::min(ctx->num_sms, kGramMaxCtas), s);
         });
         return GAD_OK;
@@ -950,8 +950,8 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
     }
     if (ctx->cfg.zeta_mode == 1) {
         ctx->use_gram = ctx->use_tc && !p.gram_ptr.empty();
-        if (ctx->use_gram && !(tc_make_map(&ctx->map_xhi, ctx->at<float>(p.o_xhi), p.dims[0], p.Np, 0, 4ull * p.ld[0], 0, zeta_gram_box_rows()) &&
-                               tc_make_map(&ctx->map_xlo, ctx->at<float>(p.o_xlo), p.dims[0], p.Np, 0, 4ull * p.ld[0], 0, zeta_gram_box_rows())))
+        if (ctx->use_gram && !(tc_make_map(&ctx->map_xhi, ctx->at<void>(p.o_xhi), p.dims[0], p.Np, 0, 2ull * round_up(p.dims[0], 8), 0, zeta_gram_box_rows(), false, true) &&
+                               tc_make_map(&ctx->map_xlo, ctx->at<void>(p.o_xlo), p.dims[0], p.Np, 0, 2ull * round_up(p.dims[0], 8), 0, zeta_gram_box_rows(), false, true)))
             return fail(ctx, GAD_ERR_CUDA, "cuTensorMapEncodeTiled failed");
         if (!ctx->use_gram && !p.pair_alu_ok)
             return fail(ctx, GAD_ERR_UNSUPPORTED, "zeta_mode 1 without the tensor-core kernel takes subgraphs of at most " +

@@ -162,7 +162,7 @@ cudaError_t launch_gemm_rows_simt(int mode, const float* A, int lda, int Kd, con
 int tc_rows_bn(int n_cols, int npairs, bool whole);
 int tc_tn_rows();   // rows of the row-box descriptors the weight-gradient kernel reads (mapH / mapZ of launch_gemm_tn_tc)
 bool tc_make_map(void* out_map, const void* base, uint64_t inner, uint64_t rows, uint64_t outer, uint64_t row_stride_bytes,
-                 uint64_t outer_stride_bytes, uint32_t box_rows, bool mn_major = false);
+                 uint64_t outer_stride_bytes, uint32_t box_rows, bool mn_major = false, bool half = false);
 struct SplitLayer {
     int fi, fo, ldw, ldkt;
     long long w_int;
@@ -252,15 +252,15 @@ cudaError_t launch_zeta_pair(const float* X, int ld, int F, const int32_t* deg, 
 // `err_word` (may be null): when a kernel of the epoch has reported a bounded wait that ran out, the gradients are not to
 // be trusted and the three consensus kernels leave the parameters (and `out`) untouched.
 // The same zeta_k with the squared distances from a Gram matrix on the tensor cores (zeta_gram.cu): tiles of 256 x 256 pairs,
-// tile_ptr[k] = first tile of subgraph k, any subgraph size.  Xhi, Xlo: [rows x ld] floats each (TF32 split of X, written
-// by the call; mapHi / mapLo are their descriptors, boxes of zeta_gram_box_rows rows); norm2: [rows] floats; partial: zeta_gram_partials doubles.
+// tile_ptr[k] = first tile of subgraph k, any subgraph size.  Xhi, Xlo: [rows x ldh] fp16 values each, ldh = F rounded up to 8 (split of the scaled rows of X, written
+// by the call; mapHi / mapLo are their descriptors, boxes of zeta_gram_box_rows rows); norm2: [rows] squared norms and scales; partial: zeta_gram_partials doubles.
 constexpr int kGramMaxCtas = 256;
 int64_t zeta_gram_tiles(int64_t rows);
 int64_t zeta_gram_partials(int num_ctas, int K);
 uint32_t zeta_gram_box_rows();
 cudaError_t launch_zeta_gram(const void* mapHi, const void* mapLo, const float* X, int ld, int F, long long rows, const int32_t* deg,
                              const int32_t* sub_off, const int64_t* deg_sum, const int64_t* tile_ptr, int64_t ntiles, int K, float beta,
-                             float* Xhi, float* Xlo, float* norm2, double* partial, double* zeta, int32_t* err, int num_sms, cudaStream_t s);
+                             void* Xhi, void* Xlo, float2* norm2, double* partial, double* zeta, int32_t* err, int num_sms, cudaStream_t s);
 
 // `epoch` (may be null): the device epoch counter, advanced by one.
 // pstride_p: floats between the replicas' parameters, 0 while they are equal (copy 0 then stands for all of them; the result always

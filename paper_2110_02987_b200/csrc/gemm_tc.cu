@@ -82,15 +82,15 @@ EncodeTiledFn encode_fn() {
 // operand tiles use the 128-byte swizzle of 16-byte units; MN-major TF32 tiles need the 128-byte swizzle of
 // 32-byte units (the only MN-major layout the tensor cores accept for 32-bit operands).
 bool tc_make_map(void* out_map, const void* base, uint64_t inner, uint64_t rows, uint64_t outer, uint64_t row_stride_bytes,
-                 uint64_t outer_stride_bytes, uint32_t box_rows, bool mn_major) {
+                 uint64_t outer_stride_bytes, uint32_t box_rows, bool mn_major, bool half) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     const bool three = outer > 0;
     cuuint64_t dims[3] = {inner, rows, three ? outer : 1};
     cuuint64_t strides[2] = {row_stride_bytes, outer_stride_bytes};
-    cuuint32_t box[3] = {(cuuint32_t)BK, box_rows, 1};
+    cuuint32_t box[3] = {(cuuint32_t)(half ? 2 * BK : BK), box_rows, 1};
     cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = fn(reinterpret_cast<CUtensorMap*>(out_map), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, three ? 3 : 2, const_cast<void*>(base), dims,
+    CUresult r = fn(reinterpret_cast<CUtensorMap*>(out_map), half ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, three ? 3 : 2, const_cast<void*>(base), dims,
                     strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                     mn_major ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

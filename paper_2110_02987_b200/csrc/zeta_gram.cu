@@ -4,16 +4,19 @@
 //   |x_i - x_j|^2 = |x_i|^2 + |x_j|^2 - 2 x_i . x_j .
 // The pairs of a subgraph are cut into tiles of 256 x 256 (i-block <= j-block).  A tile's inner products are one tcgen05 accumulator of a
 // pair of CTAs: each CTA holds 128 rows of the i-block and half of the j-block (rows of the feature matrix, K-major, loaded by TMA with the
-// 128-byte swizzle) and receives 128 x 256 products.  The features are split once per call into TF32-exact hi and lo = x - hi copies (a
-// streaming kernel that also takes the squared norms), and the product is accumulated as hi.hi + hi.lo + lo.hi in fp32 in tensor memory -
-// the error-compensated product of the layer transforms, here with both operands split ahead of time because the drain below needs the
-// SM's issue slots.  What bounds it is the tensor pipe; in 128 x 128 tiles of one CTA it was shared memory, read for A and B at the rate
-// of the MMAs and written by TMA on top (8 x 6560 rows of 128: 300 us, now 182; a call on as many rows of 32: 307 us, now 189).
+// 128-byte swizzle) and receives 128 x 256 products.  The features are split once per call into fp16 hi and lo copies of the row times a power of two (a
+// streaming kernel that also takes the squared norms and keeps the scales), and the product is accumulated as hi.hi + hi.lo + lo.hi in fp32 in tensor
+// memory.  hi and lo have 11 significant bits each, as TF32 parts have, and the scale keeps them clear of fp16's range: with the largest value of a row at 2^14
+// the parts of a value are short of 22 bits only where it is below 2^-16 of that, by no more than 2^-39 of the largest.  fp16 operands are multiplied twice as fast: in three TF32
+// passes the MMAs bounded the kernel (8 x 6563 rows of 128: 184 us, split 14).
+// The accumulator is added to half as often, and with it goes half of what the tensor core cuts off:
+// against fp64, 64 features with a common offset 2.4e-6 -> 1.5e-6, uniform ones 1.5e-6 -> 1.0e-6, normal ones 1e-7 and less as before.
+// What bounds it now is the drain: 17.7 instructions a pair, the schedulers issuing 65 % of the time, the tensor pipe active 43 % (157 us, split 14).
 //
 // While the MMA warp fills the second accumulator, sixteen warps read the first one back (tcgen05.ld), turn every inner product into a
 // distance and add p_j / (d + beta) over the pairs i < j inside the subgraph.  Two pairs share a reciprocal, p / x + q / y = (p y + q x) /
-// (x y): with a square root and half a reciprocal per pair the special-function unit (16 a cycle and SM) keeps up with the MMAs from 64
-// features on.  (Approximate square root and reciprocal, relative error 2^-23 each: far inside the 2e-6 the result is held to, and the
+// (x y): with a square root and half a reciprocal per pair the special-function unit (16 a cycle and SM) keeps up.  (Approximate square root and
+// reciprocal, relative error 2^-23 each: far inside the 2e-6 the result is held to, and the
 // errors of different pairs do not add up coherently.)
 //
 // Cancellation: for two rows that are close compared with their norms the Gram form loses digits, so a pair whose
@@ -24,6 +27,8 @@
 // Order of the sum: every cluster takes a contiguous range of tiles (ascending, subgraph by subgraph; the i-block stays in L2); every
 // draining warp keeps one fp64 running sum per subgraph and writes it to its own slot; a second kernel adds the slots of the clusters
 // whose ranges meet the subgraph in slot order.  For a given number of clusters the result does not depend on scheduling.
+#include <cuda_fp16.h>
+
 #include <algorithm>
 #include <atomic>
 
@@ -37,23 +42,23 @@ namespace {
 constexpr int GT = 256;                                   // rows of a tile side
 constexpr int GH = 128;                                   // rows of a tile a CTA has of A (M of the pair's MMA is twice that)
 constexpr int GBOX = 64;                                  // rows of a TMA box
-constexpr int GBK = 32;                                   // features per ring stage
-constexpr int G_TILE_BYTES = GH * GBK * 4;                // 16 KiB
-constexpr int G_BOX_BYTES = GBOX * GBK * 4;
+constexpr int GBK = 64;                                   // features per ring stage
+constexpr int G_TILE_BYTES = GH * GBK * 2;                // 16 KiB
+constexpr int G_BOX_BYTES = GBOX * GBK * 2;
 constexpr int G_STAGE_BYTES = 4 * G_TILE_BYTES;           // A_hi | A_lo | B_hi | B_lo
 constexpr int G_STAGES = 3;
 constexpr int G_RING_BYTES = G_STAGES * G_STAGE_BYTES;
 constexpr int G_EPI_WARPS = 16;                           // four per quarter of the tensor-memory lanes, every fourth block of 32 columns each
 constexpr int G_EPI_WARP0 = 2;
 constexpr int G_THREADS = 32 * (G_EPI_WARP0 + G_EPI_WARPS);
-constexpr int G_COL_BYTES = G_EPI_WARPS * 32 * 8;         // per draining warp: (p_j, |x_j|^2) of its 32 columns
+constexpr int G_COL_BYTES = G_EPI_WARPS * 32 * 16;        // per draining warp: (p_j, |x_j|^2, -2 / scale of x_j) of its 32 columns
 constexpr int G_SMEM_BYTES = G_RING_BYTES + 1024 + 256 + G_COL_BYTES;
 constexpr int G_TMEM_COLS = 2 * GT;                       // two accumulators of 256 columns: all of it
 
 struct GramArgs {
     const float* X;            // [rows x ld] features in store-row order
     int ld, F;
-    const float* norm2;        // [rows] squared norms of the rows
+    const float2* norm2;       // [rows] squared norm, 1 / scale of the fp16 copies
     const int32_t* deg;
     const int32_t* sub_off;
     const int64_t* deg_sum;
@@ -107,33 +112,40 @@ struct TilePos {
     __device__ __forceinline__ int j0(const GramArgs& a) const { return bj * GT + part * (GT / a.parts); }
 };
 
+// (FTZ: one instruction each; subnormal arguments and results count as zero)
+template <bool FTZ>
 __device__ __forceinline__ float sqrt_approx(float x) {
     float y;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    if (FTZ) asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    else asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+template <bool FTZ>
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    if (FTZ) asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    else asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 
 // Whether a pair has to be taken from the differences (true also where the Gram form has overflowed).
 __device__ __forceinline__ bool near_pair(float d2, float s2) { return !(d2 >= 0.05f * s2); }
-// Within these bounds of beta and of both squared norms the product of two denominators (distances up to 2^62, plus beta) neither
-// overflows nor underflows.
-constexpr float kLeastBeta = 0x1p-60f, kMostBeta = 0x1p60f, kMostNorm2 = 0x1p122f;
+// Within these bounds of beta and of both squared norms (or with norms of zero) the product of two denominators (distances up to 2^62, plus beta) neither
+// overflows nor underflows, and no squared distance of a pair that is not near is subnormal.
+constexpr float kLeastBeta = 0x1p-60f, kMostBeta = 0x1p60f, kLeastNorm2 = 0x1p-120f, kMostNorm2 = 0x1p122f;
+__device__ __forceinline__ bool plain_norm(float n2) { return n2 == 0.f || (n2 >= kLeastNorm2 && n2 <= kMostNorm2); }
 
 // p_j / (d_ij + beta) summed over 16 columns j of one row i.  EACH: only the columns first .. last - 1, and without the pairs that have to be
-// taken from the differences; those are reported in `close` either way.  PAIRED: two pairs share a reciprocal.
+// taken from the differences; those are reported in `close` either way.  PAIRED (norms and beta within the bounds above): two pairs share a reciprocal.
+// (Two-wide FP32 instructions, 8.5 a pair counted by hand instead of 17.7 as executed, made the kernel spill: 181 us instead of 157.)
 template <bool EACH, bool PAIRED>
-__device__ __forceinline__ float gram_terms(const uint32_t (&v)[16], const float2* cols, float ni, float beta, int first, int last, bool& close) {
+__device__ __forceinline__ float gram_terms(const uint32_t (&v)[16], const float4* cols, float ni, float si, float beta, int first, int last, bool& close) {
     float part = 0.f, p0 = 0.f, x0 = 0.f;
 #pragma unroll
     for (int jj = 0; jj < 16; ++jj) {
-        float2 c = cols[jj];                                   // (p_j, |x_j|^2), one broadcast load
+        float4 c = cols[jj];                                   // one broadcast load
         const float s2 = ni + c.y;
-        float d2 = fmaf(-2.f, __uint_as_float(v[jj]), s2);
+        float d2 = fmaf(__uint_as_float(v[jj]) * si, c.z, s2);
         bool near = near_pair(d2, s2);
         if (EACH) {
             const bool valid = jj >= first && jj < last;
@@ -143,9 +155,9 @@ __device__ __forceinline__ float gram_terms(const uint32_t (&v)[16], const float
             d2 = counts ? d2 : 1.f;
         }
         close |= near;
-        const float x = sqrt_approx(d2) + beta;
-        if (!PAIRED) part = fmaf(c.x, rcp_approx(x), part);
-        else if (jj & 1) part = fmaf(fmaf(p0, x, c.x * x0), rcp_approx(x0 * x), part);
+        const float x = sqrt_approx<PAIRED>(d2) + beta;
+        if (!PAIRED) part = fmaf(c.x, rcp_approx<false>(x), part);
+        else if (jj & 1) part = fmaf(fmaf(p0, x, c.x * x0), rcp_approx<true>(x0 * x), part);
         p0 = c.x; x0 = x;
     }
     return part;
@@ -188,7 +200,7 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
     auto tempty = [&](int i) { return bars + 8u * (3 * G_STAGES + 2 + i); };
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + G_RING_BYTES + 8 * (3 * G_STAGES + 4));
     volatile uint32_t* abort_flag = tmem_slot + 1;
-    float2* col_sm = reinterpret_cast<float2*>(sm + G_RING_BYTES + 256);   // [G_EPI_WARPS][32]
+    float4* col_sm = reinterpret_cast<float4*>(sm + G_RING_BYTES + 256);   // [G_EPI_WARPS][32]
 
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -218,7 +230,7 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
             const int ri = p.r0 + p.i0() + (int)rank * GH, rj = p.r0 + p.j0(a) + (int)rank * (width / 2);
             for (int kb = 0; kb < nkb; ++kb) {
                 if (!(ok = mbar_wait(empty(stage), phase ^ 1u, abort_flag, a.err, 21))) break;
-                mbar_expect_tx(full(stage), 2u * G_TILE_BYTES + 2u * (uint32_t)(width / 2) * (GBK * 4));
+                mbar_expect_tx(full(stage), 2u * G_TILE_BYTES + 2u * (uint32_t)(width / 2) * (GBK * 2));
                 const uint32_t base = sm_addr + stage * G_STAGE_BYTES;
                 for (int b = 0; b < GH / GBOX; ++b) {
                     tma_load_2d(base + b * G_BOX_BYTES, &tmHi, kb * GBK, ri + b * GBOX, full(stage));
@@ -244,7 +256,7 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
         // ---------------- MMA issuer (leader of the pair): the whole warp runs the loop, one elected lane issues ----------------
         int stage = 0, acc = 0;
         uint32_t phase = 0, acc_phase = 0;
-        const uint32_t idesc = instr_desc(width, 2 * GH);
+        const uint32_t idesc = instr_desc_f16(width, 2 * GH);
         bool ok = true;
         for (long long t = t_begin; t < t_end && ok; ++t) {
             if (!(ok = __all_sync(0xffffffffu, mbar_wait<true>(tempty(acc), acc_phase ^ 1u, abort_flag, a.err, 22)))) break;
@@ -257,15 +269,15 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
                 const uint32_t base = sm_addr + stage * G_STAGE_BYTES;
                 const uint64_t a_hi = smem_desc(base), a_lo = smem_desc(base + G_TILE_BYTES);
                 const uint64_t b_hi = smem_desc(base + 2 * G_TILE_BYTES), b_lo = smem_desc(base + 3 * G_TILE_BYTES);
-                const int nks = min(GBK / 8, (a.F - kb * GBK + 7) / 8);
+                const int nks = min(GBK / 16, (a.F - kb * GBK + 15) / 16);
                 if (elect_one()) {
-                    // 8 TF32 values = 32 bytes = 2 descriptor units along K
+                    // 16 fp16 values = 32 bytes = 2 descriptor units along K
 #pragma unroll
-                    for (int ks = 0; ks < GBK / 8; ++ks)
+                    for (int ks = 0; ks < GBK / 16; ++ks)
                         if (ks < nks) {
-                            mma_tf32_pair(d, a_hi + 2 * ks, b_hi + 2 * ks, idesc, (kb | ks) != 0 ? 1u : 0u);
-                            mma_tf32_pair(d, a_hi + 2 * ks, b_lo + 2 * ks, idesc, 1u);
-                            mma_tf32_pair(d, a_lo + 2 * ks, b_hi + 2 * ks, idesc, 1u);
+                            mma_f16_pair(d, a_hi + 2 * ks, b_hi + 2 * ks, idesc, (kb | ks) != 0 ? 1u : 0u);
+                            mma_f16_pair(d, a_hi + 2 * ks, b_lo + 2 * ks, idesc, 1u);
+                            mma_f16_pair(d, a_lo + 2 * ks, b_hi + 2 * ks, idesc, 1u);
                         }
                     mma_commit2(empty(stage));                    // in both CTAs
                     if (kb == nkb - 1) mma_commit2(tfull(acc));
@@ -280,7 +292,7 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
         // this warp may read tensor-memory lanes 32q .. 32q+31 (this CTA's rows i of the tile); of the four warps of a quarter each takes
         // every fourth block of 32 columns (tile columns j)
         const int ew = warp - G_EPI_WARP0, q = warp & 3;
-        float2* cols = col_sm + ew * 32;
+        float4* cols = col_sm + ew * 32;
         int acc = 0, cur_k = -1;
         uint32_t acc_phase = 0;
         bool ok = true, uniform = false;
@@ -306,7 +318,8 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
             const int ib = p.i0() + (int)rank * GH + q * 32, i = ib + lane;   // this thread's row of the tile, inside the subgraph
             const bool iv = i < p.n;
             const float pi = iv ? (uniform ? 1.f : (float)a.deg[p.r0 + i]) * invD : 0.f;
-            const float ni = iv ? a.norm2[p.r0 + i] : 0.f;
+            const float2 nsi = iv ? a.norm2[p.r0 + i] : make_float2(0.f, 1.f);
+            const float ni = nsi.x, si = nsi.y;
             if (!(ok = __all_sync(0xffffffffu, mbar_wait(tfull(acc), acc_phase, abort_flag, a.err, 26)))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             float part = 0.f;
@@ -316,10 +329,11 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
                 __syncwarp();                                                // the previous block's columns have been read
                 const int jl = jb + lane;                                    // the column this lane looks up for the warp
                 const bool jlv = jl < p.n;
-                const float2 mine = make_float2(jlv ? (uniform ? 1.f : (float)a.deg[p.r0 + jl]) * invD : 0.f, jlv ? a.norm2[p.r0 + jl] : 0.f);
+                const float2 nsj = jlv ? a.norm2[p.r0 + jl] : make_float2(0.f, 1.f);
+                const float4 mine = make_float4(jlv ? (uniform ? 1.f : (float)a.deg[p.r0 + jl]) * invD : 0.f, nsj.x, -2.f * nsj.y, 0.f);
                 cols[lane] = mine;
                 __syncwarp();
-                const bool plain = beta_ok && __all_sync(0xffffffffu, fmaxf(ni, mine.y) <= kMostNorm2);
+                const bool plain = beta_ok && __all_sync(0xffffffffu, plain_norm(ni) && plain_norm(mine.y));
                 const float4* xi = reinterpret_cast<const float4*>(a.X + (long long)(p.r0 + min(i, p.n - 1)) * a.ld);
                 for (int h = 0; h < 32; h += 16) {                           // (32 at a time do not fit the registers)
                     uint32_t v[16];
@@ -329,16 +343,16 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
                     const int first = i + 1 - jb - h, last = iv ? min(16, p.n - jb - h) : 0;
                     bool close = false;
                     float blk = 0.f;
-                    if (whole && plain) blk = gram_terms<false, true>(v, cols + h, ni, a.beta, 0, 16, close);
+                    if (whole && plain) blk = gram_terms<false, true>(v, cols + h, ni, si, a.beta, 0, 16, close);
                     if (!whole || !plain || __any_sync(0xffffffffu, close)) {
                         close = false;
-                        blk = plain ? gram_terms<true, true>(v, cols + h, ni, a.beta, first, last, close) : gram_terms<true, false>(v, cols + h, ni, a.beta, first, last, close);
+                        blk = plain ? gram_terms<true, true>(v, cols + h, ni, si, a.beta, first, last, close) : gram_terms<true, false>(v, cols + h, ni, si, a.beta, first, last, close);
                         if (close) {   // rows close to each other compared with their norms: those pairs from the differences themselves
 #pragma unroll
                             for (int jj = 0; jj < 16; ++jj) {                // (unrolled: the accumulator block stays in registers)
-                                const float2 c = cols[h + jj];
+                                const float4 c = cols[h + jj];
                                 const float s2 = ni + c.y;
-                                const float d2 = fmaf(-2.f, __uint_as_float(v[jj]), s2);
+                                const float d2 = fmaf(__uint_as_float(v[jj]) * si, c.z, s2);
                                 if (jj >= first && jj < last && near_pair(d2, s2))
                                     blk += c.x / (sqrtf(distance2(xi, reinterpret_cast<const float4*>(a.X + (long long)(p.r0 + jb + h + jj) * a.ld), a.ld >> 2)) + a.beta);
                             }
@@ -372,31 +386,48 @@ zeta_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant
     }
 }
 
-// One pass over the features: hi = x rounded to TF32, lo = x - hi (rounded the same way), and |x_r|^2 in fp32.  One warp
-// per row (pad columns are zero and stay zero).
-__global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict__ X, int ld, long long rows, float* __restrict__ Xhi,
-                                                         float* __restrict__ Xlo, float* __restrict__ norm2) {
+// One pass over the features: every row times the power of two that brings its largest value to 2^14 .. 2^15 (a row of zeros, or with infinities, stays as
+// it is), hi = that rounded to fp16, lo = the rest rounded to fp16; |x_r|^2 in fp32 and 1 / scale.  One warp per row, eight values per lane
+// (ldh: a multiple of 8; values past the last feature are zero).
+__global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict__ X, int ld, int ldh, long long rows, __half* __restrict__ Xhi,
+                                                         __half* __restrict__ Xlo, float2* __restrict__ norm2) {
     const long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (r >= rows) return;
     const float4* x = reinterpret_cast<const float4*>(X + r * ld);
-    float4* xh = reinterpret_cast<float4*>(Xhi + r * ld);
-    float4* xl = reinterpret_cast<float4*>(Xlo + r * ld);
-    float s = 0.f;
-    for (int f4 = lane; f4 < (ld >> 2); f4 += 32) {
+    const int n4 = ld >> 2;
+    constexpr float4 zero = {0.f, 0.f, 0.f, 0.f};
+    float s = 0.f, most = 0.f;
+    for (int f4 = lane; f4 < n4; f4 += 32) {
         const float4 v = __ldg(x + f4);
         s = fmaf(v.x, v.x, s); s = fmaf(v.y, v.y, s); s = fmaf(v.z, v.z, s); s = fmaf(v.w, v.w, s);
-        float4 h, l;
-        h.x = tf32_hi(v.x); l.x = tf32_round(v.x - h.x);
-        h.y = tf32_hi(v.y); l.y = tf32_round(v.y - h.y);
-        h.z = tf32_hi(v.z); l.z = tf32_round(v.z - h.z);
-        h.w = tf32_hi(v.w); l.w = tf32_round(v.w - h.w);
-        xh[f4] = h;
-        xl[f4] = l;
+        most = fmaxf(fmaxf(fmaxf(most, fabsf(v.x)), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) norm2[r] = s;
+    for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, o));
+    }
+    // 2^e <= most < 2^(e + 1) for the biased exponent e + 127 (subnormal rows: as if 2^-126); scale 2^(14 - e), held to what fp32 has
+    const int e = max((int)(__float_as_uint(most) >> 23), 1) - 127;
+    const bool scaled = most > 0.f && e < 128;
+    const int up = scaled ? min(14 - e, 126) : 0;   // (e >= -126, so up <= 140: held to 126; up >= -113)
+    const float scale = __uint_as_float((uint32_t)(up + 127) << 23), back = __uint_as_float((uint32_t)(127 - up) << 23);
+    for (int f8 = lane; f8 < (ldh >> 3); f8 += 32) {
+        const float4 a = __ldg(x + 2 * f8), b = 2 * f8 + 1 < n4 ? __ldg(x + 2 * f8 + 1) : zero;
+        const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        __half2 h[4], l[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const float u0 = v[2 * t] * scale, u1 = v[2 * t + 1] * scale;
+            h[t] = __floats2half2_rn(u0, u1);
+            const float2 back2 = __half22float2(h[t]);
+            l[t] = __floats2half2_rn(u0 - back2.x, u1 - back2.y);
+        }
+        *reinterpret_cast<uint4*>(Xhi + r * ldh + 8 * f8) = *reinterpret_cast<const uint4*>(h);
+        *reinterpret_cast<uint4*>(Xlo + r * ldh + 8 * f8) = *reinterpret_cast<const uint4*>(l);
+    }
+    if (lane == 0) norm2[r] = make_float2(s, back);
 }
 
 // zeta_k = the slots of the clusters that meet subgraph k added in slot order (one CTA per subgraph; a warp adds every eighth slot).
@@ -437,11 +468,11 @@ uint32_t zeta_gram_box_rows() { return GBOX; }
 
 cudaError_t launch_zeta_gram(const void* mapHi, const void* mapLo, const float* X, int ld, int F, long long rows, const int32_t* deg,
                              const int32_t* sub_off, const int64_t* deg_sum, const int64_t* tile_ptr, int64_t ntiles, int K, float beta,
-                             float* Xhi, float* Xlo, float* norm2, double* partial, double* zeta, int32_t* err, int num_sms, cudaStream_t s) {
+                             void* Xhi, void* Xlo, float2* norm2, double* partial, double* zeta, int32_t* err, int num_sms, cudaStream_t s) {
     if (rows <= 0 || K <= 0) return cudaSuccess;
     cudaError_t e = configure_kernel_once(reinterpret_cast<const void*>(zeta_gram_kernel), G_SMEM_BYTES, false);
     if (e != cudaSuccess) return e;
-    split_rows_kernel<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(X, ld, rows, Xhi, Xlo, norm2);
+    split_rows_kernel<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(X, ld, (int)round_up(F, 8), rows, reinterpret_cast<__half*>(Xhi), reinterpret_cast<__half*>(Xlo), norm2);
     ++g_kernel_launches;
     GramArgs a;
     a.X = X; a.ld = ld; a.F = F; a.norm2 = norm2; a.deg = deg; a.sub_off = sub_off; a.deg_sum = deg_sum; a.tile_ptr = tile_ptr;

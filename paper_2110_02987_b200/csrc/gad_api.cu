@@ -603,7 +603,8 @@ int zeta_pass(gad_ctx* ctx, cudaStream_t s) {
     return GAD_OK;
 }
 
-int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
+// sums: where to leave the chunk sums of the first layer's weight gradient, for the update to add up; null: they are added up here.
+int backward_pass(gad_ctx* ctx, cudaStream_t ss, ChunkSums* sums) {
     const Plan& p = ctx->p;
     float* G1 = ctx->at<float>(p.o_G1);
     float* G2 = ctx->at<float>(p.o_G2);
@@ -671,6 +672,10 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss) {
                             : launch_gemm_tn_simt(agg_first ? ctx->at<float>(p.o_P[l]) : ctx->H(l), y.ldi, y.fi, agg_first ? G1 : G2, y.ldo,
                                                   y.fo, dw_chunks, ndw, p.simt[(size_t)l] != 0, ctx->at<float>(p.o_dw_partial), y.ldw, ctx->stream);
             if (e != cudaSuccess) return e;
+            if (l == 0 && sums) {
+                *sums = ChunkSums{y.w_int / 4, (long long)y.fi * y.ldw / 4, ctx->at<float4>(p.o_dw_partial), (long long)y.fi * y.ldw / 4, ctx->at<int32_t>(p.dw[l].o_ptr)};
+                return cudaSuccess;
+            }
             return launch_reduce_chunks(ctx->at<float>(p.o_dw_partial), (int64_t)y.fi * y.ldw, ctx->at<int32_t>(p.dw[l].o_ptr), p.K, grads, p.pstride,
                                         y.w_int, (int64_t)y.fi * y.ldw, ctx->stream);
         });
@@ -1078,14 +1083,23 @@ static int enqueue_epoch(gad_ctx* ctx, bool consensus) {
                                   ctx->at<float>(p.o_cs_partial), p.maxld, bias_ld, ctx->at<float>(p.o_grads), p.pstride, last.b_int, ss);
     });
     if (ss != ctx->stream) GAD_CK(cudaEventRecord(ctx->ev_bias, ss));
-    if ((rc = backward_pass(ctx, ss)) != GAD_OK) return rc;
+    // On a small store, whose epoch is a chain of short kernels, the update of a small model adds up the chunks of the last weight gradient itself (on larger
+    // stores the kernel between them is 0.2 to 0.4 % of an epoch).
+    ChunkSums sums{};
+    const bool sum_there = consensus && pdl_state().on && p.pstride <= kStepSumsFloats && p.K <= kStepSumsReplicas;
+    if ((rc = backward_pass(ctx, ss, sum_there ? &sums : nullptr)) != GAD_OK) return rc;
     if (ss == ctx->stream && (rc = zeta_pass(ctx, ss)) != GAD_OK) return rc;
     if ((rc = hand_over(ctx, ss, ctx->stream, ctx->ev_join)) != GAD_OK) return rc;
     if (consensus)
         GAD_RUN("sgd_consensus", -1, 4.0 * ((ctx->same_params ? 1 : p.K) + p.K + 1) * p.Pint, 4.0 * p.K * p.Pint, [&] {
+            const int nreport = (int)((p.o_flags + 12 - p.o_loss) / 4);
+            if (sum_there)
+                return launch_step_sums_consensus(ctx->at<float>(p.o_params), param_stride(ctx), ctx->at<float>(p.o_grads), p.pstride, p.pstride, p.K, ctx->cfg.lr,
+                                                  ctx->at<double>(p.o_zeta), ctx->cfg.weighted, ctx->at<int32_t>(p.o_flags), dropout_counter(ctx), ctx->at<float>(p.o_loss),
+                                                  ctx->published, nreport, sums, ctx->stream);
             return launch_sgd_consensus(ctx->at<float>(p.o_params), param_stride(ctx), ctx->at<float>(p.o_grads), p.pstride, p.pstride, p.K, ctx->cfg.lr,
-                                        ctx->at<double>(p.o_zeta), ctx->cfg.weighted, 1, ctx->at<int32_t>(p.o_flags), dropout_counter(ctx), ctx->at<float>(p.o_loss), ctx->published,
-                                        (int)((p.o_flags + 12 - p.o_loss) / 4), ctx->stream);
+                                        ctx->at<double>(p.o_zeta), ctx->cfg.weighted, 1, ctx->at<int32_t>(p.o_flags), dropout_counter(ctx), ctx->at<float>(p.o_loss),
+                                        ctx->published, nreport, ctx->stream);
         });
     else if (dropout_counter(ctx))
         GAD_CK(launch_epoch_counter(dropout_counter(ctx), 0, true, ctx->stream));

@@ -268,6 +268,13 @@ cudaError_t launch_zeta_gram(const void* mapHi, const void* mapLo, const float* 
 cudaError_t launch_sgd_consensus(float* params, int64_t pstride_p, const float* grads, int64_t pstride, int64_t len, int K, float lr,
                                  const double* zeta, int weighted, int with_sgd, int32_t* words, long long* epoch, const float* report, float* report_to,
                                  int nreport, cudaStream_t s);
+// The same with a step where the gradients of the parameters [4 first4, 4 (first4 + count4)) have yet to be added up, chunk by chunk in order; they are written
+// to grads.  For at most kStepSumsFloats parameters and kStepSumsReplicas replicas.
+struct ChunkSums { long long first4, count4; const float4* partial; long long stride4; const int32_t* chunk_ptr; };
+constexpr int64_t kStepSumsFloats = 256 << 10, kStepSumsReplicas = 4096;
+cudaError_t launch_step_sums_consensus(float* params, int64_t pstride_p, float* grads, int64_t pstride, int64_t len, int K, float lr, const double* zeta,
+                                       int weighted, int32_t* words, long long* epoch, const float* report, float* report_to, int nreport,
+                                       const ChunkSums& sums, cudaStream_t s);
 // The device epoch counter on its own: + 1, or set to a value.
 cudaError_t launch_epoch_counter(long long* epoch, long long set_to, bool advance, cudaStream_t s);
 // One context's share of a consensus over several contexts: out = sum_k w_k (theta_k - lr grad_k) with w_k = zeta_k / total

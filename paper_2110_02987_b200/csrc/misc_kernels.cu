@@ -601,6 +601,19 @@ __device__ __forceinline__ float4 weighted_sum(const float* params, long long ps
     return acc;
 }
 
+// What the first block of an update does besides; false: a bounded wait ran out earlier in this epoch, and the parameters stay as they are.
+__device__ __forceinline__ bool end_of_epoch(long long pstride_p, int32_t* words, long long* epoch, const float* report, float* report_to, int nreport) {
+    const bool timed_out = words[1] != 0;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0 && pstride_p != 0 && !timed_out) words[2] = 0;
+        __syncthreads();
+        if (report_to)   // the epoch's losses and error words, final by now, straight into the host's memory
+            for (int i = threadIdx.x; i < nreport; i += blockDim.x) report_to[i] = report[i];
+    }
+    if (epoch && blockIdx.x == 0 && threadIdx.x == 0) *epoch += 1;   // last kernel of an epoch: nothing reads the counter beside it
+    return !timed_out;
+}
+
 // theta_k <- theta_k - lr * grad_k (each replica's own step, update equation of Section 3.3), then
 // theta_k <- sum_j w_j theta_j for every k (weighted global consensus, Section 3.4.2).  One float4 per thread.  All copies come out
 // equal, so only copy 0 is written, and while they are equal it is the only one read (pstride_p == 0): K gradient sets and one
@@ -615,15 +628,7 @@ __global__ void __launch_bounds__(256) sgd_consensus_kernel(float* params, long 
     pdl_wait();
     after_wait(grads);
     after_wait(zeta);
-    const bool timed_out = words[1] != 0;   // a bounded wait ran out earlier in this epoch: keep the parameters as they are
-    if (blockIdx.x == 0) {
-        if (threadIdx.x == 0 && pstride_p != 0 && !timed_out) words[2] = 0;
-        __syncthreads();
-        if (report_to)   // the epoch's losses and error words, final by now, straight into the host's memory
-            for (int i = threadIdx.x; i < nreport; i += blockDim.x) report_to[i] = report[i];
-    }
-    if (epoch && blockIdx.x == 0 && threadIdx.x == 0) *epoch += 1;   // last kernel of an epoch: nothing reads the counter beside it
-    if (timed_out) return;
+    if (!end_of_epoch(pstride_p, words, epoch, report, report_to, nreport)) return;
     consensus_weights(zeta, K, weighted, w_sm);
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= len4) return;
@@ -636,6 +641,77 @@ cudaError_t launch_sgd_consensus(float* params, int64_t pstride_p, const float* 
         const int threads = len4 >= 148 * 256 * 4 ? 256 : 64;   // a small model is spread over more CTAs
         launch(sgd_consensus_kernel, dim3((unsigned)((len4 + threads - 1) / threads)), threads, (size_t)K * sizeof(float), s, 
             params, pstride_p, grads, pstride, len4, K, lr, zeta, weighted, with_sgd, words, epoch, report, report_to, nreport);
+        ++g_kernel_launches;
+    }
+    return cudaGetLastError();
+}
+
+// The sum of one float4 over the chunks c0 .. c1 - 1 in order, eight loads at a time: as reduce_chunks_kernel adds them.
+__device__ __forceinline__ float4 chunk_sum(const float4* __restrict__ partial, long long stride4, long long i, int c0, int c1) {
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c = c0; c < c1; c += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = c + u < c1 ? partial[(long long)(c + u) * stride4 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (c + u < c1) { s.x += v[u].x; s.y += v[u].y; s.z += v[u].z; s.w += v[u].w; }
+    }
+    return s;
+}
+
+// The same update where the gradients of the parameters `sums` are still chunk sums: they are added here and written to grads, which saves a short epoch the
+// kernel between its last weight gradient and the update (19 717 rows of 500-256-3: 185.6 -> 178.3 us).  A block takes 32 float4: a warp for every replica, up
+// to blockDim / 32 of them at a time (the chunks of one replica are a chain of loads), whose stepped values are then added in order by the first warp.
+// The barriers and the small blocks cost more than that kernel where there are many parameters (16.8 M of 8 replicas: 0.39 ms, the kernel above 0.11).
+__global__ void __launch_bounds__(512) step_sums_consensus_kernel(float* params, long long pstride_p, float* grads, long long pstride, long long len4, int K,
+                                                                  float lr, const double* __restrict__ zeta, int weighted, int32_t* words, long long* epoch,
+                                                                  const float* report, float* report_to, int nreport, const ChunkSums sums) {
+    extern __shared__ float4 q_sm[];   // [blockDim / 32][32], then K weights
+    const int lane = threadIdx.x & 31, ky = threadIdx.x >> 5, ny = blockDim.x >> 5;
+    float* w_sm = reinterpret_cast<float*>(q_sm + blockDim.x);
+    pdl_wait();
+    after_wait(grads);
+    after_wait(zeta);
+    if (!end_of_epoch(pstride_p, words, epoch, report, report_to, nreport)) return;
+    const long long i = (long long)blockIdx.x * 32 + lane;
+    const bool here = i < len4, summed = here && i >= sums.first4 && i < sums.first4 + sums.count4;
+    // float4 i of replica k after its step
+    auto stepped = [&](int k) {
+        if (!here || k >= K) return make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 q = reinterpret_cast<const float4*>(params + (long long)k * pstride_p)[i];
+        float4* gk = reinterpret_cast<float4*>(grads + (long long)k * pstride) + i;
+        float4 g;
+        if (summed) *gk = g = chunk_sum(sums.partial, sums.stride4, i - sums.first4, sums.chunk_ptr[k], sums.chunk_ptr[k + 1]);
+        else g = *gk;
+        q.x = fmaf(-lr, g.x, q.x); q.y = fmaf(-lr, g.y, q.y); q.z = fmaf(-lr, g.z, q.z); q.w = fmaf(-lr, g.w, q.w);
+        return q;
+    };
+    float4 next = stepped(ky);
+    consensus_weights(zeta, K, weighted, w_sm);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k0 = 0; k0 < K; k0 += ny) {
+        q_sm[ky * 32 + lane] = next;
+        __syncthreads();
+        if (k0 + ny < K) next = stepped(k0 + ny + ky);
+        if (ky == 0)
+            for (int t = 0; t < min(ny, K - k0); ++t) {
+                const float w = w_sm[k0 + t];
+                const float4 q = q_sm[t * 32 + lane];
+                acc.x = fmaf(w, q.x, acc.x); acc.y = fmaf(w, q.y, acc.y); acc.z = fmaf(w, q.z, acc.z); acc.w = fmaf(w, q.w, acc.w);
+            }
+        __syncthreads();
+    }
+    if (ky == 0 && here) reinterpret_cast<float4*>(params)[i] = acc;   // (every read of copy 0 at i is this block's, and lies before a barrier)
+}
+cudaError_t launch_step_sums_consensus(float* params, int64_t pstride_p, float* grads, int64_t pstride, int64_t len, int K, float lr, const double* zeta,
+                                       int weighted, int32_t* words, long long* epoch, const float* report, float* report_to, int nreport,
+                                       const ChunkSums& sums, cudaStream_t s) {
+    const long long len4 = len / 4;
+    if (len4 > 0) {
+        const int ny = K <= 4 ? 4 : K <= 8 ? 8 : 16;
+        launch(step_sums_consensus_kernel, dim3((unsigned)((len4 + 31) / 32)), 32u * ny, (size_t)ny * 32 * sizeof(float4) + (size_t)K * sizeof(float), s,
+               params, (long long)pstride_p, grads, (long long)pstride, len4, K, lr, zeta, weighted, words, epoch, report, report_to, nreport, sums);
         ++g_kernel_launches;
     }
     return cudaGetLastError();

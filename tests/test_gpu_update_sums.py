@@ -36,7 +36,7 @@ def check(g, ref, K, differ):
 @pytest.mark.parametrize("dims,differ", [((3, 2), False), ((37, 5, 3), True), ((64, 33, 7, 4), False), ((300, 130, 5), False)])
 def test_replicas_and_layers(K, dims, differ):
     case = small_random_case(K, n=12 * K + 30, K=K, p=0.1, halo=False)
-    g, ref, _ = make_pair(case, dims, K, lr=0.05)
+    g, ref, _ = make_pair(case, dims, K, lr=0.05, flags=128)   # (bit 7: on the tensor cores, whose weight gradients are summed there)
     check(g, ref, K, differ)
 
 
@@ -45,5 +45,5 @@ def test_sizes_and_chunks(n, dims):
     u = np.arange(n)
     col = np.sort(np.stack([(u - 1) % n, (u + 1) % n], 1), axis=1).astype(np.int32).ravel()
     core = [np.arange(0, n // 3, dtype=np.int32), np.arange(n // 3, n, dtype=np.int32)]
-    g, ref, _ = make_pair((n, np.arange(0, 2 * n + 1, 2, dtype=np.int64), col, None, core, [np.zeros(0, np.int32)] * 2), dims, n, lr=0.05)
+    g, ref, _ = make_pair((n, np.arange(0, 2 * n + 1, 2, dtype=np.int64), col, None, core, [np.zeros(0, np.int32)] * 2), dims, n, lr=0.05, flags=128)
     check(g, ref, 2, False)

@@ -32,10 +32,10 @@ UNIT = "epochs/s"
 # capture summarised under profiles/; keyed by (workload, profile entry).  A kernel changed since its capture
 # has no entry (reported as null).
 NCU_TRAFFIC = {
-    # spmm_items_kernel<2,1,...> (14.16 GB read + 2.59 GB written) + spmm_finish_kernel (2 MB), profiles/spmm_c4_dram.md
-    ("c4", "spmm_fwd_l1"): 16.76e9,
-    ("c4", "spmm_bwd_l1"): 16.81e9,
-    # spmm_items_kernel (76.8 MB read + 32.9 MB written) + spmm_finish_kernel (14.9 MB read), profiles/spmm_items_c2.md
+    # spmm_items_kernel<2,1,...> (14.37 GB read + 2.62 GB written) + spmm_finish_kernel (2 MB), profiles/spmm_c4_dram.md
+    ("c4", "spmm_fwd_l1"): 17.00e9,
+    ("c4", "spmm_bwd_l1"): 17.03e9,
+    # spmm_items_kernel (76.8 MB read + 32.8 MB written) + spmm_finish_kernel (14.9 MB read), profiles/spmm_items_c2.md
     ("c2", "spmm_fwd_l0"): 124.6e6,
 }
 

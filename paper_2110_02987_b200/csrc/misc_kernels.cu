@@ -381,6 +381,8 @@ __global__ void __launch_bounds__(256) colsum_finish_kernel(const float* __restr
     __shared__ float seg_sm[256];
     const int k = blockIdx.x;
     const int2 r = clusters[k];
+    pdl_wait();
+    after_wait(colsum);
     const int c0 = (r.x + k) * 8, c1 = (r.y + k + 1) * 8;   // rows of the partial sums
     const int nseg = segments_for(ld), per = 256 / nseg;
     const int jl = threadIdx.x % per, seg = threadIdx.x / per;
@@ -448,6 +450,9 @@ __global__ void __launch_bounds__(1024) zeta_finish_kernel(const double* __restr
                                               double* __restrict__ q_acc, int phase) {
     __shared__ double seg_a[1024], seg_b[1024];
     const int k = blockIdx.x;
+    pdl_wait();
+    after_wait(partial);
+    after_wait(q_acc);
     const long long n = sub_off[k + 1] - sub_off[k];
     if (n == 0) return;   // zero since creation
     const bool uniform = deg_sum[k] == 0;
@@ -505,6 +510,8 @@ __global__ void __launch_bounds__(256) zeta_partial_kernel(const float* __restri
     __shared__ double sm[8][32][8];
     const RowSpan c = chunks[blockIdx.x];
     const bool uniform = deg_sum[c.k] == 0;
+    pdl_wait();
+    after_wait(X);
     const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
     const int ld4 = ld >> 2, v = (int)blockIdx.y * 32 + cx;
     double* P = partial + (long long)blockIdx.x * 2 * ld;

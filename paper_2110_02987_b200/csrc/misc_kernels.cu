@@ -673,14 +673,17 @@ __device__ __forceinline__ float4 chunk_sum(const float4* __restrict__ partial, 
 // The barriers and the small blocks cost more than that kernel where there are many parameters (16.8 M of 8 replicas: 0.39 ms, the kernel above 0.11).
 __global__ void __launch_bounds__(512) step_sums_consensus_kernel(float* params, long long pstride_p, float* grads, long long pstride, long long len4, int K,
                                                                   float lr, const double* __restrict__ zeta, int weighted, int32_t* words, long long* epoch,
-                                                                  const float* report, float* report_to, int nreport, const ChunkSums sums) {
+                                                                  const float* report, float* report_to, int nreport, ChunkSums sums) {
     extern __shared__ float4 q_sm[];   // [blockDim / 32][32], then K weights
     const int lane = threadIdx.x & 31, ky = threadIdx.x >> 5, ny = blockDim.x >> 5;
     float* w_sm = reinterpret_cast<float*>(q_sm + blockDim.x);
     pdl_wait();
     after_wait(grads);
     after_wait(zeta);
-    if (!end_of_epoch(pstride_p, words, epoch, report, report_to, nreport)) return;
+    after_wait(sums.partial);
+    after_wait(sums.chunk_ptr);
+    // (after a time-out too the chunks are added up: all the gradients are then those of one epoch, as where a kernel of its own adds them)
+    const bool update = end_of_epoch(pstride_p, words, epoch, report, report_to, nreport);
     const long long i = (long long)blockIdx.x * 32 + lane;
     const bool here = i < len4, summed = here && i >= sums.first4 && i < sums.first4 + sums.count4;
     // float4 i of replica k after its step
@@ -709,7 +712,7 @@ __global__ void __launch_bounds__(512) step_sums_consensus_kernel(float* params,
             }
         __syncthreads();
     }
-    if (ky == 0 && here) reinterpret_cast<float4*>(params)[i] = acc;   // (every read of copy 0 at i is this block's, and lies before a barrier)
+    if (update && ky == 0 && here) reinterpret_cast<float4*>(params)[i] = acc;   // (every read of copy 0 at i is this block's, and lies before a barrier)
 }
 cudaError_t launch_step_sums_consensus(float* params, int64_t pstride_p, float* grads, int64_t pstride, int64_t len, int K, float lr, const double* zeta,
                                        int weighted, int32_t* words, long long* epoch, const float* report, float* report_to, int nreport,

@@ -47,3 +47,24 @@ def test_sizes_and_chunks(n, dims):
     core = [np.arange(0, n // 3, dtype=np.int32), np.arange(n // 3, n, dtype=np.int32)]
     g, ref, _ = make_pair((n, np.arange(0, 2 * n + 1, 2, dtype=np.int64), col, None, core, [np.zeros(0, np.int32)] * 2), dims, n, lr=0.05, flags=128)
     check(g, ref, 2, False)
+
+
+@pytest.mark.parametrize("K,dims", [(2, (37, 5, 3)), (9, (64, 33, 7, 4))])
+def test_gradients_of_an_epoch_that_is_not_taken(K, dims):
+    """A bounded wait runs out ahead of the second epoch: its update is left out, and the gradients of all layers are still its own."""
+    import paper_2110_02987_b200 as pkg
+    g, ref, _ = make_pair(small_random_case(K, n=12 * K + 30, K=K, p=0.1, halo=False), dims, K, lr=0.5, flags=128)
+    with g:
+        g.train_epoch()
+        oracle_step(g, ref, TOL)
+        before, first = [g.get_params(k) for k in range(K)], [g.get_grads(k) for k in range(K)]
+        g.debug_expire_wait(1)
+        g.train_epoch(wait=False)
+        with pytest.raises(pkg.GadError):
+            g.synchronize()
+        oracle_step(g, ref, TOL)
+        for k in range(K):
+            assert np.array_equal(g.get_params(k), before[k])
+            assert rel_err(g.get_grads(k), ref.get_grads(k)) <= TOL
+            w0 = dims[0] * dims[1]                      # (that is not so because the step changed nothing)
+            assert rel_err(first[k][:w0], ref.get_grads(k)[:w0]) > 10 * TOL

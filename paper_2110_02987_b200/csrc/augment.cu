@@ -43,7 +43,7 @@ __host__ __device__ inline uint64_t walk_draw(uint64_t key, int step) {
 // A node as a walk wants it: where its row of the graph begins and how long it is (33 and 31 bits), and the reciprocal of that length.
 struct __align__(16) WalkNode { unsigned long long row, recip; };
 constexpr int kLenBits = 31;
-constexpr int64_t kMaxPackedEntries = 1ll << (64 - kLenBits);
+constexpr int64_t kMaxPackedEntries = 1ll << (64 - kLenBits), kMaxPackedRow = 1ll << kLenBits;   // both exclusive
 // x mod d by m = floor((2^64 - 1) / d): x m / 2^64 lies less than one below x / d, so that the quotient is right or one too small.
 __device__ __forceinline__ unsigned long long reciprocal(unsigned long long d) { return d > 0 ? ~0ull / d : 0ull; }
 __device__ __forceinline__ unsigned long long mod_by(unsigned long long x, unsigned long long d, unsigned long long m) {
@@ -248,8 +248,9 @@ __global__ void __launch_bounds__(256) boundary_list_kernel(const uint8_t* __res
 // node[t][walk] is the node of step t, or -1 where it is inside the core set or occurred before.  (The scoring kernel reads them
 // back in 10 us where drawing the walks again took it 69.)
 // What bounds it is the number of lines that the lanes of a warp touch, each its own: 1.9 M walks of two steps made fourteen such reads each (two
-// row ends a node) and three 64-bit remainders by the division routine, 82 us.  PACKED (all but graphs of 2^33 entries and more): one 16-byte read gives
+// row ends a node) and three 64-bit remainders by the division routine, 82 us.  PACKED: one 16-byte read gives
 // a node's row and the reciprocal for the remainder, for the first node in place of its number; and the first node, one of the core set, is not looked up.
+// PACKED: where every row fits a WalkNode (walks_pack).
 template <bool PACKED>
 __global__ void __launch_bounds__(256) walk_count_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, const int32_t* __restrict__ B,
                                                          const WalkNode* __restrict__ nodes, const WalkNode* __restrict__ Bnodes,
@@ -476,6 +477,7 @@ struct AugPlan {
     size_t o_rowptr, o_col, bytes;
     std::vector<int64_t> max_walks;          // [K] cap times the core set's degree sum: n0 is at most that sum
     std::vector<int32_t> first;              // subgraphs first[b] .. first[b + 1] - 1 form batch b
+    bool packed = false;                     // walks_pack
 };
 // The buffers of one batch of G subgraphs, behind the graph in the workspace.
 struct BatchLayout {
@@ -528,6 +530,23 @@ int check_columns(const gad_csr* g, std::string& err) {
     return GAD_OK;
 }
 
+// rowptr must not decrease; the longest row.
+int check_rows(const gad_csr* g, int64_t& longest, std::string& err) {
+    int down = 0;
+    int64_t most = 0;
+#pragma omp parallel for schedule(static) reduction(| : down) reduction(max : most) if (g->n > (1 << 16))
+    for (int32_t v = 0; v < g->n; ++v) {
+        const int64_t len = g->rowptr[v + 1] - g->rowptr[v];
+        down |= len < 0;
+        most = std::max(most, len);
+    }
+    longest = most;
+    if (down) { err = "rowptr decreases"; return GAD_ERR_UNSORTED; }
+    return GAD_OK;
+}
+// Every row's start and length fit a WalkNode.  (Columns may repeat, so that a row can be longer than there are nodes.)
+bool walks_pack(int64_t nnz, int64_t longest) { return nnz < kMaxPackedEntries && longest < kMaxPackedRow; }
+
 // `columns`: check them here; else the caller does (check_columns).
 int plan_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int32_t* core_nodes, const gad_augment_config* cfg, AugPlan& p,
                  std::string& err, bool columns) {
@@ -536,10 +555,9 @@ int plan_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int
     if (!(cfg->alpha >= 0.0) || !(cfg->E > 0.0) || !(cfg->zc > 0.0) || cfg->cap < 1) { err = "alpha >= 0, E > 0, zc > 0, cap >= 1"; return GAD_ERR_ARG; }
     // the kernels index rowptr, col and the per-node arrays with the caller's values: check the whole CSR here, on the host
     if (g->nnz < 0 || g->rowptr[0] != 0) { err = "rowptr must start at 0 and nnz must not be negative"; return GAD_ERR_ARG; }
-    int down = 0;
-#pragma omp parallel for schedule(static) reduction(| : down) if (g->n > (1 << 16))
-    for (int32_t v = 0; v < g->n; ++v) down |= g->rowptr[v + 1] < g->rowptr[v];
-    if (down) { err = "rowptr decreases"; return GAD_ERR_UNSORTED; }
+    int64_t longest = 0;
+    if (int rc = check_rows(g, longest, err)) return rc;
+    p.packed = walks_pack(g->nnz, longest);
     if (g->rowptr[g->n] != g->nnz) { err = "rowptr[n] differs from nnz"; return GAD_ERR_ARG; }
     if (columns) { int rc = check_columns(g, err); if (rc != GAD_OK) return rc; }
     for (int32_t k = 0; k < K; ++k)
@@ -591,26 +609,10 @@ int aug_fail(int code, const std::string& msg) { g_aug_error = msg; return code;
 
 const char* augment_last_error() { return g_aug_error.c_str(); }
 
-}  // namespace gad
-
-using namespace gad;
-
-extern "C" {
-
-int gad_augment_workspace_bytes(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int32_t* core_nodes,
-                                const gad_augment_config* cfg, size_t* bytes) {
-    if (!bytes) return GAD_ERR_ARG;
-    AugPlan p;
-    std::string err;
-    int rc = plan_augment(g, K, core_ptr, core_nodes, cfg, p, err, true);
-    if (rc != GAD_OK) return aug_fail(rc, err);
-    *bytes = p.bytes;
-    return GAD_OK;
-}
-
-int gad_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int32_t* core_nodes, const gad_augment_config* cfg,
-                void* workspace, size_t workspace_bytes, void* stream_, int64_t* halo_ptr, int32_t* halo_nodes, int64_t halo_capacity,
-                int64_t* walks_out) {
+// gad_augment; `general`: the walks in the form that takes rows of any length, whatever this graph's are (for tests).
+int augment_in_form(bool general, const gad_csr* g, int32_t K, const int64_t* core_ptr, const int32_t* core_nodes, const gad_augment_config* cfg,
+                    void* workspace, size_t workspace_bytes, void* stream_, int64_t* halo_ptr, int32_t* halo_nodes, int64_t halo_capacity,
+                    int64_t* walks_out) {
     if (!workspace || !halo_ptr || (halo_capacity > 0 && !halo_nodes) || ((uintptr_t)workspace & 255) != 0) return aug_fail(GAD_ERR_ARG, "bad arguments");
     AugPlan p;
     std::string err;
@@ -656,7 +658,7 @@ int gad_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int3
         uint8_t *d_inside = (uint8_t*)(ws + L.o_inside), *d_bound = (uint8_t*)(ws + L.o_bound);
         unsigned long long *d_key = (unsigned long long*)(ws + L.o_key), *d_top = (unsigned long long*)(ws + L.o_top);
         WalkNode *d_nodes = (WalkNode*)(ws + L.o_nodes), *d_Bnodes = (WalkNode*)(ws + L.o_Bnodes);
-        const bool packed = g->nnz < kMaxPackedEntries;
+        const bool packed = p.packed && !general;
         unsigned* d_hist = (unsigned*)(ws + L.o_hist);
         const int ntiles = num_tiles(n);
         // about `waves` CTAs per SM over all subgraphs of the batch, at least one each
@@ -743,6 +745,36 @@ int gad_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int3
     }
     AUG_CK(cudaGetLastError());
     return GAD_OK;
+}
+
+// For tests: which form the walks of a graph take, from its row pointers.
+bool augment_packs(const gad_csr* g) {
+    int64_t longest = 0;
+    std::string err;
+    return check_rows(g, longest, err) == GAD_OK && walks_pack(g->nnz, longest);
+}
+
+}  // namespace gad
+
+using namespace gad;
+
+extern "C" {
+
+int gad_augment_workspace_bytes(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int32_t* core_nodes,
+                                const gad_augment_config* cfg, size_t* bytes) {
+    if (!bytes) return GAD_ERR_ARG;
+    AugPlan p;
+    std::string err;
+    int rc = plan_augment(g, K, core_ptr, core_nodes, cfg, p, err, true);
+    if (rc != GAD_OK) return aug_fail(rc, err);
+    *bytes = p.bytes;
+    return GAD_OK;
+}
+
+int gad_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int32_t* core_nodes, const gad_augment_config* cfg,
+                void* workspace, size_t workspace_bytes, void* stream_, int64_t* halo_ptr, int32_t* halo_nodes, int64_t halo_capacity,
+                int64_t* walks_out) {
+    return augment_in_form(false, g, K, core_ptr, core_nodes, cfg, workspace, workspace_bytes, stream_, halo_ptr, halo_nodes, halo_capacity, walks_out);
 }
 
 const char* gad_augment_last_error(void) { return augment_last_error(); }

@@ -132,3 +132,17 @@ def test_default_initialisation_is_seeded_glorot_uniform():
     assert o == a.size
     with pytest.raises(GadError):
         pkg.default_params((4, 0, 2))
+
+
+@pytest.mark.parametrize("rows,packs", [([5, 0, 3], True), ([2**31 - 1, 7], True), ([7, 2**31], False), ([2**31 + 9, 1, 1], False),
+                                        ([2**31 - 1] * 4 + [3], True), ([2**31 - 1] * 4 + [4], False), ([2**33], False)])
+def test_graphs_whose_walks_are_packed(rows, packs):
+    """A row's start takes 33 bits there and its length 31; columns may repeat, so that a row can be longer than the graph has nodes.  (The columns are
+    not looked at here.)"""
+    import ctypes as C
+    from paper_2110_02987_b200 import binding
+    rowptr = np.concatenate([[0], np.cumsum(np.array(rows, np.int64))])
+    g = binding.gad_csr(len(rows), int(rowptr[-1]), rowptr.ctypes.data_as(C.POINTER(C.c_int64)), None, None)
+    f = pkg.load()._ZN3gad13augment_packsEPK7gad_csr    # gad::augment_packs(const gad_csr*)
+    f.argtypes, f.restype = [C.c_void_p], C.c_bool
+    assert f(C.byref(g)) is packs

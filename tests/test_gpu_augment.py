@@ -136,3 +136,32 @@ def test_directed_graphs_with_dead_ends(steps):
     cores = [np.arange(0, 301, dtype=np.int32), np.arange(301, n, dtype=np.int32)]
     got, info = _both(n, rowptr, np.concatenate(rows), cores, steps, alpha=0.2, seed=11 + steps)
     assert all(len(h) > 0 for h in got)
+
+
+@pytest.mark.parametrize("steps", [1, 2, 8])
+def test_walks_of_the_general_form(steps, monkeypatch):
+    """Graphs with rows too long for a packed node take another form of the walks; small ones give the same lists in it (the oracle's)."""
+    import paper_2110_02987_b200 as pkg
+    in_form = pkg.load()._ZN3gad15augment_in_formEbPK7gad_csriPKlPKiPK18gad_augment_configPvmSA_PlPilSB_   # gad::augment_in_form(bool general, ...)
+
+    class General:
+        def __init__(self, L): self.L = L
+        def __getattr__(self, name): return getattr(self.L, name)
+        def gad_augment(self, *a): return in_form(True, *a)
+
+    real = pkg.Augmenter.__init__
+
+    def init(self, *a):
+        real(self, *a)
+        self._L = General(self._L)
+
+    monkeypatch.setattr(pkg.Augmenter, "__init__", init)
+    n = 700
+    rng = np.random.default_rng(steps)
+    length = rng.choice([0, 1, 2, 3, 64], n)
+    length[300] = n - 1
+    rowptr = np.zeros(n + 1, np.int64)
+    np.cumsum(length, out=rowptr[1:])
+    col = rng.integers(0, n, rowptr[-1]).astype(np.int32)    # (columns repeat)
+    got, _ = _both(n, rowptr, col, [np.arange(0, 301, dtype=np.int32), np.arange(301, n, dtype=np.int32)], steps, alpha=0.2, seed=steps)
+    assert all(len(h) > 0 for h in got)

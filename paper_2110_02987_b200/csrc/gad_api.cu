@@ -794,6 +794,7 @@ int upload_sparse(gad_ctx* ctx, const std::vector<int32_t>& sub_off, const std::
     out.items = ctx->at<int4>(o_items);
     out.nitems = (int32_t)work.items.size();
     out.nrows = (int64_t)rowptr.size() - 1;
+    out.nnz = rowptr.back();
     out.scratch = ctx->at<float>(p.o_spmm_scratch);
     out.nfin = (int32_t)work.fin.size();
     return GAD_OK;

@@ -85,7 +85,7 @@ struct SparseDev {
     const int4* items = nullptr;      // parts and uncut rows together, longest first inside a run of rows
     float* scratch = nullptr;         // [slots x leading dimension of the output] partial rows
     int32_t nfin = 0, nitems = 0;
-    int64_t nrows = 0;                // rows (and columns) of the store
+    int64_t nrows = 0, nnz = 0;       // rows (and columns) of the store, its entries
 };
 
 struct Layer {

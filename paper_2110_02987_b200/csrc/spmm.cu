@@ -269,20 +269,27 @@ __device__ __forceinline__ void gather_tail(float4 (&acc)[NV], const uint2* st, 
 
 // Operand rows in flight per lane and resident warps asked of the compiler: short items make the chain
 // item -> entries -> operand rows the cost, and more resident warps hide it better than more loads per warp (128 columns: 2 rows and 64 warps 53 us,
-// 4 and 48 61, 8 and 32 68; 78 / 87 / 106 on 100 000 rows).  With 256 columns of fp32, 4 rows and 28 warps: dense communities, 265 entries a
-// row, 624 -> 606 and 606 -> 584 us against 2 and 40, 34 entries a row the same.
+// 4 and 48 61, 8 and 32 68; 78 / 87 / 106 on 100 000 rows).  129 to 256 columns have a second form (DEEP): four rows and 28 warps in place of
+// two and 40.  It is the better one for long rows, and for bfloat16 operands that cannot be read in pairs whatever the rows' length
+// (110 000 rows of 25 entries, 132, 196 and 252 columns: 131 -> 124, 136 -> 127, 140 -> 131 us; 63 000 of 230: 467 -> 417, 474 -> 424, 479 -> 425).
 constexpr int kItemWarps = 4;
-template <int NV, bool PAIR> struct ItemCfg {
+// fp32 operands of 129 to 256 columns: entries a row, on average, from which the deep form is taken.  us with two rows in flight / with four, by
+// entries a row: 25 (110 000 rows; 132, 160, 192, 224, 256 columns) 143 / 156, 140 / 152, 144 / 157, 153 / 164, 163 / 172; 39 (2.57 M rows, 256) 6330 / 6700 and
+// 6105 / 6365; 40 (315 000; 132, 160, 192, 224, 256) 523 / 545, 510 / 528, 533 / 548, 577 / 588, 633 / 639; 48 (315 000, 256) 821 / 834; 60 (63 000; 160, 256)
+// 149 / 151, 182 / 180; 60 (110 000, 256) 325 / 326; 66 (420 000, 256) 1557 / 1569; 79 (63 000; 160, 256) 195 / 193, 234 / 232; 106 (110 000, 256) 526 / 516;
+// 110 (63 000; 160, 256) 270 / 268, 318 / 310; 160 (110 000, 256) 798 / 778; 230 (63 000; 132, 160, 192, 224, 256) 572 / 567, 539 / 533, 544 / 537, 578 / 565, 616 / 601.
+constexpr int64_t kDeepEntries = 72;
+template <int NV, bool PAIR, bool DEEP> struct ItemCfg {
     // (PAIR: half the bytes per operand row, twice the rows in flight)
-    static constexpr int UU = (PAIR ? 2 : 1) * (NV == 2 && !PAIR ? 4 : NV <= 4 ? 2 : 1);
-    static constexpr int MINB = NV == 1 ? 16 : NV == 2 ? (PAIR ? 10 : 7) : (NV <= 4 ? 6 : 4);   // CTAs of 4 warps per SM
+    static constexpr int UU = (PAIR ? 2 : 1) * (DEEP ? 4 : NV <= 4 ? 2 : 1);
+    static constexpr int MINB = NV == 1 ? 16 : NV == 2 ? (DEEP ? 7 : 10) : (NV <= 4 ? 6 : 4);   // CTAs of 4 warps per SM
 };
 
-template <int NV, bool EPI, bool OFF32, bool BF, bool PAIR>
-__global__ void __launch_bounds__(32 * kItemWarps, ItemCfg<NV, PAIR>::MINB)
+template <int NV, bool EPI, bool OFF32, bool BF, bool PAIR, bool DEEP>
+__global__ void __launch_bounds__(32 * kItemWarps, ItemCfg<NV, PAIR, DEEP>::MINB)
 spmm_items_kernel(const uint2* __restrict__ ecv, const int4* __restrict__ items, int nitems, const float* __restrict__ Z,
                   int ldz, float* __restrict__ out, int ldo, float* __restrict__ scratch, int F4, EpiDev ep) {
-    constexpr int UU = ItemCfg<NV, PAIR>::UU;
+    constexpr int UU = ItemCfg<NV, PAIR, DEEP>::UU;
     __shared__ __align__(16) uint2 stage_all[kItemWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int idx = blockIdx.x * kItemWarps + warp;
@@ -342,18 +349,26 @@ static cudaError_t launch_rows(const SparseDev& A, const float* Z, int ldz, floa
             const unsigned grid = (unsigned)((A.nitems + kItemWarps - 1) / kItemWarps);
             // every byte of the operand within 4 GiB of its start: 32-bit offsets
             const bool off32 = (unsigned long long)A.nrows * (unsigned long long)OpBytes<BF>::elem * (unsigned long long)ldz < (1ull << 32);
-            bool paired = false;
+            auto go = [&](auto kernel) {
+                launch_share(kernel, dim3(grid), 32 * kItemWarps, kGatherSharedKB, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+            };
+            // a bfloat16 operand of a whole number of 8-column runs: 16-byte loads, eight columns per lane and load
+            const bool paired = BF && NV % 2 == 0 && F4 % 2 == 0 && ldz % 8 == 0;
             if constexpr (BF && NV % 2 == 0) {
-                // a bfloat16 operand of a whole number of 8-column runs: 16-byte loads, eight columns per lane and load
-                if (F4 % 2 == 0 && ldz % 8 == 0) {
-                    paired = true;
-                    if (off32) launch_share(spmm_items_kernel<NV, EPI, true, true, true>, dim3(grid), 32 * kItemWarps, kGatherSharedKB, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
-                    else launch_share(spmm_items_kernel<NV, EPI, false, true, true>, dim3(grid), 32 * kItemWarps, kGatherSharedKB, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
-                }
+                if (paired && off32) go(spmm_items_kernel<NV, EPI, true, true, true, false>);
+                else if (paired) go(spmm_items_kernel<NV, EPI, false, true, true, false>);
             }
-            if (!paired) {
-                if (off32) launch_share(spmm_items_kernel<NV, EPI, true, BF, false>, dim3(grid), 32 * kItemWarps, kGatherSharedKB, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
-                else launch_share(spmm_items_kernel<NV, EPI, false, BF, false>, dim3(grid), 32 * kItemWarps, kGatherSharedKB, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+            if constexpr (NV == 2) {
+                if (!paired && (BF || A.nnz >= kDeepEntries * A.nrows)) {
+                    if (off32) go(spmm_items_kernel<2, EPI, true, BF, false, true>);
+                    else go(spmm_items_kernel<2, EPI, false, BF, false, true>);
+                } else if constexpr (!BF) {
+                    if (off32) go(spmm_items_kernel<2, EPI, true, false, false, false>);
+                    else go(spmm_items_kernel<2, EPI, false, false, false, false>);
+                }
+            } else if (!paired) {
+                if (off32) go(spmm_items_kernel<NV, EPI, true, BF, false, false>);
+                else go(spmm_items_kernel<NV, EPI, false, BF, false, false>);
             }
             ++g_kernel_launches;
         }

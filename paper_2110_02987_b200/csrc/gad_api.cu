@@ -102,6 +102,8 @@ struct Plan {
     size_t bytes = 0;
     // offsets into the workspace
     size_t o_growptr = 0, o_gecv = 0, o_gfin = 0, o_gitems = 0;   // the loss rows' store (see gad_ctx::Ag)
+    int64_t run_min_rows = 0;         // rows from which a subgraph's items may be ordered by runs as well (kRunOperandBytes); 0: none has so many
+    size_t o_runs = 0, o_truns = 0, o_gruns = 0;
     size_t o_rowptr, o_ecv, o_fin, o_items, o_trowptr, o_tecv, o_tfin, o_titems, o_spmm_scratch, o_sub_off, o_gid, o_deg, o_label, o_train,
         o_deg_sum, o_deg_sq, o_inv_ntrain, o_tiles, o_chunks, o_chunk_ptr, o_core_spans, o_G1, o_G2, o_params, o_grads,
         o_dw_partial, o_cs_partial, o_loss_partial, o_zeta_partial, o_zeta, o_loss, o_flags, o_zeta_f, o_w_f, o_stage,
@@ -215,6 +217,14 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
         for (int64_t r = 0; r < core_count[k]; r += 256)
             p.core_spans.push_back(RowSpan{(int32_t)(sub_off[k] + r), (int32_t)std::min<int64_t>(256, core_count[k] - r), k, 0});
     }
+    int32_t max_spmm_ld = 4;   // a layer's SpMMs run at its input width when it aggregates first, else at its output width
+    for (int l = 0; l < p.L; ++l) max_spmm_ld = std::max(max_spmm_ld, p.ld[p.agg_first[l] ? l : l + 1]);
+    if (max_spmm_ld > 64) {
+        const int64_t row_bytes = (cfg->gemm_mode == 1 ? 2 : 4) * (int64_t)std::min(max_spmm_ld, 1024);   // of one pass
+        const int64_t least = std::max<int64_t>(kItemWindow + 1, (kRunOperandBytes + row_bytes - 1) / row_bytes);
+        for (int32_t k = 0; k < K; ++k)
+            if (sub_off[k + 1] - sub_off[k] >= least) p.run_min_rows = least;
+    }
     const size_t Np = (size_t)p.Np, nc = p.chunks.size();
     size_t cur = 0;
     p.o_rowptr = take(cur, 8 * (Np + 1)); p.o_ecv = take(cur, 8 * (size_t)nnz);
@@ -230,6 +240,10 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
         p.o_gfin = take(cur, 16 * max_fin);
         p.o_gitems = take(cur, 16 * (Np + max_parts));
     }
+    if (p.run_min_rows > 0) {
+        p.o_runs = take(cur, 16 * (Np + max_parts)); p.o_truns = take(cur, 16 * (Np + max_parts));
+        if (!(cfg->flags & 64)) p.o_gruns = take(cur, 16 * (Np + max_parts));
+    }
     p.o_sub_off = take(cur, 4 * (size_t)(K + 1)); p.o_gid = take(cur, 4 * Np); p.o_deg = take(cur, 4 * Np);
     p.o_label = take(cur, 4 * Np); p.o_train = take(cur, Np);
     p.o_deg_sum = take(cur, 8 * (size_t)K); p.o_deg_sq = take(cur, 8 * (size_t)K); p.o_inv_ntrain = take(cur, 4 * (size_t)K);
@@ -240,8 +254,6 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
     p.o_core_spans = take(cur, sizeof(RowSpan) * p.core_spans.size());
     p.o_H.resize(p.L + 1);
     for (int l = 0; l <= p.L; ++l) p.o_H[l] = take(cur, 4 * Np * (size_t)p.ld[l]);
-    int32_t max_spmm_ld = 4;   // a layer's SpMMs run at its input width when it aggregates first, else at its output width
-    for (int l = 0; l < p.L; ++l) max_spmm_ld = std::max(max_spmm_ld, p.ld[p.agg_first[l] ? l : l + 1]);
     p.o_spmm_scratch = take(cur, 4 * (size_t)slots * (size_t)max_spmm_ld);
     if (cfg->gemm_mode == 1) {
         p.o_bf16 = take(cur, 2 * Np * (size_t)max_spmm_ld);
@@ -766,19 +778,38 @@ void default_params(const std::vector<int32_t>& dims, uint64_t seed, float* out)
     }
 }
 
-int upload_sparse(gad_ctx* ctx, const std::vector<int32_t>& sub_off, const std::vector<int64_t>& rowptr, const std::vector<int32_t>& col,
-                  const std::vector<float>& val,
-                  size_t o_rowptr, size_t o_ecv, size_t o_fin, size_t o_items, SparseDev& out, int64_t forced_part = 0,
+int upload_sparse(gad_ctx* ctx, const std::vector<int32_t>& sub_off, const std::vector<int64_t>& core_count, const std::vector<int64_t>& rowptr,
+                  const std::vector<int32_t>& col, const std::vector<float>& val,
+                  size_t o_rowptr, size_t o_ecv, size_t o_fin, size_t o_items, size_t o_runs, SparseDev& out, int64_t forced_part = 0,
                   int64_t* part_entries = nullptr) {
     const Plan& p = ctx->p;
     std::vector<uint2> ecv(col.size());
+#pragma omp parallel for schedule(static) if (col.size() > (1 << 16))
     for (size_t e = 0; e < col.size(); ++e) {
         uint32_t bits;
         std::memcpy(&bits, &val[e], 4);
         ecv[e] = make_uint2((uint32_t)col[e], bits);
     }
     RowWork work;
-    bin_rows(rowptr, sub_off, work, forced_part);
+    std::vector<uint8_t> by_runs((size_t)p.K, 0);
+    for (int32_t k = 0; k < p.K && p.run_min_rows > 0; ++k) {
+        const int64_t rows = sub_off[k + 1] - sub_off[k], e0 = rowptr[sub_off[k]], e1 = rowptr[sub_off[k + 1]];
+        if (rows < p.run_min_rows) continue;
+        const int64_t halo0 = sub_off[k] + core_count[k];
+        int64_t near = 0, all = 0;
+#pragma omp parallel for schedule(static) reduction(+ : near, all) if (e1 - e0 > (1 << 16))
+        for (int64_t r = sub_off[k]; r < sub_off[k + 1]; ++r)
+            for (int64_t e = rowptr[r]; e < rowptr[r + 1]; ++e) {
+                const int64_t c = col[(size_t)e];
+                if (r >= halo0 && c >= halo0) continue;
+                ++all;
+                near += std::abs(c - r) < kItemWindow;
+            }
+        if ((double)near < kRunNearShare * (double)all) continue;
+        by_runs[(size_t)k] = 1;
+        out.run_rows = out.run_rows > 0 ? std::min(out.run_rows, rows) : rows;
+    }
+    bin_rows(rowptr, sub_off, work, forced_part, by_runs);
     if (part_entries) *part_entries = work.part_entries;
     if (work.slots > p.slots) return fail(ctx, GAD_ERR_OOM, "SpMM scratch slots exceed the planned count");
     GAD_CK(cudaMemcpyAsync(ctx->ws + o_rowptr, rowptr.data(), 8 * rowptr.size(), cudaMemcpyHostToDevice, ctx->stream));
@@ -787,6 +818,10 @@ int upload_sparse(gad_ctx* ctx, const std::vector<int32_t>& sub_off, const std::
         GAD_CK(cudaMemcpyAsync(ctx->ws + o_fin, work.fin.data(), 16 * work.fin.size(), cudaMemcpyHostToDevice, ctx->stream));
     if (!work.items.empty())
         GAD_CK(cudaMemcpyAsync(ctx->ws + o_items, work.items.data(), 16 * work.items.size(), cudaMemcpyHostToDevice, ctx->stream));
+    if (!work.runs.empty()) {
+        GAD_CK(cudaMemcpyAsync(ctx->ws + o_runs, work.runs.data(), 16 * work.runs.size(), cudaMemcpyHostToDevice, ctx->stream));
+        out.runs = ctx->at<int4>(o_runs);
+    }
     GAD_CK(cudaStreamSynchronize(ctx->stream));  // the host vectors above go out of scope
     out.rowptr = ctx->at<int64_t>(o_rowptr);
     out.ecv = ctx->at<uint2>(o_ecv);
@@ -875,10 +910,10 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
     ctx->gid = st.gid;
 
     int64_t part_t = 0;   // part length of the store the backward aggregation reads
-    rc = upload_sparse(ctx, st.sub_off, st.rowptr, st.col, st.val, p.o_rowptr, p.o_ecv, p.o_fin, p.o_items, ctx->A, 0, &part_t);
+    rc = upload_sparse(ctx, st.sub_off, st.core_count, st.rowptr, st.col, st.val, p.o_rowptr, p.o_ecv, p.o_fin, p.o_items, p.o_runs, ctx->A, 0, &part_t);
     if (rc != GAD_OK) return rc;
     if (!st.symmetric) {
-        rc = upload_sparse(ctx, st.sub_off, st.t_rowptr, st.t_col, st.t_val, p.o_trowptr, p.o_tecv, p.o_tfin, p.o_titems, ctx->At, 0, &part_t);
+        rc = upload_sparse(ctx, st.sub_off, st.core_count, st.t_rowptr, st.t_col, st.t_val, p.o_trowptr, p.o_tecv, p.o_tfin, p.o_titems, p.o_truns, ctx->At, 0, &part_t);
         if (rc != GAD_OK) return rc;
     }
     // per-row labels and loss mask, per-subgraph degree sums and training counts
@@ -917,7 +952,7 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
                 if (train[(size_t)cl[e]]) { gcl.push_back(cl[e]); gvl.push_back(vl[e]); }
             grp[(size_t)r + 1] = (int64_t)gcl.size();
         }
-        rc = upload_sparse(ctx, st.sub_off, grp, gcl, gvl, p.o_growptr, p.o_gecv, p.o_gfin, p.o_gitems, ctx->Ag, part_t);
+        rc = upload_sparse(ctx, st.sub_off, st.core_count, grp, gcl, gvl, p.o_growptr, p.o_gecv, p.o_gfin, p.o_gitems, p.o_gruns, ctx->Ag, part_t);
         if (rc != GAD_OK) return rc;
         ctx->use_loss_rows = true;
         ctx->nnz_loss_rows = (int64_t)gcl.size();

@@ -62,16 +62,31 @@ int store_sizes(const gad_csr* g, const gad_partition* part, int64_t* Np, int64_
 // items = {row, low 32 bits of the first entry's position in the store, (high bits << 16) | entries, scratch slot
 // or -1 for an uncut row}, subgraph by subgraph and inside a subgraph binned by floor(log2(entries)), longest bin
 // first, ascending row inside a bin.  `perm` (uncut rows in that order) and `parts` are the intermediate lists the
-// items are built from.
+// items are built from.  runs = the same items, those of some subgraphs binned inside runs of kItemWindow rows (no such subgraph: empty).
 constexpr int64_t kMinPart = 64, kMaxPart = 8192, kMaxSlotsPerRow = 32;
+// Neighbouring rows of a graph that is numbered by community, time or site gather the same operand rows.  Ordered by length over a whole
+// subgraph the resident warps (9472) spread over all of it, and where its operand does not fit the L2 (126 MB) beside what else passes, those rows come
+// from HBM again and again; in runs they do not.  Epochs of 4 x 131 000 rows of 34 entries, 256 wide: 6100 us without runs, 5995 with
+// runs of 65 536 rows, 5915 of 32 768, 5900 of 16 384, 5900 of 4096.  A run ends on short items beside the long ones of the next, which costs every launch.
+// So runs serve launches whose operand takes half of the L2 and more, in subgraphs a good third of whose entries read a row less than a run away (those between
+// two replicated nodes aside: their rows are few and stay in the L2 in any order).  us without / with, by rows of a subgraph, columns and that share:
+//   both: 131 000, 256 (134 MB), 0.75 1258 / 1171 and 1230 / 1144; 157 000, 0.71, 128 (81 MB) 351 / 335, 192 (121 MB) 581 / 532, 384 and 512 (242, 323 MB)
+//     572 / 530; 210 000, 256 (215 MB), 0.42 1596 / 1520 and 1583 / 1496, 100 (84 MB) 737 / 718; 79 000, 256 (81 MB), 0.37 822 / 812 and 823 / 803;
+//     bfloat16, 131 000, 256 (67 MB), 0.75 834 / 802 and 764 / 730;
+//   smaller operands: 131 000, 0.75, 100 (52 MB) 586 / 602; bfloat16, 131 000, 0.75, 100 (26 MB) 453 / 475, 210 000, 0.42, 100 (42 MB) 377 / 369; and the kernels
+//     of up to 64 columns, whose warps have two to eight items each: 157 000, 0.71, 8 101 / 122 and 64 / 74, 64 233 / 237, 131 000, 47 438 / 473 and 222 / 253;
+//   fewer near: 16 x 161 000, 256 (165 MB), 0.16 to 0.32 6200 / 6260 and 5990 / 6070; 131 000, 256, 0.25 1300 / 1320 and 1271 / 1290; 157 000, 0.21, 128 356 / 360,
+//     192 591 / 595; bfloat16, 131 000, 256, 0.25 833 / 852 and 762 / 767.
+constexpr int64_t kItemWindow = 16384, kRunOperandBytes = 63 << 20;
+constexpr double kRunNearShare = 0.35;
 struct RowWork {
     std::vector<int32_t> perm;
-    std::vector<int4> parts, fin, items;
+    std::vector<int4> parts, fin, items, runs;
     int64_t slots = 0, part_entries = kMinPart;
 };
 int64_t part_entries_for(const std::vector<int64_t>& rowptr);
-// forced_part > 0: cut rows into parts of that many entries instead of the length part_entries_for would choose
-void bin_rows(const std::vector<int64_t>& rowptr, const std::vector<int32_t>& sub_off, RowWork& out, int64_t forced_part = 0);
+// forced_part > 0: cut rows into parts of that many entries instead of the length part_entries_for would choose.  by_runs [K]: subgraphs of `runs` cut into runs.
+void bin_rows(const std::vector<int64_t>& rowptr, const std::vector<int32_t>& sub_off, RowWork& out, int64_t forced_part, const std::vector<uint8_t>& by_runs);
 // Scratch slots bin_rows would use, from the row lengths alone.
 int64_t count_slots(const std::vector<int64_t>& rowptr);
 
@@ -82,7 +97,9 @@ struct SparseDev {
     const int64_t* rowptr = nullptr;  // [Np+1] (kept for the accessors; the kernels read the work list)
     const uint2* ecv = nullptr;       // [nnz] packed (column, value bits)
     const int4* fin = nullptr;        // rows made of several parts
-    const int4* items = nullptr;      // parts and uncut rows together, longest first inside a run of rows
+    const int4* items = nullptr;      // parts and uncut rows together, longest first inside a subgraph
+    const int4* runs = nullptr;       // the same, longest first inside a run of rows where a subgraph gains by it; or null
+    int64_t run_rows = 0;             // rows of the smallest of those subgraphs
     float* scratch = nullptr;         // [slots x leading dimension of the output] partial rows
     int32_t nfin = 0, nitems = 0;
     int64_t nrows = 0, nnz = 0;       // rows (and columns) of the store, its entries

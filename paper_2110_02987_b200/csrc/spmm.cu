@@ -3,7 +3,7 @@
 // the transposed store it is the backward aggregation dZ = A~^T dPre.
 //
 // Work list: every row, or every part of a row too long for one item, is an item {row, position of its first
-// entry, entries, scratch slot}; items are grouped by subgraph and, inside one, by runs of rows, longest first in each.  Operands wider
+// entry, entries, scratch slot}; items are grouped by subgraph, longest first in each (or in each run of rows: kRunOperandBytes).  Operands wider
 // than 64 columns take a warp per item, narrower ones a group of 4, 8 or 16 lanes per item; every lane owns 16
 // bytes of each operand row it gathers.  The parts of a cut row go to scratch slots and a second kernel adds them
 // in part order, so results never depend on scheduling.
@@ -349,8 +349,9 @@ static cudaError_t launch_rows(const SparseDev& A, const float* Z, int ldz, floa
             const unsigned grid = (unsigned)((A.nitems + kItemWarps - 1) / kItemWarps);
             // every byte of the operand within 4 GiB of its start: 32-bit offsets
             const bool off32 = (unsigned long long)A.nrows * (unsigned long long)OpBytes<BF>::elem * (unsigned long long)ldz < (1ull << 32);
+            const int4* items = A.runs && A.run_rows * (4ll * F4 * OpBytes<BF>::elem) >= kRunOperandBytes ? A.runs : A.items;
             auto go = [&](auto kernel) {
-                launch_share(kernel, dim3(grid), 32 * kItemWarps, kGatherSharedKB, s, A.ecv, A.items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
+                launch_share(kernel, dim3(grid), 32 * kItemWarps, kGatherSharedKB, s, A.ecv, items, A.nitems, Z, ldz, out, ldo, A.scratch, F4, ep);
             };
             // a bfloat16 operand of a whole number of 8-column runs: 16-byte loads, eight columns per lane and load
             const bool paired = BF && NV % 2 == 0 && F4 % 2 == 0 && ldz % 8 == 0;
@@ -440,10 +441,11 @@ __global__ void __launch_bounds__(256) check_store_kernel(const uint2* __restric
 cudaError_t launch_check_store(const SparseDev& A, long long nnz, long long slots, const int32_t* sub_off, int K, unsigned long long* bad,
                                cudaStream_t s) {
     const long long work = (long long)A.nitems + A.nfin;
-    if (work > 0) {
-        check_store_kernel<<<(unsigned)((work + 255) / 256), 256, 0, s>>>(A.ecv, nnz, A.items, A.nitems, A.fin, A.nfin, slots, A.nrows, sub_off, K, bad);
-        ++g_kernel_launches;
-    }
+    for (const int4* items : {A.items, A.runs})
+        if (items && work > 0) {
+            check_store_kernel<<<(unsigned)((work + 255) / 256), 256, 0, s>>>(A.ecv, nnz, items, A.nitems, A.fin, A.nfin, slots, A.nrows, sub_off, K, bad);
+            ++g_kernel_launches;
+        }
     return cudaGetLastError();
 }
 

@@ -279,17 +279,10 @@ int64_t count_slots(const std::vector<int64_t>& rowptr) {
     return slots;
 }
 
-// Rows whose items are ordered by length together.  Neighbouring rows of a graph that is numbered by community, time or site gather
-// the same operand rows: ordered by length over a whole subgraph the resident warps (9472) spread over all of it, and where its operand exceeds the
-// L2 (126 MB) those rows come from HBM again and again.  4 x 131 000 rows of 34 entries, 256 wide (134 MB a subgraph), 12 communities in each:
-// epochs of 6100 us without runs, 5995 with runs of 65 536 rows, 5915 of 32 768, 5900 of 16 384, 5900 of 4096; shorter runs mix long and short rows
-// in one CTA (16 x 13 000 rows of 35 entries: 1685 us with runs of 16 384, 1701 of 4096), subgraphs up to this size are one run.
-constexpr int64_t kItemWindow = 16384;
-
-void bin_rows(const std::vector<int64_t>& rowptr, const std::vector<int32_t>& sub_off, RowWork& out, int64_t forced_part) {
+void bin_rows(const std::vector<int64_t>& rowptr, const std::vector<int32_t>& sub_off, RowWork& out, int64_t forced_part, const std::vector<uint8_t>& by_runs) {
     const int64_t Np = (int64_t)rowptr.size() - 1;
     const int64_t part = forced_part > 0 ? forced_part : part_entries_for(rowptr);
-    out.perm.clear(); out.parts.clear(); out.fin.clear(); out.items.clear(); out.slots = 0; out.part_entries = part;
+    out.perm.clear(); out.parts.clear(); out.fin.clear(); out.items.clear(); out.runs.clear(); out.slots = 0; out.part_entries = part;
     std::vector<int64_t> count(64, 0);
     auto bin_of = [](int64_t len) { int b = 0; while (len > 1) { len >>= 1; ++b; } return b; };
     for (int64_t r = 0; r < Np; ++r) {
@@ -310,8 +303,8 @@ void bin_rows(const std::vector<int64_t>& rowptr, const std::vector<int32_t>& su
             out.parts.push_back(make_int4((int)r, (int)(q * pl), (int)std::min(pl, len - q * pl), (int)(out.slots + q)));
         out.slots += np;
     }
-    // the unified list: subgraph by subgraph (the operand rows one subgraph gathers stay together in L2), inside it by runs of
-    // kItemWindow rows, parts and uncut rows of a run longest first
+    // the unified list: subgraph by subgraph (the operand rows one subgraph gathers stay together in L2), parts and uncut rows of a subgraph
+    // longest first; and the same items once more with some subgraphs cut into runs of kItemWindow rows, longest first in each
     auto pack = [&](int64_t row, int64_t e0, int64_t len, int64_t slot) {
         return make_int4((int)row, (int)(uint32_t)(e0 & 0xFFFFFFFFll), (int)(uint32_t)(((e0 >> 32) << 16) | len), (int)slot);
     };
@@ -320,22 +313,30 @@ void bin_rows(const std::vector<int64_t>& rowptr, const std::vector<int32_t>& su
     for (int64_t k = 0; k < K; ++k)
         for (int64_t r = sub_off[k]; r < sub_off[k + 1]; ++r) sub_of[(size_t)r] = (int32_t)k;
     for (int4& f : out.fin) f.w = sub_of[(size_t)f.x];
-    std::vector<int64_t> first_run((size_t)K + 1, 0);
-    for (int64_t k = 0; k < K; ++k) first_run[(size_t)k + 1] = first_run[(size_t)k] + (sub_off[k + 1] - sub_off[k] + kItemWindow - 1) / kItemWindow;
-    auto key = [&](int64_t row, int64_t len) {
-        const size_t k = (size_t)sub_of[(size_t)row];
-        return (size_t)((first_run[k] + (row - sub_off[k]) / kItemWindow) * 64 + (63 - bin_of(len)));
+    auto order = [&](bool runs, std::vector<int4>& items) {
+        std::vector<int64_t> first_run((size_t)K + 1, 0), rows_of((size_t)K, 0);
+        for (size_t k = 0; k < (size_t)K; ++k) {
+            const int64_t rows = sub_off[k + 1] - sub_off[k];
+            rows_of[k] = runs && by_runs[k] ? kItemWindow : std::max<int64_t>(rows, 1);   // rows of a run
+            first_run[k + 1] = first_run[k] + (rows + rows_of[k] - 1) / rows_of[k];
+        }
+        auto key = [&](int64_t row, int64_t len) {
+            const size_t k = (size_t)sub_of[(size_t)row];
+            return (size_t)((first_run[k] + (row - sub_off[k]) / rows_of[k]) * 64 + (63 - bin_of(len)));
+        };
+        std::vector<int64_t> istart((size_t)first_run[(size_t)K] * 64 + 1, 0);
+        for (const int4& pt : out.parts) istart[key(pt.x, pt.z) + 1]++;
+        for (int32_t r : out.perm) istart[key(r, rowptr[r + 1] - rowptr[r]) + 1]++;
+        for (size_t i = 1; i < istart.size(); ++i) istart[i] += istart[i - 1];
+        items.resize((size_t)istart.back());
+        for (const int4& pt : out.parts) items[(size_t)istart[key(pt.x, pt.z)]++] = pack(pt.x, rowptr[pt.x] + pt.y, pt.z, pt.w);
+        for (int32_t r : out.perm) {
+            const int64_t len = rowptr[r + 1] - rowptr[r];
+            items[(size_t)istart[key(r, len)]++] = pack(r, rowptr[r], len, -1);
+        }
     };
-    std::vector<int64_t> istart((size_t)first_run[(size_t)K] * 64 + 1, 0);
-    for (const int4& pt : out.parts) istart[key(pt.x, pt.z) + 1]++;
-    for (int32_t r : out.perm) istart[key(r, rowptr[r + 1] - rowptr[r]) + 1]++;
-    for (size_t i = 1; i < istart.size(); ++i) istart[i] += istart[i - 1];
-    out.items.resize((size_t)istart.back());
-    for (const int4& pt : out.parts) out.items[(size_t)istart[key(pt.x, pt.z)]++] = pack(pt.x, rowptr[pt.x] + pt.y, pt.z, pt.w);
-    for (int32_t r : out.perm) {
-        const int64_t len = rowptr[r + 1] - rowptr[r];
-        out.items[(size_t)istart[key(r, len)]++] = pack(r, rowptr[r], len, -1);
-    }
+    order(false, out.items);
+    if (std::find(by_runs.begin(), by_runs.end(), 1) != by_runs.end()) order(true, out.runs);
 }
 
 }  // namespace gad

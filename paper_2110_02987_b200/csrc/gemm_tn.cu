@@ -367,7 +367,7 @@ cudaError_t launch_gemm_tn_tc(const void* mapH, const void* mapZ, int passes, in
     auto go = [&](auto kernel) {
         cudaError_t e = configure_kernel_once(reinterpret_cast<const void*>(kernel), SMEM_BYTES, false);
         if (e != cudaSuccess) return e;
-        e = launch_cluster(kernel, dim3((unsigned)(units * t.cg)), THREADS, SMEM_BYTES, (unsigned)t.cg, false, 0, s, *reinterpret_cast<const CUtensorMap*>(mapH),
+        e = launch_cluster(kernel, dim3((unsigned)(units * t.cg)), THREADS, SMEM_BYTES, (unsigned)t.cg, Early::kOverlap, 0, s, *reinterpret_cast<const CUtensorMap*>(mapH),
                    *reinterpret_cast<const CUtensorMap*>(mapZ), a);
         ++g_kernel_launches;
         return e;

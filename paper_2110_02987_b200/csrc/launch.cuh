@@ -35,8 +35,11 @@ PdlState& pdl_state();   // of this thread
 // Not where the kernels of the main sequence overlap: each change then waits for an SM that the overlap keeps busy (2708 rows: 163 -> 166 us an epoch).
 constexpr unsigned kGatherSharedKB = 32, kZetaSharedKB = 100;
 
+// When a kernel may come up ahead of the end of the one in front: never, where the whole main sequence overlaps, or as a finishing kernel too.
+enum class Early { kNever, kOverlap, kTail };
+
 template <class... P, class... Args>
-cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, unsigned cluster, bool tail, unsigned shared_kb, cudaStream_t s,
+cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, unsigned cluster, Early early, unsigned shared_kb, cudaStream_t s,
                            Args&&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = s;
@@ -48,8 +51,8 @@ cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, unsigned block, size
         ++cfg.numAttrs;
     }
     PdlState& st = pdl_state();
-    if ((st.on || st.tails) && s == st.stream) {
-        if (st.direct && (st.on || tail)) {
+    if ((st.on || st.tails) && s == st.stream && early != Early::kNever) {
+        if (st.direct && (st.on || early == Early::kTail)) {
             attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
             attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
             ++cfg.numAttrs;
@@ -65,18 +68,24 @@ cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, unsigned block, size
 }
 template <class... P, class... Args>
 cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, Args&&... args) {
-    return launch_cluster(kernel, grid, block, smem, 1, false, 0, s, std::forward<Args>(args)...);
+    return launch_cluster(kernel, grid, block, smem, 1, Early::kOverlap, 0, s, std::forward<Args>(args)...);
 }
 // The same for a kernel that asks for a share of the SM's memory (kGatherSharedKB, kZetaSharedKB).
 template <class... P, class... Args>
 cudaError_t launch_share(void (*kernel)(P...), dim3 grid, unsigned block, unsigned shared_kb, cudaStream_t s, Args&&... args) {
-    return launch_cluster(kernel, grid, block, 0, 1, false, shared_kb, s, std::forward<Args>(args)...);
+    return launch_cluster(kernel, grid, block, 0, 1, Early::kOverlap, shared_kb, s, std::forward<Args>(args)...);
+}
+// The same for a kernel of the side work.  It does not wait for the one in front (pdl_wait), so it never comes up early, on whatever stream: a pointer that
+// has passed through after_wait is no longer known to be read-only, and the importance statistics of 1200 features took 64 us that way instead of 44.
+template <class... P, class... Args>
+cudaError_t launch_beside(void (*kernel)(P...), dim3 grid, unsigned block, unsigned shared_kb, cudaStream_t s, Args&&... args) {
+    return launch_cluster(kernel, grid, block, 0, 1, Early::kNever, shared_kb, s, std::forward<Args>(args)...);
 }
 // A small kernel that only finishes what the one in front has left (rows cut into parts, sums of chunks): its blocks find room beside the
 // last ones in front on a store of any size (89 250 rows in 50 subgraphs: 912 -> 903 us an epoch; 70 000 of 60-60-60-5: 362 -> 356).
 template <class... P, class... Args>
 cudaError_t launch_tail(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, Args&&... args) {
-    return launch_cluster(kernel, grid, block, smem, 1, true, 0, s, std::forward<Args>(args)...);
+    return launch_cluster(kernel, grid, block, smem, 1, Early::kTail, 0, s, std::forward<Args>(args)...);
 }
 
 // A kernel of one or two blocks for every SM, each with work for several microseconds, does not come up early: its blocks would go where

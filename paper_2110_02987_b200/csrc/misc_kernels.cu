@@ -381,8 +381,6 @@ __global__ void __launch_bounds__(256) colsum_finish_kernel(const float* __restr
     __shared__ float seg_sm[256];
     const int k = blockIdx.x;
     const int2 r = clusters[k];
-    pdl_wait();
-    after_wait(colsum);
     const int c0 = (r.x + k) * 8, c1 = (r.y + k + 1) * 8;   // rows of the partial sums
     const int nseg = segments_for(ld), per = 256 / nseg;
     const int jl = threadIdx.x % per, seg = threadIdx.x / per;
@@ -399,7 +397,7 @@ __global__ void __launch_bounds__(256) colsum_finish_kernel(const float* __restr
     }
 }
 cudaError_t launch_colsum_finish(const float* colsum, int ld, const int2* clusters, int K, float* out, int64_t ostride, int64_t off, cudaStream_t s) {
-    launch_share(colsum_finish_kernel, dim3((unsigned)K), 256, kGatherSharedKB, s, colsum, ld, clusters, out, ostride, off);
+    launch_beside(colsum_finish_kernel, dim3((unsigned)K), 256, kGatherSharedKB, s, colsum, ld, clusters, out, ostride, off);
     ++g_kernel_launches;
     return cudaGetLastError();
 }
@@ -450,9 +448,6 @@ __global__ void __launch_bounds__(1024) zeta_finish_kernel(const double* __restr
                                               double* __restrict__ q_acc, int phase) {
     __shared__ double seg_a[1024], seg_b[1024];
     const int k = blockIdx.x;
-    pdl_wait();
-    after_wait(partial);
-    after_wait(q_acc);
     const long long n = sub_off[k + 1] - sub_off[k];
     if (n == 0) return;   // zero since creation
     const bool uniform = deg_sum[k] == 0;
@@ -510,8 +505,6 @@ __global__ void __launch_bounds__(256) zeta_partial_kernel(const float* __restri
     __shared__ double sm[8][32][8];
     const RowSpan c = chunks[blockIdx.x];
     const bool uniform = deg_sum[c.k] == 0;
-    pdl_wait();
-    after_wait(X);
     const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
     const int ld4 = ld >> 2, v = (int)blockIdx.y * 32 + cx;
     double* P = partial + (long long)blockIdx.x * 2 * ld;
@@ -556,8 +549,8 @@ cudaError_t launch_zeta(const float* X, int ld, int F, const int32_t* deg, const
                         const int32_t* chunk_ptr, const int32_t* sub_off, int K, const int64_t* deg_sum, const int64_t* deg_sq,
                         float beta, double* partial, double* zeta, double* q_acc, int phase, cudaStream_t s) {
     if (nchunks > 0) {
-        launch_share(zeta_partial_kernel, dim3((unsigned)nchunks, (unsigned)((ld / 4 + 31) / 32)), 256, kZetaSharedKB, s, X, ld, deg, chunks, sub_off, deg_sum, partial);
-        launch_share(zeta_finish_kernel, dim3((unsigned)K), 1024, kZetaSharedKB, s, partial, F, ld, chunk_ptr, sub_off, deg_sum, deg_sq, beta, zeta, q_acc, phase);
+        launch_beside(zeta_partial_kernel, dim3((unsigned)nchunks, (unsigned)((ld / 4 + 31) / 32)), 256, kZetaSharedKB, s, X, ld, deg, chunks, sub_off, deg_sum, partial);
+        launch_beside(zeta_finish_kernel, dim3((unsigned)K), 1024, kZetaSharedKB, s, partial, F, ld, chunk_ptr, sub_off, deg_sum, deg_sq, beta, zeta, q_acc, phase);
         g_kernel_launches += 2;
     }
     return cudaGetLastError();

@@ -1,5 +1,6 @@
 """Kernels that are launched through csrc/launch.cuh may come up before the kernel in front of them has finished (programmatic dependent launch), so each of
-them has to wait for it.  On the GPU a missing wait shows only where the overlap happens; here it is looked up in the sources."""
+them has to wait for it; those that do not wait go through launch_beside, which never lets a kernel come up early.  On the GPU a missing wait shows only
+where the overlap happens; here it is looked up in the sources."""
 import glob
 import os
 import re
@@ -50,8 +51,15 @@ CASES = [(f, k, body) for f, t in sources() for k, body in kernels(t).items() if
 
 def test_the_launches_are_found():
     names = {k for _, k, _ in CASES}
-    assert {"gemm_rows_kernel", "gemm_tn_kernel", "spmm_items_kernel", "spmm_finish_kernel", "reduce_chunks_kernel", "colsum_finish_kernel", "zeta_partial_kernel",
-            "zeta_finish_kernel", "step_sums_consensus_kernel", "narrow_bwd_kernel", "small_rows_kernel", "split_weights_kernel"} <= names, names
+    assert {"gemm_rows_kernel", "gemm_tn_kernel", "spmm_items_kernel", "spmm_finish_kernel", "reduce_chunks_kernel", "step_sums_consensus_kernel",
+            "narrow_bwd_kernel", "small_rows_kernel", "split_weights_kernel"} <= names, names
+
+
+def test_kernels_beside_never_come_up_early():
+    text = open(os.path.join(CSRC, "launch.cuh")).read()
+    body = text[text.index("launch_beside("):]
+    assert "Early::kNever" in body[:body.index("\n}")]
+    assert re.search(r"== st\.stream && early != Early::kNever\) \{", text)
 
 
 @pytest.mark.parametrize("file,kernel,body", CASES, ids=[k for _, k, _ in CASES])

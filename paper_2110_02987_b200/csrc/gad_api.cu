@@ -78,7 +78,7 @@ struct Plan {
     std::vector<RowSpan> zchunks;     // row chunks of the importance statistics, first chunk per subgraph [K+1]
     std::vector<int32_t> zchunk_ptr;
     size_t o_zchunks = 0, o_zchunk_ptr = 0;
-    struct DwChunks { std::vector<RowSpan> spans; std::vector<int32_t> ptr; size_t o_spans = 0, o_ptr = 0; };
+    struct DwChunks { std::vector<RowSpan> spans; std::vector<int32_t> ptr; int32_t most = 0; size_t o_spans = 0, o_ptr = 0; };   // most: of a subgraph
     std::vector<DwChunks> dw;         // [L] row chunks of each layer's weight gradient, their first chunk per subgraph [K+1]
     std::vector<int64_t> pair_ptr;    // [K+1] tiles of pairs per subgraph (zeta_mode 1 on the FP32 ALUs), else empty
     size_t o_pair_ptr = 0, o_pair_partial = 0;
@@ -199,6 +199,7 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
             for (int64_t r = sub_off[k]; r < sub_off[k + 1]; r += Rdw)
                 d.spans.push_back(RowSpan{(int32_t)r, (int32_t)std::min<int64_t>(Rdw, sub_off[k + 1] - r), k, 0});
             d.ptr[k + 1] = (int32_t)d.spans.size();
+            d.most = std::max(d.most, d.ptr[k + 1] - d.ptr[k]);
         }
         dw_floats = std::max(dw_floats, d.spans.size() * (size_t)y.fi * y.ldw);
     }
@@ -1122,7 +1123,7 @@ static int enqueue_epoch(gad_ctx* ctx, bool consensus) {
     // On a small store, whose epoch is a chain of short kernels, the update of a small model adds up the chunks of the last weight gradient itself (on larger
     // stores the kernel between them is 0.2 to 0.4 % of an epoch; behind a first layer on the FP32 ALUs it comes up early and is 0.3 us shorter than the longer update).
     ChunkSums sums{};
-    const bool sum_there = consensus && pdl_state().on && on_tc(ctx, 0) && p.pstride <= kStepSumsFloats && p.K <= kStepSumsReplicas;
+    const bool sum_there = consensus && pdl_state().on && on_tc(ctx, 0) && p.pstride <= kStepSumsFloats && p.K <= kStepSumsReplicas && p.dw[0].most <= kStepSumsChunks;
     if ((rc = backward_pass(ctx, ss, sum_there ? &sums : nullptr)) != GAD_OK) return rc;
     if (ss == ctx->stream && (rc = zeta_pass(ctx, ss)) != GAD_OK) return rc;
     if ((rc = hand_over(ctx, ss, ctx->stream, ctx->ev_join)) != GAD_OK) return rc;

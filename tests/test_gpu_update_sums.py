@@ -1,5 +1,5 @@
 """The update of small models, which adds up the chunks of the last weight gradient: numbers of replicas around what a block takes at a time, layers whose
-end falls inside a block, chunks around eight to a replica, copies that differ, and models on either side of the size from which it does not."""
+end falls inside a block, chunks around eight to a replica, copies that differ, and models on either side of the size and of the number of chunks from which it does not."""
 import numpy as np
 import pytest
 
@@ -40,7 +40,8 @@ def test_replicas_and_layers(K, dims, differ):
     check(g, ref, K, differ)
 
 
-@pytest.mark.parametrize("n,dims", [(40, (500, 511, 3)), (40, (500, 530, 3)), (6000, (9, 6, 3)), (9500, (40, 24, 3))])
+@pytest.mark.parametrize("n,dims", [(40, (500, 511, 3)), (40, (500, 530, 3)), (6000, (9, 6, 3)), (9500, (40, 24, 3)),
+                                    (1536, (40, 24, 3)), (1537, (40, 24, 3))])   # (chunks of 32 rows: 32 and 33 in the larger subgraph)
 def test_sizes_and_chunks(n, dims):
     u = np.arange(n)
     col = np.sort(np.stack([(u - 1) % n, (u + 1) % n], 1), axis=1).astype(np.int32).ravel()

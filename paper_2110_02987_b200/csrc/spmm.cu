@@ -270,7 +270,7 @@ __device__ __forceinline__ void gather_tail(float4 (&acc)[NV], const uint2* st, 
 // Operand rows in flight per lane and resident warps asked of the compiler: short items make the chain
 // item -> entries -> operand rows the cost, and more resident warps hide it better than more loads per warp (128 columns: 2 rows and 64 warps 53 us,
 // 4 and 48 61, 8 and 32 68; 78 / 87 / 106 on 100 000 rows).  129 to 256 columns have a second form (DEEP): four rows and 28 warps in place of
-// two and 40.  It is the better one for long rows, and for bfloat16 operands that cannot be read in pairs whatever the rows' length
+// two and 40.  It is the better one for long rows, for few items, and for bfloat16 operands that cannot be read in pairs whatever the rows' length
 // (110 000 rows of 25 entries, 132, 196 and 252 columns: 131 -> 124, 136 -> 127, 140 -> 131 us; 63 000 of 230: 467 -> 417, 474 -> 424, 479 -> 425).
 constexpr int kItemWarps = 4;
 // fp32 operands of 129 to 256 columns: entries a row, on average, from which the deep form is taken.  us with two rows in flight / with four, by
@@ -279,6 +279,12 @@ constexpr int kItemWarps = 4;
 // 149 / 151, 182 / 180; 60 (110 000, 256) 325 / 326; 66 (420 000, 256) 1557 / 1569; 79 (63 000; 160, 256) 195 / 193, 234 / 232; 106 (110 000, 256) 526 / 516;
 // 110 (63 000; 160, 256) 270 / 268, 318 / 310; 160 (110 000, 256) 798 / 778; 230 (63 000; 132, 160, 192, 224, 256) 572 / 567, 539 / 533, 544 / 537, 578 / 565, 616 / 601.
 constexpr int64_t kDeepEntries = 72;
+// It is also taken where a launch has few items, so that the warps that fit are not what it is short of.  By rows of the store, 136 and 256 columns, power-law rows
+// of 5 and 25 entries / rows of equal length: 1600 rows 12.9 / 10.6, 12.9 / 10.8, 17.5 / 15.2, 17.8 / 15.4 us and 8.6 / 7.6, 8.6 / 7.7, 10.6 / 8.7, 10.8 / 8.7; 6300 18.5 / 16.2, 19.0 / 16.7,
+// 19.6 / 18.9, 19.4 / 19.3 and 8.7 / 8.7, 8.7 / 9.2, 13.7 / 14.9, 14.8 / 14.9; 14 700 22.3 / 20.6, 23.7 / 23.4, 30.1 / 30.0, 31.7 / 30.5 and 12.7 / 12.9, 13.7 / 14.8, 22.0 / 22.2, 24.2 / 24.2;
+// 21 000 26.7 / 24.3, 28.6 / 27.1, 36.8 / 37.0, 39.5 / 38.6 and 15.8 / 16.8, 17.7 / 19.1, 28.2 / 29.2, 31.5 / 32.2; 42 000 37.4 / 37.5, 38.8 / 38.9, 61.2 / 63.7, 67.4 / 70.6 and 25.2 / 29.1,
+// 27.3 / 31.1, 48.6 / 50.8, 53.8 / 55.9.
+constexpr int kDeepItems = 16384;
 template <int NV, bool PAIR, bool DEEP> struct ItemCfg {
     // (PAIR: half the bytes per operand row, twice the rows in flight)
     static constexpr int UU = (PAIR ? 2 : 1) * (DEEP ? 4 : NV <= 4 ? 2 : 1);
@@ -360,7 +366,7 @@ static cudaError_t launch_rows(const SparseDev& A, const float* Z, int ldz, floa
                 else if (paired) go(spmm_items_kernel<NV, EPI, false, true, true, false>);
             }
             if constexpr (NV == 2) {
-                if (!paired && (BF || A.nnz >= kDeepEntries * A.nrows)) {
+                if (!paired && (BF || A.nnz >= kDeepEntries * A.nrows || A.nitems <= kDeepItems)) {
                     if (off32) go(spmm_items_kernel<2, EPI, true, BF, false, true>);
                     else go(spmm_items_kernel<2, EPI, false, BF, false, true>);
                 } else if constexpr (!BF) {

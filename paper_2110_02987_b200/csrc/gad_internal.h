@@ -288,10 +288,10 @@ cudaError_t launch_sgd_consensus(float* params, int64_t pstride_p, const float* 
 // The same with a step where the gradients of the parameters [4 first4, 4 (first4 + count4)) have yet to be added up, chunk by chunk in order; they are written
 // to grads.  For at most kStepSumsFloats parameters, kStepSumsReplicas replicas and kStepSumsChunks chunks in each: a warp reads a replica's chunks eight at a
 // time, one after the other.  1750 nets of up to 262 144 parameters and 48 000 rows, mean change of an epoch against a kernel of its own by the most chunks
-// a replica has: up to 8 -3.8 us, 16 -2.6, 24 -1.4, 32 -2.2, 40 -0.1, 48 +1.1, 72 +3.4, 100 and more +10 (23 700 rows of 27-129-13 in one subgraph: 127 -> 140).
-// At the limit of parameters (2700 to 42 000 rows, 2 to 50 replicas of 0.23 to 0.26 M) 0 to 10 us less.
+// a replica has: up to 8 -3.8 us, 16 -2.6, 24 -1.4, 32 -2.2, 64 0 (more than 64 000 parameters less: 1509 rows of 225-493-13, 47 chunks, 142 -> 126), 72 +3.4, 100 and more
+// +10 (23 700 rows of 27-129-13 in one subgraph: 127 -> 140).  At the limit of parameters (2700 to 42 000 rows, 2 to 50 replicas of 0.23 to 0.26 M) 0 to 10 us less.
 struct ChunkSums { long long first4, count4; const float4* partial; long long stride4; const int32_t* chunk_ptr; };
-constexpr int64_t kStepSumsFloats = 256 << 10, kStepSumsReplicas = 4096, kStepSumsChunks = 32;
+constexpr int64_t kStepSumsFloats = 256 << 10, kStepSumsReplicas = 4096, kStepSumsChunks = 64;
 cudaError_t launch_step_sums_consensus(float* params, int64_t pstride_p, float* grads, int64_t pstride, int64_t len, int K, float lr, const double* zeta,
                                        int weighted, int32_t* words, long long* epoch, const float* report, float* report_to, int nreport,
                                        const ChunkSums& sums, cudaStream_t s);

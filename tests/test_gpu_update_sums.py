@@ -41,7 +41,7 @@ def test_replicas_and_layers(K, dims, differ):
 
 
 @pytest.mark.parametrize("n,dims", [(40, (500, 511, 3)), (40, (500, 530, 3)), (6000, (9, 6, 3)), (9500, (40, 24, 3)),
-                                    (1536, (40, 24, 3)), (1537, (40, 24, 3))])   # (chunks of 32 rows: 32 and 33 in the larger subgraph)
+                                    (3072, (40, 24, 3)), (3073, (40, 24, 3))])   # (chunks of 32 rows: 64 and 65 in the larger subgraph)
 def test_sizes_and_chunks(n, dims):
     u = np.arange(n)
     col = np.sort(np.stack([(u - 1) % n, (u + 1) % n], 1), axis=1).astype(np.int32).ravel()

@@ -72,6 +72,7 @@ struct Plan {
     std::vector<int32_t> ld;          // [L+1]
     int32_t maxld = 0;
     std::vector<RowSpan> pair_tiles;  // 128-row tiles, an even number per subgraph (the last may be empty)
+    std::vector<int32_t> fwd_bn, back_bn;   // [L] output columns per tile of each layer's transform, and of the one back through it
     size_t o_pair_tiles = 0;
     std::vector<RowSpan> tiles, chunks, core_spans;
     std::vector<int32_t> chunk_ptr;   // [K+1]
@@ -217,6 +218,12 @@ int make_plan(Plan& p, int32_t n, int32_t K, const std::vector<int32_t>& sub_off
         p.chunk_ptr[k + 1] = (int32_t)p.chunks.size();
         for (int64_t r = 0; r < core_count[k]; r += 256)
             p.core_spans.push_back(RowSpan{(int32_t)(sub_off[k] + r), (int32_t)std::min<int64_t>(256, core_count[k] - r), k, 0});
+    }
+    for (int l = 0; l < p.L; ++l) {
+        const Layer& y = p.layers[l];
+        const int npairs = (int)(p.pair_tiles.size() / 2);
+        p.fwd_bn.push_back(cfg->gemm_mode == 1 ? tc_rows_bn_whole(y.fo, npairs) : tc_rows_bn(y.fo, npairs, y.fi, cfg->dropout > 0.f && p.agg_first[l] && l < p.L - 1));
+        p.back_bn.push_back(tc_rows_bn_whole(y.fi, npairs));
     }
     int32_t max_spmm_ld = 4;   // a layer's SpMMs run at its input width when it aggregates first, else at its output width
     for (int l = 0; l < p.L; ++l) max_spmm_ld = std::max(max_spmm_ld, p.ld[p.agg_first[l] ? l : l + 1]);
@@ -544,7 +551,7 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t fork = nullptr) {
             const ActEpi act = make_act(ep, 0);
             GAD_RUN("gemm_fwd", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
                 if (on_tc(ctx, l))
-                    return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 2, passes, y.fi, y.fo,
+                    return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 2, passes, y.fi, y.fo, p.fwd_bn[l],
                                                ctx->H(l + 1), y.ldo, ctx->at<RowSpan>(p.o_pair_tiles), (int)(p.pair_tiles.size() / 2), nullptr, 0, 1.f, &act,
                                                ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params);
                 return launch_gemm_rows_simt(2, ctx->at<float>(p.o_P[l]), y.ldi, y.fi, params, pstride, y.w_int, y.ldw, y.fo, ctx->H(l + 1), y.ldo,
@@ -556,7 +563,7 @@ int forward_pass(gad_ctx* ctx, bool train, cudaStream_t fork = nullptr) {
         void* zb = on_tc(ctx, l) ? bf16_of(ctx) : nullptr;
         GAD_RUN("gemm_fwd", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
             if (on_tc(ctx, l))
-                return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 0, passes, y.fi, y.fo, Z,
+                return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 0], &ctx->maps[kMapsPerLayer * l + 1], &ctx->maps[kMapsPerLayer * l + 2], 0, passes, y.fi, y.fo, p.fwd_bn[l], Z,
                                            y.ldo, ctx->at<RowSpan>(p.o_pair_tiles), (int)(p.pair_tiles.size() / 2), train ? ctx->bits(l) : nullptr, bit_words_of(y.ldi), 1.f, nullptr,
                                            ctx->at<int32_t>(p.o_flags) + 1, ctx->num_sms, ctx->stream, ctx->same_params, zb);
             return launch_gemm_rows_simt(0, ctx->H(l), y.ldi, y.fi, params, pstride, y.w_int, y.ldw, y.fo, Z, y.ldo,
@@ -697,7 +704,7 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss, ChunkSums* sums) {
             GAD_RUN("gemm_dh", l, 4.0 * p.Np * (y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
                 if (on_tc(ctx, l))
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 3], &ctx->maps[kMapsPerLayer * l + 4], &ctx->maps[kMapsPerLayer * l + 5], 1,
-                                               ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G2, y.ldi, ctx->at<RowSpan>(p.o_pair_tiles),
+                                               ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, p.back_bn[l], G2, y.ldi, ctx->at<RowSpan>(p.o_pair_tiles),
                                                (int)(p.pair_tiles.size() / 2), nullptr, 0, 1.f, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
                                                ctx->num_sms, ctx->stream, ctx->same_params);
                 return launch_gemm_rows_simt(1, G1, y.ldo, y.fo, params, pstride, y.w_int, y.ldw, y.fi, G2, y.ldi,
@@ -718,7 +725,7 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss, ChunkSums* sums) {
         GAD_RUN("gemm_dh", l, 4.0 * p.Np * (2.0 * y.fi + y.fo) + 4.0 * p.K * y.fi * y.fo, 2.0 * p.Np * y.fi * y.fo, [&] {
                 if (on_tc(ctx, l))
                     return launch_gemm_rows_tc(&ctx->maps[kMapsPerLayer * l + 3], &ctx->maps[kMapsPerLayer * l + 4], &ctx->maps[kMapsPerLayer * l + 5], 1,
-                                               ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, G1, y.ldi, ctx->at<RowSpan>(p.o_pair_tiles),
+                                               ctx->cfg.gemm_mode == 0 ? 3 : 1, y.fo, y.fi, p.back_bn[l], G1, y.ldi, ctx->at<RowSpan>(p.o_pair_tiles),
                                                (int)(p.pair_tiles.size() / 2), ctx->bits(l), bit_words_of(y.ldi), scale, nullptr, ctx->at<int32_t>(p.o_flags) + 1,
                                                ctx->num_sms, ctx->stream, ctx->same_params, out_bf16 ? bf16_of(ctx) : nullptr,
                                                sums ? ctx->at<float>(p.o_colsum) : nullptr);
@@ -1025,12 +1032,12 @@ int gad_create(gad_ctx** out, const gad_csr* g, const gad_partition* part, const
             const bool agg_first = p.agg_first[l] != 0;   // then the transform and the weight gradient read A~ H^(l), dW and dH read dPre (G1)
             float* Hin = agg_first ? ctx->at<float>(p.o_P[l]) : ctx->H(l);
             ok = ok && tc_make_map(&m[0], Hin, y.fi, p.Np, 0, 4ull * y.ldi, 0, 128);
-            ok = ok && tc_make_map(&m[1], ctx->at<float>(p.o_wt_hi[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, tc_rows_bn(y.fo, npairs, cfg->gemm_mode == 1) / 2);
-            ok = ok && tc_make_map(&m[2], ctx->at<float>(p.o_wt_lo[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, tc_rows_bn(y.fo, npairs, cfg->gemm_mode == 1) / 2);
+            ok = ok && tc_make_map(&m[1], ctx->at<float>(p.o_wt_hi[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, p.fwd_bn[l] / 2);
+            ok = ok && tc_make_map(&m[2], ctx->at<float>(p.o_wt_lo[l]), y.fi, y.fo, p.K, 4ull * y.ldi, 4ull * y.fo * y.ldi, p.fwd_bn[l] / 2);
             // input gradient: A = dZ [Np x fo] (in G2), B = W copies [K][fi][fo]
             ok = ok && tc_make_map(&m[3], ctx->at<float>(agg_first ? p.o_G1 : p.o_G2), y.fo, p.Np, 0, 4ull * y.ldo, 0, 128);
-            ok = ok && tc_make_map(&m[4], ctx->at<float>(p.o_w_hi[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, tc_rows_bn(y.fi, npairs, true) / 2);
-            ok = ok && tc_make_map(&m[5], ctx->at<float>(p.o_w_lo[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, tc_rows_bn(y.fi, npairs, true) / 2);
+            ok = ok && tc_make_map(&m[4], ctx->at<float>(p.o_w_hi[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, p.back_bn[l] / 2);
+            ok = ok && tc_make_map(&m[5], ctx->at<float>(p.o_w_lo[l]), y.fo, y.fi, p.K, 4ull * y.ldw, 4ull * y.fi * y.ldw, p.back_bn[l] / 2);
             // weight gradient: 32-row tiles of H^(l) and of dZ (in G2)
             ok = ok && tc_make_map(&m[6], Hin, y.fi, p.Np, 0, 4ull * y.ldi, 0, tc_tn_rows(), true);
             ok = ok && tc_make_map(&m[7], ctx->at<float>(agg_first ? p.o_G1 : p.o_G2), y.fo, p.Np, 0, 4ull * y.ldo, 0, tc_tn_rows(), true);

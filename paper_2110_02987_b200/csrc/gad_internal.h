@@ -176,7 +176,8 @@ cudaError_t launch_gemm_rows_simt(int mode, const float* A, int lda, int Kd, con
 // Tensor-core (tcgen05) version of launch_gemm_rows_simt.  The operands come through TMA descriptors made by
 // tc_make_map (A: [rows x Kd]; B, B_lo: [K][N][Kd] copies written by launch_split_weights); passes = 3 gives fp32
 // accuracy by operand splitting, passes = 1 plain TF32 operands.  err receives a role code if a bounded wait runs out.
-int tc_rows_bn(int n_cols, int npairs, bool whole);
+int tc_rows_bn(int n_cols, int npairs, int Kd, bool drop);   // columns per tile of a forward transform in three passes (drop: with dropout in its epilogue)
+int tc_rows_bn_whole(int n_cols, int npairs);                // of the others
 int tc_tn_rows();   // rows of the row-box descriptors the weight-gradient kernel reads (mapH / mapZ of launch_gemm_tn_tc)
 bool tc_make_map(void* out_map, const void* base, uint64_t inner, uint64_t rows, uint64_t outer, uint64_t row_stride_bytes,
                  uint64_t outer_stride_bytes, uint32_t box_rows, bool mn_major = false, bool half = false);
@@ -190,13 +191,13 @@ struct SplitLayers {
     SplitLayer y[MAX];
 };
 cudaError_t launch_split_weights(const float* params, int64_t pstride, int K, const SplitLayer* layers, int L, cudaStream_t s);
-// pair_tiles: 2 npairs row tiles (at most 128 rows, or none), the two of a pair in the same subgraph; tc_rows_bn columns
+// pair_tiles: 2 npairs row tiles (at most 128 rows, or none), the two of a pair in the same subgraph; bn (tc_rows_bn, tc_rows_bn_whole) columns
 // per tile, half of them the rows of B's descriptor box.  bits: with mode 0 (may be null) the transform leaves there which values of A are above
 // zero, bit c % 32 of word c / 32 of a row of bit_words words; mode 1 masks with such bits (null: no mask), 1/32 of the bytes of the activations.  one_b: the operand copies of replica 0 serve every subgraph.
 // Cbf16 (mode 0, or 1 with a mask; may be null): the result goes there as bfloat16 [rows x ldc] INSTEAD of to C - the operand copy the
 // reduced-precision aggregation gathers, written by its producer.  colsum (mode 1 with a mask, where tc_rows_sums_columns): the
 // column sums of the result, for launch_colsum_finish.
-cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols,
+cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols, int bn,
                                 float* C, int ldc, const RowSpan* pair_tiles, int npairs, uint32_t* bits, int bit_words, float scale,
                                 const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16 = nullptr, float* colsum = nullptr);
 inline int32_t bit_words_of(int32_t ld) { return (ld + 31) / 32; }

@@ -88,6 +88,7 @@ enum Form { kOnePass, kSharedLo, kTensorMem };
 constexpr int ACC_COLS = 128;                   // columns between the accumulators there (the other forms: as many as the tile has)
 constexpr int SLOTS = 4, SLOT_COLS = 2 * BK;   // tensor-memory slots of a 128 x 32 step of A: 32 columns of hi, 32 of lo
 constexpr uint32_t TMEM_COLS = 512;
+constexpr int kRowPairs = 74;                   // pairs of CTAs at work at a time
 
 template <int DRAIN, int FORM>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
@@ -462,19 +463,33 @@ namespace {
 // size (written and read by the split, read by three MMAs); with 256 columns a tile's two accumulators fill the tensor memory.
 int form_for(int BN, int passes) { return passes <= 1 ? kOnePass : BN <= 128 ? kTensorMem : kSharedLo; }
 
+// What a resident B (both parts) leaves for A.
+long long room_beside_b(int BN, int Kd) { return (long long)DATA_BYTES - (long long)((Kd + BK - 1) / BK) * 2 * (BN / 2) * (BK * 4); }
+// Turns of the CTA pairs that a launch of ntn column tiles takes, and whether a launch is one of few turns (in tiles of 256 columns).
+long long turns_of(int npairs, int ntn) { return ((long long)npairs * ntn + kRowPairs - 1) / kRowPairs; }
+bool few_turns(int npairs, int n_cols) { return turns_of(npairs, (n_cols + 255) / 256) < 4; }
+// Through tensor memory: whether B stays for all row tiles.  With several column tiles that means that A is read from HBM for each of them, where a streamed B
+// lets it come from L2 the second time, so that on large launches it pays only for reductions of at most four steps whose rows of A share 32-byte sectors (a
+// leading dimension that is no multiple of 8).  525 000 rows, us resident / streamed: 100 -> 256 168 / 231, 33 -> 320 without an epilogue 141 / 170; but 64 -> 256 144 / 145,
+// 128 -> 384 193 / 180, without an epilogue 192 -> 192 224 / 209, 129 -> 320 275 / 244 and 300 000 rows of 146 -> 267 246 / 181, with dropout 100 -> 300 455 / 369; and where a tile's
+// worth of columns is only just passed 100 -> 257 346 / 255, 24 -> 129 163 / 105.  Of few turns: 21 000 rows, 100 -> 150 19 / 19, 128 -> 256 21 / 20, 129 -> 300 27 / 25.
+bool keeps_b(int BN, int Kd, int n_cols, int npairs, bool drop) {
+    if (room_beside_b(BN, Kd) < SLOTS * A_BYTES) return false;
+    if (n_cols <= BN) return true;
+    if (Kd > 4 * BK) return false;
+    return few_turns(npairs, n_cols) || (!drop && round_up(Kd, 4) % 8 != 0 && (n_cols - 1) % 128 >= 8);
+}
+
 // Where the data of a CTA goes: four lo tiles if at least as many ring stages fit beside them, else two; B resident if at least
 // three ring stages fit beside it.
-void rows_layout(int BN, int Kd, int form, RowsArgs& a) {
+void rows_layout(int BN, int Kd, int n_cols, int form, RowsArgs& a) {
     const int passes = form == kOnePass ? 1 : 3;
     const int nkb = (Kd + BK - 1) / BK, nb = passes > 1 ? 2 : 1;
     const int b_bytes = BN / 2 * (BK * 4);
     if (form == kTensorMem) {   // as many stages as there are slots, at least (see the split)
-        const long long room_a = (long long)DATA_BYTES - (long long)nkb * nb * b_bytes;
         a.nlo = SLOTS;
-        // (with several column tiles a resident B means that A is read from HBM for each of them, a streamed one that it comes from L2 the second time:
-        // 256 -> 256 over 525 000 rows 316 us resident, 297 streamed; 100 -> 256 162 and 203)
-        a.resident = room_a >= SLOTS * A_BYTES && (a.ntn == 1 || nkb <= 4) ? 1 : 0;
-        a.nst = (int)std::min<long long>(MAX_STAGES, a.resident ? room_a / A_BYTES : DATA_BYTES / (A_BYTES + nb * b_bytes));
+        a.resident = keeps_b(BN, Kd, n_cols, a.npairs, a.act.drop != 0) ? 1 : 0;
+        a.nst = (int)std::min<long long>(MAX_STAGES, a.resident ? room_beside_b(BN, Kd) / A_BYTES : DATA_BYTES / (A_BYTES + nb * b_bytes));
         return;
     }
     for (a.nlo = 4;; a.nlo = 2) {
@@ -495,37 +510,50 @@ int max_clusters(int num_sms) {
 
 }  // namespace
 
-// Output columns per tile.  A tile that should hold all columns (`whole`: one pass, whose MMAs cost little beside reading A again, or a masked drain,
-// which sums columns) is as wide as the layer, up to 256.  Else the columns are cut into equal tiles of at most 128, whose A goes
-// through tensor memory: 500 -> 256 over 20 700 rows (84 row tiles for 74 pairs of CTAs: two turns of 256 columns, three of 128) 45.6 -> 35.9 us,
-// 602 -> 256 over 63 000 89 -> 78, 100 -> 256 over 525 000 170 -> 162, 256 -> 256 300 -> 297; in one pass 256 -> 256 over 210 000 rows 86 in tiles
-// of 256 columns, 104 of 128.  Where a launch has so few row tiles that most SMs would idle the columns are spread over more CTAs, down to 32
+// Output columns per tile.  Where a launch has so few row tiles that most SMs would idle the columns are spread over more CTAs, down to 32
 // (2843 rows x 1433 -> 128: 24 row tiles, 40 us with 128 columns per tile, 27 us with 32).
-int tc_rows_bn(int n_cols, int npairs, bool whole) {
-    int bn;
-    if (whole) bn = n_cols <= 32 ? 32 : n_cols <= 64 ? 64 : n_cols <= 128 ? 128 : 256;
-    else { const int ntn = (n_cols + 127) / 128; bn = (int)round_up((n_cols + ntn - 1) / ntn, 32); }
-    while (bn > 32 && (long long)npairs * ((n_cols + bn - 1) / bn) * 2 <= 74) bn = (int)round_up(bn / 2, 32);
+static int spread_columns(int bn, int n_cols, int npairs) {
+    while (bn > 32 && (long long)npairs * ((n_cols + bn - 1) / bn) * 2 <= kRowPairs) bn = (int)round_up(bn / 2, 32);
     return bn;
+}
+// The transform back through a layer, in one pass or three, and every transform in one pass, whose MMAs cost little beside reading A again (256 -> 256 over
+// 210 000 rows 86 us in tiles of 256 columns, 104 of 128): as wide as the layer, up to 256, so that a masked drain can sum the columns.
+int tc_rows_bn_whole(int n_cols, int npairs) {
+    return spread_columns(n_cols <= 32 ? 32 : n_cols <= 64 ? 64 : n_cols <= 128 ? 128 : 256, n_cols, npairs);
+}
+// A forward transform in three passes: equal tiles of at most 128 columns, whose A goes through tensor memory, or on large launches the same as above.
+// Such a tile costs about half of one of 256 columns, a little more where the drain is what the kernel waits for (reductions of up to 96 values, dropout) or B is
+// streamed beside rows of A that share sectors; there that many turns of the CTA pairs have to come out shorter.  us in tiles of 256 / of up to 128 columns:
+// 21 000 rows in 8 subgraphs (two turns or three half ones) 500 -> 256 46 / 38, 100 -> 256 24 / 20, with dropout 100 -> 257 47 / 35; 525 000 rows 24 -> 256 121 / 139, 100 -> 256
+// 178 / 168, 24 -> 150 80 / 113, 256 -> 256 280 / 287 and without an epilogue 303 / 291, 64 -> 300 220 / 166; with dropout 128 -> 150 240 / 262, 256 -> 256 381 / 412,
+// 100 -> 300 506 / 369.  1500 combinations of 24 to 500 -> 129 to 512, four sizes, with and without an epilogue and dropout: 10 % less than in wide tiles (the best of all
+// forms for each: 11), 4 % less than in narrow ones throughout, at most 10 % above the best of the two.
+int tc_rows_bn(int n_cols, int npairs, int Kd, bool drop) {
+    const int ntn = (n_cols + 127) / 128, bn = (int)round_up((n_cols + ntn - 1) / ntn, 32);
+    if (n_cols > 128 && !few_turns(npairs, n_cols)) {
+        const bool half = !drop && Kd > 96 && (round_up(Kd, 4) % 8 == 0 || Kd > 160 || keeps_b(bn, Kd, n_cols, npairs, drop));
+        if ((double)turns_of(npairs, ntn) * (half ? 0.5 : 0.55) > (double)turns_of(npairs, (n_cols + 255) / 256)) return tc_rows_bn_whole(n_cols, npairs);
+    }
+    return spread_columns(bn, n_cols, npairs);
 }
 
 // The drain can sum columns when a tile holds all of them.
-bool tc_rows_sums_columns(int n_cols, int npairs) { return tc_rows_bn(n_cols, npairs, true) >= n_cols; }
+bool tc_rows_sums_columns(int n_cols, int npairs) { return tc_rows_bn_whole(n_cols, npairs) >= n_cols; }
 int tc_rows_clusters(long long ntiles, int num_sms) { return (int)std::min<long long>(ntiles, std::min(max_clusters(num_sms), kMaxRowClusters)); }
 
-cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols,
+cudaError_t launch_gemm_rows_tc(const void* mapA, const void* mapB, const void* mapBlo, int mode, int passes, int Kd, int n_cols, int bn,
                                 float* C, int ldc, const RowSpan* pair_tiles, int npairs, uint32_t* bits, int bit_words, float scale,
                                 const ActEpi* act, int32_t* err, int num_sms, cudaStream_t s, bool one_b, void* Cbf16, float* colsum) {
     if (npairs <= 0) return cudaSuccess;
     if ((mode == 2 && !act) || (Cbf16 && mode == 2) || (Cbf16 && mode == 1 && !bits)) return cudaErrorInvalidValue;
-    if (colsum && !(mode == 1 && bits && tc_rows_sums_columns(n_cols, npairs))) return cudaErrorInvalidValue;
+    if (colsum && !(mode == 1 && bits && bn >= n_cols)) return cudaErrorInvalidValue;
     RowsArgs a;
-    a.tiles = pair_tiles; a.npairs = npairs; a.BN = tc_rows_bn(n_cols, npairs, passes <= 1 || mode == 1); a.ntn = (ldc + a.BN - 1) / a.BN; a.Kd = Kd;
+    a.tiles = pair_tiles; a.npairs = npairs; a.BN = bn; a.ntn = (ldc + a.BN - 1) / a.BN; a.Kd = Kd;
+    a.act = act ? *act : ActEpi{};
     const int form = form_for(a.BN, passes);
-    rows_layout(a.BN, Kd, form, a);
+    rows_layout(a.BN, Kd, n_cols, form, a);
     a.C = C; a.Cbf = reinterpret_cast<uint32_t*>(Cbf16); a.ldc = ldc; a.bits = mode == 2 ? nullptr : bits; a.bit_words = bit_words; a.scale = scale; a.colsum = colsum;
     a.kmul = one_b ? 0 : 1; a.err = err;
-    a.act = act ? *act : ActEpi{};
     const unsigned grid = 2u * (unsigned)tc_rows_clusters((long long)npairs * a.ntn, num_sms);
     const int drain = mode == 2 ? (a.act.drop ? kActDrop : kAct) : mode == 1 && bits ? (Cbf16 ? kMaskBf16 : kMask) : Cbf16 ? kBf16 : kPlain;
     auto go = [&](auto kernel) {

@@ -530,22 +530,17 @@ int check_columns(const gad_csr* g, std::string& err) {
     return GAD_OK;
 }
 
-// rowptr must not decrease; the longest row.
-int check_rows(const gad_csr* g, int64_t& longest, std::string& err) {
-    int down = 0;
-    int64_t most = 0;
-#pragma omp parallel for schedule(static) reduction(| : down) reduction(max : most) if (g->n > (1 << 16))
-    for (int32_t v = 0; v < g->n; ++v) {
-        const int64_t len = g->rowptr[v + 1] - g->rowptr[v];
-        down |= len < 0;
-        most = std::max(most, len);
-    }
-    longest = most;
-    if (down) { err = "rowptr decreases"; return GAD_ERR_UNSORTED; }
+// rowptr must not decrease.  lengths: the bits that occur in the rows' lengths (a negative one would bring the sign).
+int check_rows(const gad_csr* g, int64_t& lengths, std::string& err) {
+    int64_t bits = 0;
+#pragma omp parallel for schedule(static) reduction(| : bits) if (g->n > (1 << 16))
+    for (int32_t v = 0; v < g->n; ++v) bits |= g->rowptr[v + 1] - g->rowptr[v];
+    lengths = bits;
+    if (bits < 0) { err = "rowptr decreases"; return GAD_ERR_UNSORTED; }
     return GAD_OK;
 }
 // Every row's start and length fit a WalkNode.  (Columns may repeat, so that a row can be longer than there are nodes.)
-bool walks_pack(int64_t nnz, int64_t longest) { return nnz < kMaxPackedEntries && longest < kMaxPackedRow; }
+bool walks_pack(int64_t nnz, int64_t lengths) { return nnz < kMaxPackedEntries && lengths < kMaxPackedRow; }
 
 // `columns`: check them here; else the caller does (check_columns).
 int plan_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int32_t* core_nodes, const gad_augment_config* cfg, AugPlan& p,
@@ -555,9 +550,9 @@ int plan_augment(const gad_csr* g, int32_t K, const int64_t* core_ptr, const int
     if (!(cfg->alpha >= 0.0) || !(cfg->E > 0.0) || !(cfg->zc > 0.0) || cfg->cap < 1) { err = "alpha >= 0, E > 0, zc > 0, cap >= 1"; return GAD_ERR_ARG; }
     // the kernels index rowptr, col and the per-node arrays with the caller's values: check the whole CSR here, on the host
     if (g->nnz < 0 || g->rowptr[0] != 0) { err = "rowptr must start at 0 and nnz must not be negative"; return GAD_ERR_ARG; }
-    int64_t longest = 0;
-    if (int rc = check_rows(g, longest, err)) return rc;
-    p.packed = walks_pack(g->nnz, longest);
+    int64_t lengths = 0;
+    if (int rc = check_rows(g, lengths, err)) return rc;
+    p.packed = walks_pack(g->nnz, lengths);
     if (g->rowptr[g->n] != g->nnz) { err = "rowptr[n] differs from nnz"; return GAD_ERR_ARG; }
     if (columns) { int rc = check_columns(g, err); if (rc != GAD_OK) return rc; }
     for (int32_t k = 0; k < K; ++k)
@@ -749,9 +744,9 @@ int augment_in_form(bool general, const gad_csr* g, int32_t K, const int64_t* co
 
 // For tests: which form the walks of a graph take, from its row pointers.
 bool augment_packs(const gad_csr* g) {
-    int64_t longest = 0;
+    int64_t lengths = 0;
     std::string err;
-    return check_rows(g, longest, err) == GAD_OK && walks_pack(g->nnz, longest);
+    return check_rows(g, lengths, err) == GAD_OK && walks_pack(g->nnz, lengths);
 }
 
 }  // namespace gad

@@ -80,7 +80,9 @@ typedef struct {
                            * 1: reduced-precision operands with fp32 accumulation: one TF32 pass on the tensor      *
                            *    cores, and the aggregation gathers a bfloat16 copy of its operand (tolerance 5e-2)  */
     int32_t zeta_mode;    /* 0: aggregate distance term; 1: literal pairwise form, O(n'^2 F_0) per subgraph, the  *
-                           * squared distances from a Gram matrix on the tensor cores (any subgraph size; with   *
+                           * squared distances from a Gram matrix on the tensor cores (any subgraph size; every     *
+                           * row times a power of two as two fp16 halves, 22 significant bits of its larger values, *
+                           * fp32 sums, pairs close to each other from the differences in fp32; with              *
                            * flag bit 0 or 4 from the differences on the FP32 ALUs, GAD_ERR_UNSUPPORTED when a    *
                            * subgraph has more than 32768 rows); 2: the aggregate                               *
                            * term with the sum over layers of the variance equation (Section 3.4.1) kept: the  *

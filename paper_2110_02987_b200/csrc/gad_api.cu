@@ -623,8 +623,8 @@ int zeta_pass(gad_ctx* ctx, cudaStream_t s) {
     return GAD_OK;
 }
 
-// sums: where to leave the chunk sums of the first layer's weight gradient, for the update to add up; null: they are added up here.
-int backward_pass(gad_ctx* ctx, cudaStream_t ss, ChunkSums* sums) {
+// first_sums: where to leave the chunk sums of the first layer's weight gradient, for the update to add up; null: they are added up here.
+int backward_pass(gad_ctx* ctx, cudaStream_t ss, ChunkSums* first_sums) {
     const Plan& p = ctx->p;
     float* G1 = ctx->at<float>(p.o_G1);
     float* G2 = ctx->at<float>(p.o_G2);
@@ -692,8 +692,8 @@ int backward_pass(gad_ctx* ctx, cudaStream_t ss, ChunkSums* sums) {
                             : launch_gemm_tn_simt(agg_first ? ctx->at<float>(p.o_P[l]) : ctx->H(l), y.ldi, y.fi, agg_first ? G1 : G2, y.ldo,
                                                   y.fo, dw_chunks, ndw, p.simt[(size_t)l] != 0, ctx->at<float>(p.o_dw_partial), y.ldw, ctx->stream);
             if (e != cudaSuccess) return e;
-            if (l == 0 && sums) {
-                *sums = ChunkSums{y.w_int / 4, (long long)y.fi * y.ldw / 4, ctx->at<float4>(p.o_dw_partial), (long long)y.fi * y.ldw / 4, ctx->at<int32_t>(p.dw[l].o_ptr)};
+            if (l == 0 && first_sums) {
+                *first_sums = ChunkSums{y.w_int / 4, (long long)y.fi * y.ldw / 4, ctx->at<float4>(p.o_dw_partial), (long long)y.fi * y.ldw / 4, ctx->at<int32_t>(p.dw[l].o_ptr)};
                 return cudaSuccess;
             }
             return launch_reduce_chunks(ctx->at<float>(p.o_dw_partial), (int64_t)y.fi * y.ldw, ctx->at<int32_t>(p.dw[l].o_ptr), p.K, grads, p.pstride,

@@ -12,22 +12,21 @@
 // representable in TF32), and lo = x - hi rounded to TF32, and the product is accumulated as A_hi B_hi + A_hi B_lo + A_lo B_hi
 // in fp32 (the dropped A_lo B_lo term and the rounding of lo are ~2^-20 relative).  B is split once per epoch by a small kernel
 // (hi = x rounded).  For A the tile as loaded is its own hi part, because the tensor core ignores the low 13 mantissa bits
-// of an fp32 operand (hi = x truncated); eight warps write only the lo tile beside it.  With passes = 1 only A B is issued
-// on the unsplit operands (TF32 operand precision).
+// of an fp32 operand (hi = x truncated); eight warps write lo: beside the loaded tile in shared memory, or both parts into tensor memory, from
+// which the MMAs then read A (tiles of up to 128 columns).  With passes = 1 only A B is issued on the unsplit operands (TF32 operand precision).
 //
-// What bounds it is shared-memory bandwidth (128 B per clock and SM) under the tensor pipe, then HBM.  Per 32 values of the
-// reduction and 256 output columns the tensor pipe needs 1536 cycles.  One CTA alone moves 256 KB meanwhile (operand reads 144,
-// TMA 80, split 32) and another 32 for a drain that turns its tiles through shared memory: 2250 cycles.  Therefore
+// What bounds it is the tensor pipe at 256 x 256, the drain for short reductions, the chain TMA -> split -> MMA -> drain on small launches.  Per 32 values of
+// the reduction and 256 output columns the tensor pipe needs 1536 cycles; shared memory gives 128 B per clock and SM.  One CTA alone, A split there, moves
+// 256 KB meanwhile (operand reads 144, TMA 80, split 32) and another 32 for a drain that turns its tiles through shared memory: 2250 cycles.  Therefore
 //   - the CTAs of a cluster of two work as a pair (cta_group::2): each holds 128 rows of A and half of the B rows, and one
 //     MMA of M = 256 reads 4 KB of each from either CTA: 96 KB of operand reads and 48 of TMA instead of 144 and 80;
 //   - B stays in shared memory for all tiles of a CTA where it fits beside the ring (up to 256 columns x 128 values);
 //   - the drain reads tensor memory in the 16 x 256-bit shape, in which four lanes hold 32 consecutive bytes of a row: whole
 //     sectors go to global memory straight from the registers;
-//   - the ring of loaded tiles is separate from the two lo tiles, so that most of the space holds loads in flight (short
-//     reductions are a chain of TMA latency, split and MMA).
+//   - the ring of loaded tiles is separate from the split ones (two or four lo tiles, or four slots of tensor memory), so that most of the
+//     space holds loads in flight (short reductions are a chain of TMA latency, split and MMA).
 // Before this kernel (one CTA per tile, B streamed, drain through shared memory) and with it, event times inside an epoch under the power cap,
-// 525 000 rows: 100 -> 256 300 -> 187 us, 256 -> 256 346 -> 305 us (tensor pipe active 72 - 77 % of the time), 256 -> 47 181 -> 153 us; 110 000 rows,
-// 128 -> 128: 48 -> 33 us; 2843 rows, 1433 -> 128, on its own: 40 -> 27 us.
+// 525 000 rows: 100 -> 256 300 -> 168 us, 256 -> 256 346 -> 290, 256 -> 47 181 -> 153; 110 000 rows, 128 -> 128: 48 -> 33 us (27 through tensor memory).
 // Roles of a CTA: warp 0 issues TMA loads, warps 2-9 split the A tile and tell the pair's leader, warp 1 of the leader
 // issues the MMAs, warps 10-17 drain.  Every mbarrier wait is bounded: on a time-out the CTA raises an error word, stops, meets its
 // peer at the cluster barrier, frees its tensor memory and returns.
@@ -243,7 +242,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // ---------------- A split: lo = x - (x as the tensor core reads it); the pair's leader is told ----------------
         // With two lo tiles (wide outputs: the tensor pipe sets the pace) all warps share a step.  With four they form four groups
         // that take turns: what a step costs is then mostly waiting - for the barriers, the proxy fence and the arrival - so four
-        // steps are in hand at a time.  (A group's wait for a ring stage is unambiguous because nlo <= nst: once its own previous
+        // steps are in hand at a time.  (Through tensor memory a group has a warp for every quarter of the lanes, so that there are two.)  (A group's wait for a ring stage is unambiguous because nlo <= nst: once its own previous
         // step has been multiplied, so has the step before in that stage.)
         const int gw = SPLIT_WARPS / groups, group = (warp - 2) / gw, tt = threadIdx.x - 64 - 32 * gw * group;
         constexpr bool leaves_bits = DRAIN == kPlain || DRAIN == kBf16;

@@ -78,7 +78,7 @@ EncodeTiledFn encode_fn() {
 
 }  // namespace
 
-// fp32 tensor [outer (z)] x [rows (y)] x [inner (x)], box = 32 floats x box_rows x 1, zero fill outside.  K-major
+// fp32 tensor [outer (z)] x [rows (y)] x [inner (x)], box = 32 floats (`half`: 64 fp16 values) x box_rows x 1, zero fill outside.  K-major
 // operand tiles use the 128-byte swizzle of 16-byte units; MN-major TF32 tiles need the 128-byte swizzle of
 // 32-byte units (the only MN-major layout the tensor cores accept for 32-bit operands).
 bool tc_make_map(void* out_map, const void* base, uint64_t inner, uint64_t rows, uint64_t outer, uint64_t row_stride_bytes,

@@ -14,6 +14,7 @@
 // output tile) drains while the next one is multiplied.
 // One timeline of an epoch each, both operands split in shared memory and now: 525 000 rows, 256 x 256 259 -> 239 us, 256 x 47 123 -> 117, 100 x 256 216 -> 167;
 // 94 000 rows in 50 subgraphs, 128 x 128 35.7 -> 27.9, 500 x 128 94.5 -> 75; 110 000 rows, 128 x 128 34.5 -> 29.2.
+// (Single CTAs: a thread spills 4 bytes at the 96 registers that 18 warps leave it.)
 #include <cuda.h>
 
 #include <algorithm>

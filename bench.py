@@ -32,9 +32,9 @@ UNIT = "epochs/s"
 # capture summarised under profiles/; keyed by (workload, profile entry).  A kernel changed since its capture
 # has no entry (reported as null).
 NCU_TRAFFIC = {
-    # spmm_items_kernel<2,1,...> (14.37 GB read + 2.62 GB written) + spmm_finish_kernel (2 MB), profiles/spmm_c4_dram.md
-    ("c4", "spmm_fwd_l1"): 17.00e9,
-    ("c4", "spmm_bwd_l1"): 17.03e9,
+    # spmm_items_kernel<2,1,...> (14.10 GB read + 2.60 GB written) + spmm_finish_kernel (2 MB), profiles/spmm_c4_dram.md
+    ("c4", "spmm_fwd_l1"): 16.69e9,
+    ("c4", "spmm_bwd_l1"): 16.85e9,
     # spmm_items_kernel (76.8 MB read + 32.8 MB written) + spmm_finish_kernel (14.9 MB read), profiles/spmm_items_c2.md
     ("c2", "spmm_fwd_l0"): 124.6e6,
 }
@@ -688,7 +688,7 @@ def main():
                               "note": "operand rows the gather moves on the chip (4 F bytes per stored entry) / time; this kernel's measured "
                                       "ceilings at F = 256 (bench.py --micro gather): 23.3 TB/s with the rows L1-resident, 20.5 TB/s "
                                       "L2-resident; the SM's L1 / shared-memory data stage moves 128 B per clock (37 TB/s at 1.965 GHz); under ncu the L2 "
-                                      "runs at 89 % of its peak throughput on c3 and at 75 % on a 1 M-row graph without locality"}
+                                      "runs at 91 % of its peak throughput on c3 and at 75 % on a 1 M-row graph without locality"}
     kernels = [{"name": e["name"], "ms_per_step": e["total_ms"] / prof_steps, "share": e["total_ms"] / total_prof,
                 "GBps": e["bytes_per_launch"] * e["launches"] / (e["total_ms"] * 1e-3) / 1e9 if e["total_ms"] > 0 else None,
                 "TFLOPs": e["flops_per_launch"] * e["launches"] / (e["total_ms"] * 1e-3) / 1e12 if e["total_ms"] > 0 else None}

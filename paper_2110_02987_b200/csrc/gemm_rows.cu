@@ -516,7 +516,8 @@ static int spread_columns(int bn, int n_cols, int npairs) {
     return bn;
 }
 // The transform back through a layer, in one pass or three, and every transform in one pass, whose MMAs cost little beside reading A again (256 -> 256 over
-// 210 000 rows 86 us in tiles of 256 columns, 104 of 128): as wide as the layer, up to 256, so that a masked drain can sum the columns.
+// 210 000 rows 86 us in tiles of 256 columns, 104 of 128): as wide as the layer, up to 256, so that a masked drain can sum the columns.  (So are the ways back
+// that sum none, without a mask or of more than 256 columns; narrower tiles have not been measured there.)
 int tc_rows_bn_whole(int n_cols, int npairs) {
     return spread_columns(n_cols <= 32 ? 32 : n_cols <= 64 ? 64 : n_cols <= 128 ? 128 : 256, n_cols, npairs);
 }
